@@ -74,7 +74,8 @@ struct __align__(64) GtaParams {
   int B, T, tsteps;          // tsteps = ceil(T / 64) K steps per example
   int total_items;
   const float* clip;         // [B] R_i (scale mode)
-  uint32_t noise_k0, noise_k1, noise_step;   // Gaussian stream of the fused noise (per-layer id)
+  NoiseKeys noise_keys;      // Gaussian stream of the fused noise (per-layer id)
+  uint32_t noise_step;
   const uint32_t* step_dev;  // optional device counter added to noise_step
   float noise_scale;
   float* sq_partials;        // [B][n_per] (square-sum mode)
@@ -412,7 +413,7 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
         const bool vec_ok = ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0);
         // fused Gaussian mechanism (Eq. 3): only on the final destination, never on a K-split plane
         const bool noisy = (L.noise_amp >= 0.f) && (L.nsplit == 1);
-        const NoiseKey nkey{P.noise_k0, P.noise_k1, L.tensor_id, effective_step(P.noise_step, P.step_dev)};
+        const uint32_t tensor_id = L.tensor_id, step = effective_step(P.noise_step, P.step_dev);
 #pragma unroll 1
         for (int c = c_lo; c < c_hi; ++c) {
           uint32_t r[32];
@@ -447,7 +448,7 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
                 for (int qd = 0; qd < 8; ++qd) {
                   if (col0 + 4 * qd < L.N) {
                     float z[4];
-                    normals4((j0 >> 2) + qd, nkey, z);
+                    normals4((j0 >> 2) + qd, P.noise_keys, tensor_id, step, z);
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
                       v[4 * qd + e] = noised(v[4 * qd + e], z[e], L.noise_amp, P.noise_scale);
@@ -681,7 +682,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
       items += L.tiles_m * L.tiles_n * nsplit;
     }
     if (noise) {
-      P.noise_k0 = uint32_t(noise->seed); P.noise_k1 = uint32_t(noise->seed >> 32);
+      P.noise_keys = expand_noise_keys(noise->seed);
       P.noise_step = noise->step; P.noise_scale = noise->scale;
       P.step_dev = g_step_dev;
     }

@@ -16,8 +16,9 @@ namespace {
 template <bool kFill>
 __global__ void __launch_bounds__(256)
 add_noise_kernel(float* __restrict__ out, long long n, int cols, long long ld, float amp,
-                 float scale, NoiseKey key, const uint32_t* __restrict__ step_dev, long long q0) {
-  key.step = effective_step(key.step, step_dev);
+                 float scale, const __grid_constant__ NoiseKeys keys, uint32_t tensor_id, uint32_t step,
+                 const uint32_t* __restrict__ step_dev, long long q0) {
+  step = effective_step(step, step_dev);
   const long long nq = (n + 3) >> 2;
   const bool flat = (ld == cols);
   // 16-byte accesses only on a 16-byte aligned base (the fused entry points accept any fp32
@@ -26,7 +27,7 @@ add_noise_kernel(float* __restrict__ out, long long n, int cols, long long ld, f
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < nq;
        q += (long long)gridDim.x * blockDim.x) {
     float z[4];
-    normals4((unsigned long long)(q0 + q), key, z);       // q0: first counter of a slice
+    normals4((unsigned long long)(q0 + q), keys, tensor_id, step, z);       // q0: first counter of a slice
     const long long j = q << 2;
     if (vec && j + 3 < n) {
       float4 v = kFill ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<float4*>(out + j);
@@ -46,21 +47,29 @@ add_noise_kernel(float* __restrict__ out, long long n, int cols, long long ld, f
 }
 
 // Exhaustive error scan of the fp32 Box-Muller factors.  k runs over all 2^24 values of the
-// 24-bit integer that feeds the factor.  out[0] = max relative error of r = sqrt(-2 ln u1) over
-// the inputs with r^2 <= t_max, out[1] = max absolute error of cos / sin(2 pi u2), out[2] = the
-// largest r seen, all against float64; out[3] = the r^2 threshold compiled into box_muller.
+// 24-bit integer that feeds the factor.  out[0] = max relative error of r = sqrt(-2 ln u1) (the
+// unrounded rh + rl that multiplies the direction) over the inputs with r^2 <= t_max, out[1] = max
+// absolute error of cos / sin(2 pi u2), out[2] = the largest r seen, all against float64;
+// out[3] = the r^2 threshold compiled into the generator.
 __global__ void noise_error_scan_kernel(float t_max, double* out) {
   double er = 0.0, ed = 0.0, rmax = 0.0;
   for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < (1u << 24); k += gridDim.x * blockDim.x) {
-    const float t = bm_t_f32(k);
+    float t, t2, h, l, c, s, unused;
+    F2 rh, rl, cc, ss;
+    bm_radius(k << 8, k << 8, 0u, 0u, t, t2, rh, rl);
     if (t <= t_max) {
-      const double r32 = (double)__fsqrt_rn(t);
+      unpack(rh, h, unused);
+      unpack(rl, l, unused);
+      const double r32 = (double)h + (double)l;
       const double r64 = sqrt(-2.0 * log(double(k + 1u) * 5.9604644775390625e-08));
       if (r64 > 0.0) er = fmax(er, fabs(r32 - r64) / r64);
       rmax = fmax(rmax, r64);
     }
-    float s, c;
-    bm_dir_f32(k, s, c);
+    const uint32_t v = (k << 8) + 0x20000000u;
+    bm_direction(v, v, cc, ss);
+    unpack(cc, c, unused);
+    unpack(ss, s, unused);
+    if (v & 0x80000000u) { c = -c; s = -s; }
     double s64, c64;
     sincospi(double(k) * 1.1920928955078125e-07, &s64, &c64);
     ed = fmax(ed, fmax(fabs((double)s - s64), fabs((double)c - c64)));
@@ -93,7 +102,7 @@ dp_status launch_add_noise(float* out, long long rows, int cols, long long ld, b
   // Fill mode is meant to run beside another kernel (it depends on no gradient): four blocks
   // per SM leave half of every SM's thread slots free for it.
   const int grid = (int)std::min<long long>(want, (long long)sm_count() * (fill ? 4 : 16));
-  const NoiseKey key{uint32_t(seed), uint32_t(seed >> 32), tensor_id, step};
+  const NoiseKeys keys = expand_noise_keys(seed);
   if (fill && first_use_on_this_device(reinterpret_cast<const void*>(&launch_add_noise))) {
     // same shared-memory carve-out as the TMA kernels, so that both can be resident on one SM
     DP_CUDA_OK(cudaFuncSetAttribute(add_noise_kernel<true>,
@@ -101,9 +110,11 @@ dp_status launch_add_noise(float* out, long long rows, int cols, long long ld, b
                                     cudaSharedmemCarveoutMaxShared));
   }
   if (fill)
-    add_noise_kernel<true><<<grid, 256, 0, st>>>(out, n, cols, ld, amp, scale, key, g_step_dev, first_quad);
+    add_noise_kernel<true><<<grid, 256, 0, st>>>(out, n, cols, ld, amp, scale, keys, tensor_id, step,
+                                             g_step_dev, first_quad);
   else
-    add_noise_kernel<false><<<grid, 256, 0, st>>>(out, n, cols, ld, amp, scale, key, g_step_dev, first_quad);
+    add_noise_kernel<false><<<grid, 256, 0, st>>>(out, n, cols, ld, amp, scale, keys, tensor_id, step,
+                                             g_step_dev, first_quad);
   DP_LAUNCH_OK();
   return DP_OK;
 }
