@@ -89,10 +89,12 @@ struct Item {
   int layer, tm, tn, k0, k1, split, example;
 };
 
+// `l` is the caller's running layer index: a role's items ascend, so the search goes on from the layer
+// of its previous item.  (From layer 0 it was a chain of up to 97 dependent constant loads, a line
+// each, in every role and for every tile.)
 template <bool kSqsum>
-__device__ __forceinline__ Item decode_item(const GtaParams& P, int item) {
+__device__ __forceinline__ Item decode_item(const GtaParams& P, int item, int& l) {
   Item it;
-  int l = 0;
   while (l + 1 < P.n_layers && item >= P.layer[l + 1].item_begin) ++l;
   const GtaLayer& L = P.layer[l];
   int local = item - L.item_begin;
@@ -110,26 +112,6 @@ __device__ __forceinline__ Item decode_item(const GtaParams& P, int item) {
   return it;
 }
 
-// Partial in-register transpose of a 32 x 32 tile held one row per lane (v[c] = column c): the
-// upper three lane bits are exchanged with the upper three register bits (three butterfly stages
-// of 16 exchanges).  Afterwards lane l holds, in v[4i .. 4i+3], columns 4(l>>2) .. +3 of row
-// 4i + (l&3): four consecutive columns per register quad, and the 32 lanes of quad i cover rows
-// 4i .. 4i+3 completely -- one float4 store per quad writes four whole 128-byte lines.
-__device__ __forceinline__ void warp_transpose_quads(float (&v)[32], int lane) {
-#pragma unroll
-  for (int d = 16; d >= 4; d >>= 1) {
-    const bool up = (lane & d) != 0;
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      if ((j & d) == 0) {
-        const float send = up ? v[j] : v[j + d];
-        const float recv = __shfl_xor_sync(0xffffffffu, send, d);
-        if (up) v[j] = recv; else v[j + d] = recv;
-      }
-    }
-  }
-}
-
 template <bool kScale, bool kSqsum, bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_gta_kernel(const __grid_constant__ GtaParams P) {
@@ -137,7 +119,6 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
   constexpr int kStages = Geo<kPair>::kStages;
   constexpr int kStageBytes = Geo<kPair>::kStageBytes;
   constexpr int kTileM = Geo<kPair>::kTileM;
-  constexpr int kPeers = kPair ? 2 : 1;
   // pair: rank 0 issues the MMAs; both CTAs walk the same list of work items
   const uint32_t rank = kPair ? ptx::cluster_ctarank() : 0u;
   const int first_item = kPair ? int(blockIdx.x >> 1) : int(blockIdx.x);
@@ -172,7 +153,7 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
     }
     for (int b = 0; b < 2; ++b) {
       ptx::mbar_init(&acc_full[b], 1);
-      ptx::mbar_init(&acc_empty[b], kEpiWarps * kPeers);    // epilogue warps of both CTAs
+      ptx::mbar_init(&acc_empty[b], kEpiWarps);    // this CTA's epilogue warps (pair: + 4 bytes from each of rank 1's)
     }
     ptx::mbar_init(mma_done, 1);
     for (int b = 0; b < 4; ++b) ptx::mbar_init(&red_bar[b], kEpiWarps);
@@ -202,9 +183,10 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
       const uint32_t my_bytes = is_a ? uint32_t(Geo<kPair>::kABytes) : uint32_t(kGBytes);
       const int nbox = is_a ? kBoxesA : kBoxes;
       uint32_t stage = 0, phase = 0, issued = 0;
+      int lay = 0;
       bool ok = true;
       for (int item = first_item; item < P.total_items && ok; item += item_stride) {
-        const Item it = decode_item<kSqsum>(P, item);
+        const Item it = decode_item<kSqsum>(P, item, lay);
         const uint64_t tm = reinterpret_cast<uint64_t>(is_a ? &P.tmA[it.layer] : &P.tmG[it.layer]);
         // first column of this CTA's part of the tile: its G rows, or its share of the A columns
         const int c0 = is_a ? it.tn * kBN + int(rank) * Geo<kPair>::kAColsPerCta
@@ -239,9 +221,10 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
       const uint32_t desc_lo0 = uint32_t(dbase) | ((tiles_a >> 4) & 0x3FFF);
       const uint32_t go_a = kScale ? ready_a : full_a;
       uint32_t stage = 0, phase = 0, n_item = 0;
+      int lay = 0;
       bool ok = true;
       for (int item = first_item; item < P.total_items && ok; item += item_stride, ++n_item) {
-        const Item it = decode_item<kSqsum>(P, item);
+        const Item it = decode_item<kSqsum>(P, item, lay);
         const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
         if (!(kPair ? ptx::mbar_wait_cluster(&acc_empty[buf], acc_phase ^ 1, abort_flag, P.wait_limit)
                     : ptx::mbar_wait(&acc_empty[buf], acc_phase ^ 1, abort_flag, P.wait_limit))) { ok = false; break; }
@@ -293,9 +276,10 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
       const uint32_t ready_remote = kPair ? ptx::mapa_u32(ready_a, 0) : 0u;
       const uint32_t sink_remote = kPair ? ptx::mapa_u32(ptx::smem_u32(sink), 0) : 0u;
       uint32_t cnt = 0;
+      int lay = 0;
       bool ok = true;
       for (int item = first_item; item < P.total_items && ok; item += item_stride) {
-        const Item it = decode_item<kSqsum>(P, item);
+        const Item it = decode_item<kSqsum>(P, item, lay);
         const bool scale_here = P.clip && !P.layer[it.layer].prescaled;
         // first K step of this item that belongs to this warp
         int ks = it.k0 + int((uint32_t(sw) + kScalerWarps - cnt % kScalerWarps) % kScalerWarps);
@@ -361,10 +345,26 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
     // this warp's 32-column chunks: the 8 chunks are dealt to the kEpiWarps/4 column groups
     constexpr int kGroups = kEpiWarps / 4;
     const int c_lo = ((ew >> 2) * (kBN / 32)) / kGroups, c_hi = (((ew >> 2) + 1) * (kBN / 32)) / kGroups;
+    // Frees an accumulator once this warp has read its part of it.  Across the pair it signals like
+    // the scaler warps do, not with mbarrier.arrive.release.cluster: that arrive waits until every
+    // store the warp has issued is acknowledged by the L2, thousands of cycles when all SMs write.
+    const uint32_t acc_empty_a = ptx::smem_u32(acc_empty);
+    const uint32_t acc_empty_remote = kPair ? ptx::mapa_u32(acc_empty_a, 0) : 0u;
+    const uint32_t sink_remote = kPair ? ptx::mapa_u32(ptx::smem_u32(sink), 0) : 0u;
+    auto free_acc = [&](uint32_t buf) {
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (!kPair) ptx::mbar_arrive(&acc_empty[buf]);
+        else if (rank == 0) ptx::mbar_arrive_expect_tx_a(acc_empty_a + 8 * buf, 4);
+        else ptx::st_async_signal_a(acc_empty_remote + 8 * buf, sink_remote);
+      }
+    };
     uint32_t n_item = 0;
+    int lay = 0;
     bool ok = true;
     for (int item = first_item; item < P.total_items && ok; item += item_stride, ++n_item) {
-      const Item it = decode_item<kSqsum>(P, item);
+      const Item it = decode_item<kSqsum>(P, item, lay);
       const GtaLayer& L = P.layer[it.layer];
       const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
       if (!ptx::mbar_wait_relaxed(&acc_full[buf], acc_phase, abort_flag, P.wait_limit)) { ok = false; break; }
@@ -381,12 +381,7 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
 #pragma unroll
           for (int j = 0; j < 32; ++j) { const float v = __uint_as_float(r[j]); acc = fmaf(v, v, acc); }
         }
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) {
-          if (kPair) ptx::mbar_arrive_cluster(&acc_empty[buf], 0);
-          else ptx::mbar_arrive(&acc_empty[buf]);
-        }
+        free_acc(buf);
         // the warps' sums meet through an mbarrier with a bounded wait (no blocking named
         // barrier: a warp that gave up never arrives); four slots, since the other warps can run
         // at most two items ahead of a waiting warp 0 (they need its acc_empty arrivals)
@@ -410,83 +405,71 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
         float beta;
         if (L.nsplit == 1) { dst = L.out; ld = L.ldo; beta = L.beta; }
         else { dst = L.partial + size_t(it.split) * size_t(L.M) * L.N; ld = L.N; beta = 0.f; }
-        const bool vec_ok = ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0);
+        // 32-byte (8 columns) or 16-byte accesses where the pitch and the base allow them
+        const bool vec8 = ((ld & 7) == 0) && ((reinterpret_cast<uintptr_t>(dst) & 31) == 0);
+        const bool vec4 = ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0);
         // fused Gaussian mechanism (Eq. 3): only on the final destination, never on a K-split plane
         const bool noisy = (L.noise_amp >= 0.f) && (L.nsplit == 1);
+        const float amp = L.noise_amp;
         const uint32_t tensor_id = L.tensor_id, step = effective_step(P.noise_step, P.step_dev);
 #pragma unroll 1
         for (int c = c_lo; c < c_hi; ++c) {
           uint32_t r[32];
           ptx::tmem_ld_32x32b_x32(t0 + c * 32, r);
           ptx::tmem_ld_wait();
+          // the accumulator is free as soon as its last part is in registers: the next tile's MMAs
+          // do not wait for this warp's noise and stores
+          if (c + 1 == c_hi) free_acc(buf);
           const int col0 = it.tn * kBN + c * 32;
-          const int row_base = row - lane;                   // first row of this warp's 32
-          if (row_base < L.M && col0 < L.N) {                // the same for the whole warp
-            float v[32];
+          if (row < L.M) {
+            // One row per lane, eight columns at a time: two Philox counters (N is a multiple of 4
+            // where noise is fused, so a counter never straddles rows) and one 32-byte store, a whole
+            // sector, per lane -- no in-register transpose (48 shuffles and 96 selects per chunk).
+            // Together with the early release and the running layer search: 49 GPT-2-small layers at
+            // B = 3, T = 77 (six K steps per tile) 480 -> 301 us with noise, 276 -> 215 us without;
+            // 72 GPT-2-medium layers at B = 16, T = 128: 1161 -> 973 us; B = 64, T = 256: 1.19 -> 1.13 ms.
+            float* o = dst + size_t(row) * ld + col0;
+            const unsigned long long q0 = ((unsigned long long)row * L.N + col0) >> 2;   // first counter
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-            if (row < L.M) {
-              const bool full32 = col0 + 32 <= L.N;
-              if (beta != 0.f) {
-                const float* o = dst + size_t(row) * ld + col0;
-                if (vec_ok && full32) {
+            for (int g = 0; g < 4; ++g) {
+              const int left = L.N - col0 - 8 * g;             // columns of this row from here on
+              if (left > 0) {
+                float v[8];
 #pragma unroll
-                  for (int j = 0; j < 8; ++j) {
-                    const float4 old = *reinterpret_cast<const float4*>(o + 4 * j);
-                    v[4 * j] += old.x; v[4 * j + 1] += old.y; v[4 * j + 2] += old.z; v[4 * j + 3] += old.w;
+                for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(r[8 * g + e]);
+                float* og = o + 8 * g;
+                if (beta != 0.f) {
+                  if (vec4 && left >= 8) {
+                    const float4 a = *reinterpret_cast<const float4*>(og), b = *reinterpret_cast<const float4*>(og + 4);
+                    v[0] += a.x; v[1] += a.y; v[2] += a.z; v[3] += a.w;
+                    v[4] += b.x; v[5] += b.y; v[6] += b.z; v[7] += b.w;
+                  } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) if (e < left) v[e] += og[e];
                   }
+                }
+                if (noisy) {
+#pragma unroll
+                  for (int h = 0; h < 2; ++h) {
+                    float z[4];
+                    normals4(q0 + 2 * g + h, P.noise_keys, tensor_id, step, z);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) v[4 * h + e] = noised(v[4 * h + e], z[e], amp, P.noise_scale);
+                  }
+                }
+                if (vec8 && left >= 8) {
+                  ptx::st_global_v8(og, v);
+                } else if (vec4 && left >= 8) {
+                  __stcs(reinterpret_cast<float4*>(og), make_float4(v[0], v[1], v[2], v[3]));
+                  __stcs(reinterpret_cast<float4*>(og + 4), make_float4(v[4], v[5], v[6], v[7]));
                 } else {
 #pragma unroll
-                  for (int j = 0; j < 32; ++j) if (col0 + j < L.N) v[j] += o[j];
+                  for (int e = 0; e < 8; ++e) if (e < left) og[e] = v[e];
                 }
-              }
-              if (noisy) {
-                const unsigned long long j0 = (unsigned long long)row * L.N + col0;   // stream index
-                // N is a multiple of 4 here (the host fuses only such layers), so the Philox
-                // counters of this thread's 32 columns never straddle a row
-#pragma unroll
-                for (int qd = 0; qd < 8; ++qd) {
-                  if (col0 + 4 * qd < L.N) {
-                    float z[4];
-                    normals4((j0 >> 2) + qd, P.noise_keys, tensor_id, step, z);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                      v[4 * qd + e] = noised(v[4 * qd + e], z[e], L.noise_amp, P.noise_scale);
-                  }
-                }
-              }
-            }
-            // Stores by whole lines: with one row per lane a warp store would touch 32 different
-            // 128-byte lines, 16 bytes each -- measured, those write requests took a fifth of the
-            // kernel's throughput away from the operand loads.  After the partial transpose every
-            // float4 store of the warp writes four complete rows of this 32-column chunk.
-            warp_transpose_quads(v, lane);
-            const int colq = col0 + 4 * (lane >> 2);         // this lane's four columns
-            const int rsub = lane & 3;
-            if (vec_ok && col0 + 32 <= L.N) {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const int rr = row_base + 4 * i + rsub;
-                if (rr < L.M)
-                  __stcs(reinterpret_cast<float4*>(dst + size_t(rr) * ld + colq),
-                         make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
-              }
-            } else {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const int rr = row_base + 4 * i + rsub;
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                  if (rr < L.M && colq + e < L.N) dst[size_t(rr) * ld + colq + e] = v[4 * i + e];
               }
             }
           }
-        }
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) {
-          if (kPair) ptx::mbar_arrive_cluster(&acc_empty[buf], 0);
-          else ptx::mbar_arrive(&acc_empty[buf]);
+          __syncwarp();                                        // the TMEM load is a warp operation
         }
       }
     }
