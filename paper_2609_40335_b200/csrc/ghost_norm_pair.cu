@@ -63,9 +63,10 @@ struct Item {
   int layer, example, ti, tj, a0, a1, g0, g1, pidx;
 };
 
-__device__ __forceinline__ Item decode_item(const PairParams& P, int item) {
+// `l` is the caller's running layer index: a role's items ascend, so the search goes on from the layer
+// of its previous item instead of walking the list (a constant-memory line per layer) every time.
+__device__ __forceinline__ Item decode_item(const PairParams& P, int item, int& l) {
   Item it;
-  int l = 0;
   while (l + 1 < P.n_layers && item >= P.layer[l + 1].item_begin) ++l;
   const GhostLayerPlan& L = P.layer[l];
   const int local = item - L.item_begin;
@@ -141,9 +142,10 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
     // ------------------------------------------------------------- TMA producer
     if (lane == 0) {
       uint32_t stage = 0, phase = 0, issued = 0;
+      int lay = 0;
       bool ok = true;
       for (int item = first_item; item < P.total_items && ok; item += item_stride) {
-        const Item it = decode_item(P, item);
+        const Item it = decode_item(P, item, lay);
         const bool diag = it.ti == it.tj;
         const uint32_t bytes = diag ? kTileBytes : kStageBytes;
         const int row_i = it.ti * kTile2 + int(rank) * kRows;     // this CTA's rows of block I
@@ -174,9 +176,10 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
       constexpr uint32_t idesc = ptx::idesc_bf16_f32(kTile2, kTile2, 0, 0);
       constexpr uint64_t dbase = ptx::smem_desc_base(16, 1024, ptx::SWIZZLE_128B);   // K-major
       uint32_t stage = 0, phase = 0, n_item = 0;
+      int lay = 0;
       bool ok = true;
       for (int item = first_item; item < P.total_items && ok; item += item_stride, ++n_item) {
-        const Item it = decode_item(P, item);
+        const Item it = decode_item(P, item, lay);
         const bool diag = it.ti == it.tj;
         const uint32_t ph = n_item & 1;
         for (int pass = 0; pass < 2 && ok; ++pass) {
@@ -219,9 +222,10 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
       const uint32_t ready_a = ptx::smem_u32(ready), sink_a = ptx::smem_u32(sink);
       const uint32_t ready_remote = ptx::mapa_u32(ready_a, 0), sink_remote = ptx::mapa_u32(sink_a, 0);
       uint32_t stage = 0, phase = 0;
+      int lay = 0;
       bool ok = true;
       for (int item = first_item; item < P.total_items && ok; item += item_stride) {
-        const Item it = decode_item(P, item);
+        const Item it = decode_item(P, item, lay);
         const int nsteps = (it.a1 - it.a0) + (it.g1 - it.g0);
         for (int k = 0; k < nsteps; ++k) {
           if (!ptx::mbar_wait(&full[stage], phase, abort_flag, P.wait_limit)) { ok = false; break; }
@@ -243,9 +247,10 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
     const uint32_t t_sa = tmem_base + (uint32_t(q * 32) << 16) + cg * kColsPerWarp;
     const uint32_t t_sg = t_sa + kTile2;
     uint32_t n_item = 0;
+    int lay = 0;
     bool ok = true;
     for (int item = first_item; item < P.total_items && ok; item += item_stride, ++n_item) {
-      const Item it = decode_item(P, item);
+      const Item it = decode_item(P, item, lay);
       const uint32_t ph = n_item & 1;
       // S_A -> registers, then the accumulator is free for the next item
       if (!ptx::mbar_wait_relaxed(sa_full, ph, abort_flag, P.wait_limit)) { ok = false; break; }

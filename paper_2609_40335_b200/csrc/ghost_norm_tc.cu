@@ -59,9 +59,10 @@ struct Item {
   int layer, example, ti, tj, a0, a1, g0, g1, pidx;
 };
 
-__device__ __forceinline__ Item decode_item(const GhostParams& P, int item) {
+// `l` is the caller's running layer index: a role's items ascend, so the search goes on from the layer
+// of its previous item instead of walking the list (a constant-memory line per layer) every time.
+__device__ __forceinline__ Item decode_item(const GhostParams& P, int item, int& l) {
   Item it;
-  int l = 0;
   while (l + 1 < P.n_layers && item >= P.layer[l + 1].item_begin) ++l;
   const GhostLayerPlan& L = P.layer[l];
   const int local = item - L.item_begin;
@@ -134,9 +135,10 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
     // ------------------------------------------------------------- TMA producer
     if (lane == 0) {
       uint32_t stage = 0, phase = 0, issued = 0;
+      int lay = 0;
       bool ok = true;
       for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x) {
-        const Item it = decode_item(P, item);
+        const Item it = decode_item(P, item, lay);
         const bool diag = !kDual && (kDiagOnly || (it.ti == it.tj));
         const uint32_t bytes = diag ? kTileBytes : kStageBytes;
         const int li = kDual ? 2 * it.layer : it.layer;
@@ -170,9 +172,10 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
       // K-major operand, 128-byte swizzle: 8-row groups are 1024 bytes apart
       constexpr uint64_t dbase = ptx::smem_desc_base(16, 1024, ptx::SWIZZLE_128B);
       uint32_t stage = 0, phase = 0, n_item = 0;
+      int lay = 0;
       bool ok = true;
       for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x, ++n_item) {
-        const Item it = decode_item(P, item);
+        const Item it = decode_item(P, item, lay);
         const bool diag = !kDual && (kDiagOnly || (it.ti == it.tj));
         const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
         if (!ptx::mbar_wait(&acc_empty[buf], acc_phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
@@ -209,9 +212,10 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
     const int q = warp & 3;                          // TMEM lane quarter this warp may read
     const int ew = warp - 2;
     uint32_t n_item = 0;
+    int lay = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x, ++n_item) {
-      const Item it = decode_item(P, item);
+      const Item it = decode_item(P, item, lay);
       const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
       if (!ptx::mbar_wait_relaxed(&acc_full[buf], acc_phase, abort_flag, P.wait_limit)) { ok = false; break; }
       ptx::tc_fence_after();
