@@ -7,7 +7,9 @@
 
 namespace dpg {
 
-constexpr int kGtaMaxLayers = 80;       // layers per launch (parameter-block limit)
+// Layers per launch: what fits the 32 764-byte parameter block (two tensor maps and 56 bytes per layer).
+// GPT-2 medium's 97 layers have to fit: a second launch cost a second partly filled last wave.
+constexpr int kGtaMaxLayers = 102;
 
 // Plain data: copied into kernel parameters.
 struct GtaLayer {
@@ -15,12 +17,8 @@ struct GtaLayer {
   float* partial;         // [nsplit][M][N] planes when it is
   long long ldo;
   int M, N;               // p, d
-  int tiles_m, tiles_n;   // 128 x 256 output tiles
-  int nsplit;
-  int ksteps_per_split;
   int item_begin;
   int col_begin;          // square-sum mode: first partial-sum column of this layer
-  float beta;
   int prescaled;          // 1: the clip factors were applied to this layer's narrow operand beforehand
   float noise_amp;        // sigma*C of the fused noise, negative = none
   uint32_t tensor_id;     // noise stream id of this output tensor

@@ -72,6 +72,8 @@ struct __align__(64) GtaParams {
   GtaLayer layer[kGtaMaxLayers];
   int n_layers;
   int B, T, tsteps;          // tsteps = ceil(T / 64) K steps per example
+  int nsplit, ksteps_per_split;   // K splits, the same for all layers of a call
+  float beta;
   int total_items;
   const float* clip;         // [B] R_i (scale mode)
   NoiseKeys noise_keys;      // Gaussian stream of the fused noise (per-layer id)
@@ -83,7 +85,7 @@ struct __align__(64) GtaParams {
   int* dev_status;
   long long wait_limit;      // cycles a barrier wait may take before the CTA gives up
 };
-static_assert(sizeof(GtaParams) <= 32000, "kernel parameter block too large");
+static_assert(sizeof(GtaParams) <= 32764, "kernel parameter block too large");
 
 struct Item {
   int layer, tm, tn, k0, k1, split, example;
@@ -92,22 +94,23 @@ struct Item {
 // `l` is the caller's running layer index: a role's items ascend, so the search goes on from the layer
 // of its previous item.  (From layer 0 it was a chain of up to 97 dependent constant loads, a line
 // each, in every role and for every tile.)
-template <bool kSqsum>
+template <bool kSqsum, int kTileM>
 __device__ __forceinline__ Item decode_item(const GtaParams& P, int item, int& l) {
   Item it;
   while (l + 1 < P.n_layers && item >= P.layer[l + 1].item_begin) ++l;
   const GtaLayer& L = P.layer[l];
   int local = item - L.item_begin;
   it.layer = l;
-  it.tn = local % L.tiles_n; local /= L.tiles_n;
-  it.tm = local % L.tiles_m; local /= L.tiles_m;
+  const int tiles_n = (L.N + kBN - 1) / kBN, tiles_m = (L.M + kTileM - 1) / kTileM;
+  it.tn = local % tiles_n; local /= tiles_n;
+  it.tm = local % tiles_m; local /= tiles_m;
   if (kSqsum) {
     it.example = local; it.split = 0;
     it.k0 = local * P.tsteps; it.k1 = it.k0 + P.tsteps;
   } else {
     it.example = -1; it.split = local;
-    it.k0 = local * L.ksteps_per_split;
-    it.k1 = min(it.k0 + L.ksteps_per_split, P.B * P.tsteps);
+    it.k0 = local * P.ksteps_per_split;
+    it.k1 = min(it.k0 + P.ksteps_per_split, P.B * P.tsteps);
   }
   return it;
 }
@@ -186,7 +189,7 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
       int lay = 0;
       bool ok = true;
       for (int item = first_item; item < P.total_items && ok; item += item_stride) {
-        const Item it = decode_item<kSqsum>(P, item, lay);
+        const Item it = decode_item<kSqsum, kTileM>(P, item, lay);
         const uint64_t tm = reinterpret_cast<uint64_t>(is_a ? &P.tmA[it.layer] : &P.tmG[it.layer]);
         // first column of this CTA's part of the tile: its G rows, or its share of the A columns
         const int c0 = is_a ? it.tn * kBN + int(rank) * Geo<kPair>::kAColsPerCta
@@ -224,7 +227,7 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
       int lay = 0;
       bool ok = true;
       for (int item = first_item; item < P.total_items && ok; item += item_stride, ++n_item) {
-        const Item it = decode_item<kSqsum>(P, item, lay);
+        const Item it = decode_item<kSqsum, kTileM>(P, item, lay);
         const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
         if (!(kPair ? ptx::mbar_wait_cluster(&acc_empty[buf], acc_phase ^ 1, abort_flag, P.wait_limit)
                     : ptx::mbar_wait(&acc_empty[buf], acc_phase ^ 1, abort_flag, P.wait_limit))) { ok = false; break; }
@@ -279,7 +282,7 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
       int lay = 0;
       bool ok = true;
       for (int item = first_item; item < P.total_items && ok; item += item_stride) {
-        const Item it = decode_item<kSqsum>(P, item, lay);
+        const Item it = decode_item<kSqsum, kTileM>(P, item, lay);
         const bool scale_here = P.clip && !P.layer[it.layer].prescaled;
         // first K step of this item that belongs to this warp
         int ks = it.k0 + int((uint32_t(sw) + kScalerWarps - cnt % kScalerWarps) % kScalerWarps);
@@ -364,7 +367,7 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
     int lay = 0;
     bool ok = true;
     for (int item = first_item; item < P.total_items && ok; item += item_stride, ++n_item) {
-      const Item it = decode_item<kSqsum>(P, item, lay);
+      const Item it = decode_item<kSqsum, kTileM>(P, item, lay);
       const GtaLayer& L = P.layer[it.layer];
       const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
       if (!ptx::mbar_wait_relaxed(&acc_full[buf], acc_phase, abort_flag, P.wait_limit)) { ok = false; break; }
@@ -390,12 +393,13 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
         if (lane == 0) { epi_red[slot * kEpiWarps + ew] = acc; ptx::mbar_arrive(&red_bar[slot]); }
         if (ew == 0) {
           if (!ptx::mbar_wait_relaxed(&red_bar[slot], red_phase, abort_flag, P.wait_limit)) { ok = false; break; }
-          const long long slot_idx = (long long)it.example * P.n_per + L.col_begin + it.tm * L.tiles_n + it.tn;
+          const int tiles_n = (L.N + kBN - 1) / kBN;
+          const long long slot_idx = (long long)it.example * P.n_per + L.col_begin + it.tm * tiles_n + it.tn;
           if (lane == 0 && dp_in_range(slot_idx, (long long)P.B * P.n_per, P.dev_status)) {
             float s = 0.f;
 #pragma unroll
             for (int e = 0; e < kEpiWarps; ++e) s += epi_red[slot * kEpiWarps + e];
-            P.sq_partials[size_t(it.example) * P.n_per + L.col_begin + it.tm * L.tiles_n + it.tn] = s;
+            P.sq_partials[slot_idx] = s;
           }
         }
       } else {
@@ -403,13 +407,13 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
         float* dst;
         long long ld;
         float beta;
-        if (L.nsplit == 1) { dst = L.out; ld = L.ldo; beta = L.beta; }
+        if (P.nsplit == 1) { dst = L.out; ld = L.ldo; beta = P.beta; }
         else { dst = L.partial + size_t(it.split) * size_t(L.M) * L.N; ld = L.N; beta = 0.f; }
         // 32-byte (8 columns) or 16-byte accesses where the pitch and the base allow them
         const bool vec8 = ((ld & 7) == 0) && ((reinterpret_cast<uintptr_t>(dst) & 31) == 0);
         const bool vec4 = ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0);
         // fused Gaussian mechanism (Eq. 3): only on the final destination, never on a K-split plane
-        const bool noisy = (L.noise_amp >= 0.f) && (L.nsplit == 1);
+        const bool noisy = (L.noise_amp >= 0.f) && (P.nsplit == 1);
         const float amp = L.noise_amp;
         const uint32_t tensor_id = L.tensor_id, step = effective_step(P.noise_step, P.step_dev);
 #pragma unroll 1
@@ -647,10 +651,8 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
       if (s != DP_OK) return s;
       s = make_tmap_bf16_3d(&P.tmA[g - g0], D.A, D.lda, D.d, T, B, 64, kBK);
       if (s != DP_OK) return s;
-      L.out = outs[g]; L.ldo = ldos[g]; L.beta = beta;
+      L.out = outs[g]; L.ldo = ldos[g];
       L.M = D.p; L.N = D.d;
-      L.tiles_m = ceil_div(D.p, Geo<kUsePair>::kTileM); L.tiles_n = ceil_div(D.d, kBN);
-      L.nsplit = nsplit; L.ksteps_per_split = kps;
       L.partial = nullptr;
       if (nsplit > 1) {
         L.partial = reinterpret_cast<float*>(pw);
@@ -662,7 +664,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
       const bool fuse = noise && nsplit == 1 && (D.d % 4 == 0);
       L.noise_amp = fuse ? noise->amp : -1.f;
       L.tensor_id = noise ? noise->tensor_ids[g] : 0u;
-      items += L.tiles_m * L.tiles_n * nsplit;
+      items += ceil_div(D.p, Geo<kUsePair>::kTileM) * ceil_div(D.d, kBN) * nsplit;
     }
     if (noise) {
       P.noise_keys = expand_noise_keys(noise->seed);
@@ -671,6 +673,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
     }
     P.n_layers = g1 - g0; P.B = B; P.T = T; P.tsteps = tsteps;
     P.total_items = items;
+    P.nsplit = nsplit; P.ksteps_per_split = kps; P.beta = beta;
     P.clip = clip;
     P.dev_status = dev_status;
     P.wait_limit = g_wait_limit;
@@ -716,15 +719,14 @@ dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& p
       if (s != DP_OK) return s;
       GtaLayer& L = P.layer[g - g0];
       L.M = D.p; L.N = D.d;
-      L.tiles_m = plan.direct[li].tiles_m; L.tiles_n = plan.direct[li].tiles_n;
-      L.nsplit = 1; L.ksteps_per_split = 0;
       L.col_begin = plan.direct[li].col_begin;
       L.item_begin = items;
-      items += B * L.tiles_m * L.tiles_n;
+      items += B * plan.direct[li].tiles_m * plan.direct[li].tiles_n;
     }
     P.n_layers = int(g1 - g0);
     P.B = B; P.T = T; P.tsteps = ceil_div(T, kBK);
     P.total_items = items;
+    P.nsplit = 1;
     P.sq_partials = partials; P.n_per = plan.n_per;
     P.dev_status = dev_status;
     P.wait_limit = g_wait_limit;

@@ -57,7 +57,7 @@ struct __align__(64) PairParams {
   int* dev_status;
   long long wait_limit;
 };
-static_assert(sizeof(PairParams) <= 32000, "kernel parameter block too large");
+static_assert(sizeof(PairParams) <= 32764, "kernel parameter block too large");
 
 struct Item {
   int layer, example, ti, tj, a0, a1, g0, g1, pidx;

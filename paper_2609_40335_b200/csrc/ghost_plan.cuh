@@ -8,7 +8,9 @@
 
 namespace dpg {
 
-constexpr int kGhostMaxLayers = 96;     // layers per tensor-core launch (parameter-block limit)
+// Layers per tensor-core launch (two tensor maps and 28 bytes each in the parameter block); GPT-2
+// medium's 97 layers have to fit.
+constexpr int kGhostMaxLayers = 112;
 
 // Plain data: copied into kernel parameters.
 struct GhostLayerPlan {
