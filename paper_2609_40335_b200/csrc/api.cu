@@ -346,7 +346,7 @@ dp_status dp_ghost_norms(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, 
 // ------------------------------------------------------------------------ embedding norms
 size_t dp_embed_norms_ws_bytes(int32_t B, int32_t T, int32_t d) {
   if (B <= 0 || T <= 0 || d <= 0) return 0;
-  return align_up(size_t(B) * ceil_div(d, kEmbedColsPerBlock) * sizeof(float), 256);
+  return align_up(size_t(B) * ceil_div(d, kEmbedColsPerBlock) * embed_norm_parts(B, T, d) * sizeof(float), 256);
 }
 
 dp_status dp_embed_norms(const int32_t* ids, const void* G, int64_t ldg, dp_dtype dt, int32_t B,
@@ -358,9 +358,10 @@ dp_status dp_embed_norms(const int32_t* ids, const void* G, int64_t ldg, dp_dtyp
   if (!ws || ws_bytes < dp_embed_norms_ws_bytes(B, T, d)) return DP_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   float* partials = static_cast<float*>(ws);
-  dp_status s = launch_embed_norms(ids, G, ldg, dt, B, T, d, V, partials, first_occ, dev_status, st);
+  const int parts = embed_norm_parts(B, T, d);
+  dp_status s = launch_embed_norms(ids, G, ldg, dt, B, T, d, V, parts, partials, first_occ, dev_status, st);
   if (s != DP_OK) return s;
-  return launch_reduce_partials(partials, ceil_div(d, kEmbedColsPerBlock), B, sq, 1.f, nullptr, st);
+  return launch_reduce_partials(partials, ceil_div(d, kEmbedColsPerBlock) * parts, B, sq, 1.f, nullptr, st);
 }
 
 // ------------------------------------------------------------------------ tied cross term
@@ -612,25 +613,30 @@ dp_status dp_clip_accumulate(const void* A, int64_t lda, const void* G, int64_t 
 }
 
 // ------------------------------------------------------------------ clip accumulate, embedding
-static void embed_ws_layout(int B, int T, int d, int V, size_t* off_clip, size_t* off_counts,
-                            size_t* off_seg, size_t* off_perm, size_t* off_blk, size_t* off_part,
-                            size_t* total, int* chunks) {
+// scratch of the sort: counts per id, overall and per chunk, and the ranks
+static size_t sort_totals_bytes(size_t n, int V) {
+  const size_t chunks = (n + kSortChunk - 1) / kSortChunk;
+  return align_up((chunks + 1) * V * sizeof(int), 256);
+}
+
+static void embed_ws_layout(int B, int T, int d, int V, size_t* off_clip, size_t* off_totals,
+                            size_t* off_seg, size_t* off_perm, size_t* off_rank, size_t* off_part,
+                            size_t* total) {
   const size_t n = size_t(B) * T;
-  *chunks = int((n + kSortChunk - 1) / kSortChunk);
   size_t o = 0;
   *off_clip = o;   o += align_up(size_t(B) * sizeof(float), 256);
-  *off_counts = o; o += align_up(size_t(*chunks) * V * sizeof(int), 256);
+  *off_totals = o; o += sort_totals_bytes(n, V);
   *off_seg = o;    o += align_up(size_t(V + 1) * sizeof(int), 256);
   *off_perm = o;   o += align_up(n * sizeof(int), 256);
-  *off_blk = o;    o += align_up(size_t(ceil_div(V, 1024)) * sizeof(int), 256);
+  *off_rank = o;   o += align_up(n * sizeof(int), 256);
   *off_part = o;   o += embed_scatter_partial_bytes((long long)n, d);
   *total = o;
 }
 
 size_t dp_clip_accumulate_embed_ws_bytes(int32_t B, int32_t T, int32_t d, int32_t V) {
   if (B <= 0 || T <= 0 || V <= 0 || d <= 0) return 0;
-  size_t a, b, c, e, f, g, total; int chunks;
-  embed_ws_layout(B, T, d, V, &a, &b, &c, &e, &f, &g, &total, &chunks);
+  size_t a, b, c, e, f, g, total;
+  embed_ws_layout(B, T, d, V, &a, &b, &c, &e, &f, &g, &total);
   return total;
 }
 
@@ -650,18 +656,17 @@ static dp_status clip_accumulate_embed_impl(const int32_t* ids, const void* G, i
   if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
   if (!(beta == 0.f || beta == 1.f) || !finite_pos(C)) return DP_ERR_INVALID_ARG;
   if ((long long)B * T > 0x7fffffffLL) return DP_ERR_UNSUPPORTED;
-  size_t o_clip, o_counts, o_seg, o_perm, o_blk, o_part, total; int chunks;
-  embed_ws_layout(B, T, d, V, &o_clip, &o_counts, &o_seg, &o_perm, &o_blk, &o_part, &total, &chunks);
+  size_t o_clip, o_totals, o_seg, o_perm, o_rank, o_part, total;
+  embed_ws_layout(B, T, d, V, &o_clip, &o_totals, &o_seg, &o_perm, &o_rank, &o_part, &total);
   if (!ws || ws_bytes < total) return DP_ERR_WORKSPACE;
   cudaStream_t st = (cudaStream_t)stream;
   char* w = static_cast<char*>(ws);
   float* clip_ws = reinterpret_cast<float*>(w + o_clip);
   EmbedSortWs sw;
-  sw.counts = reinterpret_cast<int*>(w + o_counts);
+  sw.totals = reinterpret_cast<int*>(w + o_totals);
   sw.seg = reinterpret_cast<int*>(w + o_seg);
   sw.perm = reinterpret_cast<int*>(w + o_perm);
-  sw.block_sums = reinterpret_cast<int*>(w + o_blk);
-  sw.chunks = chunks;
+  sw.rank = reinterpret_cast<int*>(w + o_rank);
   const int n = B * T;
   dp_status s = resolve_clip(sq, B, C, clip, &clip_ws, st);
   if (s != DP_OK) return s;
@@ -704,8 +709,8 @@ dp_status dp_clip_accumulate_embed(const int32_t* ids, const void* G, int64_t ld
 
 size_t dp_embed_sort_ws_bytes(int32_t B, int32_t T, int32_t V) {
   if (B <= 0 || T <= 0 || V <= 0) return 0;
-  const size_t chunks = (size_t(B) * T + kSortChunk - 1) / kSortChunk;
-  return align_up(chunks * V * sizeof(int), 256) + align_up(size_t(ceil_div(V, 1024)) * sizeof(int), 256);
+  const size_t n = size_t(B) * T;
+  return sort_totals_bytes(n, V) + align_up(n * sizeof(int), 256);
 }
 
 dp_status dp_embed_sort(const int32_t* ids, int32_t B, int32_t T, int32_t V, int32_t* perm,
@@ -715,10 +720,8 @@ dp_status dp_embed_sort(const int32_t* ids, int32_t B, int32_t T, int32_t V, int
   if (!ws || ws_bytes < dp_embed_sort_ws_bytes(B, T, V)) return DP_ERR_WORKSPACE;
   const int n = B * T;
   EmbedSortWs sw;
-  sw.chunks = (n + kSortChunk - 1) / kSortChunk;
-  sw.counts = static_cast<int*>(ws);
-  sw.block_sums = reinterpret_cast<int*>(static_cast<char*>(ws) +
-                                         align_up(size_t(sw.chunks) * V * sizeof(int), 256));
+  sw.totals = static_cast<int*>(ws);
+  sw.rank = reinterpret_cast<int*>(static_cast<char*>(ws) + sort_totals_bytes(size_t(n), V));
   sw.seg = seg;
   sw.perm = perm;
   return launch_embed_sort(ids, n, V, sw, dev_status, (cudaStream_t)stream);

@@ -47,6 +47,15 @@ int sm_count();
 // afterwards.  A process that drives several GPUs gets the set-up on each of them.
 bool first_use_on_this_device(const void* key);
 
+// Small kernels that run on a second stream beside a persistent TMA kernel ask for the same
+// shared-memory carve-out as that kernel: an SM changes its carve-out only when it is idle, so a
+// kernel with another preference waits until the persistent one has left the SM.
+template <typename K>
+inline cudaError_t prefer_max_shared(K* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                              cudaSharedmemCarveoutMaxShared);
+}
+
 template <typename T> __device__ __forceinline__ float to_f32(T v);
 template <> __device__ __forceinline__ float to_f32<float>(float v) { return v; }
 template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 v) {
@@ -108,6 +117,45 @@ __device__ __forceinline__ void load8<float>(const float* p, int nvalid, bool ve
     for (int e = 0; e < 8; ++e) v[e] = e < nvalid ? p[e] : 0.f;
   }
 }
+
+// Eight consecutive columns of one row, kept as loaded (a bf16 row chunk stays one 16-byte
+// register quad until it is consumed, so twice as many loads fit in flight per thread).
+template <typename T> struct Raw8;
+template <> struct Raw8<__nv_bfloat16> {
+  uint4 q;
+  __device__ __forceinline__ void zero() { q = make_uint4(0u, 0u, 0u, 0u); }
+  __device__ __forceinline__ void load(const __nv_bfloat16* p, int nvalid, bool vec) {
+    if (vec && nvalid >= 8) {
+      q = *reinterpret_cast<const uint4*>(p);
+    } else {
+      uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (e < nvalid) w[e >> 1] |= uint32_t(__bfloat16_as_ushort(p[e])) << (16 * (e & 1));
+      q = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+  __device__ __forceinline__ void unpack(float (&v)[8]) const {
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      v[2 * e] = __uint_as_float(w[e] << 16);
+      v[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
+    }
+  }
+};
+template <> struct Raw8<float> {
+  float v8[8];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v8[e] = 0.f;
+  }
+  __device__ __forceinline__ void load(const float* p, int nvalid, bool vec) { load8<float>(p, nvalid, vec, v8); }
+  __device__ __forceinline__ void unpack(float (&v)[8]) const {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = v8[e];
+  }
+};
 
 // Clip coefficient of Eq. 7 from a squared norm, IEEE sqrt and divide.  A zero norm gives 1
 // (nothing to clip).  The tied norm in + out + 2 cross can round to a tiny negative number when

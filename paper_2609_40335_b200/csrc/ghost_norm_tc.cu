@@ -282,6 +282,8 @@ __global__ void reduce_partials_kernel(const float* __restrict__ partials, int n
 
 dp_status launch_reduce_partials(const float* partials, int n_per, int B, float* sq,
                                  float factor, float* plain_out, cudaStream_t st) {
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&launch_reduce_partials)))
+    DP_CUDA_OK(prefer_max_shared(reduce_partials_kernel));
   const int warps = 4;
   reduce_partials_kernel<<<ceil_div(B, warps), warps * 32, 0, st>>>(partials, n_per, B, sq,
                                                                   factor, plain_out);

@@ -103,12 +103,8 @@ dp_status launch_add_noise(float* out, long long rows, int cols, long long ld, b
   // per SM leave half of every SM's thread slots free for it.
   const int grid = (int)std::min<long long>(want, (long long)sm_count() * (fill ? 4 : 16));
   const NoiseKeys keys = expand_noise_keys(seed);
-  if (fill && first_use_on_this_device(reinterpret_cast<const void*>(&launch_add_noise))) {
-    // same shared-memory carve-out as the TMA kernels, so that both can be resident on one SM
-    DP_CUDA_OK(cudaFuncSetAttribute(add_noise_kernel<true>,
-                                    cudaFuncAttributePreferredSharedMemoryCarveout,
-                                    cudaSharedmemCarveoutMaxShared));
-  }
+  if (fill && first_use_on_this_device(reinterpret_cast<const void*>(&launch_add_noise)))
+    DP_CUDA_OK(prefer_max_shared(add_noise_kernel<true>));
   if (fill)
     add_noise_kernel<true><<<grid, 256, 0, st>>>(out, n, cols, ld, amp, scale, keys, tensor_id, step,
                                              g_step_dev, first_quad);

@@ -6,6 +6,7 @@
 // already fully committed.  For them the scratch of the embedding norm (one partial sum per
 // example and 256-column slab) lives in a fixed array inside the library image instead of a
 // caller buffer.  Nothing here calls cudaMalloc, cudaFree or any other allocating routine.
+#include <algorithm>
 #include <mutex>
 
 #include "dp_common.cuh"
@@ -58,7 +59,8 @@ extern "C" dp_status dp_embed_norms_static(const int32_t* ids, const void* G, in
   cudaStream_t st = (cudaStream_t)stream;
   // every partial that is read below is written first by the norm kernel, so the array's
   // previous contents never matter and nothing has to be cleared
-  s = launch_embed_norms(ids, G, ldg, dt, B, T, d, V, partials, first_occ, dev_status, st);
+  const int parts = std::min(embed_norm_parts(B, T, d), kStaticScratchFloats / (B * slabs));
+  s = launch_embed_norms(ids, G, ldg, dt, B, T, d, V, parts, partials, first_occ, dev_status, st);
   if (s != DP_OK) return s;
-  return launch_reduce_partials(partials, slabs, B, sq, 1.f, nullptr, st);
+  return launch_reduce_partials(partials, slabs * parts, B, sq, 1.f, nullptr, st);
 }

@@ -50,40 +50,6 @@ __device__ __forceinline__ int find_param(const VecParams& P, int slab) {
   return k;
 }
 
-// Eight consecutive columns of one row, kept as loaded (a bf16 row chunk stays one 16-byte
-// register quad until it is consumed, so twice as many loads fit in flight per thread).
-template <typename T> struct Raw8;
-template <> struct Raw8<__nv_bfloat16> {
-  uint4 q;
-  __device__ __forceinline__ void load(const __nv_bfloat16* p, int nvalid, bool vec) {
-    if (vec && nvalid >= 8) {
-      q = *reinterpret_cast<const uint4*>(p);
-    } else {
-      uint32_t w[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        if (e < nvalid) w[e >> 1] |= uint32_t(__bfloat16_as_ushort(p[e])) << (16 * (e & 1));
-      q = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-  }
-  __device__ __forceinline__ void unpack(float (&v)[8]) const {
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      v[2 * e] = __uint_as_float(w[e] << 16);
-      v[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-    }
-  }
-};
-template <> struct Raw8<float> {
-  float v8[8];
-  __device__ __forceinline__ void load(const float* p, int nvalid, bool vec) { load8<float>(p, nvalid, vec, v8); }
-  __device__ __forceinline__ void unpack(float (&v)[8]) const {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = v8[e];
-  }
-};
-
 // sum over the rows [r0, r1) (stride 8 from warp w) of weight(row) * G[row, cols] * X[row, cols].
 // All loads of a batch are issued before any is consumed; rows past r1 re-read row r1-1 with
 // weight 0, so the loads are unconditional.  The example of a row (for its clip factor) is

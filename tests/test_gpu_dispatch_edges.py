@@ -41,3 +41,53 @@ def test_as_many_layers_as_one_launch_holds_and_one_more(n_layers):
         want = np.einsum("b,bpd->pd", clip.double().cpu().numpy(), per)
         assert np.linalg.norm(o.double().cpu().numpy() - want) < 1e-5 * np.linalg.norm(want)
     assert (np.abs(sq.double().cpu().numpy() / want_sq - 1) < 1e-5).all()
+
+
+def reference_sort(ids, V):
+    flat = ids.cpu().numpy().reshape(-1)
+    ok = np.flatnonzero((flat >= 0) & (flat < V))
+    perm = ok[np.argsort(flat[ok], kind="stable")]
+    return perm, np.concatenate([[0], np.cumsum(np.bincount(flat[ok], minlength=V))])
+
+
+# one block up to 4096 tokens and 8192 ids; chunks of 1024 up to 32768 tokens, of 4096 beyond
+@pytest.mark.parametrize("B,T,V", [(1, 1, 1), (1, 31, 5), (2, 2048, 8192), (1, 4097, 100), (3, 1365, 8193),
+                                   (8, 4096, 300), (1, 32769, 70000), (3, 13107, 9)])
+def test_token_sort_at_the_edges_of_its_variants(B, T, V):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B * T)
+    ids = torch.randint(-1, V + 1, (B, T), generator=g, device="cuda", dtype=torch.int32)   # -1, V: out of range
+    if T > 100:
+        ids[:, 50:T // 2] = min(2, V - 1)                # one id far more frequent than the others
+    perm = torch.full((B * T,), -7, dtype=torch.int32, device="cuda")
+    seg = torch.empty(V + 1, dtype=torch.int32, device="cuda")
+    dp.dp_embed_sort(ids, V, perm, seg)
+    want_perm, want_seg = reference_sort(ids, V)
+    assert np.array_equal(seg.cpu().numpy(), want_seg)
+    got = perm.cpu().numpy()
+    assert np.array_equal(got[:len(want_perm)], want_perm)
+    assert (got[len(want_perm):] == -7).all()
+
+
+# 48 rows of one id are summed by one warp, 49 by eight; rows are cut into parts of at least 64
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("T,frequent", [(48, 48), (49, 49), (64, 48), (65, 49), (129, 80), (1000, 500), (4096, 2100)])
+def test_embedding_norm_with_frequent_tokens(dtype, T, frequent):
+    B, d, V = 2, 264, 5000
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    ids = torch.randint(0, V, (B, T), generator=g, device="cuda", dtype=torch.int32)
+    for i in range(B):
+        ids[i, torch.randperm(T, generator=g, device="cuda")[:frequent]] = 3 + i
+    G = torch.randn(B, T, d, generator=g, device="cuda").to(torch.float32 if dtype == "f32" else torch.bfloat16)
+    sq = torch.zeros(B, device="cuda")
+    first = torch.empty(B, T, dtype=torch.int32, device="cuda")
+    dp.dp_embed_norms(ids, G, V, sq, first_occ=first)
+    for i in range(B):
+        row = ids[i].cpu().numpy()
+        table = np.zeros((V, d))
+        np.add.at(table, row, G[i].double().cpu().numpy())
+        want = (table ** 2).sum()
+        assert abs(float(sq[i]) / want - 1) < 1e-5       # fp32 sums of at most 2100 terms
+        uniq, where = np.unique(row, return_index=True)
+        assert np.array_equal(first[i].cpu().numpy(), where[np.searchsorted(uniq, row)])
