@@ -295,6 +295,42 @@ dp_status dp_noise_step_device(const uint32_t* dev_counter);
 dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale,
                         uint64_t seed, uint32_t tensor_id, uint32_t step, void* stream);
 
+/* ---- one whole step (norms, clip factors, clipped sums, noise) in one call ----
+ * What the calls above compute one by one, enqueued on two streams: `stream` carries the layer
+ * norms, the vector norms, the tied cross term, the clip factors and the grouped clipped sums;
+ * `side_stream` the embedding norms, the token sorts, the tables' noise (or zeros) and, once the
+ * clip factors exist, the row sums of tables that no GEMM writes.  A caller that steps thousands of
+ * times pays one call instead of a dozen.  Nothing is kept between calls.
+ * layers [host, n_layers; the LM head, if any, is the last one], with outs / ldos / tensor_ids as in
+ * dp_clip_accumulate_noise_grouped (tied: the head's out is wte).  vectors, vector_outs, vector_ids
+ * as in dp_clip_accumulate_vectors.  pos_ids NULL: no position table.  with_noise 0: the bare
+ * clipped sums.  sq, clip [dev, B] and norms, cross [dev, B or NULL; cross is needed when tied] are
+ * overwritten; side_sq [dev, B], perm / seg and pos_perm / pos_seg [dev, as in dp_embed_sort] are
+ * scratch, as are ws (the largest *_ws_bytes of the calls on `stream`, and
+ * dp_clip_accumulate_embed_ws_bytes when tied) and side_ws (the largest of dp_embed_norms_ws_bytes,
+ * dp_embed_sort_ws_bytes and dp_clip_accumulate_embed_ws_bytes over both tables).  events: four
+ * cudaEvent_t of the caller that order the two streams; `stream` has waited for `side_stream` at the
+ * end.  phases: DP_STEP_ALL, or the three phases one after the other with the same descriptor (so
+ * that a caller can time them). */
+enum { DP_STEP_NORMS = 1, DP_STEP_GEMM = 2, DP_STEP_REST = 4, DP_STEP_ALL = 7 };
+typedef struct {
+  dp_linear_desc* layers;  float* const* outs;  const int64_t* ldos;  const uint32_t* tensor_ids;
+  const dp_vector_desc* vectors;  float* const* vector_outs;  const uint32_t* vector_ids;
+  const int32_t* ids;  const void* G_emb;  int64_t ldge;
+  const int32_t* pos_ids;
+  float* wte;  int64_t ld_wte;
+  float* wpe;  int64_t ld_wpe;
+  float* sq;  float* clip;  float* norms;  float* cross;  float* side_sq;
+  int32_t* perm;  int32_t* seg;  int32_t* pos_perm;  int32_t* pos_seg;
+  void* ws;  size_t ws_bytes;  void* side_ws;  size_t side_ws_bytes;
+  int32_t* dev_status;  void* stream;  void* side_stream;  void* events[4];
+  uint64_t seed;
+  int32_t n_layers, n_vectors, dtype, B, T, V, d, pos_rows, tied, with_noise;
+  float C, sigma;
+  uint32_t step, wte_id, wpe_id;
+} dp_step_desc;
+dp_status dp_step_enqueue(const dp_step_desc* desc, int32_t phases);
+
 /* ---- privacy accounting on the host (no device work) ----
  * The paper calibrates sigma with a Renyi-DP accountant from the target epsilon (3 in the main
  * experiments), delta = N^-1.1, the sampling rate q = batch / N and the number of steps.  One step

@@ -20,6 +20,7 @@ DP_DEV_BAD_ID, DP_DEV_TIMEOUT, DP_DEV_BOUNDS = 1, 2, 4
 _LIB_PATH = os.environ.get("DP_GHOST_LIB") or os.path.join(os.path.dirname(os.path.abspath(__file__)),
                                                        "libdp_ghost.so")
 _lib = None
+_native = None
 
 
 class DpGhostError(RuntimeError):
@@ -39,6 +40,24 @@ class _VectorDesc(C.Structure):
                 ("p", C.c_int32)]
 
 
+class _StepDesc(C.Structure):
+    _fields_ = [(n, C.c_void_p) for n in ("layers", "outs", "ldos", "tensor_ids", "vectors", "vector_outs",
+                                          "vector_ids", "ids", "G_emb")]
+    _fields_ += [("ldge", C.c_int64), ("pos_ids", C.c_void_p), ("wte", C.c_void_p), ("ld_wte", C.c_int64),
+                 ("wpe", C.c_void_p), ("ld_wpe", C.c_int64)]
+    _fields_ += [(n, C.c_void_p) for n in ("sq", "clip", "norms", "cross", "side_sq", "perm", "seg",
+                                           "pos_perm", "pos_seg")]
+    _fields_ += [("ws", C.c_void_p), ("ws_bytes", C.c_size_t), ("side_ws", C.c_void_p),
+                 ("side_ws_bytes", C.c_size_t), ("dev_status", C.c_void_p), ("stream", C.c_void_p),
+                 ("side_stream", C.c_void_p), ("events", C.c_void_p * 4), ("seed", C.c_uint64)]
+    _fields_ += [(n, C.c_int32) for n in ("n_layers", "n_vectors", "dtype", "B", "T", "V", "d", "pos_rows",
+                                          "tied", "with_noise")]
+    _fields_ += [("C", C.c_float), ("sigma", C.c_float), ("step", C.c_uint32), ("wte_id", C.c_uint32),
+                 ("wpe_id", C.c_uint32)]
+
+
+STEP_NORMS, STEP_GEMM, STEP_REST, STEP_ALL = 1, 2, 4, 7
+
 EXPORTS = ["dp_vector_norms", "dp_vector_norms_ws_bytes", "dp_clip_accumulate_vectors",
            "dp_clip_accumulate_vectors_ws_bytes", "dp_ghost_norms", "dp_ghost_norms_ws_bytes", "dp_embed_norms", "dp_embed_norms_ws_bytes",
            "dp_embed_norms_static",
@@ -52,7 +71,7 @@ EXPORTS = ["dp_vector_norms", "dp_vector_norms_ws_bytes", "dp_clip_accumulate_ve
            "dp_last_cuda_error", "dp_version", "dp_kernel_launches", "dp_debug_force_fma",
            "dp_debug_noise_error_scan", "dp_debug_bounds_checked", "dp_debug_bounds_probe",
            "dp_debug_tensor_map_encodes", "dp_debug_set_wait_limit",
-           "dp_debug_ghost_single", "dp_set_reserved_sms"]
+           "dp_debug_ghost_single", "dp_set_reserved_sms", "dp_step_enqueue"]
 
 
 def lib_path() -> str:
@@ -118,6 +137,7 @@ def load():
     L.dp_fill_noise.argtypes = [vp, i64, f32, f32, f32, C.c_uint64, C.c_uint32, C.c_uint32, vp]
     L.dp_add_noise_slice.argtypes = [vp, i64, i64, f32, f32, f32, C.c_uint64, C.c_uint32, C.c_uint32, vp]
     L.dp_noise_step_device.argtypes = [vp]
+    L.dp_step_enqueue.argtypes = [C.POINTER(_StepDesc), i32]
     L.dp_rdp_epsilon.argtypes = [C.c_double, C.c_double, i64, C.c_double, vp, vp]
     L.dp_sigma_for_epsilon.argtypes = [C.c_double, i64, C.c_double, C.c_double, C.c_double, vp]
     L.dp_status_string.argtypes = [i32]
@@ -177,12 +197,36 @@ def _dt(t: torch.Tensor) -> int:
 
 def _rows_ld(t: torch.Tensor) -> int:
     """Leading dimension of a (..., ld) tensor whose leading axes are densely packed."""
-    if t.stride(-1) != 1:
+    st = t.stride()
+    ld = st[-2]
+    if st[-1] != 1:
         raise DpGhostError(1, "marshal", "innermost stride must be 1")
-    ld = t.stride(-2)
-    if t.dim() == 3 and t.stride(0) != t.shape[1] * ld:
+    if len(st) == 3 and st[0] != t.size(1) * ld:
         raise DpGhostError(1, "marshal", "examples must be contiguous blocks of T rows")
     return ld
+
+
+def _marshal():
+    """The native half of the marshalling (csrc/marshal.cpp)."""
+    global _native
+    if _native is None:
+        try:
+            from . import _marshal as m
+        except ImportError as e:
+            raise DpGhostError(-1, "load", f"{e}: build the package first; there is no fallback") from e
+        _native = m
+    return _native
+
+
+def _outputs(tensors):
+    """Device pointers and leading strides of several output tensors: two ctypes arrays."""
+    n = len(tensors)
+    buf = _marshal().outputs(tensors)
+    if buf is None:
+        for t in tensors:
+            _ptr(t)
+        raise DpGhostError(1, "marshal", "outputs must be tensors")
+    return (C.c_void_p * n).from_buffer(buf), (C.c_int64 * n).from_buffer(buf, 8 * n)
 
 
 def _ws(nbytes: int, ws: Optional[torch.Tensor], device) -> torch.Tensor:
@@ -203,17 +247,19 @@ class Linear:
 
 
 def _descs(layers: Sequence[Linear]):
-    arr = (_LinearDesc * len(layers))()
-    for k, l in enumerate(layers):
-        arr[k].A = _ptr(l.A)
-        arr[k].lda = _rows_ld(l.A)
-        arr[k].d = l.d if l.d is not None else l.A.shape[-1]
-        arr[k].G = _ptr(l.G)
-        arr[k].ldg = _rows_ld(l.G)
-        arr[k].p = l.p if l.p is not None else l.G.shape[-1]
-        arr[k].mode = l.mode
-        arr[k].mode_used = -1
-    return arr
+    buf = _marshal().linears(layers)
+    if buf is None:
+        for l in layers:                       # one of these says what is wrong
+            _ptr(l.A), _ptr(l.G), _rows_ld(l.A), _rows_ld(l.G)
+        raise DpGhostError(1, "marshal", "layers need tensors A and G of at least two axes")
+    return (_LinearDesc * len(layers)).from_buffer(buf)
+
+
+def _write_modes(layers: Sequence[Linear], arr) -> List[int]:
+    used = memoryview(arr).cast("B").cast("I")[12::14].tolist()    # 14 32-bit words per record
+    for l, u in zip(layers, used):
+        l.mode_used = u
+    return used
 
 
 def dp_ghost_norms_ws_bytes(layers: Sequence[Linear], B: int, T: int) -> int:
@@ -232,10 +278,7 @@ def dp_ghost_norms(layers: Sequence[Linear], B: int, T: int, sq: torch.Tensor, w
     st = L.dp_ghost_norms(arr, len(layers), dt, B, T, _ptr(sq), _ptr(ws), ws.numel() * ws.element_size(),
                           _ptr(dev_status), _stream(stream))
     _check(st, "dp_ghost_norms")
-    used = [int(arr[k].mode_used) for k in range(len(layers))]
-    for l, u in zip(layers, used):
-        l.mode_used = u
-    return used
+    return _write_modes(layers, arr)
 
 
 def dp_embed_norms(ids: torch.Tensor, G: torch.Tensor, V: int, sq: torch.Tensor, d=None,
@@ -260,14 +303,14 @@ class Vector:
 
 
 def _vdescs(params: Sequence[Vector]):
-    arr = (_VectorDesc * len(params))()
-    for k, v in enumerate(params):
-        arr[k].G = _ptr(v.G)
-        arr[k].ldg = _rows_ld(v.G)
-        arr[k].X = _ptr(v.X)
-        arr[k].ldx = _rows_ld(v.X) if v.X is not None else 0
-        arr[k].p = v.p if v.p is not None else v.G.shape[-1]
-    return arr
+    buf = _marshal().vectors(params)
+    if buf is None:
+        for v in params:
+            _ptr(v.G), _rows_ld(v.G)
+            if v.X is not None:
+                _ptr(v.X), _rows_ld(v.X)
+        raise DpGhostError(1, "marshal", "parameters need tensors of at least two axes")
+    return (_VectorDesc * len(params)).from_buffer(buf)
 
 
 def dp_vector_norms_ws_bytes(params: Sequence[Vector], B: int, T: int) -> int:
@@ -297,7 +340,7 @@ def dp_clip_accumulate_vectors(params: Sequence[Vector], B: int, T: int, sq, C_:
     L = load()
     arr = _vdescs(params)
     n = len(params)
-    optr = (C.c_void_p * n)(*[_ptr(o) for o in outs])
+    optr, _ = _outputs(outs)
     need = int(L.dp_clip_accumulate_vectors_ws_bytes(arr, n, B, T))
     ws = _ws(need, ws, outs[0].device)
     if noise is None:
@@ -387,8 +430,7 @@ def dp_clip_accumulate_grouped(layers: Sequence[Linear], B: int, T: int, sq, C_:
     arr = _descs(layers)
     dt = _dt(layers[0].A)
     n = len(layers)
-    optr = (C.c_void_p * n)(*[_ptr(o) for o in outs])
-    ldos = (C.c_int64 * n)(*[o.stride(0) for o in outs])
+    optr, ldos = _outputs(outs)
     need = int(L.dp_clip_accumulate_grouped_ws_bytes(arr, n, dt, B, T))
     ws = _ws(need, ws, outs[0].device)
     st = L.dp_clip_accumulate_grouped(arr, n, dt, B, T, _ptr(sq), float(C_), _ptr(clip), optr, ldos,
@@ -407,8 +449,7 @@ def dp_clip_accumulate_noise_grouped(layers: Sequence[Linear], B: int, T: int, s
     arr = _descs(layers)
     dt = _dt(layers[0].A)
     n = len(layers)
-    optr = (C.c_void_p * n)(*[_ptr(o) for o in outs])
-    ldos = (C.c_int64 * n)(*[o.stride(0) for o in outs])
+    optr, ldos = _outputs(outs)
     tids = (C.c_uint32 * n)(*[int(t) for t in tensor_ids])
     need = int(L.dp_clip_accumulate_grouped_ws_bytes(arr, n, dt, B, T))
     ws = _ws(need, ws, outs[0].device)
@@ -510,6 +551,34 @@ def dp_fill_noise(out: torch.Tensor, sigma: float, C_: float, scale: float, seed
     st = L.dp_fill_noise(_ptr(out), n, float(sigma), float(C_), float(scale), int(seed) & (2 ** 64 - 1),
                          int(tensor_id), int(step), _stream(stream))
     _check(st, "dp_fill_noise")
+
+
+def dp_step_enqueue(layers, outs, tensor_ids, vectors, vector_outs, vector_ids, *, ids, G_emb, pos_ids, wte, wpe,
+                    sq, clip, norms, cross, side_sq, perm, seg, pos_perm, pos_seg, ws, side_ws, dev_status,
+                    stream, side_stream, events, V, d, tied, noise, C_, sigma, seed, step, wte_id, wpe_id,
+                    phases=STEP_ALL):
+    """The whole step (or some of its phases) in one library call; see the header."""
+    L = load()
+    n, nv = len(layers), len(vectors)
+    arr = _descs(layers) if n else None
+    varr = _vdescs(vectors) if nv else None
+    (optr, ldos), (vptr, _) = _outputs(outs), _outputs(vector_outs)
+    tids, vids = (C.c_uint32 * n)(*tensor_ids), (C.c_uint32 * nv)(*vector_ids)
+    at = C.addressof
+    B, T = ids.shape
+    S = _StepDesc(
+        at(arr) if n else None, at(optr) if n else None, at(ldos) if n else None, at(tids),
+        at(varr) if nv else None, at(vptr) if nv else None, at(vids), _ptr(ids), _ptr(G_emb), _rows_ld(G_emb),
+        _ptr(pos_ids), _ptr(wte), wte.stride(0), _ptr(wpe), wpe.stride(0) if wpe is not None else 0, _ptr(sq),
+        _ptr(clip), _ptr(norms), _ptr(cross), _ptr(side_sq), _ptr(perm), _ptr(seg), _ptr(pos_perm),
+        _ptr(pos_seg), _ptr(ws), ws.nbytes, _ptr(side_ws), side_ws.nbytes, _ptr(dev_status), _stream(stream),
+        _stream(side_stream), (C.c_void_p * 4)(*events), int(seed) & (2 ** 64 - 1), n, nv, _dt(G_emb), B, T, V, d,
+        wpe.shape[0] if wpe is not None else 0, int(bool(tied)), int(bool(noise)), float(C_), float(sigma),
+        int(step) & 0xFFFFFFFF, wte_id, wpe_id)
+    st = L.dp_step_enqueue(C.byref(S), phases)
+    _check(st, "dp_step_enqueue")
+    if n and phases & STEP_NORMS:
+        _write_modes(layers, arr)
 
 
 def dp_rdp_epsilon(q: float, sigma: float, steps: int, delta: float):

@@ -1,4 +1,5 @@
-"""Builds csrc/*.cu into libdp_ghost.so (sm_100a only) next to this file.
+"""Builds csrc/*.cu into libdp_ghost.so (sm_100a only) and csrc/marshal.cpp into the Python
+extension _marshal.so, next to this file.
 
     python -m paper_2609_40335_b200.build [--force] [--verbose] [--check]
 
@@ -21,6 +22,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ_DIR = os.path.join(HERE, "build")
 LIB_PATH = os.path.join(HERE, "libdp_ghost.so")
 CHECK_LIB_PATH = os.path.join(HERE, "libdp_ghost_check.so")
+MARSHAL_PATH = os.path.join(HERE, "_marshal.so")
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC"]
 
@@ -66,6 +68,8 @@ def build(force: bool = False, verbose: bool = False, check: bool = False) -> st
         r = subprocess.run(cmd, capture_output=True, text=True)
         return cmd, r
 
+    if not check:
+        build_marshal(force)
     with cf.ThreadPoolExecutor(max_workers=min(8, max(1, len(jobs)))) as ex:
         for cmd, r in ex.map(run, jobs):
             if verbose or r.returncode != 0:
@@ -79,6 +83,27 @@ def build(force: bool = False, verbose: bool = False, check: bool = False) -> st
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
     return lib_path
+
+
+def build_marshal(force: bool = False) -> str:
+    """Compile the extension that reads the tensors of a call (see csrc/marshal.cpp)."""
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    src = os.path.join(CSRC, "marshal.cpp")
+    header = os.path.join(os.path.dirname(HERE), "include", "dp_ghost.h")
+    if force or _stale(MARSHAL_PATH, [src, header]):
+        lib = os.path.join(root, "lib")
+        cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+               "-I" + os.path.join(root, "include"), "-I" + sysconfig.get_paths()["include"], src, "-o", MARSHAL_PATH,
+               "-L" + lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-Wl,-rpath," + lib]
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        if r.returncode != 0:
+            sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+            raise RuntimeError("compiling marshal.cpp failed")
+    return MARSHAL_PATH
 
 
 if __name__ == "__main__":

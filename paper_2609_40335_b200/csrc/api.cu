@@ -183,7 +183,7 @@ static int resolve_mode(const dp_linear_desc& L, int T) {
 
 // norm of one fp32 layer on the tensor cores; ws holds the widened operands and the partial sums
 static dp_status f32_norm_tc(const dp_linear_desc& L, int B, int T, int mode, float* sq, char* ws,
-                             int* dev_status, cudaStream_t st) {
+                             int* dev_status, cudaStream_t st, bool overwrite) {
   const bool direct = mode == DP_NORM_DIRECT;
   SplitLayer S = split_layout(L, B, T, !direct, ws);
   float* partials = reinterpret_cast<float*>(ws + S.bytes);
@@ -198,7 +198,7 @@ static dp_status f32_norm_tc(const dp_linear_desc& L, int B, int T, int mode, fl
     const GhostPlan plan = plan_ghost_norms(&S.one, 1, B, T, sm_count(), false);
     s = launch_ghost_norm_tc(&S.one, plan, B, T, partials, dev_status, st, &S.other);
     if (s != DP_OK) return s;
-    return launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st);
+    return launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st, overwrite);
   }
   // DIRECT: G'^T A' per example over 3T token rows
   s = launch_split_rows(A, L.lda, B, T, L.d, nullptr, 1, const_cast<void*>(S.one.A), st);
@@ -209,7 +209,7 @@ static dp_status f32_norm_tc(const dp_linear_desc& L, int B, int T, int mode, fl
   const GhostPlan plan = plan_ghost_norms(&S.one, 1, B, 3 * T, sm_count(), false);
   s = launch_direct_norm_tc(&S.one, plan, B, 3 * T, partials, dev_status, st);
   if (s != DP_OK) return s;
-  return launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st);
+  return launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st, overwrite);
 }
 
 }  // namespace dpg
@@ -297,9 +297,10 @@ size_t dp_ghost_norms_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, d
   return align_up(size_t(B) * plan.n_per * sizeof(float), 256);
 }
 
-dp_status dp_ghost_norms(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B,
-                         int32_t T, float* sq, void* ws, size_t ws_bytes, int32_t* dev_status,
-                         void* stream) {
+// overwrite: sq is written instead of added to (its first contribution of a step)
+static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B,
+                                  int32_t T, float* sq, void* ws, size_t ws_bytes, int32_t* dev_status,
+                                  void* stream, bool overwrite) {
   if (!layers || n_layers <= 0 || B <= 0 || T <= 0 || !sq) return DP_ERR_INVALID_ARG;
   if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
@@ -315,11 +316,12 @@ dp_status dp_ghost_norms(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, 
       dp_status s;
       if (dt == DP_F32 && f32_on_tensor_cores(layers[l], T)) {
         if (!ws || !aligned16(ws)) return DP_ERR_WORKSPACE;
-        s = f32_norm_tc(layers[l], B, T, plan.mode_used[l], sq, static_cast<char*>(ws), dev_status, st);
+        s = f32_norm_tc(layers[l], B, T, plan.mode_used[l], sq, static_cast<char*>(ws), dev_status, st, overwrite);
       } else {
-        s = launch_norms_fma(layers[l], dt, plan.mode_used[l], B, T, sq, st);
+        s = launch_norms_fma(layers[l], dt, plan.mode_used[l], B, T, sq, st, overwrite);
       }
       if (s != DP_OK) return s;
+      overwrite = false;
       layers[l].mode_used = plan.mode_used[l];
     }
     return DP_OK;
@@ -337,10 +339,16 @@ dp_status dp_ghost_norms(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, 
     s = launch_direct_norm_tc(layers, plan, B, T, partials, dev_status, st);
     if (s != DP_OK) return s;
   }
-  s = launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st);
+  s = launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st, overwrite);
   if (s != DP_OK) return s;
   for (int l = 0; l < n_layers; ++l) layers[l].mode_used = plan.mode_used[l];
   return DP_OK;
+}
+
+dp_status dp_ghost_norms(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B,
+                         int32_t T, float* sq, void* ws, size_t ws_bytes, int32_t* dev_status,
+                         void* stream) {
+  return ghost_norms_impl(layers, n_layers, dt, B, T, sq, ws, ws_bytes, dev_status, stream, false);
 }
 
 // ------------------------------------------------------------------------ embedding norms
@@ -349,9 +357,9 @@ size_t dp_embed_norms_ws_bytes(int32_t B, int32_t T, int32_t d) {
   return align_up(size_t(B) * ceil_div(d, kEmbedColsPerBlock) * embed_norm_parts(B, T, d) * sizeof(float), 256);
 }
 
-dp_status dp_embed_norms(const int32_t* ids, const void* G, int64_t ldg, dp_dtype dt, int32_t B,
-                         int32_t T, int32_t d, int32_t V, float* sq, int32_t* first_occ, void* ws,
-                         size_t ws_bytes, int32_t* dev_status, void* stream) {
+static dp_status embed_norms_impl(const int32_t* ids, const void* G, int64_t ldg, dp_dtype dt, int32_t B,
+                                  int32_t T, int32_t d, int32_t V, float* sq, int32_t* first_occ, void* ws,
+                                  size_t ws_bytes, int32_t* dev_status, void* stream, bool overwrite) {
   if (!ids || !G || !sq || B <= 0 || T <= 0 || d <= 0 || V <= 0 || ldg < d) return DP_ERR_INVALID_ARG;
   if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
   if (T > kEmbedMaxT) return DP_ERR_UNSUPPORTED;
@@ -361,7 +369,14 @@ dp_status dp_embed_norms(const int32_t* ids, const void* G, int64_t ldg, dp_dtyp
   const int parts = embed_norm_parts(B, T, d);
   dp_status s = launch_embed_norms(ids, G, ldg, dt, B, T, d, V, parts, partials, first_occ, dev_status, st);
   if (s != DP_OK) return s;
-  return launch_reduce_partials(partials, ceil_div(d, kEmbedColsPerBlock) * parts, B, sq, 1.f, nullptr, st);
+  return launch_reduce_partials(partials, ceil_div(d, kEmbedColsPerBlock) * parts, B, sq, 1.f, nullptr, st,
+                                overwrite);
+}
+
+dp_status dp_embed_norms(const int32_t* ids, const void* G, int64_t ldg, dp_dtype dt, int32_t B,
+                         int32_t T, int32_t d, int32_t V, float* sq, int32_t* first_occ, void* ws,
+                         size_t ws_bytes, int32_t* dev_status, void* stream) {
+  return embed_norms_impl(ids, G, ldg, dt, B, T, d, V, sq, first_occ, ws, ws_bytes, dev_status, stream, false);
 }
 
 // ------------------------------------------------------------------------ tied cross term
@@ -783,6 +798,143 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
   if (!aligned16(out)) return DP_ERR_ALIGNMENT;
   return launch_add_noise(out, n, 1, 1, true, sigma * C, scale, seed, tensor_id, step,
                           (cudaStream_t)stream);
+}
+
+// ------------------------------------------------------------------------------ whole step
+static dp_status check_step(const dp_step_desc* S) {
+  if (!S || S->B <= 0 || S->T <= 0 || S->V <= 0 || S->d <= 0 || S->n_layers < 0 || S->n_vectors < 0)
+    return DP_ERR_INVALID_ARG;
+  if (!S->ids || !S->G_emb || !S->wte || !S->sq || !S->clip || !S->side_sq || !S->perm || !S->seg)
+    return DP_ERR_INVALID_ARG;
+  if (S->n_layers && (!S->layers || !S->outs || !S->ldos || (S->with_noise && !S->tensor_ids)))
+    return DP_ERR_INVALID_ARG;
+  if (S->tied && (S->n_layers == 0 || !S->cross)) return DP_ERR_INVALID_ARG;
+  if (S->pos_ids && (!S->wpe || !S->pos_perm || !S->pos_seg || S->pos_rows <= 0)) return DP_ERR_INVALID_ARG;
+  for (int k = 0; k < 4; ++k) if (!S->events[k]) return DP_ERR_INVALID_ARG;
+  if (S->with_noise && !noise_args_ok(S->sigma, S->C, 1.f)) return DP_ERR_INVALID_ARG;
+  return DP_OK;
+}
+
+// A table that no GEMM writes starts as its noise (or as zeros), so that the row sums can be added.
+static dp_status start_table(const dp_step_desc* S, float* table, int64_t ld, int64_t rows, uint32_t tid,
+                             cudaStream_t st) {
+  if (S->with_noise)
+    return launch_add_noise(table, rows, S->d, ld, true, S->sigma * S->C, 1.f, S->seed, tid, S->step, st);
+  DP_CUDA_OK(cudaMemset2DAsync(table, size_t(ld) * sizeof(float), 0, size_t(S->d) * sizeof(float),
+                               size_t(rows), st));
+  return DP_OK;
+}
+
+// events: [0] the step began, [1] embedding norms done, [2] row sums done, [3] clip factors exist
+static dp_status step_norms(const dp_step_desc* S) {
+  cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
+  const dp_dtype dt = (dp_dtype)S->dtype;
+  dp_status s;
+  DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[0], main));
+  if (S->n_layers) {
+    s = ghost_norms_impl(S->layers, S->n_layers, dt, S->B, S->T, S->sq, S->ws, S->ws_bytes, S->dev_status,
+                         main, true);
+    if (s != DP_OK) return s;
+  } else {
+    DP_CUDA_OK(cudaMemsetAsync(S->sq, 0, size_t(S->B) * sizeof(float), main));
+  }
+  // Side stream: all that needs neither the big norm kernel nor the clip factors.  It is enqueued
+  // after that kernel: what is already resident keeps the kernel's CTAs out until it ends, what
+  // arrives second shares the SMs with them.
+  DP_CUDA_OK(cudaStreamWaitEvent(side, (cudaEvent_t)S->events[0], 0));     // earlier readers are done
+  s = embed_norms_impl(S->ids, S->G_emb, S->ldge, dt, S->B, S->T, S->d, S->V, S->side_sq, nullptr, S->side_ws,
+                       S->side_ws_bytes, S->dev_status, side, true);
+  if (s != DP_OK) return s;
+  if (S->pos_ids) {
+    s = embed_norms_impl(S->pos_ids, S->G_emb, S->ldge, dt, S->B, S->T, S->d, S->T, S->side_sq, nullptr,
+                         S->side_ws, S->side_ws_bytes, S->dev_status, side, false);
+    if (s != DP_OK) return s;
+  }
+  DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[1], side));
+  s = dp_embed_sort(S->ids, S->B, S->T, S->V, S->perm, S->seg, S->side_ws, S->side_ws_bytes, S->dev_status, side);
+  if (s != DP_OK) return s;
+  if (S->pos_ids) {
+    s = dp_embed_sort(S->pos_ids, S->B, S->T, S->pos_rows, S->pos_perm, S->pos_seg, S->side_ws,
+                      S->side_ws_bytes, S->dev_status, side);
+    if (s != DP_OK) return s;
+    s = start_table(S, S->wpe, S->ld_wpe, S->pos_rows, S->wpe_id, side);
+    if (s != DP_OK) return s;
+  }
+  if (!S->tied) {
+    s = start_table(S, S->wte, S->ld_wte, S->V, S->wte_id, side);
+    if (s != DP_OK) return s;
+  }
+  // main stream again
+  if (S->n_vectors) {
+    s = dp_vector_norms(S->vectors, S->n_vectors, dt, S->B, S->T, S->sq, S->ws, S->ws_bytes, main);
+    if (s != DP_OK) return s;
+  }
+  if (S->tied) {
+    const dp_linear_desc& lm = S->layers[S->n_layers - 1];
+    s = dp_tied_cross_term(S->ids, S->G_emb, S->ldge, lm.A, lm.lda, lm.G, lm.ldg, dt, S->B, S->T, S->d, S->V,
+                           S->sq, S->cross, S->ws, S->ws_bytes, S->dev_status, main);
+    if (s != DP_OK) return s;
+  }
+  DP_CUDA_OK(cudaStreamWaitEvent(main, (cudaEvent_t)S->events[1], 0));
+  // the two accumulators join in one fixed order of additions, then Eq. 7
+  s = launch_clip_factors(S->sq, S->B, S->C, S->clip, S->norms, main, S->side_sq, S->sq);
+  if (s != DP_OK) return s;
+  DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[3], main));
+  return DP_OK;
+}
+
+static dp_status step_gemm(const dp_step_desc* S) {
+  if (!S->n_layers) return DP_OK;
+  const dp_dtype dt = (dp_dtype)S->dtype;
+  if (S->with_noise)
+    return dp_clip_accumulate_noise_grouped(S->layers, S->n_layers, dt, S->B, S->T, nullptr, S->C, S->clip,
+                                            S->outs, S->ldos, 0.f, S->sigma, 1.f, S->seed, S->tensor_ids,
+                                            S->step, S->ws, S->ws_bytes, S->dev_status, S->stream);
+  return dp_clip_accumulate_grouped(S->layers, S->n_layers, dt, S->B, S->T, nullptr, S->C, S->clip, S->outs,
+                                    S->ldos, 0.f, S->ws, S->ws_bytes, S->dev_status, S->stream);
+}
+
+static dp_status step_rest(const dp_step_desc* S) {
+  cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
+  const dp_dtype dt = (dp_dtype)S->dtype;
+  dp_status s;
+  // Row sums of tables that no GEMM writes need the clip factors only: on the side stream they run
+  // where the GEMM's last wave leaves SMs idle.
+  DP_CUDA_OK(cudaStreamWaitEvent(side, (cudaEvent_t)S->events[3], 0));
+  if (!S->tied) {
+    s = dp_clip_accumulate_embed_sorted(S->ids, S->G_emb, S->ldge, dt, S->B, S->T, S->d, S->V, nullptr, S->C,
+                                        S->clip, S->wte, S->ld_wte, 1.f, S->perm, S->seg, S->side_ws,
+                                        S->side_ws_bytes, S->dev_status, side);
+    if (s != DP_OK) return s;
+  }
+  if (S->pos_ids) {
+    s = dp_clip_accumulate_embed_sorted(S->pos_ids, S->G_emb, S->ldge, dt, S->B, S->T, S->d, S->pos_rows, nullptr,
+                                        S->C, S->clip, S->wpe, S->ld_wpe, 1.f, S->pos_perm, S->pos_seg,
+                                        S->side_ws, S->side_ws_bytes, S->dev_status, side);
+    if (s != DP_OK) return s;
+  }
+  DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[2], side));
+  DP_CUDA_OK(cudaStreamWaitEvent(main, (cudaEvent_t)S->events[2], 0));
+  if (S->tied) {                       // onto the head's sum and noise
+    s = dp_clip_accumulate_embed_sorted(S->ids, S->G_emb, S->ldge, dt, S->B, S->T, S->d, S->V, nullptr, S->C,
+                                        S->clip, S->wte, S->ld_wte, 1.f, S->perm, S->seg, S->ws,
+                                        S->ws_bytes, S->dev_status, main);
+    if (s != DP_OK) return s;
+  }
+  if (S->n_vectors)
+    return dp_clip_accumulate_vectors(S->vectors, S->n_vectors, dt, S->B, S->T, nullptr, S->C, S->clip,
+                                      S->vector_outs, 0.f, S->with_noise, S->sigma, 1.f, S->seed,
+                                      S->vector_ids, S->step, S->ws, S->ws_bytes, main);
+  return DP_OK;
+}
+
+dp_status dp_step_enqueue(const dp_step_desc* S, int32_t phases) {
+  dp_status s = check_step(S);
+  if (s != DP_OK) return s;
+  if (phases & DP_STEP_NORMS) { s = step_norms(S); if (s != DP_OK) return s; }
+  if (phases & DP_STEP_GEMM) { s = step_gemm(S); if (s != DP_OK) return s; }
+  if (phases & DP_STEP_REST) { s = step_rest(S); if (s != DP_OK) return s; }
+  return DP_OK;
 }
 
 }  // extern "C"

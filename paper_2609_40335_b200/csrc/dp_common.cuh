@@ -188,8 +188,9 @@ constexpr int kBoundsChecked = 0;
 #endif
 
 // ---- launchers implemented across the .cu files (all enqueue on `st`, no sync) ----
-// sq[i] += factor * sum_j partials[i*n_per + j] (fixed order); plain_out[i] = that sum if given
-dp_status launch_reduce_partials(const float* partials, int n_per, int B, float* sq,
-                                 float factor, float* plain_out, cudaStream_t st);
+// sq[i] += factor * sum_j partials[i*n_per + j] (fixed order); plain_out[i] = that sum if given.
+// overwrite: sq[i] = ... instead (the first contribution to an accumulator nobody zeroed)
+dp_status launch_reduce_partials(const float* partials, int n_per, int B, float* sq, float factor,
+                                 float* plain_out, cudaStream_t st, bool overwrite = false);
 
 }  // namespace dpg

@@ -13,7 +13,7 @@ namespace {
 template <typename T>
 __global__ void ghost_norm_fma_kernel(const T* __restrict__ A, long long lda, int d,
                                       const T* __restrict__ G, long long ldg, int p, int Tn,
-                                      float* __restrict__ sq) {
+                                      float* __restrict__ sq, int overwrite) {
   __shared__ float red[32];
   const int i = blockIdx.x;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -38,13 +38,13 @@ __global__ void ghost_norm_fma_kernel(const T* __restrict__ A, long long lda, in
     acc += (t == s ? 1.f : 2.f) * da * dg;
   }
   const float tot = block_sum(lane == 0 ? acc : 0.f, red);
-  if (threadIdx.x == 0) sq[i] += tot;
+  if (threadIdx.x == 0) sq[i] = (overwrite ? 0.f : sq[i]) + tot;
 }
 
 template <typename T>
 __global__ void direct_norm_fma_kernel(const T* __restrict__ A, long long lda, int d,
                                        const T* __restrict__ G, long long ldg, int p, int Tn,
-                                       float* __restrict__ sq) {
+                                       float* __restrict__ sq, int overwrite) {
   __shared__ float red[32];
   const int i = blockIdx.x;
   const T* Ai = A + size_t(i) * Tn * lda;
@@ -58,7 +58,7 @@ __global__ void direct_norm_fma_kernel(const T* __restrict__ A, long long lda, i
     acc = fmaf(v, v, acc);
   }
   const float tot = block_sum(acc, red);
-  if (threadIdx.x == 0) sq[i] += tot;
+  if (threadIdx.x == 0) sq[i] = (overwrite ? 0.f : sq[i]) + tot;
 }
 
 // 64 x 64 output tile per block of 256 threads, 16 token rows per shared-memory step
@@ -159,21 +159,21 @@ __global__ void clip_factors_kernel(const float* __restrict__ sq, int B, float C
 
 template <typename T>
 static dp_status norms_fma_t(const dp_linear_desc& L, int mode, int B, int Tn, float* sq,
-                             cudaStream_t st) {
+                             cudaStream_t st, int overwrite) {
   if (mode == DP_NORM_GHOST)
     ghost_norm_fma_kernel<T><<<B, 256, 0, st>>>((const T*)L.A, L.lda, L.d, (const T*)L.G, L.ldg,
-                                               L.p, Tn, sq);
+                                               L.p, Tn, sq, overwrite);
   else
     direct_norm_fma_kernel<T><<<B, 256, 0, st>>>((const T*)L.A, L.lda, L.d, (const T*)L.G, L.ldg,
-                                                L.p, Tn, sq);
+                                                L.p, Tn, sq, overwrite);
   DP_LAUNCH_OK();
   return DP_OK;
 }
 
 dp_status launch_norms_fma(const dp_linear_desc& L, dp_dtype dt, int mode, int B, int T, float* sq,
-                           cudaStream_t st) {
-  return dt == DP_F32 ? norms_fma_t<float>(L, mode, B, T, sq, st)
-                      : norms_fma_t<__nv_bfloat16>(L, mode, B, T, sq, st);
+                           cudaStream_t st, bool overwrite) {
+  return dt == DP_F32 ? norms_fma_t<float>(L, mode, B, T, sq, st, overwrite)
+                      : norms_fma_t<__nv_bfloat16>(L, mode, B, T, sq, st, overwrite);
 }
 
 dp_status launch_clip_accumulate_fma(const void* A, int64_t lda, const void* G, int64_t ldg,

@@ -7,7 +7,7 @@
 namespace dpg {
 
 dp_status launch_norms_fma(const dp_linear_desc& L, dp_dtype dt, int mode, int B, int T, float* sq,
-                           cudaStream_t st);
+                           cudaStream_t st, bool overwrite = false);
 dp_status launch_clip_accumulate_fma(const void* A, int64_t lda, const void* G, int64_t ldg,
                                      dp_dtype dt, int B, int T, int d, int p, const float* clip,
                                      float* out, int64_t ldo, float beta, cudaStream_t st);

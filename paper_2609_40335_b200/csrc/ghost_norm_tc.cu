@@ -265,7 +265,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
 
 __global__ void reduce_partials_kernel(const float* __restrict__ partials, int n_per, int B,
                                        float* __restrict__ sq, float factor,
-                                       float* __restrict__ plain_out) {
+                                       float* __restrict__ plain_out, int overwrite) {
   const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (i >= B) return;
@@ -274,19 +274,19 @@ __global__ void reduce_partials_kernel(const float* __restrict__ partials, int n
   s = warp_sum(s);
   if (lane == 0) {
     if (plain_out) plain_out[i] = s;
-    if (sq) sq[i] += factor * s;
+    if (sq) sq[i] = (overwrite ? 0.f : sq[i]) + factor * s;
   }
 }
 
 }  // namespace
 
 dp_status launch_reduce_partials(const float* partials, int n_per, int B, float* sq,
-                                 float factor, float* plain_out, cudaStream_t st) {
+                                 float factor, float* plain_out, cudaStream_t st, bool overwrite) {
   if (first_use_on_this_device(reinterpret_cast<const void*>(&launch_reduce_partials)))
     DP_CUDA_OK(prefer_max_shared(reduce_partials_kernel));
   const int warps = 4;
   reduce_partials_kernel<<<ceil_div(B, warps), warps * 32, 0, st>>>(partials, n_per, B, sq,
-                                                                  factor, plain_out);
+                                                                  factor, plain_out, overwrite ? 1 : 0);
   DP_LAUNCH_OK();
   return DP_OK;
 }

@@ -300,31 +300,6 @@ def clip_noise_phase(ds: DeviceStep, seed: int, step: int, scale: float = 1.0, s
     _clip_vectors(ds, 0.0, noise=(seed, step, scale), stream=stream)
 
 
-def prefill_embedding_noise(ds: DeviceStep, seed: int, step: int, scale: float = 1.0,
-                            after: Optional[torch.cuda.Event] = None) -> torch.cuda.Event:
-    """Start the noise fill of the embedding tables on a side stream.  The fill depends on no
-    gradient, so it overlaps the (HBM-bound) norm phase; returns the event to wait for.
-    after: event that orders the fill behind the previous users of the tables (default: all
-    work enqueued so far on the current stream)."""
-    if ds.side_stream is None:
-        ds.side_stream = torch.cuda.Stream(device=ds.sq.device)
-    main = torch.cuda.current_stream()
-    tid = tensor_ids(ds)
-    side = ds.side_stream
-    if after is not None:
-        side.wait_event(after)
-    else:
-        side.wait_stream(main)                   # previous step's readers of the tables are done
-    names = ["wpe"] if ds.positions else []
-    if not (ds.tied and ds.lm is not None):
-        names.append("wte")                      # tied: the head GEMM writes the table first
-    for name in names:
-        dp.dp_fill_noise(ds.outs[name], ds.sigma, ds.C, scale, seed, tid[name], step, stream=side)
-    ev = torch.cuda.Event()
-    ev.record(side)
-    return ev
-
-
 def prefill_all_noise(ds: DeviceStep, seed: int, step: int) -> torch.cuda.Event:
     """Fill EVERY output tensor with its noise on the side stream (scale 1).  The fills are
     ALU-bound and depend on no gradient, the norm phase is HBM-bound: they share the SMs."""
@@ -359,51 +334,24 @@ def clip_onto_noise(ds: DeviceStep, filled: torch.cuda.Event) -> None:
     _clip_vectors(ds, 1.0)
 
 
-def clip_after_prefill(ds: DeviceStep, seed: int, step: int, filled: torch.cuda.Event,
-                       scale: float = 1.0, gemm_events=None) -> None:
-    """Clipped sums when the embedding tables already hold their noise (see prefill).
-    gemm_events: optional (start, stop) CUDA events recorded around the grouped GEMM call."""
-    kw = dict(ws=ds.ws, dev_status=ds.dev_status)
-    tid = tensor_ids(ds)
-    layers = list(ds.linears)
-    names = [f"linear{k}" for k in range(len(ds.linears))]
-    if ds.lm is not None:
-        layers.append(ds.lm)
-        names.append("wte" if ds.tied else "lm_head")
-    if layers:
-        if gemm_events:
-            gemm_events[0].record(torch.cuda.current_stream())
-        # sq=None: ds.clip already holds the factors (overlapped_norms computed them)
-        dp.dp_clip_accumulate_noise_grouped(layers, ds.B, ds.T, None, ds.C, [ds.outs[n] for n in names],
-                                            ds.sigma, scale, seed, [tid[n] for n in names], step,
-                                            beta=0.0, clip=ds.clip, **kw)
-        if gemm_events:
-            gemm_events[1].record(torch.cuda.current_stream())
-    torch.cuda.current_stream().wait_event(filled)
-    # beta = 1: rows are added onto the noise (untied) or onto head sum + noise (tied); the token
-    # sorts were made beside the norm phase
-    sb = ds.side
-    dp.dp_clip_accumulate_embed_sorted(ds.ids, ds.G_emb, ds.V, None, ds.C, ds.outs["wte"], sb["perm"],
-                                       sb["seg"], beta=1.0, d=ds.d_model, clip=ds.clip, **kw)
-    if ds.positions:
-        dp.dp_clip_accumulate_embed_sorted(ds.pos_ids, ds.G_emb, WPE_ROWS, None, ds.C, ds.outs["wpe"],
-                                           sb["pos_perm"], sb["pos_seg"], beta=1.0, d=ds.d_model,
-                                           clip=ds.clip, **kw)
-    _clip_vectors(ds, 0.0, noise=(seed, step, scale), factors=True)
-
-
 def _side_buffers(ds: DeviceStep) -> dict:
     """Buffers of the side stream (allocated once): it runs beside the main stream, so it needs its
     own workspace and its own norm accumulator; the token sorts it makes are kept for the scatter."""
     if ds.side is None:
         dev = ds.sq.device
         L = dp.load()
-        rows = max(ds.V, WPE_ROWS if ds.positions else 0)
-        need = max(int(L.dp_embed_norms_ws_bytes(ds.B, ds.T, ds.d_model)),
-                   int(L.dp_embed_sort_ws_bytes(ds.B, ds.T, rows)), 256)
+        need = max(256, int(L.dp_embed_norms_ws_bytes(ds.B, ds.T, ds.d_model)))
+        for rows in [ds.V] + ([WPE_ROWS] if ds.positions else []):
+            need = max(need, int(L.dp_embed_sort_ws_bytes(ds.B, ds.T, rows)),
+                       int(L.dp_clip_accumulate_embed_ws_bytes(ds.B, ds.T, ds.d_model, rows)))
+        if ds.side_stream is None:
+            ds.side_stream = torch.cuda.Stream(device=dev)
+        events = [torch.cuda.Event() for _ in range(4)]
+        for e in events:
+            e.record(ds.side_stream)         # creates the CUDA event behind the object
         ds.side = dict(
             ws=torch.empty(need, dtype=torch.uint8, device=dev),
-            sq=torch.zeros(ds.B, dtype=torch.float32, device=dev),
+            sq=torch.zeros(ds.B, dtype=torch.float32, device=dev), events=events,
             perm=torch.empty(ds.B * ds.T, dtype=torch.int32, device=dev),
             seg=torch.empty(ds.V + 1, dtype=torch.int32, device=dev),
             pos_perm=torch.empty(ds.B * ds.T, dtype=torch.int32, device=dev) if ds.positions else None,
@@ -411,65 +359,74 @@ def _side_buffers(ds: DeviceStep) -> dict:
     return ds.side
 
 
+def _enqueue(ds: DeviceStep, seed: int, step: int, phases: int, noise: bool = True) -> None:
+    """Phases of the step through the library's one-call form (dp_step_enqueue)."""
+    sb, outs = _side_buffers(ds), ds.outs
+    names = [f"linear{k}" for k in range(len(ds.linears))]
+    vnames = [f"vector{k}" for k in range(len(ds.vectors))]
+    layers = ds.linears
+    if ds.lm is not None:
+        layers = layers + [ds.lm]
+        names.append("wte" if ds.tied else "lm_head")
+    tid = tensor_ids(ds)
+    dp.dp_step_enqueue(
+        layers, [outs[n] for n in names], [tid[n] for n in names], ds.vectors, [outs[n] for n in vnames],
+        [tid[n] for n in vnames], ids=ds.ids, G_emb=ds.G_emb, pos_ids=ds.pos_ids if ds.positions else None,
+        wte=outs["wte"], wpe=outs["wpe"] if ds.positions else None, sq=ds.sq, clip=ds.clip, norms=ds.norms,
+        cross=ds.cross, side_sq=sb["sq"], perm=sb["perm"], seg=sb["seg"], pos_perm=sb["pos_perm"],
+        pos_seg=sb["pos_seg"], ws=ds.ws, side_ws=sb["ws"], dev_status=ds.dev_status, stream=None,
+        side_stream=ds.side_stream, events=[e.cuda_event for e in sb["events"]], V=ds.V, d=ds.d_model,
+        tied=ds.tied and ds.lm is not None, noise=noise, C_=ds.C, sigma=ds.sigma, seed=seed, step=step,
+        wte_id=tid["wte"], wpe_id=tid["wpe"] if ds.positions else 0, phases=phases)
+
+
 def overlapped_norms(ds: DeviceStep, seed: int, step: int) -> torch.cuda.Event:
     """Norm phase with everything that does not need the big norm kernel running BESIDE it on a
-    side stream: the embedding norms (small kernels), the token sorts of the scatter (they need
-    only the ids) and the embedding tables' noise fill (ALU-bound, depends on no gradient).  The
-    side work is enqueued right AFTER the big kernel: measured on B200, work that is already
-    resident keeps the norm kernel's CTAs out until it ends, while work that arrives second shares
-    the SMs.  Returns the event after which the tables hold their noise and the sorts exist."""
-    main = torch.cuda.current_stream()
-    if ds.side_stream is None:
-        ds.side_stream = torch.cuda.Stream(device=ds.sq.device)
-    side, sb = ds.side_stream, _side_buffers(ds)
-    start = torch.cuda.Event()
-    start.record(main)
-    ds.sq.zero_()
-    every = ds.linears + ([ds.lm] if ds.lm else [])
-    if every:
-        dp.dp_ghost_norms(every, ds.B, ds.T, ds.sq, ws=ds.ws, dev_status=ds.dev_status)
-    # ---- side stream
-    side.wait_event(start)                       # previous step's readers of these buffers are done
-    with torch.cuda.stream(side):
-        sb["sq"].zero_()
-    kw = dict(ws=sb["ws"], dev_status=ds.dev_status, stream=side)
-    dp.dp_embed_norms(ds.ids, ds.G_emb, ds.V, sb["sq"], **kw)
-    if ds.positions:
-        dp.dp_embed_norms(ds.pos_ids, ds.G_emb, ds.T, sb["sq"], **kw)
-    normed = torch.cuda.Event()
-    normed.record(side)
-    dp.dp_embed_sort(ds.ids, ds.V, sb["perm"], sb["seg"], **kw)
-    if ds.positions:
-        dp.dp_embed_sort(ds.pos_ids, WPE_ROWS, sb["pos_perm"], sb["pos_seg"], **kw)
-    filled = prefill_embedding_noise(ds, seed, step, after=start)
-    # ---- main stream again
-    if ds.vectors:
-        dp.dp_vector_norms(ds.vectors, ds.B, ds.T, ds.sq, ws=ds.ws)
-    if ds.tied:
-        dp.dp_tied_cross_term(ds.ids, ds.G_emb, ds.lm.A, ds.lm.G, ds.V, sq=ds.sq, cross=ds.cross,
-                              d=ds.d_model, ws=ds.ws, dev_status=ds.dev_status)
-    main.wait_event(normed)
-    # join the two accumulators (one fixed order of additions: deterministic) and take Eq. 7
-    dp.dp_clip_factors_sum(ds.sq, sb["sq"], ds.C, clip=ds.clip, norms=ds.norms)
-    return filled
+    side stream: the embedding norms, the token sorts of the scatter (they need only the ids) and
+    the embedding tables' noise (ALU-bound, depends on no gradient).  clip_after_prefill completes
+    the step; it takes the returned event (the clip factors exist)."""
+    _enqueue(ds, seed, step, dp.STEP_NORMS)
+    return ds.side["events"][3]
+
+
+def clip_after_prefill(ds: DeviceStep, seed: int, step: int, filled: torch.cuda.Event,
+                       scale: float = 1.0, gemm_events=None) -> None:
+    """Clipped sums after overlapped_norms (the tables hold their noise, the sorts exist).
+    gemm_events: optional (start, stop) CUDA events recorded around the grouped GEMM call."""
+    if scale != 1.0:
+        raise ValueError("the overlapped step draws its noise at scale 1")
+    cur = torch.cuda.current_stream()
+    cur.wait_event(filled)
+    if gemm_events:
+        gemm_events[0].record(cur)
+    _enqueue(ds, seed, step, dp.STEP_GEMM)
+    if gemm_events:
+        gemm_events[1].record(cur)
+    _enqueue(ds, seed, step, dp.STEP_REST)
 
 
 def dp_step(ds: DeviceStep, seed: int = 0, step: int = 0, noise: bool = True, fused: bool = True,
             overlap: bool = True, stream=None, events=None) -> None:
     """norms -> clipped sums -> noise.
 
-    fused=True draws the linear-layer noise inside the clipped-sum GEMM; with overlap=True the
-    embedding tables' noise is filled on a side stream while the norms run (scale 1 only).
+    fused=True draws the linear-layer noise inside the clipped-sum GEMM; with overlap=True what does
+    not need the layer norms runs on a side stream beside them (on the current stream only).
     """
-    if noise and fused and overlap and stream is None:
+    if fused and overlap and stream is None:
+        if not events:
+            _enqueue(ds, seed, step, dp.STEP_ALL, noise)
+            return
         # events (optional, default path only): five CUDA events recorded at step start, after the
         # norm phase, around the grouped GEMM call and at step end
         cur = torch.cuda.current_stream()
-        if events: events[0].record(cur)
-        filled = overlapped_norms(ds, seed, step)
-        if events: events[1].record(cur)
-        clip_after_prefill(ds, seed, step, filled, gemm_events=(events[2], events[3]) if events else None)
-        if events: events[4].record(cur)
+        events[0].record(cur)
+        _enqueue(ds, seed, step, dp.STEP_NORMS, noise)
+        events[1].record(cur)
+        events[2].record(cur)
+        _enqueue(ds, seed, step, dp.STEP_GEMM, noise)
+        events[3].record(cur)
+        _enqueue(ds, seed, step, dp.STEP_REST, noise)
+        events[4].record(cur)
         return
     norms_phase(ds, stream)
     if noise and fused:
