@@ -83,9 +83,9 @@ typedef struct {
  * All layers share B, T and dt.  DP_BF16 runs on tcgen05 tensor cores.  DP_F32 layers with
  * T >= 32 and d, p >= 64 run there too: every fp32 operand is split into two bf16 terms in the
  * workspace (x = hi + lo up to 2^-17) and each product is taken as hi*hi' + hi*lo' + lo*hi' with
- * fp32 accumulation -- about 1e-5 relative, inside the 1e-4 of fp32 inputs; it needs a workspace of
- * about three times the layer's inputs (dp_ghost_norms_ws_bytes says how much; layers run one after
- * the other through it).  Smaller fp32 layers run on plain fp32 FMA kernels and need none. */
+ * fp32 accumulation -- about 1e-5 relative, inside the 1e-4 of fp32 inputs.  The workspace
+ * (dp_ghost_norms_ws_bytes) is about three times the inputs of the largest layer; as many layers as fit
+ * run together, and a larger workspace holds more.  Smaller fp32 layers run on plain fp32 FMA kernels and need none. */
 dp_status dp_ghost_norms(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt,
                          int32_t B, int32_t T, float* sq,
                          void* ws, size_t ws_bytes, int32_t* dev_status, void* stream);

@@ -142,73 +142,68 @@ static bool f32_on_tensor_cores(const dp_linear_desc& L, int T) {
   return !g_force_fma && T >= 32 && L.d >= 64 && L.p >= 64;
 }
 
-// One layer's widened operands inside a workspace: `a` and `g` (and, column form, their second
-// sides `a2`, `g2`), then whatever the kernels need behind them.
-struct SplitLayer {
-  dp_linear_desc one, other;     // descriptors of the widened bf16 operands
-  size_t bytes;                  // workspace taken by the operands
-};
-
-static SplitLayer split_layout(const dp_linear_desc& L, int B, int T, bool column_form, char* base) {
-  SplitLayer S;
-  memset(&S, 0, sizeof(S));
-  const size_t na = split_bytes((long long)B * T, L.d), ng = split_bytes((long long)B * T, L.p);
-  const int dp_ = split_padded(L.d), pp = split_padded(L.p);
-  S.one.mode = S.other.mode = DP_NORM_GHOST;
-  if (column_form) {             // (B*T, 3*padded) operands, two sides each
-    S.one.A = base; S.one.G = base + na; S.other.A = base + na + ng; S.other.G = base + 2 * na + ng;
-    S.one.d = S.other.d = 3 * dp_; S.one.p = S.other.p = 3 * pp;
-    S.one.lda = S.other.lda = 3 * dp_; S.one.ldg = S.other.ldg = 3 * pp;
-    S.bytes = 2 * (na + ng);
-  } else {                       // (B, 3T, padded) operands
-    S.one.A = base; S.one.G = base + na;
-    S.one.d = L.d; S.one.p = L.p; S.one.lda = dp_; S.one.ldg = pp;
-    S.bytes = na + ng;
-  }
-  return S;
-}
-
-static size_t f32_norm_ws_bytes(const dp_linear_desc& L, int B, int T, int mode, int sms) {
-  const bool direct = mode == DP_NORM_DIRECT;
-  SplitLayer S = split_layout(L, B, T, !direct, nullptr);
-  S.one.mode = mode;
-  const GhostPlan plan = plan_ghost_norms(&S.one, 1, B, direct ? 3 * T : T, sms, false);
-  return S.bytes + align_up(size_t(B) * plan.n_per * sizeof(float), 256);
-}
-
 static int resolve_mode(const dp_linear_desc& L, int T) {
   if (L.mode != DP_NORM_AUTO) return L.mode;
   return ((long long)T * T > (long long)L.d * L.p) ? DP_NORM_DIRECT : DP_NORM_GHOST;
 }
 
-// norm of one fp32 layer on the tensor cores; ws holds the widened operands and the partial sums
-static dp_status f32_norm_tc(const dp_linear_desc& L, int B, int T, int mode, float* sq, char* ws,
-                             int* dev_status, cudaStream_t st, bool overwrite) {
-  const bool direct = mode == DP_NORM_DIRECT;
-  SplitLayer S = split_layout(L, B, T, !direct, ws);
-  float* partials = reinterpret_cast<float*>(ws + S.bytes);
-  dp_status s;
-  const float* A = static_cast<const float*>(L.A);
-  const float* G = static_cast<const float*>(L.G);
-  if (!direct) {
-    s = launch_split_cols(A, L.lda, (int64_t)B * T, L.d, const_cast<void*>(S.one.A), const_cast<void*>(S.other.A), st);
-    if (s != DP_OK) return s;
-    s = launch_split_cols(G, L.ldg, (int64_t)B * T, L.p, const_cast<void*>(S.one.G), const_cast<void*>(S.other.G), st);
-    if (s != DP_OK) return s;
-    const GhostPlan plan = plan_ghost_norms(&S.one, 1, B, T, sm_count(), false);
-    s = launch_ghost_norm_tc(&S.one, plan, B, T, partials, dev_status, st, &S.other);
-    if (s != DP_OK) return s;
-    return launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st, overwrite);
+// Layers whose split operands share the workspace and run through the kernels together.  How many
+// there are follows from the workspace at hand: it holds the largest layer with room to spare (the
+// *_ws_bytes functions see to that), and so several ordinary layers beside a head-sized one.
+struct SplitGroup {
+  std::vector<int> index;               // into the caller's layers
+  std::vector<dp_linear_desc> desc;     // the same layers on their split operands
+  std::vector<SplitJob> jobs;
+  size_t bytes = 0;                     // workspace taken by the split operands
+  size_t bound = 0;                     // norms: by all of it, at most
+  long long tiles = 0;                  // sums: output tiles
+  size_t out_bytes = 0;                 // and one fp32 plane of every output
+
+  void add(const dp_linear_desc& L, int l, int B, int T, bool scale_g, char* base) {
+    dp_linear_desc D = L;
+    const long long rows = (long long)B * T;
+    D.mode = resolve_mode(L, T);
+    D.A = base + bytes; D.lda = split_padded(L.d);
+    jobs.push_back({static_cast<const float*>(L.A), L.lda, L.d, false, base + bytes});
+    bytes += split_bytes(rows, L.d);
+    D.G = base + bytes; D.ldg = split_padded(L.p);
+    jobs.push_back({static_cast<const float*>(L.G), L.ldg, L.p, scale_g, base + bytes});
+    bytes += split_bytes(rows, L.p);
+    index.push_back(l);
+    desc.push_back(D);
+    tiles += gta_tiles(L);
+    out_bytes += align_up(size_t(L.p) * size_t(L.d) * sizeof(float), 256);
   }
-  // DIRECT: G'^T A' per example over 3T token rows
-  s = launch_split_rows(A, L.lda, B, T, L.d, nullptr, 1, const_cast<void*>(S.one.A), st);
+};
+
+static size_t split_layer_bytes(const dp_linear_desc& L, int B, int T) {
+  return split_bytes((long long)B * T, L.d) + split_bytes((long long)B * T, L.p);
+}
+
+// What a layer takes of the workspace for its norm.  Planned alone it is cut into at least as many
+// chunks (partial sums) as in company, so the sums of these bound a group's needs.
+static size_t f32_norm_bytes(const dp_linear_desc& L, int B, int T, int sms) {
+  dp_linear_desc one = L;
+  one.mode = resolve_mode(L, T);
+  const GhostPlan plan = plan_ghost_norms(&one, 1, B, T, sms, false);
+  return split_layer_bytes(L, B, T) + align_up(size_t(B) * plan.n_per * sizeof(float), 256);
+}
+
+// norms of a group of fp32 layers: split, Gram or gradient-tile kernels, one reduction
+static dp_status f32_norm_group(const SplitGroup& g, int B, int T, float* sq, char* ws, int* dev_status,
+                                cudaStream_t st, bool overwrite) {
+  const GhostPlan plan = plan_ghost_norms(g.desc.data(), (int)g.desc.size(), B, T, sm_count(), false);
+  float* partials = reinterpret_cast<float*>(ws + g.bytes);
+  dp_status s = launch_split(g.jobs.data(), (int)g.jobs.size(), B, T, nullptr, st);
   if (s != DP_OK) return s;
-  s = launch_split_rows(G, L.ldg, B, T, L.p, nullptr, 2, const_cast<void*>(S.one.G), st);
-  if (s != DP_OK) return s;
-  S.one.mode = DP_NORM_DIRECT;
-  const GhostPlan plan = plan_ghost_norms(&S.one, 1, B, 3 * T, sm_count(), false);
-  s = launch_direct_norm_tc(&S.one, plan, B, 3 * T, partials, dev_status, st);
-  if (s != DP_OK) return s;
+  if (!plan.ghost_layers.empty()) {
+    s = launch_ghost_norm_tc(g.desc.data(), plan, B, T, partials, dev_status, st, true);
+    if (s != DP_OK) return s;
+  }
+  if (!plan.direct_layers.empty()) {
+    s = launch_direct_norm_tc(g.desc.data(), plan, B, T, 3, partials, dev_status, st);
+    if (s != DP_OK) return s;
+  }
   return launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st, overwrite);
 }
 
@@ -290,7 +285,7 @@ size_t dp_ghost_norms_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, d
     size_t need = 0;
     for (int l = 0; l < n_layers; ++l)
       if (f32_on_tensor_cores(layers[l], T))
-        need = std::max(need, f32_norm_ws_bytes(layers[l], B, T, resolve_mode(layers[l], T), sm_count()));
+        need = std::max(need, f32_norm_bytes(layers[l], B, T, sm_count()) + 2 * split_layer_bytes(layers[l], B, T));
     return need;
   }
   const GhostPlan plan = plan_ghost_norms(layers, n_layers, B, T, sm_count());
@@ -312,19 +307,32 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
   const GhostPlan plan = plan_ghost_norms(layers, n_layers, B, T, sm_count());
   if (!tc) {
     if (dt == DP_F32 && dp_ghost_norms_ws_bytes(layers, n_layers, dt, B, T) > ws_bytes) return DP_ERR_WORKSPACE;
+    SplitGroup group;
+    char* base = static_cast<char*>(ws);
+    auto flush = [&]() {
+      if (group.index.empty()) return DP_OK;
+      const dp_status s = f32_norm_group(group, B, T, sq, base, dev_status, st, overwrite);
+      overwrite = false;
+      group = SplitGroup();
+      return s;
+    };
     for (int l = 0; l < n_layers; ++l) {
-      dp_status s;
+      dp_status s = DP_OK;
       if (dt == DP_F32 && f32_on_tensor_cores(layers[l], T)) {
         if (!ws || !aligned16(ws)) return DP_ERR_WORKSPACE;
-        s = f32_norm_tc(layers[l], B, T, plan.mode_used[l], sq, static_cast<char*>(ws), dev_status, st, overwrite);
+        const size_t more = f32_norm_bytes(layers[l], B, T, sm_count());
+        if (group.bound + more > ws_bytes) s = flush();
+        if (s != DP_OK) return s;
+        group.bound += more;
+        group.add(layers[l], l, B, T, false, base);
       } else {
         s = launch_norms_fma(layers[l], dt, plan.mode_used[l], B, T, sq, st, overwrite);
+        overwrite = false;
       }
       if (s != DP_OK) return s;
-      overwrite = false;
       layers[l].mode_used = plan.mode_used[l];
     }
-    return DP_OK;
+    return flush();
   }
   const size_t need = align_up(size_t(B) * plan.n_per * sizeof(float), 256);
   if (!ws || ws_bytes < need) return DP_ERR_WORKSPACE;
@@ -336,7 +344,7 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
     if (s != DP_OK) return s;
   }
   if (!plan.direct_layers.empty()) {
-    s = launch_direct_norm_tc(layers, plan, B, T, partials, dev_status, st);
+    s = launch_direct_norm_tc(layers, plan, B, T, 1, partials, dev_status, st);
     if (s != DP_OK) return s;
   }
   s = launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st, overwrite);
@@ -504,14 +512,13 @@ size_t dp_clip_accumulate_grouped_ws_bytes(const dp_linear_desc* layers, int32_t
                                            dp_dtype dt, int32_t B, int32_t T) {
   if (!layers || n_layers <= 0 || B <= 0 || T <= 0) return 0;
   size_t n = align_up(size_t(B) * sizeof(float), 256);          // clip factors
-  if (dt == DP_BF16 && !g_force_fma) n += gta_partial_bytes(layers, n_layers, B, T, sm_count());
-  if (dt == DP_F32) {            // widened operands of one layer at a time + its K-split planes
+  if (dt == DP_BF16 && !g_force_fma) n += gta_partial_bytes(layers, n_layers, B, T, 1, sm_count());
+  if (dt == DP_F32) {            // split operands of the largest layer, half as much again, and its K-split planes
     size_t need = 0;
     for (int l = 0; l < n_layers; ++l)
-      if (f32_on_tensor_cores(layers[l], T)) {
-        SplitLayer S = split_layout(layers[l], B, T, false, nullptr);
-        need = std::max(need, S.bytes + gta_partial_bytes(&S.one, 1, B, 3 * T, sm_count()));
-      }
+      if (f32_on_tensor_cores(layers[l], T))
+        need = std::max(need, split_layer_bytes(layers[l], B, T) * 3 / 2 +
+                                  gta_partial_bytes(layers + l, 1, B, T, 3, sm_count()));
     n += need;
   }
   return n;
@@ -540,23 +547,38 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
   dp_status s = resolve_clip(sq, B, C, clip, &clip_ws, st);
   if (s != DP_OK) return s;
   if (!tc) {
-    char* split_ws = static_cast<char*>(ws) + align_up(size_t(B) * sizeof(float), 256);
+    const size_t head = align_up(size_t(B) * sizeof(float), 256);
+    char* base = static_cast<char*>(ws) + head;
+    SplitGroup group;
+    auto flush = [&]() {
+      if (group.index.empty()) return DP_OK;
+      // R_i multiplies G in fp32 before the split, so the GEMM runs unscaled (clip = NULL)
+      dp_status s = launch_split(group.jobs.data(), (int)group.jobs.size(), B, T, clip_ws, st);
+      if (s != DP_OK) return s;
+      std::vector<float*> out;
+      std::vector<int64_t> ldo;
+      std::vector<uint32_t> ids;
+      for (int l : group.index) {
+        out.push_back(outs[l]); ldo.push_back(ldos[l]);
+        if (noise) ids.push_back(noise->tensor_ids[l]);
+      }
+      GtaNoise nz;
+      if (noise) { nz = *noise; nz.tensor_ids = ids.data(); }
+      s = launch_clip_accumulate_tc(group.desc.data(), (int)group.desc.size(), B, T, 3, nullptr, out.data(),
+                                    ldo.data(), beta, noise ? &nz : nullptr,
+                                    reinterpret_cast<float*>(base + group.bytes), dev_status, st);
+      group = SplitGroup();
+      return s;
+    };
     for (int l = 0; l < n_layers; ++l) {
       if (dt == DP_F32 && f32_on_tensor_cores(layers[l], T)) {
-        // R_i multiplies G in fp32 before the split, so the GEMM runs unscaled (clip = NULL)
-        SplitLayer S = split_layout(layers[l], B, T, false, split_ws);
-        s = launch_split_rows(static_cast<const float*>(layers[l].A), layers[l].lda, B, T, layers[l].d,
-                              nullptr, 1, const_cast<void*>(S.one.A), st);
+        // the K split, and with it the planes of partial sums, follows from the group's tiles
+        const size_t out = align_up(size_t(layers[l].p) * size_t(layers[l].d) * sizeof(float), 256);
+        const int ns = gta_choose_nsplit(group.tiles + gta_tiles(layers[l]), B, T, 3, sm_count());
+        const size_t planes = ns > 1 ? size_t(ns) * (group.out_bytes + out) : 0;
+        if (head + group.bytes + split_layer_bytes(layers[l], B, T) + planes > ws_bytes) s = flush();
         if (s != DP_OK) return s;
-        s = launch_split_rows(static_cast<const float*>(layers[l].G), layers[l].ldg, B, T, layers[l].p,
-                              clip_ws, 2, const_cast<void*>(S.one.G), st);
-        if (s != DP_OK) return s;
-        GtaNoise one_noise;
-        if (noise) { one_noise = *noise; one_noise.tensor_ids = noise->tensor_ids + l; }
-        s = launch_clip_accumulate_tc(&S.one, 1, B, 3 * T, nullptr, outs + l, ldos + l, beta,
-                                      noise ? &one_noise : nullptr,
-                                      reinterpret_cast<float*>(split_ws + S.bytes), dev_status, st);
-        if (s != DP_OK) return s;
+        group.add(layers[l], l, B, T, true, base);
         continue;
       }
       s = launch_clip_accumulate_fma(layers[l].A, layers[l].lda, layers[l].G, layers[l].ldg, dt, B, T,
@@ -568,11 +590,11 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
         if (s != DP_OK) return s;
       }
     }
-    return DP_OK;
+    return flush();
   }
   float* partial = reinterpret_cast<float*>(static_cast<char*>(ws) +
                                             align_up(size_t(B) * sizeof(float), 256));
-  return launch_clip_accumulate_tc(layers, n_layers, B, T, clip_ws, outs, ldos, beta, noise, partial,
+  return launch_clip_accumulate_tc(layers, n_layers, B, T, 1, clip_ws, outs, ldos, beta, noise, partial,
                                    dev_status, st);
 }
 

@@ -32,18 +32,21 @@ struct GtaNoise {
   const uint32_t* tensor_ids;   // [n_layers]
 };
 
-int gta_choose_nsplit(const dp_linear_desc* layers, int n_layers, int B, int T, int sms);
-// scratch of a grouped call behind the clip factors: K-split planes (if any) and the pre-scaled
-// copies of very narrow operands
-size_t gta_partial_bytes(const dp_linear_desc* layers, int n_layers, int B, int T, int sms);
+// terms = 3: the operands are (2B, T, .) planes of high and low bf16 terms (fp32 inputs) and a product
+// takes three K steps per 64 tokens; terms = 1: plain bf16 operands.
+long long gta_tiles(const dp_linear_desc& L);           // output tiles of one layer
+int gta_choose_nsplit(long long tiles, int B, int T, int terms, int sms);
+// scratch of a grouped call behind the clip factors: K-split planes (if any) and, terms = 1, the
+// pre-scaled copies of very narrow operands
+size_t gta_partial_bytes(const dp_linear_desc* layers, int n_layers, int B, int T, int terms, int sms);
 
 // One persistent launch over the output tiles of all layers (plus split-K reduces if needed).
-dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, int B, int T,
+dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, int B, int T, int terms,
                                     const float* clip, float* const* outs, const int64_t* ldos,
                                     float beta, const GtaNoise* noise, float* partial_ws,
                                     int* dev_status, cudaStream_t st);
 
-dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
+dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T, int terms,
                                 float* partials, int* dev_status, cudaStream_t st);
 
 }  // namespace dpg

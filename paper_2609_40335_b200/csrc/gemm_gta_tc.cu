@@ -71,7 +71,8 @@ struct __align__(64) GtaParams {
   CUtensorMap tmA[kGtaMaxLayers];
   GtaLayer layer[kGtaMaxLayers];
   int n_layers;
-  int B, T, tsteps;          // tsteps = ceil(T / 64) K steps per example
+  int B, T, tsteps;          // tsteps = terms * ceil(T / 64) K steps per example
+  int terms;                 // 3: split fp32 operands (hi hi, hi lo, lo hi per 64 tokens), else 1
   int nsplit, ksteps_per_split;   // K splits, the same for all layers of a call
   float beta;
   int total_items;
@@ -194,16 +195,23 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
         // first column of this CTA's part of the tile: its G rows, or its share of the A columns
         const int c0 = is_a ? it.tn * kBN + int(rank) * Geo<kPair>::kAColsPerCta
                             : it.tm * kTileM + int(rank) * kBM;
-        int ex = it.k0 / P.tsteps, ts = it.k0 - ex * P.tsteps;
+        // K step -> example, token block and (split operands) which of the three products
+        int ex = it.k0 / P.tsteps, ts = it.k0 - ex * P.tsteps, term = 0;
+        const int terms = P.terms, low_term = is_a ? 1 : 2, tblocks = P.tsteps / terms;
+        if (terms > 1) { term = ts % terms; ts /= terms; }
         for (int ks = it.k0; ks < it.k1; ++ks) {
           if (!ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
           const uint32_t bar = full_a + 8 * stage;
           const uint32_t dst = tiles_a + stage * kStageBytes + (is_a ? kGBytes : 0);
           ptx::mbar_arrive_expect_tx_a(bar, my_bytes);
           for (int j = 0; j < nbox; ++j)
-            ptx::tma_load_3d_a(dst + j * kBoxBytes, tm, bar, c0 + j * 64, ts * kBK, ex);
+            ptx::tma_load_3d_a(dst + j * kBoxBytes, tm, bar, c0 + j * 64, ts * kBK,
+                               terms > 1 ? 2 * ex + (term == low_term) : ex);
           ++issued;
-          if (++ts == P.tsteps) { ts = 0; ++ex; }
+          if (++term == terms) {
+            term = 0;
+            if (++ts == tblocks) { ts = 0; ++ex; }
+          }
           if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
       }
@@ -584,11 +592,18 @@ dp_status launch_gta(const GtaParams& P, int units, cudaStream_t st) {
 
 // K-split factor shared by all layers of one grouped call: 1 when the output tiles alone give
 // every SM at least two items, otherwise enough splits to get there (>= 4 K steps per split).
-int gta_choose_nsplit(const dp_linear_desc* layers, int n_layers, int B, int T, int sms) {
+long long gta_tiles(const dp_linear_desc& L) {
+  return (long long)ceil_div(L.p, Geo<kUsePair>::kTileM) * ceil_div(L.d, kBN);
+}
+
+static long long gta_tiles(const dp_linear_desc* layers, int n_layers) {
   long long tiles = 0;
-  for (int l = 0; l < n_layers; ++l)
-    tiles += (long long)ceil_div(layers[l].p, Geo<kUsePair>::kTileM) * ceil_div(layers[l].d, kBN);
-  const int ksteps = B * ceil_div(T, kBK);
+  for (int l = 0; l < n_layers; ++l) tiles += gta_tiles(layers[l]);
+  return tiles;
+}
+
+int gta_choose_nsplit(long long tiles, int B, int T, int terms, int sms) {
+  const int ksteps = B * terms * ceil_div(T, kBK);
   const int units = kUsePair ? sms / 2 : sms;          // persistent CTAs or CTA pairs
   if (tiles >= 2LL * units) return 1;
   long long ns = std::max<long long>(1, (2LL * units) / std::max<long long>(tiles, 1));
@@ -596,26 +611,26 @@ int gta_choose_nsplit(const dp_linear_desc* layers, int n_layers, int B, int T, 
   return (int)std::max<long long>(1, ns);
 }
 
-size_t gta_partial_bytes(const dp_linear_desc* layers, int n_layers, int B, int T, int sms) {
-  const int ns = gta_choose_nsplit(layers, n_layers, B, T, sms);
+size_t gta_partial_bytes(const dp_linear_desc* layers, int n_layers, int B, int T, int terms, int sms) {
+  const int ns = gta_choose_nsplit(gta_tiles(layers, n_layers), B, T, terms, sms);
   size_t n = 0;
   for (int l = 0; l < n_layers; ++l) {
     if (ns > 1) n += align_up(size_t(ns) * size_t(layers[l].p) * size_t(layers[l].d) * sizeof(float), 256);
-    if (prescale_layer(layers[l])) n += prescale_bytes(layers[l], B, T);
+    if (terms == 1 && prescale_layer(layers[l])) n += prescale_bytes(layers[l], B, T);
   }
   return n;
 }
 
-dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, int B, int T,
+dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, int B, int T, int terms,
                                     const float* clip, float* const* outs, const int64_t* ldos,
                                     float beta, const GtaNoise* noise, float* partial_ws,
                                     int* dev_status, cudaStream_t st) {
   dp_status s = set_attr_once<kClipScale, false, kUsePair>();
   if (s != DP_OK) return s;
   const int sms = sm_count();
-  const int tsteps = ceil_div(T, kBK);
+  const int tsteps = terms * ceil_div(T, kBK), planes = terms > 1 ? 2 * B : B;
   const int ksteps = B * tsteps;
-  int nsplit = gta_choose_nsplit(layers, n_layers, B, T, sms);
+  int nsplit = gta_choose_nsplit(gta_tiles(layers, n_layers), B, T, terms, sms);
   const int kps = ceil_div(ksteps, nsplit);
   nsplit = ceil_div(ksteps, kps);                       // drop empty trailing splits
   char* pw = reinterpret_cast<char*>(partial_ws);
@@ -647,9 +662,9 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
         if (narrow_a) { D.A = copy; D.lda = cp; } else { D.G = copy; D.ldg = cp; }
         L.prescaled = 1;
       }
-      s = make_tmap_bf16_3d(&P.tmG[g - g0], D.G, D.ldg, D.p, T, B, 64, kBK);
+      s = make_tmap_bf16_3d(&P.tmG[g - g0], D.G, D.ldg, D.p, T, planes, 64, kBK);
       if (s != DP_OK) return s;
-      s = make_tmap_bf16_3d(&P.tmA[g - g0], D.A, D.lda, D.d, T, B, 64, kBK);
+      s = make_tmap_bf16_3d(&P.tmA[g - g0], D.A, D.lda, D.d, T, planes, 64, kBK);
       if (s != DP_OK) return s;
       L.out = outs[g]; L.ldo = ldos[g];
       L.M = D.p; L.N = D.d;
@@ -671,7 +686,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
       P.noise_step = noise->step; P.noise_scale = noise->scale;
       P.step_dev = g_step_dev;
     }
-    P.n_layers = g1 - g0; P.B = B; P.T = T; P.tsteps = tsteps;
+    P.n_layers = g1 - g0; P.B = B; P.T = T; P.tsteps = tsteps; P.terms = terms;
     P.total_items = items;
     P.nsplit = nsplit; P.ksteps_per_split = kps; P.beta = beta;
     P.clip = clip;
@@ -700,11 +715,11 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
 }
 
 
-dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
+dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T, int terms,
                                 float* partials, int* dev_status, cudaStream_t st) {
   dp_status s = set_attr_once<false, true, false>();
   if (s != DP_OK) return s;
-  const int sms = sm_count();
+  const int sms = sm_count(), planes = terms > 1 ? 2 * B : B;
   for (size_t g0 = 0; g0 < plan.direct_layers.size(); g0 += kGtaMaxLayers) {
     const size_t g1 = std::min(plan.direct_layers.size(), g0 + kGtaMaxLayers);
     GtaParams P;
@@ -713,9 +728,9 @@ dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& p
     for (size_t g = g0; g < g1; ++g) {
       const int li = plan.direct_layers[g];
       const dp_linear_desc& D = layers[li];
-      s = make_tmap_bf16_3d(&P.tmG[g - g0], D.G, D.ldg, D.p, T, B, 64, kBK);
+      s = make_tmap_bf16_3d(&P.tmG[g - g0], D.G, D.ldg, D.p, T, planes, 64, kBK);
       if (s != DP_OK) return s;
-      s = make_tmap_bf16_3d(&P.tmA[g - g0], D.A, D.lda, D.d, T, B, 64, kBK);
+      s = make_tmap_bf16_3d(&P.tmA[g - g0], D.A, D.lda, D.d, T, planes, 64, kBK);
       if (s != DP_OK) return s;
       GtaLayer& L = P.layer[g - g0];
       L.M = D.p; L.N = D.d;
@@ -724,7 +739,7 @@ dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& p
       items += B * plan.direct[li].tiles_m * plan.direct[li].tiles_n;
     }
     P.n_layers = int(g1 - g0);
-    P.B = B; P.T = T; P.tsteps = ceil_div(T, kBK);
+    P.B = B; P.T = T; P.tsteps = terms * ceil_div(T, kBK); P.terms = terms;
     P.total_items = items;
     P.nsplit = 1;
     P.sq_partials = partials; P.n_per = plan.n_per;

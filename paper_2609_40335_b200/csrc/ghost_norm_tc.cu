@@ -32,11 +32,13 @@ constexpr int kKStep = 64;                       // bf16 columns per stage row (
 constexpr int kTileBytes = kTile * kKStep * 2;   // 16 KiB
 // A stage holds row tile ti and, for off-diagonal tile pairs, row tile tj.  When T <= 128 every
 // pair is diagonal, so stages shrink to one tile and twice as many are kept in flight (the
-// kernel is HBM-bound there: bytes in flight are what counts).
-template <bool kDiagOnly>
+// kernel is HBM-bound there: bytes in flight are what counts).  Split operands (fp32 inputs) bring
+// two tiles, high and low terms, for each.
+template <bool kDiagOnly, bool kSplit>
 struct GhostGeo {
-  static constexpr int kStageBytes = kDiagOnly ? kTileBytes : 2 * kTileBytes;
-  static constexpr int kStages = kDiagOnly ? 12 : 6;
+  static constexpr int kTermBytes = (kSplit ? 2 : 1) * kTileBytes;       // one row tile, all its terms
+  static constexpr int kStageBytes = (kDiagOnly ? 1 : 2) * kTermBytes;
+  static constexpr int kStages = 12 * kTileBytes / kStageBytes;
   static constexpr size_t kSmemBytes = size_t(kStages) * kStageBytes + 1024 /*alignment slack*/ + 512;
 };
 constexpr int kThreads = 192;
@@ -86,16 +88,15 @@ __device__ __forceinline__ Item decode_item(const GhostParams& P, int item, int&
   return it;
 }
 
-// kDual: the two sides of each Gram product come from two different tensors (maps 2l and 2l+1 of
-// a layer): the fp32 path, where S = X Y^T with X = [hi | hi | lo] and Y = [hi | lo | hi] of the
-// operand split into two bf16 terms.  S is still symmetric, so tile pairs are enumerated as before,
-// but a diagonal pair also needs both loads.
-template <bool kDiagOnly, bool kDual = false>
+// kSplit: fp32 operands stored as two bf16 planes per example (see split_kernels.cu).  Every Gram
+// tile is then S = hi hi^T + hi lo^T + lo hi^T, three MMAs per K step on tiles loaded once.
+template <bool kDiagOnly, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
-  static_assert(!(kDiagOnly && kDual), "the two-tensor form always loads two tiles per stage");
-  constexpr int kStages = GhostGeo<kDiagOnly>::kStages;
-  constexpr int kStageBytes = GhostGeo<kDiagOnly>::kStageBytes;
+  using Geo = GhostGeo<kDiagOnly, kSplit>;
+  constexpr int kStages = Geo::kStages;
+  constexpr int kStageBytes = Geo::kStageBytes;
+  constexpr int kTermBytes = Geo::kTermBytes;
   extern __shared__ uint8_t smem_raw[];
   // 128-byte swizzled tiles need 1024-byte alignment
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -139,21 +140,23 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
       bool ok = true;
       for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x) {
         const Item it = decode_item(P, item, lay);
-        const bool diag = !kDual && (kDiagOnly || (it.ti == it.tj));
-        const uint32_t bytes = diag ? kTileBytes : kStageBytes;
-        const int li = kDual ? 2 * it.layer : it.layer;
+        const bool diag = kDiagOnly || (it.ti == it.tj);
+        const uint32_t bytes = diag ? kTermBytes : kStageBytes;
+        const int ex = kSplit ? 2 * it.example : it.example;     // (high) plane of the example
         for (int pass = 0; pass < 2 && ok; ++pass) {
-          const CUtensorMap* tm = pass == 0 ? &P.tmA[li] : &P.tmG[li];
-          const CUtensorMap* tm2 = kDual ? tm + 1 : tm;     // the other side of the product
+          const CUtensorMap* tm = pass == 0 ? &P.tmA[it.layer] : &P.tmG[it.layer];
           const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
           for (int k = k0; k < k1; ++k) {
             if (!ptx::mbar_wait(&empty[stage], phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
             uint8_t* dst = tiles + size_t(stage) * kStageBytes;
             ptx::mbar_arrive_expect_tx(&full[stage], bytes);
-            ptx::tma_load_3d(dst, tm, &full[stage], k * kKStep, it.ti * kTile, it.example);
-            if (!diag)
-              ptx::tma_load_3d(dst + kTileBytes, tm2, &full[stage], k * kKStep, it.tj * kTile,
-                               it.example);
+            ptx::tma_load_3d(dst, tm, &full[stage], k * kKStep, it.ti * kTile, ex);
+            if (kSplit) ptx::tma_load_3d(dst + kTileBytes, tm, &full[stage], k * kKStep, it.ti * kTile, ex + 1);
+            if (!diag) {
+              ptx::tma_load_3d(dst + kTermBytes, tm, &full[stage], k * kKStep, it.tj * kTile, ex);
+              if (kSplit)
+                ptx::tma_load_3d(dst + kTermBytes + kTileBytes, tm, &full[stage], k * kKStep, it.tj * kTile, ex + 1);
+            }
             ++issued;
             if (++stage == kStages) { stage = 0; phase ^= 1; }
           }
@@ -176,7 +179,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
       bool ok = true;
       for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x, ++n_item) {
         const Item it = decode_item(P, item, lay);
-        const bool diag = !kDual && (kDiagOnly || (it.ti == it.tj));
+        const bool diag = kDiagOnly || (it.ti == it.tj);
         const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
         if (!ptx::mbar_wait(&acc_empty[buf], acc_phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
         ptx::tc_fence_after();
@@ -187,13 +190,16 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
             if (!ptx::mbar_wait(&full[stage], phase, abort_flag, P.wait_limit)) { ok = false; break; }
             ptx::tc_fence_after();
             const uint32_t sa = ptx::smem_u32(tiles + size_t(stage) * kStageBytes);
-            const uint32_t sb = diag ? sa : sa + kTileBytes;
+            const uint32_t sb = diag ? sa : sa + kTermBytes;
 #pragma unroll
             for (int kk = 0; kk < kKStep / 16; ++kk) {
               // 16 bf16 = 32 bytes further along K inside the swizzle atom
-              ptx::mma_bf16_ss(d_tmem, ptx::smem_desc(dbase, sa + kk * 32),
-                               ptx::smem_desc(dbase, sb + kk * 32), idesc,
-                               (k > 0 || kk > 0) ? 1u : 0u);
+              const uint64_t ah = ptx::smem_desc(dbase, sa + kk * 32), bh = ptx::smem_desc(dbase, sb + kk * 32);
+              ptx::mma_bf16_ss(d_tmem, ah, bh, idesc, (k > 0 || kk > 0) ? 1u : 0u);
+              if (kSplit) {
+                ptx::mma_bf16_ss(d_tmem, ah, ptx::smem_desc(dbase, sb + kTileBytes + kk * 32), idesc, 1u);
+                ptx::mma_bf16_ss(d_tmem, ptx::smem_desc(dbase, sa + kTileBytes + kk * 32), bh, idesc, 1u);
+              }
             }
             ptx::mma_commit(&empty[stage]);          // stage reusable once these MMAs retire
             if (++stage == kStages) { stage = 0; phase ^= 1; }
@@ -291,46 +297,41 @@ dp_status launch_reduce_partials(const float* partials, int n_per, int B, float*
   return DP_OK;
 }
 
+namespace {
+
+template <bool kDiagOnly, bool kSplit>
+dp_status launch_variant(const GhostParams& P, cudaStream_t st) {
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_tc_kernel<kDiagOnly, kSplit>)))
+    DP_CUDA_OK(cudaFuncSetAttribute(ghost_norm_tc_kernel<kDiagOnly, kSplit>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)GhostGeo<kDiagOnly, kSplit>::kSmemBytes));
+  const int grid = std::min(P.total_items, sm_count());
+  ghost_norm_tc_kernel<kDiagOnly, kSplit><<<grid, kThreads, GhostGeo<kDiagOnly, kSplit>::kSmemBytes, st>>>(P);
+  DP_LAUNCH_OK();
+  return DP_OK;
+}
+
+}  // namespace
+
 // Enqueue the tensor-core ghost norm for the planned layers; partial sums land in
 // plan.partials layout inside `partials` (the caller reduces them afterwards).
 dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
-                               float* partials, int* dev_status, cudaStream_t st,
-                               const dp_linear_desc* other_side) {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&launch_ghost_norm_tc))) {
-    DP_CUDA_OK(cudaFuncSetAttribute(ghost_norm_tc_kernel<true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)GhostGeo<true>::kSmemBytes));
-    DP_CUDA_OK(cudaFuncSetAttribute(ghost_norm_tc_kernel<false>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)GhostGeo<false>::kSmemBytes));
-    DP_CUDA_OK(cudaFuncSetAttribute(ghost_norm_tc_kernel<false, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)GhostGeo<false>::kSmemBytes));
-  }
-  const bool dual = other_side != nullptr;
-  const size_t per_launch = dual ? kGhostMaxLayers / 2 : kGhostMaxLayers;
+                               float* partials, int* dev_status, cudaStream_t st, bool split) {
   const int nt = ceil_div(T, kTile);
+  const int planes = split ? 2 * B : B;
   // layers are processed in groups that fit one parameter block
-  for (size_t g0 = 0; g0 < plan.ghost_layers.size(); g0 += per_launch) {
-    const size_t g1 = std::min(plan.ghost_layers.size(), g0 + per_launch);
+  for (size_t g0 = 0; g0 < plan.ghost_layers.size(); g0 += kGhostMaxLayers) {
+    const size_t g1 = std::min(plan.ghost_layers.size(), g0 + kGhostMaxLayers);
     GhostParams P;
     memset(&P, 0, sizeof(P));
     int items = 0;
     for (size_t g = g0; g < g1; ++g) {
       const int li = plan.ghost_layers[g];
       const dp_linear_desc& L = layers[li];
-      const size_t slot = dual ? 2 * (g - g0) : (g - g0);
-      dp_status s = make_tmap_bf16_3d(&P.tmA[slot], L.A, L.lda, L.d, T, B, kKStep, kTile);
+      dp_status s = make_tmap_bf16_3d(&P.tmA[g - g0], L.A, L.lda, L.d, T, planes, kKStep, kTile);
       if (s != DP_OK) return s;
-      s = make_tmap_bf16_3d(&P.tmG[slot], L.G, L.ldg, L.p, T, B, kKStep, kTile);
+      s = make_tmap_bf16_3d(&P.tmG[g - g0], L.G, L.ldg, L.p, T, planes, kKStep, kTile);
       if (s != DP_OK) return s;
-      if (dual) {
-        const dp_linear_desc& R = other_side[li];
-        s = make_tmap_bf16_3d(&P.tmA[slot + 1], R.A, R.lda, R.d, T, B, kKStep, kTile);
-        if (s != DP_OK) return s;
-        s = make_tmap_bf16_3d(&P.tmG[slot + 1], R.G, R.ldg, R.p, T, B, kKStep, kTile);
-        if (s != DP_OK) return s;
-      }
       GhostLayerPlan lp = plan.layer[li];
       lp.item_begin = items;
       items += B * plan.ntp * lp.nsplit;
@@ -343,14 +344,9 @@ dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& pl
     P.partials = partials;
     P.dev_status = dev_status;
     P.wait_limit = g_wait_limit;
-    const int grid = std::min(items, sm_count());
-    if (dual)
-      ghost_norm_tc_kernel<false, true><<<grid, kThreads, GhostGeo<false>::kSmemBytes, st>>>(P);
-    else if (nt == 1)
-      ghost_norm_tc_kernel<true><<<grid, kThreads, GhostGeo<true>::kSmemBytes, st>>>(P);
-    else
-      ghost_norm_tc_kernel<false><<<grid, kThreads, GhostGeo<false>::kSmemBytes, st>>>(P);
-    DP_LAUNCH_OK();
+    const dp_status s = split ? (nt == 1 ? launch_variant<true, true>(P, st) : launch_variant<false, true>(P, st))
+                              : (nt == 1 ? launch_variant<true, false>(P, st) : launch_variant<false, false>(P, st));
+    if (s != DP_OK) return s;
   }
   return DP_OK;
 }

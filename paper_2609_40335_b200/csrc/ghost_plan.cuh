@@ -47,10 +47,8 @@ GhostPlan plan_ghost_norms(const dp_linear_desc* layers, int n_layers, int B, in
 dp_status launch_ghost_norm_pair(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
                                  float* partials, int* dev_status, cudaStream_t st);
 
-// other_side != NULL: the second operand of every Gram product is taken from other_side[l] (same
-// shapes as layers[l]) instead of layers[l] itself (the split fp32 path).
+// split: the operands are (2B, T, .) planes of high and low bf16 terms (fp32 inputs).
 dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
-                               float* partials, int* dev_status, cudaStream_t st,
-                               const dp_linear_desc* other_side = nullptr);
+                               float* partials, int* dev_status, cudaStream_t st, bool split = false);
 
 }  // namespace dpg

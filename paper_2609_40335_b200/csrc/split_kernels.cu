@@ -5,12 +5,11 @@
 // the "3 x TF32" scheme with 16 instead of 21 mantissa bits, far inside the 1e-4 the fp32 path has
 // to meet, and at three bf16 MMAs cheaper than three TF32 MMAs (which run at half the bf16 rate).
 //
-// The three products become ONE ordinary product of two widened operands, so the bf16 kernels
-// run unchanged:
-//   contraction over columns (the Gram matrices of the ghost norm):
-//       X = [hi | hi | lo],  Y = [hi | lo | hi]   ->  X Y^T = hi hi^T + hi lo^T + lo hi^T
-//   contraction over tokens (G^T A of the clipped sum and of the DIRECT norm): per example
-//       G' = [hi ; hi ; lo] (3T rows),  A' = [hi ; lo ; hi]   ->  G'^T A' = the three products.
+// An operand is stored once, as two planes per example (as many bytes as the fp32 original); the
+// Gram and G^T A kernels pick the plane of each side of each product by the tensor map's example
+// coordinate.  (Widened copies [hi | hi | lo] and [hi | lo | hi] took three to six times the
+// workspace and traffic and, the workspace being sized for one layer, a dozen launches per layer:
+// 24 layers and a head of DistilGPT2 at B = 8, T = 128 took 236 launches, now 12.)
 // For the clipped sum the clip factor R_i (Eq. 7) multiplies G in fp32 BEFORE the split, so the
 // GEMM itself runs unscaled and no bf16 rounding of R_i * g occurs.
 #include <cuda_bf16.h>
@@ -24,70 +23,87 @@ namespace dpg {
 
 namespace {
 
-__device__ __forceinline__ void split2(float x, __nv_bfloat16& hi, __nv_bfloat16& lo) {
-  hi = __float2bfloat16_rn(x);
-  lo = __float2bfloat16_rn(x - __bfloat162float(hi));
-}
+constexpr int kMaxJobs = 208;          // tensors per launch (parameter block)
+constexpr int kChunksPerBlock = 1024;  // 8-column chunks per block of 256 threads
 
-// X, Y: (rows, 3*cp) bf16; column blocks of width cp (c rounded up to 8; the padding is zero)
+struct SplitTensor {
+  const float* src;
+  __nv_bfloat16* dst;
+  long long lds;
+  int c, per_row;                      // columns, 8-column chunks per row
+  int block_begin, scaled;
+};
+struct SplitParams {
+  SplitTensor t[kMaxJobs];
+  int n, T;
+  long long rows;                      // B * T
+  const float* clip;
+};
+
+// HBM-bound: 4 bytes read and 4 written per element, 32 + 32 per thread and step
 __global__ void __launch_bounds__(256)
-split_cols_kernel(const float* __restrict__ src, long long lds, long long rows, int c, int cp,
-                  __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ Y) {
-  const long long total = rows * cp;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long r = e / cp;
-    const int col = int(e - r * cp);
-    __nv_bfloat16 hi = __float2bfloat16_rn(0.f), lo = hi;
-    if (col < c) split2(src[r * lds + col], hi, lo);
-    __nv_bfloat16* x = X + r * 3 * cp + col;
-    __nv_bfloat16* y = Y + r * 3 * cp + col;
-    x[0] = hi; x[cp] = hi; x[2 * cp] = lo;
-    y[0] = hi; y[cp] = lo; y[2 * cp] = hi;
+split_kernel(const __grid_constant__ SplitParams P) {
+  int lo = 0, hi = P.n - 1;            // the tensor this block belongs to
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (int(blockIdx.x) >= P.t[mid].block_begin) lo = mid; else hi = mid - 1;
   }
-}
-
-// dst: (B, 3T, cp) bf16: rows [0,T) / [T,2T) / [2T,3T) of example i hold the three terms
-// {hi,hi,lo} (lo_slab = 2) or {hi,lo,hi} (lo_slab = 1) of scale[i] * src[i]
-__global__ void __launch_bounds__(256)
-split_rows_kernel(const float* __restrict__ src, long long lds, int B, int T, int c, int cp,
-                  const float* __restrict__ scale, int lo_slab, __nv_bfloat16* __restrict__ dst) {
-  const long long total = (long long)B * T * cp;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long r = e / cp;                   // token row i*T + t
-    const int col = int(e - r * cp);
-    const int i = int(r / T), t = int(r - (long long)i * T);
-    __nv_bfloat16 hi = __float2bfloat16_rn(0.f), lo = hi;
-    if (col < c) split2(src[r * lds + col] * (scale ? scale[i] : 1.f), hi, lo);
-    __nv_bfloat16* d0 = dst + ((long long)i * 3 * T + t) * cp + col;
+  const SplitTensor& S = P.t[lo];
+  const bool vec = ((reinterpret_cast<uintptr_t>(S.src) & 15) == 0) && ((S.lds & 3) == 0);
+  const long long total = P.rows * S.per_row;
+  const long long first = (long long)(int(blockIdx.x) - S.block_begin) * kChunksPerBlock;
+  const size_t plane = size_t(P.T) * S.per_row * 8;        // elements of one plane
+  const long long row0 = first / S.per_row;                // the block's first row and chunk in it
+  const unsigned off0 = unsigned(first - row0 * S.per_row);
 #pragma unroll
-    for (int sl = 0; sl < 3; ++sl) d0[(long long)sl * T * cp] = (sl == lo_slab) ? lo : hi;
+  for (int k = 0; k < kChunksPerBlock / 256; ++k) {
+    const unsigned off = off0 + k * 256 + threadIdx.x;
+    const unsigned dr = off / unsigned(S.per_row);
+    if (first + k * 256 + threadIdx.x >= total) break;
+    const unsigned r = unsigned(row0) + dr;                // token row i*T + t
+    const int col = int(off - dr * S.per_row) * 8;
+    const int i = int(r / unsigned(P.T)), t = int(r - unsigned(i) * P.T);
+    float v[8];
+    load8<float>(S.src + (long long)r * S.lds + col, S.c - col, vec, v);      // columns >= c read as zero
+    if (S.scaled) {
+      const float f = __ldg(P.clip + i);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] *= f;
+    }
+    uint4 h, l;
+    __nv_bfloat162* h2 = reinterpret_cast<__nv_bfloat162*>(&h);
+    __nv_bfloat162* l2 = reinterpret_cast<__nv_bfloat162*>(&l);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      h2[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+      const float2 b = __bfloat1622float2(h2[j]);
+      l2[j] = __floats2bfloat162_rn(v[2 * j] - b.x, v[2 * j + 1] - b.y);
+    }
+    __nv_bfloat16* d = S.dst + size_t(2 * i) * plane + size_t(t) * S.per_row * 8 + col;
+    *reinterpret_cast<uint4*>(d) = h;
+    *reinterpret_cast<uint4*>(d + plane) = l;
   }
-}
-
-int grid_for(long long total) {
-  return (int)std::min<long long>((total + 255) / 256, (long long)sm_count() * 16);
 }
 
 }  // namespace
 
-dp_status launch_split_cols(const float* src, int64_t lds, int64_t rows, int c, void* X, void* Y,
-                            cudaStream_t st) {
-  const int cp = split_padded(c);
-  split_cols_kernel<<<grid_for(rows * cp), 256, 0, st>>>(src, lds, rows, c, cp,
-                                                       static_cast<__nv_bfloat16*>(X),
-                                                       static_cast<__nv_bfloat16*>(Y));
-  DP_LAUNCH_OK();
-  return DP_OK;
-}
-
-dp_status launch_split_rows(const float* src, int64_t lds, int B, int T, int c, const float* scale,
-                            int lo_slab, void* dst, cudaStream_t st) {
-  const int cp = split_padded(c);
-  split_rows_kernel<<<grid_for((long long)B * T * cp), 256, 0, st>>>(
-      src, lds, B, T, c, cp, scale, lo_slab, static_cast<__nv_bfloat16*>(dst));
-  DP_LAUNCH_OK();
+dp_status launch_split(const SplitJob* jobs, int n, int B, int T, const float* clip, cudaStream_t st) {
+  for (int j0 = 0; j0 < n; j0 += kMaxJobs) {
+    SplitParams P;
+    P.n = std::min(n - j0, kMaxJobs);
+    P.T = T; P.rows = (long long)B * T; P.clip = clip;
+    long long blocks = 0;
+    for (int k = 0; k < P.n; ++k) {
+      const SplitJob& J = jobs[j0 + k];
+      SplitTensor& S = P.t[k];
+      S.src = J.src; S.dst = static_cast<__nv_bfloat16*>(J.dst); S.lds = J.lds; S.c = J.c;
+      S.per_row = split_padded(J.c) / 8; S.scaled = J.scaled ? 1 : 0; S.block_begin = int(blocks);
+      blocks += (P.rows * S.per_row + kChunksPerBlock - 1) / kChunksPerBlock;
+    }
+    if (blocks > 0x7fffffffLL) return DP_ERR_UNSUPPORTED;
+    split_kernel<<<(unsigned)blocks, 256, 0, st>>>(P);
+    DP_LAUNCH_OK();
+  }
   return DP_OK;
 }
 

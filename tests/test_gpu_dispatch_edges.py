@@ -91,3 +91,35 @@ def test_embedding_norm_with_frequent_tokens(dtype, T, frequent):
         assert abs(float(sq[i]) / want - 1) < 1e-5       # fp32 sums of at most 2100 terms
         uniq, where = np.unique(row, return_index=True)
         assert np.array_equal(first[i].cpu().numpy(), where[np.searchsorted(uniq, row)])
+
+
+# fp32 layers share the workspace in groups: all at once, one at a time (the reported size holds the
+# largest with little to spare), and mixed with layers that stay on the FMA kernels
+@pytest.mark.parametrize("extra", [0, 1 << 26])
+@pytest.mark.parametrize("T", [32, 128, 129, 260])
+def test_fp32_layers_in_groups(extra, T):
+    B = 2
+    shapes = [(64, 64), (136, 72), (64, 300), (40, 64), (520, 256), (65, 131)]
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    layers = [dp.Linear(torch.randn(B, T, d, generator=g, device="cuda"),
+                        0.1 * torch.randn(B, T, p, generator=g, device="cuda"), d=d, p=p) for d, p in shapes]
+    layers[1].mode = dp.DP_NORM_DIRECT
+
+    def ws(need):
+        return torch.empty(max(need, 256) + extra, dtype=torch.uint8, device="cuda")
+
+    sq = torch.zeros(B, device="cuda")
+    dp.dp_ghost_norms(layers, B, T, sq, ws=ws(dp.dp_ghost_norms_ws_bytes(layers, B, T)))
+    clip = torch.tensor([0.3, 1.0], device="cuda")
+    outs = [torch.ones(p, d, device="cuda") for d, p in shapes]
+    dp.dp_clip_accumulate_grouped(layers, B, T, None, 1.0, outs, beta=1.0, clip=clip,
+                                  ws=ws(dp.dp_clip_accumulate_grouped_ws_bytes(layers, B, T)))
+    want_sq = np.zeros(B)
+    for l, o in zip(layers, outs):
+        per = np.einsum("btp,btd->bpd", f64(l.G, l.p), f64(l.A, l.d))
+        want_sq += (per ** 2).sum((1, 2))
+        want = 1.0 + np.einsum("b,bpd->pd", clip.double().cpu().numpy(), per)
+        assert np.linalg.norm(o.double().cpu().numpy() - want) < 2e-5 * np.linalg.norm(want)   # two bf16 terms
+    assert (np.abs(sq.double().cpu().numpy() / want_sq - 1) < 2e-5).all()
+
