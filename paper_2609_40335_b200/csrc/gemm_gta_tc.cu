@@ -503,17 +503,82 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
   }
 }
 
-// out = beta*out + sum over K splits of the partial planes, in split order
-__global__ void splitk_reduce_kernel(const float* __restrict__ partial, int nsplit, int M, int N,
-                                     float* __restrict__ out, long long ldo, float beta) {
-  const size_t total = size_t(M) * N;
-  for (size_t e = size_t(blockIdx.x) * blockDim.x + threadIdx.x; e < total;
-       e += size_t(gridDim.x) * blockDim.x) {
-    const int r = int(e / N), c = int(e - size_t(r) * N);
-    float s = 0.f;
-    for (int k = 0; k < nsplit; ++k) s += partial[size_t(k) * total + e];
-    float* o = out + size_t(r) * ldo + c;
-    *o = (beta != 0.f) ? (*o + s) : s;
+// out = beta*out + sum over K splits of the partial planes, in split order, then the Gaussian
+// mechanism of Eq. 3 -- for all layers of the launch in one kernel (a reduce and a noise pass per
+// layer were two launches each).  A thread owns one Philox counter: four consecutive elements of
+// the row-major output.
+struct ReduceLayer {
+  float* out;
+  const float* partial;
+  long long ldo;
+  int M, N, block_begin;
+  uint32_t tensor_id;
+};
+struct ReduceParams {
+  ReduceLayer layer[kGtaMaxLayers];
+  int n_layers, nsplit, with_noise;
+  float beta, amp, scale;
+  NoiseKeys keys;
+  uint32_t step;
+  const uint32_t* step_dev;
+};
+constexpr int kReduceQuads = 512;                    // quads per block of 256 threads
+
+__global__ void __launch_bounds__(256)
+splitk_reduce_kernel(const __grid_constant__ ReduceParams P) {
+  int lo = 0, hi = P.n_layers - 1;                   // the layer this block belongs to
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (int(blockIdx.x) >= P.layer[mid].block_begin) lo = mid; else hi = mid - 1;
+  }
+  const ReduceLayer& L = P.layer[lo];
+  const size_t total = size_t(L.M) * L.N;
+  const bool vec = (total & 3) == 0;                 // planes are 256-byte aligned
+  const bool ovec = (L.N & 3) == 0 && (L.ldo & 3) == 0 && (reinterpret_cast<uintptr_t>(L.out) & 15) == 0;
+  const uint32_t step = effective_step(P.step, P.step_dev);
+#pragma unroll
+  for (int k = 0; k < kReduceQuads / 256; ++k) {
+    const size_t q = size_t(int(blockIdx.x) - L.block_begin) * kReduceQuads + k * 256 + threadIdx.x;
+    const size_t e0 = 4 * q;
+    if (e0 >= total) break;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (vec) {
+      const float* src = L.partial + e0;
+#pragma unroll 4
+      for (int s = 0; s < P.nsplit; ++s) {
+        const float4 x = __ldcs(reinterpret_cast<const float4*>(src + size_t(s) * total));
+        v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+      }
+    } else {
+      for (int s = 0; s < P.nsplit; ++s)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) if (e0 + e < total) v[e] += L.partial[size_t(s) * total + e0 + e];
+    }
+    float z[4];
+    if (P.with_noise) normals4(q, P.keys, L.tensor_id, step, z);
+    const size_t r = e0 / L.N, c = e0 - r * L.N;
+    float* o = L.out + r * L.ldo + c;
+    if (ovec) {
+      if (P.beta != 0.f) {
+        const float4 x = *reinterpret_cast<const float4*>(o);
+        v[0] = x.x + v[0]; v[1] = x.y + v[1]; v[2] = x.z + v[2]; v[3] = x.w + v[3];
+      }
+      if (P.with_noise)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = noised(v[e], z[e], P.amp, P.scale);
+      *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (e0 + e < total) {
+          const size_t re = (e0 + e) / L.N;
+          float* oe = L.out + re * L.ldo + (e0 + e - re * L.N);
+          float x = (P.beta != 0.f) ? (*oe + v[e]) : v[e];
+          if (P.with_noise) x = noised(x, z[e], P.amp, P.scale);
+          *oe = x;
+        }
+      }
+    }
   }
 }
 
@@ -695,14 +760,24 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
     const int units = std::min(items, kUsePair ? sms / 2 : sms);
     s = launch_gta<kClipScale, false, kUsePair>(P, units, st);
     if (s != DP_OK) return s;
+    if (nsplit > 1) {
+      ReduceParams R;
+      R.n_layers = P.n_layers; R.nsplit = nsplit; R.with_noise = noise ? 1 : 0; R.beta = beta;
+      R.amp = noise ? noise->amp : 0.f; R.scale = noise ? noise->scale : 1.f;
+      R.keys = expand_noise_keys(noise ? noise->seed : 0);
+      R.step = noise ? noise->step : 0; R.step_dev = noise ? g_step_dev : nullptr;
+      long long blocks = 0;
+      for (int k = 0; k < P.n_layers; ++k) {
+        const GtaLayer& L = P.layer[k];
+        R.layer[k] = {L.out, L.partial, L.ldo, L.M, L.N, int(blocks), L.tensor_id};
+        blocks += ((long long)L.M * L.N + 4 * kReduceQuads - 1) / (4 * kReduceQuads);
+      }
+      splitk_reduce_kernel<<<(unsigned)blocks, 256, 0, st>>>(R);
+      DP_LAUNCH_OK();
+      continue;
+    }
     for (int g = g0; g < g1; ++g) {
       const GtaLayer& L = P.layer[g - g0];
-      if (nsplit > 1) {
-        const size_t total = size_t(L.M) * L.N;
-        const int blocks = (int)std::min<size_t>((total + 255) / 256, size_t(sms) * 8);
-        splitk_reduce_kernel<<<blocks, 256, 0, st>>>(L.partial, nsplit, L.M, L.N, L.out, L.ldo, beta);
-        DP_LAUNCH_OK();
-      }
       if (noise && L.noise_amp < 0.f) {        // not fused for this layer: stand-alone pass
         const dp_status ns = launch_add_noise(L.out, L.M, L.N, L.ldo, false, noise->amp,
                                               noise->scale, noise->seed, noise->tensor_ids[g],

@@ -123,3 +123,26 @@ def test_fp32_layers_in_groups(extra, T):
         assert np.linalg.norm(o.double().cpu().numpy() - want) < 2e-5 * np.linalg.norm(want)   # two bf16 terms
     assert (np.abs(sq.double().cpu().numpy() / want_sq - 1) < 2e-5).all()
 
+
+# one reduction for the K-split planes of all layers: widths that are and are not multiples of 4
+@pytest.mark.parametrize("shapes", [[(64, 64), (256, 300)], [(50, 70), (33, 41), (3, 5)]])
+@pytest.mark.parametrize("noise", [False, True])
+def test_k_split_planes_of_several_layers(shapes, noise):
+    B, T = 16, 64
+    layers = [dp.Linear(bf16((B, T, d), 1.0, k, ld=(d + 7) // 8 * 8), bf16((B, T, p), 0.1, 50 + k, ld=(p + 7) // 8 * 8),
+                        d=d, p=p) for k, (d, p) in enumerate(shapes)]
+    clip = torch.full((B,), 0.5, device="cuda")
+    start = [torch.randn(p, d, device="cuda") for d, p in shapes]
+    plain, outs = [t.clone() for t in start], [t.clone() for t in start]
+    dp.dp_clip_accumulate_grouped(layers, B, T, None, 1.0, plain, beta=1.0, clip=clip)
+    if noise:
+        ids = list(range(5, 5 + len(shapes)))
+        dp.dp_clip_accumulate_noise_grouped(layers, B, T, None, 1.0, outs, 0.7, 0.5, 11, ids, 2, beta=1.0, clip=clip)
+        for t, i in zip(plain, ids):
+            dp.dp_add_noise(t, 0.7, 1.0, 0.5, 11, i, 2)
+        for a, b in zip(plain, outs):
+            assert torch.equal(a, b)
+    else:
+        for l, o, s in zip(layers, plain, start):
+            want = s.double().cpu().numpy() + 0.5 * np.einsum("btp,btd->pd", f64(l.G, l.p), f64(l.A, l.d))
+            assert np.linalg.norm(o.double().cpu().numpy() - want) < 1e-5 * np.linalg.norm(want)
