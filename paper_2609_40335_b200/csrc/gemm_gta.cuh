@@ -46,6 +46,22 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
                                     float beta, const GtaNoise* noise, float* partial_ws,
                                     int* dev_status, cudaStream_t st);
 
+// Items of two output tiles sharing an operand, for calls with tiles enough (gemm_gta_big.cu).
+struct GtaBigJob {
+  const void* A;
+  int64_t lda;
+  const void* G;
+  int64_t ldg;
+  int d, p;
+  float* out;
+  int64_t ldo;
+  int prescaled;
+  float noise_amp;        // sigma*C of the fused noise, negative = none
+  uint32_t tensor_id;
+};
+dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, const float* clip, float beta,
+                         const GtaNoise* noise, int* dev_status, cudaStream_t st);
+
 dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T, int terms,
                                 float* partials, int* dev_status, cudaStream_t st);
 

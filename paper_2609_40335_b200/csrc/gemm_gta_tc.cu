@@ -18,7 +18,8 @@
 // the fused Gaussian noise, which is latency-bound per warp -- hence so many); two TMEM
 // accumulators overlap the epilogue with the next tile.
 //
-// Clipped sums run on CTA PAIRS (cta_group::2, cluster of 2): a 256 x 256 output tile per pair,
+// Clipped sums run on CTA PAIRS (cta_group::2, cluster of 2; here those with few output tiles, the others
+// in gemm_gta_big.cu): a 256 x 256 output tile per pair,
 // each CTA loading its own 128 G rows and half of the A tile's columns, rank 0 issuing the MMAs
 // for both, stage-free and accumulator-ready signals multicast to both CTAs by tcgen05.commit,
 // scaler and epilogue warps of rank 1 arriving on rank 0's barriers.  The DIRECT-norm variant
@@ -28,6 +29,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <vector>
 
 #include "dp_common.cuh"
 #include "gemm_gta.cuh"
@@ -698,6 +700,9 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
   int nsplit = gta_choose_nsplit(gta_tiles(layers, n_layers), B, T, terms, sms);
   const int kps = ceil_div(ksteps, nsplit);
   nsplit = ceil_div(ksteps, kps);                       // drop empty trailing splits
+  // Two tiles per item need the tiles for it: at least two per CTA pair (the bound below which K is split;
+  // with fewer, one-tile items spread over more SMs).
+  const bool use_big = gta_tiles(layers, n_layers) >= 2LL * (sms / 2);
   char* pw = reinterpret_cast<char*>(partial_ws);
   char* pre = pw;                                       // pre-scaled copies sit behind the K-split planes
   if (pw && nsplit > 1)
@@ -707,6 +712,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
     const int g1 = std::min(n_layers, g0 + kGtaMaxLayers);
     GtaParams P;
     memset(&P, 0, sizeof(P));
+    std::vector<GtaBigJob> big;
     int items = 0;
     for (int g = g0; g < g1; ++g) {
       dp_linear_desc D = layers[g];
@@ -727,10 +733,12 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
         if (narrow_a) { D.A = copy; D.lda = cp; } else { D.G = copy; D.ldg = cp; }
         L.prescaled = 1;
       }
-      s = make_tmap_bf16_3d(&P.tmG[g - g0], D.G, D.ldg, D.p, T, planes, 64, kBK);
-      if (s != DP_OK) return s;
-      s = make_tmap_bf16_3d(&P.tmA[g - g0], D.A, D.lda, D.d, T, planes, 64, kBK);
-      if (s != DP_OK) return s;
+      if (!use_big) {
+        s = make_tmap_bf16_3d(&P.tmG[g - g0], D.G, D.ldg, D.p, T, planes, 64, kBK);
+        if (s != DP_OK) return s;
+        s = make_tmap_bf16_3d(&P.tmA[g - g0], D.A, D.lda, D.d, T, planes, 64, kBK);
+        if (s != DP_OK) return s;
+      }
       L.out = outs[g]; L.ldo = ldos[g];
       L.M = D.p; L.N = D.d;
       L.partial = nullptr;
@@ -744,6 +752,8 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
       const bool fuse = noise && nsplit == 1 && (D.d % 4 == 0);
       L.noise_amp = fuse ? noise->amp : -1.f;
       L.tensor_id = noise ? noise->tensor_ids[g] : 0u;
+      if (use_big)
+        big.push_back({D.A, D.lda, D.G, D.ldg, D.d, D.p, L.out, L.ldo, L.prescaled, L.noise_amp, L.tensor_id});
       items += ceil_div(D.p, Geo<kUsePair>::kTileM) * ceil_div(D.d, kBN) * nsplit;
     }
     if (noise) {
@@ -758,7 +768,8 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
     P.dev_status = dev_status;
     P.wait_limit = g_wait_limit;
     const int units = std::min(items, kUsePair ? sms / 2 : sms);
-    s = launch_gta<kClipScale, false, kUsePair>(P, units, st);
+    s = use_big ? launch_gta_big(big.data(), (int)big.size(), B, T, terms, clip, beta, noise, dev_status, st)
+                : launch_gta<kClipScale, false, kUsePair>(P, units, st);
     if (s != DP_OK) return s;
     if (nsplit > 1) {
       ReduceParams R;

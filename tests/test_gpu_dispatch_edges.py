@@ -146,3 +146,58 @@ def test_k_split_planes_of_several_layers(shapes, noise):
         for l, o, s in zip(layers, plain, start):
             want = s.double().cpu().numpy() + 0.5 * np.einsum("btp,btd->pd", f64(l.G, l.p), f64(l.A, l.d))
             assert np.linalg.norm(o.double().cpu().numpy() - want) < 1e-5 * np.linalg.norm(want)
+
+
+# two-tile items: both orientations, leftover lines of tiles paired along their length, a last corner tile,
+# items converted to single tiles in a last wave, partial tiles, widths that are no multiple of 4 or 8
+BIG_SHAPES = [[(257, 19001)], [(19000, 250)], [(700, 13000), (100, 3000), (64, 64)], [(511, 6500), (2600, 1281), (768, 768)],
+              [(768, 14300)]]
+
+
+@pytest.mark.parametrize("shapes", BIG_SHAPES)
+@pytest.mark.parametrize("beta,noise,B,T", [(0.0, False, 3, 50), (1.0, True, 3, 50), (0.0, True, 1, 7), (0.0, True, 20, 64)])
+def test_two_tile_items(shapes, beta, noise, B, T):
+    layers = [dp.Linear(bf16((B, T, d), 1.0, k, ld=(d + 7) // 8 * 8), bf16((B, T, p), 0.1, 50 + k, ld=(p + 7) // 8 * 8),
+                        d=d, p=p) for k, (d, p) in enumerate(shapes)]
+    clip = torch.tensor([2.0 ** -(i % 3) for i in range(B)], device="cuda")
+    start = [torch.randn(p, d, device="cuda") for d, p in shapes]
+    outs, st = [t.clone() for t in start], torch.zeros(1, dtype=torch.int32, device="cuda")
+    dp.dp_clip_accumulate_grouped(layers, B, T, None, 1.0, outs, beta=beta, clip=clip, dev_status=st)
+    for l, o, s in zip(layers, outs, start):
+        g = l.G[..., :l.p].double().cpu() * clip.double().cpu()[:, None, None]
+        want = g.reshape(-1, l.p).T @ l.A[..., :l.d].double().cpu().reshape(-1, l.d) + beta * s.double().cpu()
+        # powers of two: R_i * x is exact in bf16, what is left is fp32 accumulation
+        assert float((o.double().cpu() - want).norm() / want.norm()) < 1e-5
+    if noise:
+        again = [t.clone() for t in start]
+        ids = list(range(3, 3 + len(shapes)))
+        dp.dp_clip_accumulate_noise_grouped(layers, B, T, None, 1.0, again, 0.9, 0.5, 7, ids, 1, beta=beta, clip=clip,
+                                            dev_status=st)
+        for a, o, i in zip(again, outs, ids):
+            dp.dp_add_noise(o, 0.9, 1.0, 0.5, 7, i, 1)
+            assert torch.equal(a, o)
+    assert int(st.item()) == 0
+
+
+def test_two_tile_items_give_up_cleanly():
+    """A wait limit of zero: the kernel flags DP_DEV_TIMEOUT and returns; the same call then succeeds."""
+    B, T, d, p = 32, 128, 512, 19000               # long enough a contraction that some wait is not over at once
+    layer = [dp.Linear(bf16((B, T, d), 1.0, 1), bf16((B, T, p), 0.1, 2), d=d, p=p)]
+    clip = torch.full((B,), 0.3, device="cuda")
+    lib = dp.load()
+
+    def run():
+        out, st = torch.zeros(p, d, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+        dp.dp_clip_accumulate_grouped(layer, B, T, None, 1.0, [out], clip=clip, dev_status=st)
+        torch.cuda.synchronize()
+        return out, int(st.item())
+
+    good, flag = run()
+    assert flag == 0
+    prev = lib.dp_debug_set_wait_limit(0)
+    try:
+        assert run()[1] & dp.DP_DEV_TIMEOUT
+    finally:
+        lib.dp_debug_set_wait_limit(prev)
+    again, flag = run()
+    assert flag == 0 and torch.equal(good, again)
