@@ -137,44 +137,51 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
   ptx::cluster_sync_all();        // the partner's barriers exist before anyone arrives on them
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tiles_a = ptx::smem_u32(tiles), full_a = ptx::smem_u32(full), empty_a = ptx::smem_u32(empty);
 
   if (warp == 0) {
     // ------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued = 0;
-      int lay = 0;
-      bool ok = true;
-      for (int item = first_item; item < P.total_items && ok; item += item_stride) {
-        const Item it = decode_item(P, item, lay);
-        const bool diag = it.ti == it.tj;
-        const uint32_t bytes = diag ? kTileBytes : kStageBytes;
-        const int row_i = it.ti * kTile2 + int(rank) * kRows;     // this CTA's rows of block I
-        const int row_j = it.tj * kTile2 + int(rank) * kRows;     // and of block J
-        for (int pass = 0; pass < 2 && ok; ++pass) {
-          const CUtensorMap* tm = pass == 0 ? &P.tmA[it.layer] : &P.tmG[it.layer];
-          const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
-          for (int k = k0; k < k1; ++k) {
-            if (!ptx::mbar_wait(&empty[stage], phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
-            uint8_t* dst = tiles + size_t(stage) * kStageBytes;
-            ptx::mbar_arrive_expect_tx(&full[stage], bytes);
-            ptx::tma_load_3d(dst, tm, &full[stage], k * kKStep, row_i, it.example);
-            if (!diag) ptx::tma_load_3d(dst + kTileBytes, tm, &full[stage], k * kKStep, row_j, it.example);
-            ++issued;
-            if (++stage == kStages) { stage = 0; phase ^= 1; }
+    // producer, issuer and relay: the whole warp runs the loop, an elected lane issues (see ptx::warp_ok)
+    uint32_t stage = 0, phase = 0, issued = 0;
+    int lay = 0;
+    bool ok = true;
+    for (int item = first_item; item < P.total_items && ok; item += item_stride) {
+      const Item it = decode_item(P, item, lay);
+      const bool diag = it.ti == it.tj;
+      const uint32_t bytes = diag ? kTileBytes : kStageBytes;
+      const int row_i = it.ti * kTile2 + int(rank) * kRows;     // this CTA's rows of block I
+      const int row_j = it.tj * kTile2 + int(rank) * kRows;     // and of block J
+      for (int pass = 0; pass < 2 && ok; ++pass) {
+        const uint64_t tm = reinterpret_cast<uint64_t>(pass == 0 ? &P.tmA[it.layer] : &P.tmG[it.layer]);
+        const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
+        for (int k = k0; k < k1; ++k) {
+          ok = ptx::warp_ok(ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit));
+          if (!ok) break;
+          const uint32_t dst = tiles_a + stage * kStageBytes, bar = full_a + 8 * stage;
+          if (ptx::elect_one()) {
+            ptx::mbar_arrive_expect_tx_a(bar, bytes);
+            ptx::tma_load_3d_a(dst, tm, bar, k * kKStep, row_i, it.example);
+            if (!diag) ptx::tma_load_3d_a(dst + kTileBytes, tm, bar, k * kKStep, row_j, it.example);
           }
+          __syncwarp();
+          ++issued;
+          if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
       }
-      if (!ok) {
-        *abort_flag = 1;
-        if (P.dev_status) atomicOr(P.dev_status, DP_DEV_TIMEOUT);
-        ptx::drain_issued_copies(full, kStages, issued);
-      }
+    }
+    if (!ok && ptx::elect_one()) {
+      *abort_flag = 1;
+      if (P.dev_status) atomicOr(P.dev_status, DP_DEV_TIMEOUT);
+      ptx::drain_issued_copies(full, kStages, issued);
     }
   } else if (warp == 1) {
     // --------------------------------------------------------------- MMA issuer
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       constexpr uint32_t idesc = ptx::idesc_bf16_f32(kTile2, kTile2, 0, 0);
       constexpr uint64_t dbase = ptx::smem_desc_base(16, 1024, ptx::SWIZZLE_128B);   // K-major
+      constexpr uint32_t desc_hi = uint32_t(dbase >> 32);
+      const uint32_t desc_lo0 = uint32_t(dbase) | ((tiles_a >> 4) & 0x3FFF);
+      const uint32_t ready_a = ptx::smem_u32(ready);
       uint32_t stage = 0, phase = 0, n_item = 0;
       int lay = 0;
       bool ok = true;
@@ -185,27 +192,30 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
         for (int pass = 0; pass < 2 && ok; ++pass) {
           // the accumulator of this pass must have been read out for the previous item
           uint64_t* freed = pass == 0 ? sa_empty : sg_empty;
-          if (!ptx::mbar_wait_cluster(freed, ph ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
+          ok = ptx::warp_ok(ptx::mbar_wait_cluster(freed, ph ^ 1, abort_flag, P.wait_limit));
+          if (!ok) break;
           ptx::tc_fence_after();
           const uint32_t d_tmem = tmem_base + pass * kTile2;
           const int nsteps = pass == 0 ? it.a1 - it.a0 : it.g1 - it.g0;
           for (int k = 0; k < nsteps; ++k) {
-            if (!ptx::mbar_wait_cluster(&ready[stage], phase, abort_flag, P.wait_limit)) { ok = false; break; }
+            ok = ptx::warp_ok(ptx::mbar_wait_cluster_a(ready_a + 8 * stage, phase, abort_flag, P.wait_limit));
+            if (!ok) break;
             ptx::tc_fence_after();
-            const uint32_t sa = ptx::smem_u32(tiles + size_t(stage) * kStageBytes);
-            const uint32_t sb = diag ? sa : sa + kTileBytes;
+            const uint32_t sa = desc_lo0 + stage * (kStageBytes >> 4);
+            const uint32_t sb = diag ? sa : sa + (kTileBytes >> 4);
+            if (ptx::elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < kKStep / 16; ++kk)
-              ptx::mma_bf16_ss_pair(d_tmem, ptx::smem_desc(dbase, sa + kk * 32),
-                                    ptx::smem_desc(dbase, sb + kk * 32), idesc,
-                                    (k > 0 || kk > 0) ? 1u : 0u);
-            ptx::mma_commit_pair(&empty[stage], 3);
+              for (int kk = 0; kk < kKStep / 16; ++kk)
+                ptx::mma_bf16_ss_pair_lh(d_tmem, sa + kk * 2, sb + kk * 2, desc_hi, idesc, (k > 0 || kk > 0) ? 1u : 0u);
+              ptx::mma_commit_pair_a(empty_a + 8 * stage, 3);
+              if (k + 1 == nsteps) ptx::mma_commit_pair(pass == 0 ? sa_full : sg_full, 3);
+            }
+            __syncwarp();
             if (++stage == kStages) { stage = 0; phase ^= 1; }
           }
-          if (ok) ptx::mma_commit_pair(pass == 0 ? sa_full : sg_full, 3);
         }
       }
-      if (!ok) {
+      if (!ok && ptx::elect_one()) {
         *abort_flag = 1;
         if (P.dev_status) atomicOr(P.dev_status, DP_DEV_TIMEOUT);
         ptx::drain_issued_mmas(mma_done, true);
@@ -218,26 +228,28 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
     // acquired its `full` barrier (so the TMA data are visible to it), delivers those 4 bytes with
     // an asynchronous store into rank 0's shared memory whose completion on the barrier is a
     // release at cluster scope.
-    if (lane == 0) {
-      const uint32_t ready_a = ptx::smem_u32(ready), sink_a = ptx::smem_u32(sink);
-      const uint32_t ready_remote = ptx::mapa_u32(ready_a, 0), sink_remote = ptx::mapa_u32(sink_a, 0);
-      uint32_t stage = 0, phase = 0;
-      int lay = 0;
-      bool ok = true;
-      for (int item = first_item; item < P.total_items && ok; item += item_stride) {
-        const Item it = decode_item(P, item, lay);
-        const int nsteps = (it.a1 - it.a0) + (it.g1 - it.g0);
-        for (int k = 0; k < nsteps; ++k) {
-          if (!ptx::mbar_wait(&full[stage], phase, abort_flag, P.wait_limit)) { ok = false; break; }
+    const uint32_t ready_a = ptx::smem_u32(ready), sink_a = ptx::smem_u32(sink);
+    const uint32_t ready_remote = ptx::mapa_u32(ready_a, 0), sink_remote = ptx::mapa_u32(sink_a, 0);
+    uint32_t stage = 0, phase = 0;
+    int lay = 0;
+    bool ok = true;
+    for (int item = first_item; item < P.total_items && ok; item += item_stride) {
+      const Item it = decode_item(P, item, lay);
+      const int nsteps = (it.a1 - it.a0) + (it.g1 - it.g0);
+      for (int k = 0; k < nsteps; ++k) {
+        ok = ptx::warp_ok(ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit));
+        if (!ok) break;
+        if (ptx::elect_one()) {
           if (rank == 0) ptx::mbar_arrive_expect_tx_a(ready_a + 8 * stage, 4);
           else ptx::st_async_signal_a(ready_remote + 8 * stage, sink_remote + 4 * stage);
-          if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
+        __syncwarp();
+        if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
-      if (!ok) {
-        *abort_flag = 1;
-        if (P.dev_status) atomicOr(P.dev_status, DP_DEV_TIMEOUT);
-      }
+    }
+    if (!ok && ptx::elect_one()) {
+      *abort_flag = 1;
+      if (P.dev_status) atomicOr(P.dev_status, DP_DEV_TIMEOUT);
     }
   } else if (warp >= kEpiWarp0) {
     // ----------------------------------------------------------------- epilogue

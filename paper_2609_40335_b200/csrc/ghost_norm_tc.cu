@@ -131,87 +131,96 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tiles_a = ptx::smem_u32(tiles), full_a = ptx::smem_u32(full), empty_a = ptx::smem_u32(empty);
 
   if (warp == 0) {
     // ------------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0, issued = 0;
-      int lay = 0;
-      bool ok = true;
-      for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x) {
-        const Item it = decode_item(P, item, lay);
-        const bool diag = kDiagOnly || (it.ti == it.tj);
-        const uint32_t bytes = diag ? kTermBytes : kStageBytes;
-        const int ex = kSplit ? 2 * it.example : it.example;     // (high) plane of the example
-        for (int pass = 0; pass < 2 && ok; ++pass) {
-          const CUtensorMap* tm = pass == 0 ? &P.tmA[it.layer] : &P.tmG[it.layer];
-          const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
-          for (int k = k0; k < k1; ++k) {
-            if (!ptx::mbar_wait(&empty[stage], phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
-            uint8_t* dst = tiles + size_t(stage) * kStageBytes;
-            ptx::mbar_arrive_expect_tx(&full[stage], bytes);
-            ptx::tma_load_3d(dst, tm, &full[stage], k * kKStep, it.ti * kTile, ex);
-            if (kSplit) ptx::tma_load_3d(dst + kTileBytes, tm, &full[stage], k * kKStep, it.ti * kTile, ex + 1);
+    // producer and issuer: the whole warp runs the loop, an elected lane issues (see ptx::warp_ok)
+    uint32_t stage = 0, phase = 0, issued = 0;
+    int lay = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x) {
+      const Item it = decode_item(P, item, lay);
+      const bool diag = kDiagOnly || (it.ti == it.tj);
+      const uint32_t bytes = diag ? kTermBytes : kStageBytes;
+      const int ex = kSplit ? 2 * it.example : it.example;     // (high) plane of the example
+      for (int pass = 0; pass < 2 && ok; ++pass) {
+        const uint64_t tm = reinterpret_cast<uint64_t>(pass == 0 ? &P.tmA[it.layer] : &P.tmG[it.layer]);
+        const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
+        for (int k = k0; k < k1; ++k) {
+          ok = ptx::warp_ok(ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit));
+          if (!ok) break;
+          const uint32_t dst = tiles_a + stage * kStageBytes, bar = full_a + 8 * stage;
+          if (ptx::elect_one()) {
+            ptx::mbar_arrive_expect_tx_a(bar, bytes);
+            ptx::tma_load_3d_a(dst, tm, bar, k * kKStep, it.ti * kTile, ex);
+            if (kSplit) ptx::tma_load_3d_a(dst + kTileBytes, tm, bar, k * kKStep, it.ti * kTile, ex + 1);
             if (!diag) {
-              ptx::tma_load_3d(dst + kTermBytes, tm, &full[stage], k * kKStep, it.tj * kTile, ex);
+              ptx::tma_load_3d_a(dst + kTermBytes, tm, bar, k * kKStep, it.tj * kTile, ex);
               if (kSplit)
-                ptx::tma_load_3d(dst + kTermBytes + kTileBytes, tm, &full[stage], k * kKStep, it.tj * kTile, ex + 1);
+                ptx::tma_load_3d_a(dst + kTermBytes + kTileBytes, tm, bar, k * kKStep, it.tj * kTile, ex + 1);
             }
-            ++issued;
-            if (++stage == kStages) { stage = 0; phase ^= 1; }
           }
+          __syncwarp();
+          ++issued;
+          if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
       }
-      if (!ok) {
-        *abort_flag = 1;
-        if (P.dev_status) atomicOr(P.dev_status, DP_DEV_TIMEOUT);
-        ptx::drain_issued_copies(full, kStages, issued);   // copies in flight land before exit
-      }
+    }
+    if (!ok && ptx::elect_one()) {
+      *abort_flag = 1;
+      if (P.dev_status) atomicOr(P.dev_status, DP_DEV_TIMEOUT);
+      ptx::drain_issued_copies(full, kStages, issued);   // copies in flight land before exit
     }
   } else if (warp == 1) {
     // --------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      constexpr uint32_t idesc = ptx::idesc_bf16_f32(kTile, kTile, 0, 0);
-      // K-major operand, 128-byte swizzle: 8-row groups are 1024 bytes apart
-      constexpr uint64_t dbase = ptx::smem_desc_base(16, 1024, ptx::SWIZZLE_128B);
-      uint32_t stage = 0, phase = 0, n_item = 0;
-      int lay = 0;
-      bool ok = true;
-      for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x, ++n_item) {
-        const Item it = decode_item(P, item, lay);
-        const bool diag = kDiagOnly || (it.ti == it.tj);
-        const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
-        if (!ptx::mbar_wait(&acc_empty[buf], acc_phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
-        ptx::tc_fence_after();
-        for (int pass = 0; pass < 2 && ok; ++pass) {
-          const uint32_t d_tmem = tmem_base + buf * 256 + pass * 128;
-          const int nsteps = pass == 0 ? it.a1 - it.a0 : it.g1 - it.g0;
-          for (int k = 0; k < nsteps; ++k) {
-            if (!ptx::mbar_wait(&full[stage], phase, abort_flag, P.wait_limit)) { ok = false; break; }
-            ptx::tc_fence_after();
-            const uint32_t sa = ptx::smem_u32(tiles + size_t(stage) * kStageBytes);
-            const uint32_t sb = diag ? sa : sa + kTermBytes;
+    constexpr uint32_t idesc = ptx::idesc_bf16_f32(kTile, kTile, 0, 0);
+    // K-major operand, 128-byte swizzle: 8-row groups are 1024 bytes apart; 16 bf16 = 32 bytes
+    // further along K inside the swizzle atom
+    constexpr uint64_t dbase = ptx::smem_desc_base(16, 1024, ptx::SWIZZLE_128B);
+    constexpr uint32_t desc_hi = uint32_t(dbase >> 32);
+    const uint32_t desc_lo0 = uint32_t(dbase) | ((tiles_a >> 4) & 0x3FFF);
+    uint32_t stage = 0, phase = 0, n_item = 0;
+    int lay = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x, ++n_item) {
+      const Item it = decode_item(P, item, lay);
+      const bool diag = kDiagOnly || (it.ti == it.tj);
+      const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
+      ok = ptx::warp_ok(ptx::mbar_wait(&acc_empty[buf], acc_phase ^ 1, abort_flag, P.wait_limit));
+      if (!ok) break;
+      ptx::tc_fence_after();
+      for (int pass = 0; pass < 2 && ok; ++pass) {
+        const uint32_t d_tmem = tmem_base + buf * 256 + pass * 128;
+        const int nsteps = pass == 0 ? it.a1 - it.a0 : it.g1 - it.g0;
+        for (int k = 0; k < nsteps; ++k) {
+          ok = ptx::warp_ok(ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit));
+          if (!ok) break;
+          ptx::tc_fence_after();
+          const uint32_t sa = desc_lo0 + stage * (kStageBytes >> 4);
+          const uint32_t sb = diag ? sa : sa + (kTermBytes >> 4);
+          if (ptx::elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < kKStep / 16; ++kk) {
-              // 16 bf16 = 32 bytes further along K inside the swizzle atom
-              const uint64_t ah = ptx::smem_desc(dbase, sa + kk * 32), bh = ptx::smem_desc(dbase, sb + kk * 32);
-              ptx::mma_bf16_ss(d_tmem, ah, bh, idesc, (k > 0 || kk > 0) ? 1u : 0u);
+              const uint32_t ah = sa + kk * 2, bh = sb + kk * 2, low = kTileBytes >> 4;
+              ptx::mma_bf16_ss_lh(d_tmem, ah, bh, desc_hi, idesc, (k > 0 || kk > 0) ? 1u : 0u);
               if (kSplit) {
-                ptx::mma_bf16_ss(d_tmem, ah, ptx::smem_desc(dbase, sb + kTileBytes + kk * 32), idesc, 1u);
-                ptx::mma_bf16_ss(d_tmem, ptx::smem_desc(dbase, sa + kTileBytes + kk * 32), bh, idesc, 1u);
+                ptx::mma_bf16_ss_lh(d_tmem, ah, bh + low, desc_hi, idesc, 1u);
+                ptx::mma_bf16_ss_lh(d_tmem, ah + low, bh, desc_hi, idesc, 1u);
               }
             }
-            ptx::mma_commit(&empty[stage]);          // stage reusable once these MMAs retire
-            if (++stage == kStages) { stage = 0; phase ^= 1; }
+            ptx::mma_commit_a(empty_a + 8 * stage);      // stage reusable once these MMAs retire
+            if (pass == 1 && k + 1 == nsteps) ptx::mma_commit(&acc_full[buf]);     // both Gram tiles complete
           }
+          __syncwarp();
+          if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
-        if (ok) ptx::mma_commit(&acc_full[buf]);     // both Gram tiles complete
       }
-      if (!ok) {
-        *abort_flag = 1;
-        if (P.dev_status) atomicOr(P.dev_status, DP_DEV_TIMEOUT);
-        ptx::drain_issued_mmas(mma_done, false);
-      }
+    }
+    if (!ok && ptx::elect_one()) {
+      *abort_flag = 1;
+      if (P.dev_status) atomicOr(P.dev_status, DP_DEV_TIMEOUT);
+      ptx::drain_issued_mmas(mma_done, false);
     }
   } else {
     // ----------------------------------------------------------------- epilogue
