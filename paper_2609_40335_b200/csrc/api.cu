@@ -842,6 +842,7 @@ static dp_status start_table(const dp_step_desc* S, float* table, int64_t ld, in
                              cudaStream_t st) {
   if (S->with_noise)
     return launch_add_noise(table, rows, S->d, ld, true, S->sigma * S->C, 1.f, S->seed, tid, S->step, st);
+  if (ld == S->d) return launch_clear(table, size_t(rows) * size_t(ld) * sizeof(float), st);
   DP_CUDA_OK(cudaMemset2DAsync(table, size_t(ld) * sizeof(float), 0, size_t(S->d) * sizeof(float),
                                size_t(rows), st));
   return DP_OK;

@@ -211,8 +211,7 @@ dp_status launch_cross_term_tc(const int* ids, const void* Ge, int64_t ldge, con
                                int64_t ldal, const void* Gl, int64_t ldgl, int B, int T, int d, int V,
                                float* partials, int* dev_status, cudaStream_t st) {
   if (first_use_on_this_device(reinterpret_cast<const void*>(&cross_term_tc_kernel)))
-    DP_CUDA_OK(cudaFuncSetAttribute(cross_term_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kSmemBytes));
+    DP_CUDA_OK(allow_shared(cross_term_tc_kernel, kSmemBytes));
   CrossParams P;
   memset(&P, 0, sizeof(P));
   dp_status s = make_tmap_bf16_3d(&P.tmE, Ge, ldge, d, T, B, kKStep, kTile);

@@ -47,13 +47,20 @@ int sm_count();
 // afterwards.  A process that drives several GPUs gets the set-up on each of them.
 bool first_use_on_this_device(const void* key);
 
-// Small kernels that run on a second stream beside a persistent TMA kernel ask for the same
-// shared-memory carve-out as that kernel: an SM changes its carve-out only when it is idle, so a
-// kernel with another preference waits until the persistent one has left the SM.
+// Persistent TMA kernels and the small ones that run beside them on a second stream all ask for the
+// largest shared-memory carve-out: an SM changes its carve-out only when it is idle, so a kernel
+// with another preference waits until the persistent one has left the SM.
 template <typename K>
 inline cudaError_t prefer_max_shared(K* kernel) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                               cudaSharedmemCarveoutMaxShared);
+}
+// dynamic shared memory of a TMA kernel, with that carve-out (without it embedding norms enqueued
+// beside ghost_norm_tc_kernel began 25 us before it ended instead of with it)
+template <typename K>
+inline cudaError_t allow_shared(K* kernel, size_t bytes) {
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  return e != cudaSuccess ? e : prefer_max_shared(kernel);
 }
 
 template <typename T> __device__ __forceinline__ float to_f32(T v);

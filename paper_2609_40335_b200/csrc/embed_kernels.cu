@@ -283,6 +283,23 @@ embed_norm_kernel(const int* __restrict__ ids, const T* __restrict__ G, long lon
   if (threadIdx.x == 0) partials[(size_t(i) * slabs + slab) * parts + part] = s;
 }
 
+// ------------------------------------------------------------------ side-stream kernels
+// The kernels from here on run on a second stream beside the persistent tensor-core kernels, whose CTAs
+// leave 4096 registers per SM (gemm_gta_big_kernel also 33 KiB of shared memory): blocks of 128
+// threads with 32 registers (one warp per quarter of an SM, whose register file they share out) fit
+// beside one; larger ones, such as the 256 and 1024 threads that these kernels had, wait until it has
+// ended.  The step, sustained: GPT-2 small B = 64, T = 256 with positions 5442 -> 5349 us, DistilGPT2 with all
+// its vectors B = 21, T = 203 1447 -> 1383, untied B = 32, T = 128 983 -> 937 (with the persistent kernels asking
+// for the carve-out, see allow_shared).
+constexpr int kSideThreads = 128;
+
+// zeros; a memset's own kernel does not fit beside a persistent one
+__global__ void __launch_bounds__(kSideThreads, 16) clear_kernel(uint4* __restrict__ p, size_t n16) {
+  const size_t stride = size_t(gridDim.x) * kSideThreads;
+#pragma unroll 4
+  for (size_t k = size_t(blockIdx.x) * kSideThreads + threadIdx.x; k < n16; k += stride) p[k] = make_uint4(0, 0, 0, 0);
+}
+
 // ------------------------------------------------------------------ sort kernels
 // Stable counting sort of the token ids: perm lists the positions by (id, position), seg[v] = number
 // of positions with id < v.
@@ -361,7 +378,8 @@ sort_one_block_kernel(const int* __restrict__ ids, int n, int V, int* __restrict
   }
 }
 
-__global__ void __launch_bounds__(kSortThreads)
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, 2048 / kThreads)
 sort_rank_kernel(const int* __restrict__ ids, int n, int V, int chunk_len, int* __restrict__ counts,
                  int* __restrict__ totals, int* __restrict__ rank, int* __restrict__ dev_status) {
   extern __shared__ __align__(16) int sm_i[];
@@ -371,7 +389,7 @@ sort_rank_kernel(const int* __restrict__ ids, int n, int V, int chunk_len, int* 
   const TokenGroups g{sm_i, sm_i + n32, sm_i + 2 * n32, keys, keys + slots};
   load_ids(ids + j0, m, V, g.id, dev_status);
   group_tokens(g, keys, keys + slots, slots, m);
-  for (int t = threadIdx.x; t < m; t += kSortThreads) {
+  for (int t = threadIdx.x; t < m; t += kThreads) {
     rank[j0 + t] = g.rank[t];
     const int id = g.id[t];
     if (id >= 0 && g.size[t] > 0) {
@@ -382,17 +400,26 @@ sort_rank_kernel(const int* __restrict__ ids, int n, int V, int chunk_len, int* 
 }
 
 // exclusive scan of the totals: block b adds up the totals before its 1024 entries itself (L2 reads)
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(kSideThreads, 16)
 sort_scan_kernel(const int* __restrict__ totals, int V, int* __restrict__ seg) {
-  __shared__ int wsum[32], wbase[32];
+  constexpr int kWarps = kSideThreads / 32;
+  static_assert(kSideThreads * 8 == 1024, "eight entries per thread");
+  __shared__ int wsum[kWarps], wbase[kWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int base = 0;
-  for (int v = threadIdx.x; v < blockIdx.x * 1024; v += 1024) base += totals[v];
+  const int4* t4 = reinterpret_cast<const int4*>(totals);
+#pragma unroll 4
+  for (int v = threadIdx.x; v < blockIdx.x * 256; v += kSideThreads) {
+    const int4 y = t4[v];
+    base += (y.x + y.y) + (y.z + y.w);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) base += __shfl_xor_sync(0xffffffffu, base, o);
-  const int v = blockIdx.x * 1024 + threadIdx.x;
-  const int x = v < V ? totals[v] : 0;
-  int inc = x;                                         // inclusive scan inside the warp
+  const int v0 = blockIdx.x * 1024 + 8 * threadIdx.x;
+  int x[8], s = 0;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) { x[e] = v0 + e < V ? totals[v0 + e] : 0; s += x[e]; }
+  int inc = s;                                         // inclusive scan inside the warp
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int y = __shfl_up_sync(0xffffffffu, inc, o);
@@ -400,18 +427,21 @@ sort_scan_kernel(const int* __restrict__ totals, int V, int* __restrict__ seg) {
   }
   if (lane == 31) { wsum[w] = inc; wbase[w] = base; }
   __syncthreads();
-  int before = 0;
-  for (int k = 0; k < 32; ++k) before += wbase[k] + (k < w ? wsum[k] : 0);
-  const int excl = before + inc - x;
-  if (v < V) seg[v] = excl;
-  if (v == V - 1) seg[V] = excl + x;
+  int run = inc - s;
+#pragma unroll
+  for (int k = 0; k < kWarps; ++k) run += wbase[k] + (k < w ? wsum[k] : 0);
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    if (v0 + e <= V) seg[v0 + e] = run;                // entry V: all tokens
+    run += x[e];
+  }
 }
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSideThreads, 16)
 sort_place_kernel(const int* __restrict__ ids, int n, int V, int chunk_len, const int* __restrict__ counts,
                   const int* __restrict__ rank, const int* __restrict__ seg, int* __restrict__ perm,
                   int* __restrict__ dev_status) {
-  const int j = blockIdx.x * 256 + threadIdx.x;
+  const int j = blockIdx.x * kSideThreads + threadIdx.x;
   if (j >= n) return;
   const int id = ids[j];
   if (id < 0 || id >= V) return;
@@ -423,12 +453,12 @@ sort_place_kernel(const int* __restrict__ ids, int n, int V, int chunk_len, cons
 }
 
 // ------------------------------------------------------------------ segmented row sum
-// The sorted order is cut into 32-position chunks; grid = (chunks, 256-column slabs).
+// The sorted order is cut into 32-position chunks; grid = (chunks, 128-column slabs).
 //   pass 1 (embed_scatter_kernel): a block finds the segments (runs of one token id) that meet
-//     its chunk.  Short segments (<= 32 rows) are summed by one warp each, from their head, in
-//     sorted order, and written to the table.  Rows of LONG segments (a frequent token) are
-//     summed per chunk by the whole block -- warp w takes rows w, w+8, ... and the eight warp
-//     sums are added in warp order -- into a partial buffer [chunk][slot][column]; slot 0 is the
+//     its chunk.  Short segments (<= 32 rows) are summed by the warp in whose quarter of the chunk
+//     they start, in sorted order, and written to the table.  Rows of LONG segments (a frequent
+//     token) are summed per chunk by the whole block -- warp w takes rows w, w+4, ... and the four
+//     warp sums are added in warp order -- into a partial buffer [chunk][slot][column]; slot 0 is the
 //     segment that continues from the previous chunk, slot 1 the one that starts in this chunk
 //     (a 32-position chunk can meet at most one of each).
 //   pass 2 (embed_scatter_combine_kernel): the block whose chunk holds a long segment's head
@@ -437,111 +467,133 @@ sort_place_kernel(const int* __restrict__ ids, int n, int V, int chunk_len, cons
 // and a very frequent token is spread over as many blocks as it has chunks.
 constexpr int kScatChunk = 32;     // sorted positions per block
 constexpr int kScatShort = 32;     // longest segment handled by a single warp
-constexpr int kScatBatch = 4;      // row loads in flight per lane
+constexpr int kScatCols = 128;     // columns per block, four per lane
+constexpr int kScatWarps = kSideThreads / 32;
+
+// four consecutive values of one row
+template <typename T> struct Raw4;
+template <> struct Raw4<__nv_bfloat16> {
+  uint2 q;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p, int nvalid, bool vec) {
+    if (vec && nvalid >= 4) {
+      q = *reinterpret_cast<const uint2*>(p);
+    } else {
+      uint32_t w[2] = {0u, 0u};
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (e < nvalid) w[e >> 1] |= uint32_t(__bfloat16_as_ushort(p[e])) << (16 * (e & 1));
+      q = make_uint2(w[0], w[1]);
+    }
+  }
+  __device__ __forceinline__ float4 unpack() const {
+    return make_float4(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xffff0000u),
+                       __uint_as_float(q.y << 16), __uint_as_float(q.y & 0xffff0000u));
+  }
+};
+template <> struct Raw4<float> {
+  float4 q;
+  __device__ __forceinline__ void load(const float* p, int nvalid, bool vec) {
+    if (vec && nvalid >= 4) q = *reinterpret_cast<const float4*>(p);
+    else q = make_float4(p[0], nvalid > 1 ? p[1] : 0.f, nvalid > 2 ? p[2] : 0.f, nvalid > 3 ? p[3] : 0.f);
+  }
+  __device__ __forceinline__ float4 unpack() const { return q; }
+};
+__device__ __forceinline__ void fma4(float4& a, float r, const float4& x) {
+  a.x = fmaf(r, x.x, a.x); a.y = fmaf(r, x.y, a.y); a.z = fmaf(r, x.z, a.z); a.w = fmaf(r, x.w, a.w);
+}
 
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSideThreads, 16)
 embed_scatter_kernel(const int* __restrict__ ids, const T* __restrict__ G, long long ldg, int Tn,
                      int d, const float* __restrict__ clip, const int* __restrict__ perm,
                      const int* __restrict__ seg, int V, float* __restrict__ out, long long ldo,
                      float beta, float scale, float* __restrict__ long_part, int n_rows,
                      int* __restrict__ dev_status) {
-  __shared__ float part[8][kEmbedColsPerBlock];
-  __shared__ int s_pos[kScatChunk + kScatShort];
+  constexpr int kBatch = sizeof(T) == 2 ? 4 : 2;         // row loads in flight per lane
+  static_assert(kScatChunk + kScatShort <= kSideThreads, "one staged row per thread");
+  __shared__ float4 part[kScatWarps][kScatCols / 4];
+  __shared__ int s_pos[kScatChunk + kScatShort], s_end[kScatChunk + kScatShort], s_n[kScatChunk];
   __shared__ float s_r[kScatChunk + kScatShort];
-  __shared__ int s_hk[kScatChunk], s_hv[kScatChunk], s_hn[kScatChunk];
-  __shared__ unsigned s_mask, s_long0, s_long1;
+  __shared__ unsigned s_short, s_long0, s_long1;
   const int n_valid = seg[V];
   const int kc = blockIdx.x * kScatChunk;
   if (kc >= n_valid) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 
-  // ---- classify the chunk's positions (warp 0) and stage positions / clip factors of the
-  //      chunk and of the kScatShort rows after it (threads 0..63)
-  int my_v = -1, my_n = 0;
-  bool head = false;
-  if (threadIdx.x < kScatChunk) {
+  // ---- stage positions and clip factors of the chunk and of the kScatShort rows after it, and
+  //      classify the chunk's positions (warp 0)
+  {
     const int k = kc + threadIdx.x;
-    int s0 = 0;
-    if (k < n_valid) {
-      const int pos = perm[k];
-      if (dp_in_range(pos, n_rows, dev_status)) my_v = ids[pos];
-      if (dp_in_range(my_v, V, dev_status)) {
-        s0 = seg[my_v];
-        my_n = seg[my_v + 1] - s0;
-        head = (s0 == k);
-      }
-    }
-    const bool is_long = my_n > kScatShort;
-    const unsigned m = __ballot_sync(0xffffffffu, head);
-    const unsigned l0 = __ballot_sync(0xffffffffu, is_long && s0 < kc);     // continues from before
-    const unsigned l1 = __ballot_sync(0xffffffffu, is_long && s0 >= kc);    // starts in this chunk
-    if (lane == 0) { s_mask = m; s_long0 = l0; s_long1 = l1; }
-  }
-  if (threadIdx.x < kScatChunk + kScatShort) {
-    const int k = kc + threadIdx.x;
-    if (k < n_valid) {
-      int pos = perm[k];
+    int pos = 0;
+    const bool staged = threadIdx.x < kScatChunk + kScatShort;
+    if (staged && k < n_valid) {
+      pos = perm[k];
       if (!dp_in_range(pos, n_rows, dev_status)) pos = 0;   // checked build: flagged, row 0 stands in
       s_pos[threadIdx.x] = pos;
       s_r[threadIdx.x] = clip[pos / Tn];
     }
-  }
-  __syncthreads();
-  const int n_heads = __popc(s_mask);
-  if (threadIdx.x < kScatChunk && head) {
-    const int slot = __popc(s_mask & ((1u << lane) - 1u));
-    s_hk[slot] = kc + threadIdx.x;
-    s_hv[slot] = my_v;
-    s_hn[slot] = my_n;
-  }
-  __syncthreads();
-
-  const int c = blockIdx.y * kEmbedColsPerBlock + lane * 8;
-  const int nvalid = min(8, d - c);
-  const bool vec = ((reinterpret_cast<uintptr_t>(G) & 15) == 0) && ((ldg * sizeof(T)) % 16 == 0);
-  const bool ovec = ((reinterpret_cast<uintptr_t>(out) & 15) == 0) && ((ldo & 3) == 0);
-
-  // ---- short segments: one warp each, rows in sorted order
-  for (int h = w; h < n_heads; h += 8) {
-    const int n = s_hn[h];
-    if (n > kScatShort || nvalid <= 0) continue;
-    const int o0 = s_hk[h] - kc, v = s_hv[h];          // rows o0 .. o0+n-1 of the staged window
-    float acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-    for (int b0 = 0; b0 < n; b0 += kScatBatch) {
-      float vals[kScatBatch][8];
-      float r[kScatBatch];
-#pragma unroll
-      for (int b = 0; b < kScatBatch; ++b) {
-        if (b0 + b < n) {
-          r[b] = s_r[o0 + b0 + b];
-          load8<T>(G + size_t(s_pos[o0 + b0 + b]) * ldg + c, nvalid, vec, vals[b]);
-        } else {
-          r[b] = 0.f;
-#pragma unroll
-          for (int e = 0; e < 8; ++e) vals[b][e] = 0.f;
+    if (staged) s_end[threadIdx.x] = -1;
+    if (w == 0) {
+      int v = -1, n = 0, s0 = 0;
+      if (k < n_valid) {
+        v = ids[pos];
+        if (dp_in_range(v, V, dev_status)) {
+          s0 = seg[v];
+          n = seg[v + 1] - s0;
         }
       }
-#pragma unroll
-      for (int b = 0; b < kScatBatch; ++b)
-#pragma unroll
-        for (int e = 0; e < 8; ++e) acc[e] = fmaf(r[b], vals[b][e], acc[e]);
+      const bool head = n > 0 && s0 == k, is_long = n > kScatShort;
+      const unsigned sh = __ballot_sync(0xffffffffu, head && !is_long);
+      const unsigned l0 = __ballot_sync(0xffffffffu, is_long && s0 < kc);     // continues from before
+      const unsigned l1 = __ballot_sync(0xffffffffu, is_long && s0 >= kc);    // starts in this chunk
+      if (lane == 0) { s_short = sh; s_long0 = l0; s_long1 = l1; }
+      s_n[lane] = n;
+      __syncwarp();
     }
-    float* o = out + size_t(v) * ldo + c;
-    if (ovec && nvalid == 8) {
-      float4 a = make_float4(acc[0] * scale, acc[1] * scale, acc[2] * scale, acc[3] * scale);
-      float4 b = make_float4(acc[4] * scale, acc[5] * scale, acc[6] * scale, acc[7] * scale);
-      if (beta != 0.f) {
-        const float4 oa = *reinterpret_cast<const float4*>(o), ob = *reinterpret_cast<const float4*>(o + 4);
-        a.x += oa.x; a.y += oa.y; a.z += oa.z; a.w += oa.w;
-        b.x += ob.x; b.y += ob.y; b.z += ob.z; b.w += ob.w;
+    __syncthreads();
+    if (w == 0 && ((s_short >> lane) & 1u)) s_end[lane + s_n[lane] - 1] = ids[pos];   // id at a segment's last row
+  }
+  __syncthreads();
+
+  const int c = blockIdx.y * kScatCols + lane * 4;
+  const int nvalid = min(4, d - c);
+  const bool vec = (reinterpret_cast<uintptr_t>(G) % (4 * sizeof(T)) == 0) && ((ldg & 3) == 0);
+  const bool ovec = ((reinterpret_cast<uintptr_t>(out) & 15) == 0) && ((ldo & 3) == 0) && nvalid == 4;
+
+  // ---- short segments: a warp takes those that start in its part of the chunk.  Their rows lie one after
+  //      the other (a long segment can only be the chunk's last), so batches of loads run across them.
+  constexpr int kPerWarp = kScatChunk / kScatWarps;
+  const unsigned mine = s_short & (((1u << kPerWarp) - 1u) << (kPerWarp * w));
+  if (mine != 0u && nvalid > 0) {
+    const int last = 31 - __clz(mine), end = last + s_n[last];
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int o0 = __ffs(mine) - 1; o0 < end; o0 += kBatch) {
+      Raw4<T> g[kBatch];
+#pragma unroll
+      for (int b = 0; b < kBatch; ++b)
+        if (o0 + b < end) g[b].load(G + size_t(s_pos[o0 + b]) * ldg + c, nvalid, vec);
+#pragma unroll
+      for (int b = 0; b < kBatch; ++b) {
+        if (o0 + b >= end) break;
+        fma4(acc, s_r[o0 + b], g[b].unpack());
+        const int v = s_end[o0 + b];
+        if (v >= 0) {
+          float* o = out + size_t(v) * ldo + c;
+          if (ovec) {
+            float4 p = make_float4(acc.x * scale, acc.y * scale, acc.z * scale, acc.w * scale);
+            if (beta != 0.f) {
+              const float4 q = *reinterpret_cast<const float4*>(o);
+              p.x += q.x; p.y += q.y; p.z += q.z; p.w += q.w;
+            }
+            *reinterpret_cast<float4*>(o) = p;
+          } else {
+            const float a[4] = {acc.x, acc.y, acc.z, acc.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) if (e < nvalid) o[e] = (beta != 0.f ? o[e] : 0.f) + a[e] * scale;
+          }
+          acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
       }
-      *reinterpret_cast<float4*>(o) = a;
-      *reinterpret_cast<float4*>(o + 4) = b;
-    } else {
-      for (int e = 0; e < nvalid; ++e) o[e] = (beta != 0.f ? o[e] : 0.f) + acc[e] * scale;
     }
   }
 
@@ -551,39 +603,25 @@ embed_scatter_kernel(const int* __restrict__ ids, const T* __restrict__ G, long 
     const unsigned m = slot == 0 ? s_long0 : s_long1;
     if (m == 0u) continue;                               // uniform over the block
     const int a = __ffs(m) - 1, b = 32 - __clz(m);       // the rows form one run [a, b)
-    float acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     if (nvalid > 0) {
-      float vals[kScatBatch][8];
+      for (int k0 = a + w; k0 < b; k0 += kScatWarps * kBatch) {
+        Raw4<T> g[kBatch];
 #pragma unroll
-      for (int j = 0; j < kScatBatch; ++j) {
-        const int k = a + w + 8 * j;
-        if (k < b) {
-          load8<T>(G + size_t(s_pos[k]) * ldg + c, nvalid, vec, vals[j]);
-        } else {
+        for (int j = 0; j < kBatch; ++j)
+          if (k0 + kScatWarps * j < b) g[j].load(G + size_t(s_pos[k0 + kScatWarps * j]) * ldg + c, nvalid, vec);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) vals[j][e] = 0.f;
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < kScatBatch; ++j) {
-        const int k = a + w + 8 * j;
-        if (k < b) {
-          const float r = s_r[k];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) acc[e] = fmaf(r, vals[j][e], acc[e]);
-        }
+        for (int j = 0; j < kBatch; ++j)
+          if (k0 + kScatWarps * j < b) fma4(acc, s_r[k0 + kScatWarps * j], g[j].unpack());
       }
     }
-#pragma unroll
-    for (int e = 0; e < 8; ++e) part[w][lane * 8 + e] = acc[e];
+    part[w][lane] = acc;
     __syncthreads();
-    const int cc = blockIdx.y * kEmbedColsPerBlock + threadIdx.x;
+    const int cc = blockIdx.y * kScatCols + threadIdx.x;
     if (cc < d) {
       float sum = 0.f;
 #pragma unroll
-      for (int ww = 0; ww < 8; ++ww) sum += part[ww][threadIdx.x];
+      for (int ww = 0; ww < kScatWarps; ++ww) sum += reinterpret_cast<const float*>(part[ww])[threadIdx.x];
       long_part[(size_t(blockIdx.x) * 2 + slot) * d + cc] = sum;
     }
     __syncthreads();
@@ -591,7 +629,7 @@ embed_scatter_kernel(const int* __restrict__ ids, const T* __restrict__ G, long 
 }
 
 // pass 2: table row of every long segment = beta*row + scale * (its partials in chunk order)
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSideThreads, 16)
 embed_scatter_combine_kernel(const int* __restrict__ ids, const int* __restrict__ perm,
                              const int* __restrict__ seg, int V, int d,
                              const float* __restrict__ long_part, float* __restrict__ out,
@@ -623,10 +661,11 @@ embed_scatter_combine_kernel(const int* __restrict__ ids, const int* __restrict_
   __syncthreads();
   const int n = s_n;
   if (n == 0) return;
-  const int cc = blockIdx.y * kEmbedColsPerBlock + threadIdx.x;
+  const int cc = blockIdx.y * kSideThreads + threadIdx.x;
   if (cc >= d) return;
   const int c0 = blockIdx.x, c1 = (s_k0 + n - 1) / kScatChunk;
   float sum = long_part[(size_t(c0) * 2 + 1) * d + cc];            // starts in its own chunk
+#pragma unroll 8
   for (int cch = c0 + 1; cch <= c1; ++cch) sum += long_part[(size_t(cch) * 2 + 0) * d + cc];
   float* o = out + size_t(s_v) * ldo + cc;
   sum *= scale;
@@ -666,15 +705,31 @@ dp_status launch_embed_norms(const int* ids, const void* G, int64_t ldg, dp_dtyp
   return DP_OK;
 }
 
+dp_status launch_clear(void* p, size_t bytes, cudaStream_t st) {
+  if ((reinterpret_cast<uintptr_t>(p) & 15) != 0) {
+    DP_CUDA_OK(cudaMemsetAsync(p, 0, bytes, st));
+    return DP_OK;
+  }
+  const size_t n16 = bytes / 16;
+  if (n16) {
+    if (first_use_on_this_device(reinterpret_cast<const void*>(&launch_clear)))
+      DP_CUDA_OK(prefer_max_shared(clear_kernel));
+    const size_t blocks = std::min((n16 + kSideThreads - 1) / kSideThreads, size_t(sm_count()) * 16);
+    clear_kernel<<<(unsigned)blocks, kSideThreads, 0, st>>>(static_cast<uint4*>(p), n16);
+    DP_LAUNCH_OK();
+  }
+  if (bytes & 15) DP_CUDA_OK(cudaMemsetAsync(static_cast<char*>(p) + n16 * 16, 0, bytes & 15, st));
+  return DP_OK;
+}
+
 dp_status launch_embed_sort(const int* ids, int n, int V, const EmbedSortWs& ws, int* dev_status,
                             cudaStream_t st) {
   if (first_use_on_this_device(reinterpret_cast<const void*>(&launch_embed_sort))) {
     DP_CUDA_OK(cudaFuncSetAttribute(sort_one_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)group_smem_bytes(kSortOneBlock)));
-    DP_CUDA_OK(cudaFuncSetAttribute(sort_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)group_smem_bytes(kSortOneBlock)));
+    DP_CUDA_OK(allow_shared(sort_rank_kernel<kSideThreads>, group_smem_bytes(kSortChunk)));
+    DP_CUDA_OK(allow_shared(sort_rank_kernel<4 * kSideThreads>, group_smem_bytes(4 * kSortChunk)));
     DP_CUDA_OK(prefer_max_shared(sort_one_block_kernel));
-    DP_CUDA_OK(prefer_max_shared(sort_rank_kernel));
     DP_CUDA_OK(prefer_max_shared(sort_scan_kernel));
     DP_CUDA_OK(prefer_max_shared(sort_place_kernel));
   }
@@ -687,15 +742,20 @@ dp_status launch_embed_sort(const int* ids, int n, int V, const EmbedSortWs& ws,
   // counts of the chunks before a token few
   const int chunk_len = n <= 32 * kSortChunk ? kSortChunk : 4 * kSortChunk;
   const int chunks = ceil_div(n, chunk_len);
-  DP_CUDA_OK(cudaMemsetAsync(ws.totals, 0, (size_t(V) + size_t(chunks) * V) * sizeof(int), st));
   int* counts = ws.totals + V;
-  sort_rank_kernel<<<chunks, kSortThreads, group_smem_bytes(chunk_len), st>>>(ids, n, V, chunk_len, counts,
-                                                                              ws.totals, ws.rank, dev_status);
+  dp_status s = launch_clear(ws.totals, align_up((size_t(V) + size_t(chunks) * V) * sizeof(int), 16), st);
+  if (s != DP_OK) return s;
+  if (chunk_len == kSortChunk)
+    sort_rank_kernel<kSideThreads><<<chunks, kSideThreads, group_smem_bytes(chunk_len), st>>>(
+        ids, n, V, chunk_len, counts, ws.totals, ws.rank, dev_status);
+  else
+    sort_rank_kernel<4 * kSideThreads><<<chunks, 4 * kSideThreads, group_smem_bytes(chunk_len), st>>>(
+        ids, n, V, chunk_len, counts, ws.totals, ws.rank, dev_status);
   DP_LAUNCH_OK();
-  sort_scan_kernel<<<ceil_div(V, 1024), 1024, 0, st>>>(ws.totals, V, ws.seg);
+  sort_scan_kernel<<<ceil_div(V + 1, 1024), kSideThreads, 0, st>>>(ws.totals, V, ws.seg);
   DP_LAUNCH_OK();
-  sort_place_kernel<<<ceil_div(n, 256), 256, 0, st>>>(ids, n, V, chunk_len, counts, ws.rank, ws.seg, ws.perm,
-                                                      dev_status);
+  sort_place_kernel<<<ceil_div(n, kSideThreads), kSideThreads, 0, st>>>(ids, n, V, chunk_len, counts, ws.rank,
+                                                                       ws.seg, ws.perm, dev_status);
   DP_LAUNCH_OK();
   return DP_OK;
 }
@@ -730,17 +790,18 @@ dp_status launch_embed_scatter(const int* ids, const void* G, int64_t ldg, dp_dt
     DP_CUDA_OK(prefer_max_shared(embed_scatter_kernel<__nv_bfloat16>));
     DP_CUDA_OK(prefer_max_shared(embed_scatter_combine_kernel));
   }
-  dim3 grid(ceil_div(n, kScatChunk), ceil_div(d, kEmbedColsPerBlock));
+  static_assert(kScatCols == kSideThreads, "both passes take 128 columns per block");
+  const dim3 grid(ceil_div(n, kScatChunk), ceil_div(d, kScatCols));
   if (dt == DP_F32)
-    embed_scatter_kernel<float><<<grid, 256, 0, st>>>(ids, (const float*)G, ldg, T, d, clip, perm,
+    embed_scatter_kernel<float><<<grid, kSideThreads, 0, st>>>(ids, (const float*)G, ldg, T, d, clip, perm,
                                                      seg, V, out, ldo, 1.f, scale, long_part, n,
                                                      dev_status);
   else
-    embed_scatter_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(ids, (const __nv_bfloat16*)G, ldg, T,
+    embed_scatter_kernel<__nv_bfloat16><<<grid, kSideThreads, 0, st>>>(ids, (const __nv_bfloat16*)G, ldg, T,
                                                              d, clip, perm, seg, V, out, ldo, 1.f,
                                                              scale, long_part, n, dev_status);
   DP_LAUNCH_OK();
-  embed_scatter_combine_kernel<<<grid, 256, 0, st>>>(ids, perm, seg, V, d, long_part, out, ldo, 1.f,
+  embed_scatter_combine_kernel<<<grid, kSideThreads, 0, st>>>(ids, perm, seg, V, d, long_part, out, ldo, 1.f,
                                                      scale, n, dev_status);
   DP_LAUNCH_OK();
   return DP_OK;

@@ -209,6 +209,8 @@ dp_status launch_cross_term_fma(const int* ids, const void* Ge, int64_t ldge, co
 
 dp_status launch_clip_factors(const float* sq, int B, float C, float* clip, float* norms,
                               cudaStream_t st, const float* extra, float* sq_out) {
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&launch_clip_factors)))
+    DP_CUDA_OK(prefer_max_shared(clip_factors_kernel));
   clip_factors_kernel<<<ceil_div(B, 128), 128, 0, st>>>(sq, B, C, clip, norms, extra, sq_out);
   DP_LAUNCH_OK();
   return DP_OK;

@@ -37,6 +37,7 @@ constexpr int kSortChunk = 1024;
 // Most tokens and ids that one block sorts by itself: one launch instead of four (10.4 -> 4.5 us at 64
 // tokens, 1000 ids); its scan over 50 257 ids by one SM would take 40 us.
 constexpr int kSortOneBlock = 4096, kSortOneBlockIds = 8192;
+dp_status launch_clear(void* p, size_t bytes, cudaStream_t st);
 dp_status launch_embed_sort(const int* ids, int n, int V, const EmbedSortWs& ws, int* dev_status,
                             cudaStream_t st);
 dp_status launch_embed_scatter(const int* ids, const void* G, int64_t ldg, dp_dtype dt, int n,
@@ -49,7 +50,7 @@ dp_status launch_bounds_probe(long long idx, long long n, int* dev_status, cudaS
 size_t embed_scatter_partial_bytes(long long n, int d);
 
 // logical (rows, cols) tensor with row pitch ld; element j = row*cols + col of the stream.
-// fill: write scale*amp*z without reading out.
+// fill: write scale*amp*z without reading out (first_quad: add mode only).
 dp_status launch_add_noise(float* out, long long rows, int cols, long long ld, bool fill, float amp,
                            float scale, uint64_t seed, uint32_t tensor_id, uint32_t step,
                            cudaStream_t st, long long first_quad = 0);

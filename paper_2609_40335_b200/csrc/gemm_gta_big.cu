@@ -478,8 +478,7 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
 dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, const float* clip, float beta,
                          const GtaNoise* noise, int* dev_status, cudaStream_t st) {
   if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_big_kernel)))
-    DP_CUDA_OK(cudaFuncSetAttribute(gemm_gta_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kSmemBytes));
+    DP_CUDA_OK(allow_shared(gemm_gta_big_kernel, kSmemBytes));
   BigParams P;
   memset(&P, 0, sizeof(P));
   const int planes = terms > 1 ? 2 * B : B;

@@ -629,9 +629,7 @@ constexpr bool kUsePair = true;
 template <bool kScale, bool kSqsum, bool kPair>
 dp_status set_attr_once() {
   if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_kernel<kScale, kSqsum, kPair>)))
-    DP_CUDA_OK(cudaFuncSetAttribute(gemm_gta_kernel<kScale, kSqsum, kPair>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)Geo<kPair>::kSmemBytes));
+    DP_CUDA_OK(allow_shared(gemm_gta_kernel<kScale, kSqsum, kPair>, Geo<kPair>::kSmemBytes));
   return DP_OK;
 }
 
@@ -726,6 +724,8 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
         pre += prescale_bytes(D, B, T);
         const long long rows = (long long)B * T;
         const int blocks = (int)std::min<long long>((rows * (cp >> 3) + 255) / 256, (long long)sms * 16);
+        if (first_use_on_this_device(reinterpret_cast<const void*>(&prescale_rows_kernel)))
+          DP_CUDA_OK(prefer_max_shared(prescale_rows_kernel));
         prescale_rows_kernel<<<blocks, 256, 0, st>>>(
             static_cast<const __nv_bfloat16*>(narrow_a ? D.A : D.G), narrow_a ? D.lda : D.ldg, copy, cp,
             rows, T, c, clip);

@@ -328,8 +328,7 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
 dp_status launch_ghost_norm_pair(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
                                  float* partials, int* dev_status, cudaStream_t st) {
   if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_pair_kernel)))
-    DP_CUDA_OK(cudaFuncSetAttribute(ghost_norm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kSmemBytes));
+    DP_CUDA_OK(allow_shared(ghost_norm_pair_kernel, kSmemBytes));
   const int nt = ceil_div(T, kTile2);
   for (size_t g0 = 0; g0 < plan.ghost_layers.size(); g0 += kGhostMaxLayers) {
     const size_t g1 = std::min(plan.ghost_layers.size(), g0 + kGhostMaxLayers);

@@ -311,9 +311,7 @@ namespace {
 template <bool kDiagOnly, bool kSplit>
 dp_status launch_variant(const GhostParams& P, cudaStream_t st) {
   if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_tc_kernel<kDiagOnly, kSplit>)))
-    DP_CUDA_OK(cudaFuncSetAttribute(ghost_norm_tc_kernel<kDiagOnly, kSplit>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)GhostGeo<kDiagOnly, kSplit>::kSmemBytes));
+    DP_CUDA_OK(allow_shared(ghost_norm_tc_kernel<kDiagOnly, kSplit>, GhostGeo<kDiagOnly, kSplit>::kSmemBytes));
   const int grid = std::min(P.total_items, sm_count());
   ghost_norm_tc_kernel<kDiagOnly, kSplit><<<grid, kThreads, GhostGeo<kDiagOnly, kSplit>::kSmemBytes, st>>>(P);
   DP_LAUNCH_OK();

@@ -46,6 +46,34 @@ add_noise_kernel(float* __restrict__ out, long long n, int cols, long long ld, f
   }
 }
 
+// The same for a contiguous 16-byte aligned tensor, shaped to run beside the persistent tensor-core kernels:
+// those leave each quarter of an SM room for one warp of 32 registers and, some of them, no shared
+// memory at all, hence blocks of 128 threads with 32 registers and 32-bit counters (a launch covers at
+// most kFillSlice of them; first_hi and first_lo are those of the slice's first).  At B = 64, T = 256 the 38.6 M
+// elements of a 50257 x 768 table are drawn inside gemm_gta_big_kernel's time; blocks of 256 threads with 44
+// registers came after it and took 250 us (see embed_kernels.cu for the steps' times).
+constexpr int kFillThreads = 128;
+constexpr long long kFillSlice = 1LL << 30;
+
+__global__ void __launch_bounds__(kFillThreads, 16)
+fill_noise_kernel(float* __restrict__ out, uint32_t nq, int tail, float amp, float scale,
+                  const __grid_constant__ NoiseKeys keys, uint32_t tensor_id, uint32_t step,
+                  const uint32_t* __restrict__ step_dev, uint32_t first_hi, uint32_t first_lo) {
+  step = effective_step(step, step_dev);
+  for (uint32_t q = blockIdx.x * kFillThreads + threadIdx.x; q < nq; q += gridDim.x * kFillThreads) {
+    float z[4];
+    normals4(((unsigned long long)first_hi << 32) | (first_lo + q), keys, tensor_id, step, z);
+    float* o = out + 4 * size_t(q);
+    if (tail == 0 || q + 1 < nq) {
+      *reinterpret_cast<float4*>(o) = make_float4(noised(0.f, z[0], amp, scale), noised(0.f, z[1], amp, scale),
+                                                  noised(0.f, z[2], amp, scale), noised(0.f, z[3], amp, scale));
+    } else {                                               // the last counter's `tail` elements
+#pragma unroll
+      for (int e = 0; e < 3; ++e) if (e < tail) o[e] = noised(0.f, z[e], amp, scale);
+    }
+  }
+}
+
 // Exhaustive error scan of the fp32 Box-Muller factors.  k runs over all 2^24 values of the
 // 24-bit integer that feeds the factor.  out[0] = max relative error of r = sqrt(-2 ln u1) (the
 // unrounded rh + rl that multiplies the direction) over the inputs with r^2 <= t_max, out[1] = max
@@ -98,19 +126,27 @@ dp_status launch_add_noise(float* out, long long rows, int cols, long long ld, b
   const long long n = rows * cols;
   if (n == 0) return DP_OK;
   const long long nq = (n + 3) >> 2;
-  const long long want = (nq + 255) / 256;
-  // Fill mode is meant to run beside another kernel (it depends on no gradient): four blocks
-  // per SM leave half of every SM's thread slots free for it.
-  const int grid = (int)std::min<long long>(want, (long long)sm_count() * (fill ? 4 : 16));
   const NoiseKeys keys = expand_noise_keys(seed);
-  if (fill && first_use_on_this_device(reinterpret_cast<const void*>(&launch_add_noise)))
-    DP_CUDA_OK(prefer_max_shared(add_noise_kernel<true>));
+  if (fill && ld == cols && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+    if (first_use_on_this_device(reinterpret_cast<const void*>(&launch_add_noise)))
+      DP_CUDA_OK(prefer_max_shared(fill_noise_kernel));
+    for (long long q0 = 0; q0 < nq; q0 += kFillSlice) {
+      const long long m = std::min(nq - q0, kFillSlice), q = first_quad + q0;
+      const int tail = q0 + m == nq ? int(n & 3) : 0;
+      const int grid = (int)std::min<long long>((m + kFillThreads - 1) / kFillThreads, (long long)sm_count() * 16);
+      fill_noise_kernel<<<grid, kFillThreads, 0, st>>>(out + 4 * q0, uint32_t(m), tail, amp, scale, keys, tensor_id,
+                                                       step, g_step_dev, uint32_t(q >> 32), uint32_t(q));
+      DP_LAUNCH_OK();
+    }
+    return DP_OK;
+  }
+  const int grid = (int)std::min<long long>((nq + 255) / 256, (long long)sm_count() * 16);
   if (fill)
-    add_noise_kernel<true><<<grid, 256, 0, st>>>(out, n, cols, ld, amp, scale, keys, tensor_id, step,
-                                             g_step_dev, first_quad);
+    add_noise_kernel<true><<<grid, 256, 0, st>>>(out, n, cols, ld, amp, scale, keys, tensor_id, step, g_step_dev,
+                                                 first_quad);
   else
-    add_noise_kernel<false><<<grid, 256, 0, st>>>(out, n, cols, ld, amp, scale, keys, tensor_id, step,
-                                             g_step_dev, first_quad);
+    add_noise_kernel<false><<<grid, 256, 0, st>>>(out, n, cols, ld, amp, scale, keys, tensor_id, step, g_step_dev,
+                                                  first_quad);
   DP_LAUNCH_OK();
   return DP_OK;
 }

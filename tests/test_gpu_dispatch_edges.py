@@ -201,3 +201,41 @@ def test_two_tile_items_give_up_cleanly():
         lib.dp_debug_set_wait_limit(prev)
     again, flag = run()
     assert flag == 0 and torch.equal(good, again)
+
+
+# the fill kernel writes whole counters of an aligned tensor, its last one element by element; a launch of it
+# covers 148 * 16 * 128 counters per pass
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 511, 512, 513, 4 * 148 * 16 * 128 + 6])
+def test_noise_fill_equals_noise_on_zeros(n):
+    filled = torch.full((n + 4,), 7.0, device="cuda")
+    added = torch.zeros(n, device="cuda")
+    dp.dp_fill_noise(filled, 0.7, 1.5, 0.5, 11, 3, 9, n=n)
+    dp.dp_add_noise(added, 0.7, 1.5, 0.5, 11, 3, 9)
+    assert torch.equal(filled[:n], added)                # the same stream, bit for bit
+    assert (filled[n:] == 7.0).all()
+
+
+# row sums: four columns per lane, 128 per block, a warp per quarter of a chunk of 32 sorted positions;
+# segments of up to 32 rows belong to one warp, longer ones to all blocks they meet
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("d,ldo,ldg", [(1, 1, 1), (3, 4, 6), (127, 131, 128), (128, 128, 128), (129, 132, 132), (264, 264, 266)])
+def test_row_sums_at_the_edges(dtype, d, ldo, ldg):
+    B, T, V = 2, 210, 40
+    lengths = [1, 7, 8, 9, 31, 32, 33, 64, 2, 1, 30, 1, 32, 100, 3, 66]
+    assert sum(lengths) == B * T
+    ids = torch.repeat_interleave(torch.arange(len(lengths)), torch.tensor(lengths))
+    g = torch.Generator()
+    g.manual_seed(d)
+    ids = ids[torch.randperm(B * T, generator=g)].to(torch.int32).view(B, T).cuda()
+    G = torch.randn(B, T, ldg, generator=g).to(torch.float32 if dtype == "f32" else torch.bfloat16).cuda()
+    clip = torch.rand(B, generator=g).cuda()
+    out = torch.full((V, ldo), 5.0, device="cuda")
+    dp.dp_clip_accumulate_embed(ids, G, V, None, 1.0, out, d=d, clip=clip)
+    want = torch.zeros(V, d, dtype=torch.float64, device="cuda")
+    rows = (G[..., :d].double() * clip.double()[:, None, None]).reshape(B * T, d)
+    want.index_add_(0, ids.flatten().long(), rows)
+    # fp32 sums of at most 100 terms of size |R g|: n eps times their sum of magnitudes
+    size = torch.zeros_like(want).index_add_(0, ids.flatten().long(), rows.abs())
+    assert ((out[:, :d].double() - want).abs() <= 110 * 2.0 ** -24 * size).all()
+    if ldo > d:
+        assert (out[:, d:] == 5.0).all()
