@@ -581,14 +581,9 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
         group.add(layers[l], l, B, T, true, base);
         continue;
       }
-      s = launch_clip_accumulate_fma(layers[l].A, layers[l].lda, layers[l].G, layers[l].ldg, dt, B, T,
-                                     layers[l].d, layers[l].p, clip_ws, outs[l], ldos[l], beta, st);
+      s = launch_clip_accumulate_fma(layers[l], dt, B, T, clip_ws, outs[l], ldos[l], beta, noise,
+                                     noise ? noise->tensor_ids[l] : 0u, st);
       if (s != DP_OK) return s;
-      if (noise) {
-        s = launch_add_noise(outs[l], layers[l].p, layers[l].d, ldos[l], false, noise->amp,
-                             noise->scale, noise->seed, noise->tensor_ids[l], noise->step, st);
-        if (s != DP_OK) return s;
-      }
     }
     return flush();
   }

@@ -8,9 +8,11 @@ namespace dpg {
 
 dp_status launch_norms_fma(const dp_linear_desc& L, dp_dtype dt, int mode, int B, int T, float* sq,
                            cudaStream_t st, bool overwrite = false);
-dp_status launch_clip_accumulate_fma(const void* A, int64_t lda, const void* G, int64_t ldg,
-                                     dp_dtype dt, int B, int T, int d, int p, const float* clip,
-                                     float* out, int64_t ldo, float beta, cudaStream_t st);
+// noise: added onto the sum (inside the kernel where d is a multiple of 4), NULL = none
+struct GtaNoise;
+dp_status launch_clip_accumulate_fma(const dp_linear_desc& L, dp_dtype dt, int B, int T, const float* clip,
+                                     float* out, int64_t ldo, float beta, const GtaNoise* noise,
+                                     uint32_t tensor_id, cudaStream_t st);
 // partials: [B * ceil(T/16)] floats, example-major
 dp_status launch_cross_term_fma(const int* ids, const void* Ge, int64_t ldge, const void* Al,
                                 int64_t ldal, const void* Gl, int64_t ldgl, dp_dtype dt, int B,

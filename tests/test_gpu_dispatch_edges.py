@@ -239,3 +239,36 @@ def test_row_sums_at_the_edges(dtype, d, ldo, ldg):
     assert ((out[:, :d].double() - want).abs() <= 110 * 2.0 ** -24 * size).all()
     if ldo > d:
         assert (out[:, d:] == 5.0).all()
+
+
+# layers that stay on the fp32 kernels: tiles of 32 or 64 outputs (64 from 148 of them on), noise inside the
+# kernel where d is a multiple of 4; sums and noise are the same bits as in two calls
+@pytest.mark.parametrize("d,p,B,T", [(64, 64, 4, 16), (32, 33, 1, 1), (4, 7, 3, 5), (30, 40, 2, 31), (62, 70, 1, 33),
+                                     (768, 800, 2, 9), (770, 769, 2, 9)])
+def test_fp32_kernels_with_noise(d, p, B, T):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d + p)
+    A = torch.randn(B, T, d, generator=g, device="cuda")
+    G = torch.randn(B, T, p, generator=g, device="cuda")
+    clip = torch.rand(B, generator=g, device="cuda")
+    layers = [dp.Linear(A, G, d=d, p=p)]
+    out, noisy = torch.full((p, d), 3.0, device="cuda"), torch.full((p, d), 3.0, device="cuda")
+    before = dp.dp_debug_force_fma(True)
+    try:
+        dp.dp_clip_accumulate_grouped(layers, B, T, None, 1.0, [out], beta=1.0, clip=clip)
+        dp.dp_clip_accumulate_noise_grouped(layers, B, T, None, 1.0, [noisy], 0.7, 0.5, 5, [2], 3, beta=1.0, clip=clip)
+        sq = torch.zeros(B, device="cuda")
+        dp.dp_ghost_norms(layers, B, T, sq)
+    finally:
+        dp.dp_debug_force_fma(before)
+    G64, A64 = (G * clip[:, None, None]).double(), A.double()
+    want = 3.0 + torch.einsum("btp,btd->pd", G64, A64)
+    size = 3.0 + torch.einsum("btp,btd->pd", G64.abs(), A64.abs())
+    assert ((out.double() - want).abs() <= (B * T + 2) * 2.0 ** -24 * size).all()
+    dp.dp_add_noise(out, 0.7, 1.0, 0.5, 5, 2, 3)
+    assert torch.equal(out, noisy)
+    grads = torch.einsum("btp,btd->bpd", G.double(), A64)
+    norms = (grads ** 2).sum((1, 2))
+    # sums of at most T^2 products of dots of max(d, p) terms; their magnitudes add up to |A|^2 |G|^2
+    size = (A64 ** 2).sum((1, 2)) * (G.double() ** 2).sum((1, 2))
+    assert ((sq.double() - norms).abs() <= 2.0 ** -24 * (64 + T * T / 32) * size).all()
