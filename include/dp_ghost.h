@@ -308,7 +308,8 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
  * overwritten; side_sq [dev, B], perm / seg and pos_perm / pos_seg [dev, as in dp_embed_sort] are
  * scratch, as are ws (the largest *_ws_bytes of the calls on `stream`, and
  * dp_clip_accumulate_embed_ws_bytes when tied) and side_ws (the largest of dp_embed_norms_ws_bytes,
- * dp_embed_sort_ws_bytes and dp_clip_accumulate_embed_ws_bytes over both tables).  events: four
+ * dp_embed_sort_ws_bytes and dp_clip_accumulate_embed_ws_bytes over both tables; with
+ * dp_embed_norms_ws_bytes more per table one kernel adds up all the norms' partial sums).  events: four
  * cudaEvent_t of the caller that order the two streams; `stream` has waited for `side_stream` at the
  * end.  phases: DP_STEP_ALL, or the three phases one after the other with the same descriptor (so
  * that a caller can time them). */

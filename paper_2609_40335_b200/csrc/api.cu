@@ -295,7 +295,8 @@ size_t dp_ghost_norms_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, d
 // overwrite: sq is written instead of added to (its first contribution of a step)
 static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B,
                                   int32_t T, float* sq, void* ws, size_t ws_bytes, int32_t* dev_status,
-                                  void* stream, bool overwrite) {
+                                  void* stream, bool overwrite, NormSource* left = nullptr) {
+  // left: the last reduction is not done; *left says where its partial sums are (or sq itself)
   if (!layers || n_layers <= 0 || B <= 0 || T <= 0 || !sq) return DP_ERR_INVALID_ARG;
   if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
@@ -332,6 +333,7 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
       if (s != DP_OK) return s;
       layers[l].mode_used = plan.mode_used[l];
     }
+    if (left) *left = NormSource{sq, 1, 1.f, nullptr};
     return flush();
   }
   const size_t need = align_up(size_t(B) * plan.n_per * sizeof(float), 256);
@@ -347,7 +349,8 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
     s = launch_direct_norm_tc(layers, plan, B, T, 1, partials, dev_status, st);
     if (s != DP_OK) return s;
   }
-  s = launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st, overwrite);
+  if (left) *left = NormSource{partials, plan.n_per, 1.f, nullptr};
+  else s = launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st, overwrite);
   if (s != DP_OK) return s;
   for (int l = 0; l < n_layers; ++l) layers[l].mode_used = plan.mode_used[l];
   return DP_OK;
@@ -367,7 +370,8 @@ size_t dp_embed_norms_ws_bytes(int32_t B, int32_t T, int32_t d) {
 
 static dp_status embed_norms_impl(const int32_t* ids, const void* G, int64_t ldg, dp_dtype dt, int32_t B,
                                   int32_t T, int32_t d, int32_t V, float* sq, int32_t* first_occ, void* ws,
-                                  size_t ws_bytes, int32_t* dev_status, void* stream, bool overwrite) {
+                                  size_t ws_bytes, int32_t* dev_status, void* stream, bool overwrite,
+                                  NormSource* left = nullptr) {
   if (!ids || !G || !sq || B <= 0 || T <= 0 || d <= 0 || V <= 0 || ldg < d) return DP_ERR_INVALID_ARG;
   if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
   if (T > kEmbedMaxT) return DP_ERR_UNSUPPORTED;
@@ -377,8 +381,9 @@ static dp_status embed_norms_impl(const int32_t* ids, const void* G, int64_t ldg
   const int parts = embed_norm_parts(B, T, d);
   dp_status s = launch_embed_norms(ids, G, ldg, dt, B, T, d, V, parts, partials, first_occ, dev_status, st);
   if (s != DP_OK) return s;
-  return launch_reduce_partials(partials, ceil_div(d, kEmbedColsPerBlock) * parts, B, sq, 1.f, nullptr, st,
-                                overwrite);
+  const int n_per = ceil_div(d, kEmbedColsPerBlock) * parts;
+  if (left) { *left = NormSource{partials, n_per, 1.f, nullptr}; return DP_OK; }
+  return launch_reduce_partials(partials, n_per, B, sq, 1.f, nullptr, st, overwrite);
 }
 
 dp_status dp_embed_norms(const int32_t* ids, const void* G, int64_t ldg, dp_dtype dt, int32_t B,
@@ -396,10 +401,10 @@ size_t dp_tied_cross_term_ws_bytes(int32_t B, int32_t T, int32_t d, int32_t V) {
   return align_up(size_t(B) * per * sizeof(float), 256);
 }
 
-dp_status dp_tied_cross_term(const int32_t* ids, const void* G_emb, int64_t ldge, const void* A_lm,
-                             int64_t ldal, const void* G_lm, int64_t ldgl, dp_dtype dt, int32_t B,
-                             int32_t T, int32_t d, int32_t V, float* sq, float* cross, void* ws,
-                             size_t ws_bytes, int32_t* dev_status, void* stream) {
+static dp_status cross_term_impl(const int32_t* ids, const void* G_emb, int64_t ldge, const void* A_lm,
+                                 int64_t ldal, const void* G_lm, int64_t ldgl, dp_dtype dt, int32_t B,
+                                 int32_t T, int32_t d, int32_t V, float* sq, float* cross, void* ws,
+                                 size_t ws_bytes, int32_t* dev_status, void* stream, NormSource* left) {
   if (!ids || !G_emb || !A_lm || !G_lm || B <= 0 || T <= 0 || d <= 0 || V <= 0)
     return DP_ERR_INVALID_ARG;
   if (!sq && !cross) return DP_ERR_INVALID_ARG;
@@ -422,7 +427,16 @@ dp_status dp_tied_cross_term(const int32_t* ids, const void* G_emb, int64_t ldge
     per = ceil_div(T, 16);
   }
   if (s != DP_OK) return s;
+  if (left) { *left = NormSource{partials, per, 2.f, cross}; return DP_OK; }
   return launch_reduce_partials(partials, per, B, sq, 2.f, cross, st);
+}
+
+dp_status dp_tied_cross_term(const int32_t* ids, const void* G_emb, int64_t ldge, const void* A_lm,
+                             int64_t ldal, const void* G_lm, int64_t ldgl, dp_dtype dt, int32_t B,
+                             int32_t T, int32_t d, int32_t V, float* sq, float* cross, void* ws,
+                             size_t ws_bytes, int32_t* dev_status, void* stream) {
+  return cross_term_impl(ids, G_emb, ldge, A_lm, ldal, G_lm, ldgl, dt, B, T, d, V, sq, cross, ws, ws_bytes,
+                         dev_status, stream, nullptr);
 }
 
 // ------------------------------------------------------- bias / LayerNorm parameters
@@ -440,8 +454,8 @@ size_t dp_vector_norms_ws_bytes(const dp_vector_desc* prm, int32_t n, int32_t B,
   return align_up(size_t(B) * vector_total_slabs(prm, n) * sizeof(float), 256);
 }
 
-dp_status dp_vector_norms(const dp_vector_desc* prm, int32_t n, dp_dtype dt, int32_t B, int32_t T,
-                          float* sq, void* ws, size_t ws_bytes, void* stream) {
+static dp_status vector_norms_impl(const dp_vector_desc* prm, int32_t n, dp_dtype dt, int32_t B, int32_t T,
+                                   float* sq, void* ws, size_t ws_bytes, void* stream, NormSource* left) {
   const dp_status c = check_vectors(prm, n, B, T);
   if (c != DP_OK) return c;
   if (!sq || (dt != DP_F32 && dt != DP_BF16)) return DP_ERR_INVALID_ARG;
@@ -451,7 +465,13 @@ dp_status dp_vector_norms(const dp_vector_desc* prm, int32_t n, dp_dtype dt, int
   const int n_per = vector_total_slabs(prm, n);
   dp_status s = launch_vector_norms(prm, n, dt, B, T, partials, n_per, st);
   if (s != DP_OK) return s;
+  if (left) { *left = NormSource{partials, n_per, 1.f, nullptr}; return DP_OK; }
   return launch_reduce_partials(partials, n_per, B, sq, 1.f, nullptr, st);
+}
+
+dp_status dp_vector_norms(const dp_vector_desc* prm, int32_t n, dp_dtype dt, int32_t B, int32_t T,
+                          float* sq, void* ws, size_t ws_bytes, void* stream) {
+  return vector_norms_impl(prm, n, dt, B, T, sq, ws, ws_bytes, stream, nullptr);
 }
 
 static size_t vector_partial_bytes(const dp_vector_desc* prm, int32_t n, int32_t B, int32_t T) {
@@ -498,7 +518,8 @@ dp_status dp_clip_accumulate_vectors(const dp_vector_desc* prm, int32_t n, dp_dt
 dp_status dp_clip_factors_sum(float* sq, const float* sq_extra, int32_t B, float C, float* clip,
                               float* norms, void* stream) {
   if (!sq || !sq_extra || B <= 0 || !finite_pos(C)) return DP_ERR_INVALID_ARG;
-  return launch_clip_factors(sq, B, C, clip, norms, (cudaStream_t)stream, sq_extra, sq);
+  const NormSources N{{{sq, 1, 1.f, nullptr}, {sq_extra, 1, 1.f, nullptr}}, 1, 2};
+  return launch_finish_norms(N, B, C, sq, clip, norms, (cudaStream_t)stream);
 }
 
 dp_status dp_clip_factors(const float* sq, int32_t B, float C, float* clip, float* norms,
@@ -847,33 +868,46 @@ static dp_status start_table(const dp_step_desc* S, float* table, int64_t ld, in
 static dp_status step_norms(const dp_step_desc* S) {
   cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
   const dp_dtype dt = (dp_dtype)S->dtype;
+  const int B = S->B, T = S->T;
   dp_status s;
+  NormSources N;                 // partial sums that the last kernel of this phase adds up
+  N.n = 0;
+  size_t held = 0;               // bytes at the head of ws that hold such sums
+  char* ws = static_cast<char*>(S->ws);
   DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[0], main));
   if (S->n_layers) {
-    s = ghost_norms_impl(S->layers, S->n_layers, dt, S->B, S->T, S->sq, S->ws, S->ws_bytes, S->dev_status,
-                         main, true);
+    s = ghost_norms_impl(S->layers, S->n_layers, dt, B, T, S->sq, S->ws, S->ws_bytes, S->dev_status, main, true,
+                         &N.src[0]);
     if (s != DP_OK) return s;
-  } else {
-    DP_CUDA_OK(cudaMemsetAsync(S->sq, 0, size_t(S->B) * sizeof(float), main));
+    if (N.src[0].partials == S->ws) held = align_up(size_t(B) * N.src[0].n_per * sizeof(float), 256);
+    N.n = 1;
   }
   // Side stream: all that needs neither the big norm kernel nor the clip factors.  It is enqueued
   // after that kernel: what is already resident keeps the kernel's CTAs out until it ends, what
   // arrives second shares the SMs with them.
   DP_CUDA_OK(cudaStreamWaitEvent(side, (cudaEvent_t)S->events[0], 0));     // earlier readers are done
-  s = embed_norms_impl(S->ids, S->G_emb, S->ldge, dt, S->B, S->T, S->d, S->V, S->side_sq, nullptr, S->side_ws,
-                       S->side_ws_bytes, S->dev_status, side, true);
-  if (s != DP_OK) return s;
-  if (S->pos_ids) {
-    s = embed_norms_impl(S->pos_ids, S->G_emb, S->ldge, dt, S->B, S->T, S->d, S->T, S->side_sq, nullptr,
-                         S->side_ws, S->side_ws_bytes, S->dev_status, side, false);
+  // The embedding norms' partial sums stay at the end of side_ws, out of the sorts' way, where it has room.
+  const size_t each = dp_embed_norms_ws_bytes(B, T, S->d), tables = S->pos_ids ? 2 : 1;
+  const size_t sorts = std::max(dp_embed_sort_ws_bytes(B, T, S->V),
+                                S->pos_ids ? dp_embed_sort_ws_bytes(B, T, S->pos_rows) : size_t(0));
+  char* side_ws = static_cast<char*>(S->side_ws);
+  size_t side_bytes = S->side_ws_bytes & ~size_t(255);
+  const bool keep = side_bytes >= sorts + tables * each;
+  NormSource embed[2];
+  for (size_t k = 0; k < tables; ++k) {
+    char* w = side_ws;
+    if (keep) { side_bytes -= each; w += side_bytes; }
+    s = embed_norms_impl(k ? S->pos_ids : S->ids, S->G_emb, S->ldge, dt, B, T, S->d, k ? T : S->V, S->side_sq, nullptr,
+                         w, keep ? each : S->side_ws_bytes, S->dev_status, side, k == 0, keep ? &embed[k] : nullptr);
     if (s != DP_OK) return s;
   }
+  if (!keep) embed[0] = NormSource{S->side_sq, 1, 1.f, nullptr};
   DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[1], side));
-  s = dp_embed_sort(S->ids, S->B, S->T, S->V, S->perm, S->seg, S->side_ws, S->side_ws_bytes, S->dev_status, side);
+  s = dp_embed_sort(S->ids, B, T, S->V, S->perm, S->seg, side_ws, side_bytes, S->dev_status, side);
   if (s != DP_OK) return s;
   if (S->pos_ids) {
-    s = dp_embed_sort(S->pos_ids, S->B, S->T, S->pos_rows, S->pos_perm, S->pos_seg, S->side_ws,
-                      S->side_ws_bytes, S->dev_status, side);
+    s = dp_embed_sort(S->pos_ids, B, T, S->pos_rows, S->pos_perm, S->pos_seg, side_ws, side_bytes, S->dev_status,
+                      side);
     if (s != DP_OK) return s;
     s = start_table(S, S->wpe, S->ld_wpe, S->pos_rows, S->wpe_id, side);
     if (s != DP_OK) return s;
@@ -882,20 +916,42 @@ static dp_status step_norms(const dp_step_desc* S) {
     s = start_table(S, S->wte, S->ld_wte, S->V, S->wte_id, side);
     if (s != DP_OK) return s;
   }
-  // main stream again
+  // main stream again.  Where ws has no room behind the sums it holds, they are added up first.
+  auto room = [&](size_t need) {
+    if (held + need <= S->ws_bytes) return DP_OK;
+    for (int k = 0; k < N.n; ++k) {
+      if (N.src[k].partials == S->sq) continue;
+      const dp_status r = launch_reduce_partials(N.src[k].partials, N.src[k].n_per, B, S->sq, N.src[k].factor,
+                                                 N.src[k].plain_out, main, k == 0);
+      if (r != DP_OK) return r;
+    }
+    if (N.n) { N.src[0] = NormSource{S->sq, 1, 1.f, nullptr}; N.n = 1; }
+    held = 0;
+    return DP_OK;
+  };
   if (S->n_vectors) {
-    s = dp_vector_norms(S->vectors, S->n_vectors, dt, S->B, S->T, S->sq, S->ws, S->ws_bytes, main);
+    const size_t need = dp_vector_norms_ws_bytes(S->vectors, S->n_vectors, B, T);
+    s = room(need);
     if (s != DP_OK) return s;
+    s = vector_norms_impl(S->vectors, S->n_vectors, dt, B, T, S->sq, ws + held, S->ws_bytes - held, main, &N.src[N.n]);
+    if (s != DP_OK) return s;
+    ++N.n;
+    held += need;
   }
   if (S->tied) {
     const dp_linear_desc& lm = S->layers[S->n_layers - 1];
-    s = dp_tied_cross_term(S->ids, S->G_emb, S->ldge, lm.A, lm.lda, lm.G, lm.ldg, dt, S->B, S->T, S->d, S->V,
-                           S->sq, S->cross, S->ws, S->ws_bytes, S->dev_status, main);
+    s = room(dp_tied_cross_term_ws_bytes(B, T, S->d, S->V));
     if (s != DP_OK) return s;
+    s = cross_term_impl(S->ids, S->G_emb, S->ldge, lm.A, lm.lda, lm.G, lm.ldg, dt, B, T, S->d, S->V, S->sq, S->cross,
+                        ws + held, S->ws_bytes - held, S->dev_status, main, &N.src[N.n]);
+    if (s != DP_OK) return s;
+    ++N.n;
   }
+  N.n_main = N.n;
+  N.src[N.n++] = embed[0];
+  if (keep && tables == 2) N.src[N.n++] = embed[1];
   DP_CUDA_OK(cudaStreamWaitEvent(main, (cudaEvent_t)S->events[1], 0));
-  // the two accumulators join in one fixed order of additions, then Eq. 7
-  s = launch_clip_factors(S->sq, S->B, S->C, S->clip, S->norms, main, S->side_sq, S->sq);
+  s = launch_finish_norms(N, B, S->C, S->sq, S->clip, S->norms, main);
   if (s != DP_OK) return s;
   DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[3], main));
   return DP_OK;

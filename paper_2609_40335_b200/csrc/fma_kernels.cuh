@@ -19,8 +19,15 @@ dp_status launch_cross_term_fma(const int* ids, const void* Ge, int64_t ldge, co
                                 int T, int d, int V, float* partials, int* dev_status,
                                 cudaStream_t st);
 dp_status launch_clip_factors(const float* sq, int B, float C, float* clip, float* norms,
-                              cudaStream_t st, const float* extra = nullptr,
-                              float* sq_out = nullptr);
+                              cudaStream_t st);
+// Partial sums of squared norms that a step has left in workspaces: [B][n_per] floats each.
+struct NormSource { const float* partials; int n_per; float factor; float* plain_out; };
+struct NormSources {
+  NormSource src[6];
+  int n_main, n;             // src[0 .. n_main) are added up, src[n_main .. n) are, then the two sums
+};
+dp_status launch_finish_norms(const NormSources& S, int B, float C, float* sq, float* clip, float* norms,
+                              cudaStream_t st);
 
 // embedding
 constexpr int kEmbedMaxT = 4096;

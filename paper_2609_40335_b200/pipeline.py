@@ -344,6 +344,8 @@ def _side_buffers(ds: DeviceStep) -> dict:
         for rows in [ds.V] + ([WPE_ROWS] if ds.positions else []):
             need = max(need, int(L.dp_embed_sort_ws_bytes(ds.B, ds.T, rows)),
                        int(L.dp_clip_accumulate_embed_ws_bytes(ds.B, ds.T, ds.d_model, rows)))
+        # the norms' partial sums lie behind what the sorts use
+        need = (need + 255) // 256 * 256 + 2 * int(L.dp_embed_norms_ws_bytes(ds.B, ds.T, ds.d_model))
         if ds.side_stream is None:
             ds.side_stream = torch.cuda.Stream(device=dev)
         events = [torch.cuda.Event() for _ in range(4)]
