@@ -14,7 +14,8 @@
 // first `skew` K steps of an item feed sub-tile 0 only, the steps up to the last feed both, and sub-tile
 // 1 makes up for the steps it missed at the end.  While one sub-tile's accumulator is read -- and its
 // Gaussian noise drawn, which takes thousands of cycles -- the tensor cores work on the other.  The
-// price is loading X of `skew` steps twice and running those steps at half the products per stage.
+// price is loading X of `skew` steps twice and running those steps at half the products per stage (with
+// few K steps it is not paid: skew 0).
 // (Drawing the noise beside the item's MMAs and parking it, or the sums, in the output cost 8 % of the
 // kernel in output traffic.)
 //
@@ -513,8 +514,12 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
   P.terms = terms; P.tsteps = terms * ceil_div(T, kBK); P.ksteps = B * P.tsteps;
   // Long enough to read one accumulator, and to draw its noise, while the other is fed: with noise 4, 6, 8,
   // 10, 12, 24 and 40 steps gave 2341, 2278, 2252, 2265, 2283, 2407 and 2513 us (B = 16, T = 512).  The same
-  // without noise, which would do with 2, so that a sum does not depend on whether noise is fused.
-  P.skew = std::min(P.ksteps, 8);
+  // without noise, which would do with 2 or none, so that a sum does not depend on whether noise is fused.
+  // With few K steps the epilogue is all there is and the staggered steps only cost loads: no skew below 16.
+  // Sustained, with noise: 215.0 -> 204.6 us at 6 steps (B = 3, T = 77, 48 GPT-2-small layers), 243.5 -> 232.6 at 8
+  // (B = 4, T = 128), but 298.6 -> 305.9 at 16 and 772 -> 790 at 32.  (Without noise
+  // 258.7 -> 241.6 at 16 as well.)
+  P.skew = P.ksteps < 16 ? 0 : 8;
   P.beta = beta; P.clip = clip;
   if (noise) {
     P.noise_keys = expand_noise_keys(noise->seed);

@@ -155,7 +155,8 @@ BIG_SHAPES = [[(257, 19001)], [(19000, 250)], [(700, 13000), (100, 3000), (64, 6
 
 
 @pytest.mark.parametrize("shapes", BIG_SHAPES)
-@pytest.mark.parametrize("beta,noise,B,T", [(0.0, False, 3, 50), (1.0, True, 3, 50), (0.0, True, 1, 7), (0.0, True, 20, 64)])
+@pytest.mark.parametrize("beta,noise,B,T", [(0.0, False, 3, 50), (1.0, True, 3, 50), (0.0, True, 1, 7), (0.0, True, 15, 64),
+                                            (0.0, True, 16, 64)])
 def test_two_tile_items(shapes, beta, noise, B, T):
     layers = [dp.Linear(bf16((B, T, d), 1.0, k, ld=(d + 7) // 8 * 8), bf16((B, T, p), 0.1, 50 + k, ld=(p + 7) // 8 * 8),
                         d=d, p=p) for k, (d, p) in enumerate(shapes)]
