@@ -306,13 +306,15 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
  * as in dp_clip_accumulate_vectors.  pos_ids NULL: no position table.  with_noise 0: the bare
  * clipped sums.  sq, clip [dev, B] and norms, cross [dev, B or NULL; cross is needed when tied] are
  * overwritten; side_sq [dev, B], perm / seg and pos_perm / pos_seg [dev, as in dp_embed_sort] are
- * scratch, as are ws (the largest *_ws_bytes of the calls on `stream`, and
+ * scratch, as are ws (the largest *_ws_bytes of the calls on `stream`, dp_step_ws_bytes if fp32 layers
+ * are to be split once instead of for the norms and again for the sums, and
  * dp_clip_accumulate_embed_ws_bytes when tied) and side_ws (the largest of dp_embed_norms_ws_bytes,
  * dp_embed_sort_ws_bytes and dp_clip_accumulate_embed_ws_bytes over both tables; with
  * dp_embed_norms_ws_bytes more per table one kernel adds up all the norms' partial sums).  events: four
  * cudaEvent_t of the caller that order the two streams; `stream` has waited for `side_stream` at the
  * end.  phases: DP_STEP_ALL, or the three phases one after the other with the same descriptor (so
  * that a caller can time them). */
+size_t dp_step_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B, int32_t T);
 enum { DP_STEP_NORMS = 1, DP_STEP_GEMM = 2, DP_STEP_REST = 4, DP_STEP_ALL = 7 };
 typedef struct {
   dp_linear_desc* layers;  float* const* outs;  const int64_t* ldos;  const uint32_t* tensor_ids;

@@ -71,7 +71,7 @@ EXPORTS = ["dp_vector_norms", "dp_vector_norms_ws_bytes", "dp_clip_accumulate_ve
            "dp_last_cuda_error", "dp_version", "dp_kernel_launches", "dp_debug_force_fma",
            "dp_debug_noise_error_scan", "dp_debug_bounds_checked", "dp_debug_bounds_probe",
            "dp_debug_tensor_map_encodes", "dp_debug_set_wait_limit",
-           "dp_debug_ghost_single", "dp_set_reserved_sms", "dp_step_enqueue"]
+           "dp_debug_ghost_single", "dp_set_reserved_sms", "dp_step_enqueue", "dp_step_ws_bytes"]
 
 
 def lib_path() -> str:
@@ -90,6 +90,8 @@ def load():
     L.dp_ghost_norms.argtypes = [C.POINTER(_LinearDesc), i32, i32, i32, i32, vp, vp, sz, vp, vp]
     L.dp_ghost_norms_ws_bytes.argtypes = [C.POINTER(_LinearDesc), i32, i32, i32, i32]
     L.dp_ghost_norms_ws_bytes.restype = sz
+    L.dp_step_ws_bytes.argtypes = [C.POINTER(_LinearDesc), i32, i32, i32, i32]
+    L.dp_step_ws_bytes.restype = sz
     L.dp_embed_norms.argtypes = [vp, vp, i64, i32, i32, i32, i32, i32, vp, vp, vp, sz, vp, vp]
     VP = C.POINTER(_VectorDesc)
     L.dp_vector_norms.argtypes = [VP, i32, i32, i32, i32, vp, vp, sz, vp]
@@ -551,6 +553,11 @@ def dp_fill_noise(out: torch.Tensor, sigma: float, C_: float, scale: float, seed
     st = L.dp_fill_noise(_ptr(out), n, float(sigma), float(C_), float(scale), int(seed) & (2 ** 64 - 1),
                          int(tensor_id), int(step), _stream(stream))
     _check(st, "dp_fill_noise")
+
+
+def dp_step_ws_bytes(layers: Sequence[Linear], B: int, T: int) -> int:
+    """Workspace with which a step splits fp32 layers once (0: nothing to gain); see the header."""
+    return int(load().dp_step_ws_bytes(_descs(layers), len(layers), _dt(layers[0].A), B, T))
 
 
 def dp_step_enqueue(layers, outs, tensor_ids, vectors, vector_outs, vector_ids, *, ids, G_emb, pos_ids, wte, wpe,

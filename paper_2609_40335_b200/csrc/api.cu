@@ -159,15 +159,16 @@ struct SplitGroup {
   long long tiles = 0;                  // sums: output tiles
   size_t out_bytes = 0;                 // and one fp32 plane of every output
 
-  void add(const dp_linear_desc& L, int l, int B, int T, bool scale_g, char* base) {
+  // scale: the narrower operand is to be multiplied by the clip factors
+  void add(const dp_linear_desc& L, int l, int B, int T, bool scale, char* base) {
     dp_linear_desc D = L;
     const long long rows = (long long)B * T;
     D.mode = resolve_mode(L, T);
     D.A = base + bytes; D.lda = split_padded(L.d);
-    jobs.push_back({static_cast<const float*>(L.A), L.lda, L.d, false, base + bytes});
+    jobs.push_back({static_cast<const float*>(L.A), L.lda, L.d, scale && L.d <= L.p, base + bytes});
     bytes += split_bytes(rows, L.d);
     D.G = base + bytes; D.ldg = split_padded(L.p);
-    jobs.push_back({static_cast<const float*>(L.G), L.ldg, L.p, scale_g, base + bytes});
+    jobs.push_back({static_cast<const float*>(L.G), L.ldg, L.p, scale && L.d > L.p, base + bytes});
     bytes += split_bytes(rows, L.p);
     index.push_back(l);
     desc.push_back(D);
@@ -189,9 +190,10 @@ static size_t f32_norm_bytes(const dp_linear_desc& L, int B, int T, int sms) {
   return split_layer_bytes(L, B, T) + align_up(size_t(B) * plan.n_per * sizeof(float), 256);
 }
 
-// norms of a group of fp32 layers: split, Gram or gradient-tile kernels, one reduction
+// norms of a group of fp32 layers: split, Gram or gradient-tile kernels, one reduction (or, with `left`,
+// the place of the partial sums)
 static dp_status f32_norm_group(const SplitGroup& g, int B, int T, float* sq, char* ws, int* dev_status,
-                                cudaStream_t st, bool overwrite) {
+                                cudaStream_t st, bool overwrite, NormSource* left) {
   const GhostPlan plan = plan_ghost_norms(g.desc.data(), (int)g.desc.size(), B, T, sm_count(), false);
   float* partials = reinterpret_cast<float*>(ws + g.bytes);
   dp_status s = launch_split(g.jobs.data(), (int)g.jobs.size(), B, T, nullptr, st);
@@ -204,6 +206,7 @@ static dp_status f32_norm_group(const SplitGroup& g, int B, int T, float* sq, ch
     s = launch_direct_norm_tc(g.desc.data(), plan, B, T, 3, partials, dev_status, st);
     if (s != DP_OK) return s;
   }
+  if (left) { *left = NormSource{partials, plan.n_per, 1.f, nullptr}; return DP_OK; }
   return launch_reduce_partials(partials, plan.n_per, B, sq, 1.f, nullptr, st, overwrite);
 }
 
@@ -295,8 +298,10 @@ size_t dp_ghost_norms_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, d
 // overwrite: sq is written instead of added to (its first contribution of a step)
 static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B,
                                   int32_t T, float* sq, void* ws, size_t ws_bytes, int32_t* dev_status,
-                                  void* stream, bool overwrite, NormSource* left = nullptr) {
+                                  void* stream, bool overwrite, NormSource* left = nullptr,
+                                  SplitGroup* kept = nullptr) {
   // left: the last reduction is not done; *left says where its partial sums are (or sq itself)
+  // kept: the split operands of fp32 layers, where they stay in ws all together; empty if they do not
   if (!layers || n_layers <= 0 || B <= 0 || T <= 0 || !sq) return DP_ERR_INVALID_ARG;
   if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
@@ -310,10 +315,14 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
     if (dt == DP_F32 && dp_ghost_norms_ws_bytes(layers, n_layers, dt, B, T) > ws_bytes) return DP_ERR_WORKSPACE;
     SplitGroup group;
     char* base = static_cast<char*>(ws);
+    if (left) *left = NormSource{sq, 1, 1.f, nullptr};
+    int flushed = 0;
     auto flush = [&]() {
       if (group.index.empty()) return DP_OK;
-      const dp_status s = f32_norm_group(group, B, T, sq, base, dev_status, st, overwrite);
+      const bool all = (int)group.index.size() == n_layers;
+      const dp_status s = f32_norm_group(group, B, T, sq, base, dev_status, st, overwrite, all ? left : nullptr);
       overwrite = false;
+      if (kept) { if (flushed++ == 0) *kept = std::move(group); else *kept = SplitGroup(); }
       group = SplitGroup();
       return s;
     };
@@ -333,7 +342,6 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
       if (s != DP_OK) return s;
       layers[l].mode_used = plan.mode_used[l];
     }
-    if (left) *left = NormSource{sq, 1, 1.f, nullptr};
     return flush();
   }
   const size_t need = align_up(size_t(B) * plan.n_per * sizeof(float), 256);
@@ -549,7 +557,7 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
                                       int32_t B, int32_t T, const float* sq, float C, float* clip,
                                       float* const* outs, const int64_t* ldos, float beta,
                                       const GtaNoise* noise, void* ws, size_t ws_bytes,
-                                      int32_t* dev_status, void* stream) {
+                                      int32_t* dev_status, void* stream, const SplitGroup* kept = nullptr) {
   if (!layers || n_layers <= 0 || !outs || !ldos || (!sq && !clip) || B <= 0 || T <= 0) return DP_ERR_INVALID_ARG;
   if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
   if (!(beta == 0.f || beta == 1.f) || !finite_pos(C)) return DP_ERR_INVALID_ARG;
@@ -573,7 +581,7 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
     SplitGroup group;
     auto flush = [&]() {
       if (group.index.empty()) return DP_OK;
-      // R_i multiplies G in fp32 before the split, so the GEMM runs unscaled (clip = NULL)
+      // R_i multiplies the narrower operand in fp32 before the split, so the GEMM runs unscaled (clip = NULL)
       dp_status s = launch_split(group.jobs.data(), (int)group.jobs.size(), B, T, clip_ws, st);
       if (s != DP_OK) return s;
       std::vector<float*> out;
@@ -591,8 +599,25 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
       group = SplitGroup();
       return s;
     };
+    if (kept && !kept->index.empty() && !sq &&
+        kept->bytes + gta_partial_bytes(kept->desc.data(), (int)kept->desc.size(), B, T, 3, sm_count()) <= ws_bytes) {
+      // the norms' split operands are still there: only the narrower one of each layer is split again, scaled
+      group = *kept;
+      base = static_cast<char*>(ws);
+      group.jobs.clear();
+      for (size_t k = 0; k < kept->index.size(); ++k) {
+        SplitJob J = kept->jobs[2 * k + (layers[kept->index[k]].d <= layers[kept->index[k]].p ? 0 : 1)];
+        J.scaled = true;
+        group.jobs.push_back(J);
+      }
+      s = flush();
+      if (s != DP_OK) return s;
+    } else {
+      kept = nullptr;
+    }
     for (int l = 0; l < n_layers; ++l) {
       if (dt == DP_F32 && f32_on_tensor_cores(layers[l], T)) {
+        if (kept) continue;
         // the K split, and with it the planes of partial sums, follows from the group's tiles
         const size_t out = align_up(size_t(layers[l].p) * size_t(layers[l].d) * sizeof(float), 256);
         const int ns = gta_choose_nsplit(group.tiles + gta_tiles(layers[l]), B, T, 3, sm_count());
@@ -839,6 +864,22 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
 }
 
 // ------------------------------------------------------------------------------ whole step
+// Workspace with which fp32 layers are split once per step: the group of all of them, the norms' partial
+// sums, the K-split planes.  Beyond 16 GiB the layers go through less in groups.
+size_t dp_step_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B, int32_t T) {
+  if (!layers || n_layers <= 0 || B <= 0 || T <= 0 || dt != DP_F32) return 0;
+  std::vector<dp_linear_desc> on;
+  size_t need = 0;
+  for (int l = 0; l < n_layers; ++l)
+    if (f32_on_tensor_cores(layers[l], T)) {
+      need += f32_norm_bytes(layers[l], B, T, sm_count());
+      on.push_back(layers[l]);
+    }
+  if (on.empty()) return 0;
+  need += gta_partial_bytes(on.data(), (int)on.size(), B, T, 3, sm_count());
+  return need <= (size_t(16) << 30) ? need : 0;
+}
+
 static dp_status check_step(const dp_step_desc* S) {
   if (!S || S->B <= 0 || S->T <= 0 || S->V <= 0 || S->d <= 0 || S->n_layers < 0 || S->n_vectors < 0)
     return DP_ERR_INVALID_ARG;
@@ -865,7 +906,7 @@ static dp_status start_table(const dp_step_desc* S, float* table, int64_t ld, in
 }
 
 // events: [0] the step began, [1] embedding norms done, [2] row sums done, [3] clip factors exist
-static dp_status step_norms(const dp_step_desc* S) {
+static dp_status step_norms(const dp_step_desc* S, SplitGroup* kept) {
   cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
   const dp_dtype dt = (dp_dtype)S->dtype;
   const int B = S->B, T = S->T;
@@ -877,10 +918,13 @@ static dp_status step_norms(const dp_step_desc* S) {
   DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[0], main));
   if (S->n_layers) {
     s = ghost_norms_impl(S->layers, S->n_layers, dt, B, T, S->sq, S->ws, S->ws_bytes, S->dev_status, main, true,
-                         &N.src[0]);
+                         &N.src[0], kept);
     if (s != DP_OK) return s;
-    if (N.src[0].partials == S->ws) held = align_up(size_t(B) * N.src[0].n_per * sizeof(float), 256);
     N.n = 1;
+    if (N.src[0].partials != S->sq)
+      held = size_t(reinterpret_cast<const char*>(N.src[0].partials) - ws) +
+             align_up(size_t(B) * N.src[0].n_per * sizeof(float), 256);
+    if (kept) held = std::max(held, kept->bytes);
   }
   // Side stream: all that needs neither the big norm kernel nor the clip factors.  It is enqueued
   // after that kernel: what is already resident keeps the kernel's CTAs out until it ends, what
@@ -919,6 +963,7 @@ static dp_status step_norms(const dp_step_desc* S) {
   // main stream again.  Where ws has no room behind the sums it holds, they are added up first.
   auto room = [&](size_t need) {
     if (held + need <= S->ws_bytes) return DP_OK;
+    if (kept) *kept = SplitGroup();
     for (int k = 0; k < N.n; ++k) {
       if (N.src[k].partials == S->sq) continue;
       const dp_status r = launch_reduce_partials(N.src[k].partials, N.src[k].n_per, B, S->sq, N.src[k].factor,
@@ -957,15 +1002,12 @@ static dp_status step_norms(const dp_step_desc* S) {
   return DP_OK;
 }
 
-static dp_status step_gemm(const dp_step_desc* S) {
+static dp_status step_gemm(const dp_step_desc* S, const SplitGroup* kept) {
   if (!S->n_layers) return DP_OK;
-  const dp_dtype dt = (dp_dtype)S->dtype;
-  if (S->with_noise)
-    return dp_clip_accumulate_noise_grouped(S->layers, S->n_layers, dt, S->B, S->T, nullptr, S->C, S->clip,
-                                            S->outs, S->ldos, 0.f, S->sigma, 1.f, S->seed, S->tensor_ids,
-                                            S->step, S->ws, S->ws_bytes, S->dev_status, S->stream);
-  return dp_clip_accumulate_grouped(S->layers, S->n_layers, dt, S->B, S->T, nullptr, S->C, S->clip, S->outs,
-                                    S->ldos, 0.f, S->ws, S->ws_bytes, S->dev_status, S->stream);
+  const GtaNoise noise{S->sigma * S->C, 1.f, S->seed, S->step, S->tensor_ids};
+  return clip_accumulate_impl(S->layers, S->n_layers, (dp_dtype)S->dtype, S->B, S->T, nullptr, S->C, S->clip, S->outs,
+                              S->ldos, 0.f, S->with_noise ? &noise : nullptr, S->ws, S->ws_bytes, S->dev_status,
+                              S->stream, kept);
 }
 
 static dp_status step_rest(const dp_step_desc* S) {
@@ -1005,8 +1047,11 @@ static dp_status step_rest(const dp_step_desc* S) {
 dp_status dp_step_enqueue(const dp_step_desc* S, int32_t phases) {
   dp_status s = check_step(S);
   if (s != DP_OK) return s;
-  if (phases & DP_STEP_NORMS) { s = step_norms(S); if (s != DP_OK) return s; }
-  if (phases & DP_STEP_GEMM) { s = step_gemm(S); if (s != DP_OK) return s; }
+  // fp32 layers: within one call the sums can use the norms' split operands
+  SplitGroup split;
+  SplitGroup* kept = phases == DP_STEP_ALL && S->dtype == DP_F32 ? &split : nullptr;
+  if (phases & DP_STEP_NORMS) { s = step_norms(S, kept); if (s != DP_OK) return s; }
+  if (phases & DP_STEP_GEMM) { s = step_gemm(S, kept); if (s != DP_OK) return s; }
   if (phases & DP_STEP_REST) { s = step_rest(S); if (s != DP_OK) return s; }
   return DP_OK;
 }

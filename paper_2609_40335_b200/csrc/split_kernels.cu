@@ -10,8 +10,10 @@
 // coordinate.  (Widened copies [hi | hi | lo] and [hi | lo | hi] took three to six times the
 // workspace and traffic and, the workspace being sized for one layer, a dozen launches per layer:
 // 24 layers and a head of DistilGPT2 at B = 8, T = 128 took 236 launches, now 12.)
-// For the clipped sum the clip factor R_i (Eq. 7) multiplies G in fp32 BEFORE the split, so the
-// GEMM itself runs unscaled and no bf16 rounding of R_i * g occurs.
+// For the clipped sum the clip factor R_i (Eq. 7) multiplies the narrower operand in fp32 BEFORE the
+// split, so the GEMM itself runs unscaled and no bf16 rounding of R_i * g occurs.  In a whole step the other
+// operand's planes are those of the norms, where the workspace holds all layers: 999 -> 865 us (DistilGPT2,
+// B = 8, T = 128, the second split 180 -> 44).
 #include <cuda_bf16.h>
 
 #include <algorithm>

@@ -162,6 +162,14 @@ def allocate(ds: DeviceStep) -> None:
         need = max(need, int(L.dp_clip_accumulate_embed_ws_bytes(ds.B, ds.T, ds.d_model, WPE_ROWS)))
     if ds.tied:
         need = max(need, int(L.dp_tied_cross_term_ws_bytes(ds.B, ds.T, ds.d_model, ds.V)))
+    if every:
+        once = dp.dp_step_ws_bytes(every, ds.B, ds.T)
+        if once:                      # the norms' partial sums of vectors and cross term lie behind it
+            if ds.vectors:
+                once += dp.dp_vector_norms_ws_bytes(ds.vectors, ds.B, ds.T)
+            if ds.tied:
+                once += int(L.dp_tied_cross_term_ws_bytes(ds.B, ds.T, ds.d_model, ds.V))
+        need = max(need, once)
     ds.ws = torch.empty(need, dtype=torch.uint8, device=dev)
 
 

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2609_40335_b200 import binding as dp
+from paper_2609_40335_b200 import binding as dp, pipeline
 
 pytestmark = pytest.mark.gpu
 
@@ -273,3 +273,49 @@ def test_fp32_kernels_with_noise(d, p, B, T):
     # sums of at most T^2 products of dots of max(d, p) terms; their magnitudes add up to |A|^2 |G|^2
     size = (A64 ** 2).sum((1, 2)) * (G.double() ** 2).sum((1, 2))
     assert ((sq.double() - norms).abs() <= 2.0 ** -24 * (64 + T * T / 32) * size).all()
+
+
+# fp32 step: split operands kept from the norms for the sums (ample workspace), layers in groups (the least
+# workspace), one layer on the FMA kernels among them; against the same step call by call
+@pytest.mark.parametrize("ample", [False, True])
+@pytest.mark.parametrize("kind", ["plain", "tied", "vectors", "fma", "direct"])
+def test_fp32_step_with_kept_operands(ample, kind):
+    B, T, V, d = 3, 40, 700, 72
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+
+    def normal(cols, std):
+        return torch.empty(B, T, cols, device="cuda").normal_(0.0, std, generator=g)
+
+    shapes = [(d, 3 * d), (3 * d, d), (d, d)] + ([(d, 8)] if kind == "fma" else [])
+    linears = [dp.Linear(normal(i, 1.0), normal(o, 0.05), d=i, p=o) for i, o in shapes]
+    if kind == "direct":
+        linears[1].mode = dp.DP_NORM_DIRECT
+    ids = torch.randint(0, V, (B, T), generator=g, device="cuda", dtype=torch.int32)
+    vec = dict(dtype=torch.float32, device="cuda")
+    ds = pipeline.DeviceStep(
+        B=B, T=T, V=V, C=1.0, sigma=0.8, tied=kind == "tied", positions=False, linears=linears,
+        lm=dp.Linear(normal(d, 1.0), normal(V, 0.02), d=d, p=V), ids=ids, pos_ids=None, G_emb=normal(d, 0.05), d_model=d,
+        sq=torch.zeros(B, **vec), clip=torch.zeros(B, **vec), norms=torch.zeros(B, **vec),
+        cross=torch.zeros(B, **vec) if kind == "tied" else None,
+        dev_status=torch.zeros(1, dtype=torch.int32, device="cuda"))
+    if kind == "vectors":
+        ds.vectors = [dp.Vector(normal(d, 0.05), normal(d, 1.0), p=d), dp.Vector(linears[0].G, None, p=3 * d)]
+    pipeline.allocate(ds)
+    full = ds.ws.numel()
+    if not ample:
+        every = ds.linears + [ds.lm]
+        least = max(dp.dp_ghost_norms_ws_bytes(every, B, T), dp.dp_clip_accumulate_grouped_ws_bytes(every, B, T),
+                    int(dp.load().dp_clip_accumulate_embed_ws_bytes(B, T, d, V)))
+        assert least < full
+        ds.ws = torch.empty(least, dtype=torch.uint8, device="cuda")
+    pipeline.dp_step(ds, noise=False, overlap=False)
+    want = {n: t.clone() for n, t in ds.outs.items()}
+    want_sq = ds.sq.clone()
+    for t in ds.outs.values():
+        t.fill_(9.0)
+    pipeline.dp_step(ds, noise=False)
+    assert torch.allclose(ds.sq, want_sq, rtol=1e-5)     # the same products, summed in groups of another size
+    for n, t in ds.outs.items():
+        assert float((t - want[n]).norm()) <= 1e-5 * float(want[n].norm()), n
+    assert int(ds.dev_status.item()) == 0
