@@ -40,22 +40,6 @@ class _VectorDesc(C.Structure):
                 ("p", C.c_int32)]
 
 
-class _StepDesc(C.Structure):
-    _fields_ = [(n, C.c_void_p) for n in ("layers", "outs", "ldos", "tensor_ids", "vectors", "vector_outs",
-                                          "vector_ids", "ids", "G_emb")]
-    _fields_ += [("ldge", C.c_int64), ("pos_ids", C.c_void_p), ("wte", C.c_void_p), ("ld_wte", C.c_int64),
-                 ("wpe", C.c_void_p), ("ld_wpe", C.c_int64)]
-    _fields_ += [(n, C.c_void_p) for n in ("sq", "clip", "norms", "cross", "side_sq", "perm", "seg",
-                                           "pos_perm", "pos_seg")]
-    _fields_ += [("ws", C.c_void_p), ("ws_bytes", C.c_size_t), ("side_ws", C.c_void_p),
-                 ("side_ws_bytes", C.c_size_t), ("dev_status", C.c_void_p), ("stream", C.c_void_p),
-                 ("side_stream", C.c_void_p), ("events", C.c_void_p * 4), ("seed", C.c_uint64)]
-    _fields_ += [(n, C.c_int32) for n in ("n_layers", "n_vectors", "dtype", "B", "T", "V", "d", "pos_rows",
-                                          "tied", "with_noise")]
-    _fields_ += [("C", C.c_float), ("sigma", C.c_float), ("step", C.c_uint32), ("wte_id", C.c_uint32),
-                 ("wpe_id", C.c_uint32)]
-
-
 STEP_NORMS, STEP_GEMM, STEP_REST, STEP_ALL = 1, 2, 4, 7
 
 EXPORTS = ["dp_vector_norms", "dp_vector_norms_ws_bytes", "dp_clip_accumulate_vectors",
@@ -139,7 +123,7 @@ def load():
     L.dp_fill_noise.argtypes = [vp, i64, f32, f32, f32, C.c_uint64, C.c_uint32, C.c_uint32, vp]
     L.dp_add_noise_slice.argtypes = [vp, i64, i64, f32, f32, f32, C.c_uint64, C.c_uint32, C.c_uint32, vp]
     L.dp_noise_step_device.argtypes = [vp]
-    L.dp_step_enqueue.argtypes = [C.POINTER(_StepDesc), i32]
+    L.dp_step_enqueue.argtypes = [vp, i32]
     L.dp_rdp_epsilon.argtypes = [C.c_double, C.c_double, i64, C.c_double, vp, vp]
     L.dp_sigma_for_epsilon.argtypes = [C.c_double, i64, C.c_double, C.c_double, C.c_double, vp]
     L.dp_status_string.argtypes = [i32]
@@ -566,26 +550,18 @@ def dp_step_enqueue(layers, outs, tensor_ids, vectors, vector_outs, vector_ids, 
                     phases=STEP_ALL):
     """The whole step (or some of its phases) in one library call; see the header."""
     L = load()
-    n, nv = len(layers), len(vectors)
-    arr = _descs(layers) if n else None
-    varr = _vdescs(vectors) if nv else None
-    (optr, ldos), (vptr, _) = _outputs(outs), _outputs(vector_outs)
-    tids, vids = (C.c_uint32 * n)(*tensor_ids), (C.c_uint32 * nv)(*vector_ids)
-    at = C.addressof
-    B, T = ids.shape
-    S = _StepDesc(
-        at(arr) if n else None, at(optr) if n else None, at(ldos) if n else None, at(tids),
-        at(varr) if nv else None, at(vptr) if nv else None, at(vids), _ptr(ids), _ptr(G_emb), _rows_ld(G_emb),
-        _ptr(pos_ids), _ptr(wte), wte.stride(0), _ptr(wpe), wpe.stride(0) if wpe is not None else 0, _ptr(sq),
-        _ptr(clip), _ptr(norms), _ptr(cross), _ptr(side_sq), _ptr(perm), _ptr(seg), _ptr(pos_perm),
-        _ptr(pos_seg), _ptr(ws), ws.nbytes, _ptr(side_ws), side_ws.nbytes, _ptr(dev_status), _stream(stream),
-        _stream(side_stream), (C.c_void_p * 4)(*events), int(seed) & (2 ** 64 - 1), n, nv, _dt(G_emb), B, T, V, d,
-        wpe.shape[0] if wpe is not None else 0, int(bool(tied)), int(bool(noise)), float(C_), float(sigma),
-        int(step) & 0xFFFFFFFF, wte_id, wpe_id)
-    st = L.dp_step_enqueue(C.byref(S), phases)
+    tensors = (ids, G_emb, pos_ids, wte, wpe, sq, clip, norms, cross, side_sq, perm, seg, pos_perm, pos_seg, ws,
+               side_ws, dev_status)
+    st = _marshal().step(
+        C.cast(L.dp_step_enqueue, C.c_void_p).value, layers, outs, tensor_ids, vectors, vector_outs, vector_ids, tensors,
+        (None if stream is None else _stream(stream), _stream(side_stream), *events, int(seed), _dt(G_emb), V, d,
+         bool(tied), bool(noise), int(step), wte_id, wpe_id, phases), C_, sigma)
+    if st is None:                             # one of these says what is wrong
+        _descs(layers), _vdescs(vectors), _outputs(outs), _outputs(vector_outs), _rows_ld(G_emb)
+        for t in tensors:
+            _ptr(t)
+        raise DpGhostError(1, "marshal", "dp_step_enqueue: arguments of the wrong kind or number")
     _check(st, "dp_step_enqueue")
-    if n and phases & STEP_NORMS:
-        _write_modes(layers, arr)
 
 
 def dp_rdp_epsilon(q: float, sigma: float, steps: int, delta: float):

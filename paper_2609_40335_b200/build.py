@@ -97,8 +97,9 @@ def build_marshal(force: bool = False) -> str:
         lib = os.path.join(root, "lib")
         cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
                f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-               "-I" + os.path.join(root, "include"), "-I" + sysconfig.get_paths()["include"], src, "-o", MARSHAL_PATH,
-               "-L" + lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-Wl,-rpath," + lib]
+               "-I" + os.path.join(root, "include"), "-I" + sysconfig.get_paths()["include"],
+               "-I" + os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"), src, "-o", MARSHAL_PATH,
+               "-L" + lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath," + lib]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
