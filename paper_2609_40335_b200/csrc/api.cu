@@ -404,7 +404,7 @@ dp_status dp_embed_norms(const int32_t* ids, const void* G, int64_t ldg, dp_dtyp
 size_t dp_tied_cross_term_ws_bytes(int32_t B, int32_t T, int32_t d, int32_t V) {
   (void)d; (void)V;
   if (B <= 0 || T <= 0) return 0;
-  // enough for either kernel: one partial per 16-token slab (fp32 path) or per 128 x 128 tile
+  // enough for either kernel: one partial per 16-token slab (fp32 path) or per tile
   const int per = std::max(ceil_div(T, 16), cross_term_tc_partials_per_example(T));
   return align_up(size_t(B) * per * sizeof(float), 256);
 }

@@ -319,3 +319,24 @@ def test_fp32_step_with_kept_operands(ample, kind):
     for n, t in ds.outs.items():
         assert float((t - want[n]).norm()) <= 1e-5 * float(want[n].norm()), n
     assert int(ds.dev_status.item()) == 0
+
+
+# tiles of 128 tokens x 32 positions, several per block from 2 x 148 tiles on
+@pytest.mark.parametrize("B,T,d,V", [(1, 1, 64, 40), (2, 31, 72, 300), (3, 33, 64, 300), (2, 129, 136, 1000), (75, 128, 64, 100),
+                                     (130, 97, 64, 64)])
+def test_cross_term_tiles(B, T, d, V):
+    G_emb, A_lm = bf16((B, T, d), 0.1, 1), bf16((B, T, d), 1.0, 2)
+    G_lm = bf16((B, T, V), 0.1, 3, ld=(V + 7) // 8 * 8)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B + T)
+    ids = torch.randint(0, V, (B, T), generator=g, device="cuda", dtype=torch.int32)
+    sq, cross = torch.ones(B, device="cuda"), torch.zeros(B, device="cuda")
+    dp.dp_tied_cross_term(ids, G_emb, A_lm, G_lm, V, sq=sq, cross=cross, d=d)
+    M = torch.einsum("btd,bsd->bts", G_emb.double(), A_lm.double())
+    W = torch.gather(G_lm[..., :V].double().transpose(1, 2), 1, ids.long()[:, :, None].expand(B, T, T))   # [b, t, s]
+    want, size = (M * W).sum((1, 2)), (M * W).abs().sum((1, 2))
+    # fp32 sums: d terms per entry of M (sizes |g||a|), then T*T entries in chains of 32
+    entry = torch.einsum("btd,bsd->bts", G_emb.double().abs(), A_lm.double().abs())
+    bound = 2.0 ** -24 * ((d + 8) * (entry * W.abs()).sum((1, 2)) + 64 * size)
+    assert ((cross.double() - want).abs() <= bound).all()
+    assert ((sq.double() - 1.0 - 2.0 * want).abs() <= 2.0 * bound + 2.0 ** -22 * (1.0 + size)).all()
