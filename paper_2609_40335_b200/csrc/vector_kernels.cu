@@ -45,9 +45,12 @@ struct VecParams {
 };
 
 __device__ __forceinline__ int find_param(const VecParams& P, int slab) {
-  int k = 0;
-  while (k + 1 < P.n && slab >= P.prm[k + 1].slab_begin) ++k;
-  return k;
+  int lo = 0, hi = P.n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (slab >= P.prm[mid].slab_begin) lo = mid; else hi = mid - 1;
+  }
+  return lo;
 }
 
 // sum over the rows [r0, r1) (stride 8 from warp w) of weight(row) * G[row, cols] * X[row, cols].
