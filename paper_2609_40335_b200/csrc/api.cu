@@ -280,17 +280,36 @@ int32_t dp_debug_force_fma(int32_t on) {
 }
 
 // ---------------------------------------------------------------------------- ghost norms
+static bool on_tensor_cores(const dp_linear_desc& L, dp_dtype dt, int T) {
+  return dt == DP_F32 ? f32_on_tensor_cores(L, T) : !g_force_fma;
+}
+
+// split operands of the largest layer three times over (what runs together follows from the room), and ...
+static size_t f32_norms_bytes(const dp_linear_desc* layers, int n_layers, dp_dtype dt, int B, int T) {
+  size_t need = 0;
+  for (int l = 0; l < n_layers; ++l)
+    if (dt == DP_F32 && f32_on_tensor_cores(layers[l], T))
+      need = std::max(need, f32_norm_bytes(layers[l], B, T, sm_count()) + 2 * split_layer_bytes(layers[l], B, T));
+  return need;
+}
+
+// ... the partial sums of the ghost norms on the fp32 kernels
+static int fma_norms_partials(const dp_linear_desc* layers, int n_layers, dp_dtype dt, int T) {
+  int n = 0;
+  for (int l = 0; l < n_layers; ++l)
+    if (!on_tensor_cores(layers[l], dt, T) && resolve_mode(layers[l], T) == DP_NORM_GHOST)
+      n += gram_fma_partials(layers[l], T);
+  return n;
+}
+static size_t fma_norms_bytes(const dp_linear_desc* layers, int n_layers, dp_dtype dt, int B, int T) {
+  return align_up(size_t(B) * fma_norms_partials(layers, n_layers, dt, T) * sizeof(float), 256);
+}
+
 size_t dp_ghost_norms_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt,
                                int32_t B, int32_t T) {
   if (!layers || n_layers <= 0 || B <= 0 || T <= 0) return 0;
-  if (g_force_fma) return 0;
-  if (dt == DP_F32) {            // layers run one after the other through the same workspace
-    size_t need = 0;
-    for (int l = 0; l < n_layers; ++l)
-      if (f32_on_tensor_cores(layers[l], T))
-        need = std::max(need, f32_norm_bytes(layers[l], B, T, sm_count()) + 2 * split_layer_bytes(layers[l], B, T));
-    return need;
-  }
+  if (dt == DP_F32 || g_force_fma)
+    return f32_norms_bytes(layers, n_layers, dt, B, T) + fma_norms_bytes(layers, n_layers, dt, B, T);
   const GhostPlan plan = plan_ghost_norms(layers, n_layers, B, T, sm_count());
   return align_up(size_t(B) * plan.n_per * sizeof(float), 256);
 }
@@ -312,10 +331,37 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
   }
   const GhostPlan plan = plan_ghost_norms(layers, n_layers, B, T, sm_count());
   if (!tc) {
-    if (dt == DP_F32 && dp_ghost_norms_ws_bytes(layers, n_layers, dt, B, T) > ws_bytes) return DP_ERR_WORKSPACE;
+    const size_t split_need = f32_norms_bytes(layers, n_layers, dt, B, T);
+    if (split_need > ws_bytes) return DP_ERR_WORKSPACE;
     SplitGroup group;
     char* base = static_cast<char*>(ws);
     if (left) *left = NormSource{sq, 1, 1.f, nullptr};
+    // ghost norms on the fp32 kernels: all layers in one launch, their partial sums at the workspace's end
+    // (at its start if nothing else needs it); without room for them a launch per layer
+    std::vector<int> fma;
+    for (int l = 0; l < n_layers; ++l)
+      if (!on_tensor_cores(layers[l], dt, T) && plan.mode_used[l] == DP_NORM_GHOST) fma.push_back(l);
+    const size_t fma_need = fma_norms_bytes(layers, n_layers, dt, B, T);
+    const bool together = !fma.empty() && ws && aligned16(ws) && split_need + fma_need <= ws_bytes;
+    if (together) {
+      char* at = base;
+      if (split_need) {
+        ws_bytes = (ws_bytes - fma_need) & ~size_t(255);
+        at += ws_bytes;
+      }
+      float* partials = reinterpret_cast<float*>(at);
+      const int n_per = fma_norms_partials(layers, n_layers, dt, T);
+      dp_status s = launch_gram_norms_fma(layers, fma.data(), (int)fma.size(), dt, B, T, partials, n_per, st);
+      if (s != DP_OK) return s;
+      for (int l : fma) layers[l].mode_used = plan.mode_used[l];
+      if (left && (int)fma.size() == n_layers) {
+        *left = NormSource{partials, n_per, 1.f, nullptr};
+        return DP_OK;
+      }
+      s = launch_reduce_partials(partials, n_per, B, sq, 1.f, nullptr, st, overwrite);
+      if (s != DP_OK) return s;
+      overwrite = false;
+    }
     int flushed = 0;
     auto flush = [&]() {
       if (group.index.empty()) return DP_OK;
@@ -328,6 +374,7 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
     };
     for (int l = 0; l < n_layers; ++l) {
       dp_status s = DP_OK;
+      if (together && !on_tensor_cores(layers[l], dt, T) && plan.mode_used[l] == DP_NORM_GHOST) continue;
       if (dt == DP_F32 && f32_on_tensor_cores(layers[l], T)) {
         if (!ws || !aligned16(ws)) return DP_ERR_WORKSPACE;
         const size_t more = f32_norm_bytes(layers[l], B, T, sm_count());
@@ -599,6 +646,7 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
       group = SplitGroup();
       return s;
     };
+    std::vector<int> fma;                // layers on the fp32 kernels: one launch for all of them
     if (kept && !kept->index.empty() && !sq &&
         kept->bytes + gta_partial_bytes(kept->desc.data(), (int)kept->desc.size(), B, T, 3, sm_count()) <= ws_bytes) {
       // the norms' split operands are still there: only the narrower one of each layer is split again, scaled
@@ -627,11 +675,12 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
         group.add(layers[l], l, B, T, true, base);
         continue;
       }
-      s = launch_clip_accumulate_fma(layers[l], dt, B, T, clip_ws, outs[l], ldos[l], beta, noise,
-                                     noise ? noise->tensor_ids[l] : 0u, st);
-      if (s != DP_OK) return s;
+      fma.push_back(l);
     }
-    return flush();
+    s = flush();
+    if (s != DP_OK || fma.empty()) return s;
+    return launch_clip_accumulate_fma(layers, fma.data(), (int)fma.size(), dt, B, T, clip_ws, outs, ldos, beta, noise,
+                                      st);
   }
   float* partial = reinterpret_cast<float*>(static_cast<char*>(ws) +
                                             align_up(size_t(B) * sizeof(float), 256));
@@ -876,7 +925,7 @@ size_t dp_step_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype
       on.push_back(layers[l]);
     }
   if (on.empty()) return 0;
-  need += gta_partial_bytes(on.data(), (int)on.size(), B, T, 3, sm_count());
+  need += gta_partial_bytes(on.data(), (int)on.size(), B, T, 3, sm_count()) + fma_norms_bytes(layers, n_layers, dt, B, T);
   return need <= (size_t(16) << 30) ? need : 0;
 }
 

@@ -8,11 +8,16 @@ namespace dpg {
 
 dp_status launch_norms_fma(const dp_linear_desc& L, dp_dtype dt, int mode, int B, int T, float* sq,
                            cudaStream_t st, bool overwrite = false);
-// noise: added onto the sum (inside the kernel where d is a multiple of 4), NULL = none
+// ghost norms of layers[index[0 .. n)] in one launch: partial sums [B][n_per], gram_fma_partials per layer
+int gram_fma_partials(const dp_linear_desc& L, int T);
+dp_status launch_gram_norms_fma(const dp_linear_desc* layers, const int* index, int n, dp_dtype dt, int B, int T,
+                                float* partials, int n_per, cudaStream_t st);
+// clipped sums of layers[index[0 .. n)]; noise: added onto them (inside the kernel where d is a multiple
+// of 4), NULL = none
 struct GtaNoise;
-dp_status launch_clip_accumulate_fma(const dp_linear_desc& L, dp_dtype dt, int B, int T, const float* clip,
-                                     float* out, int64_t ldo, float beta, const GtaNoise* noise,
-                                     uint32_t tensor_id, cudaStream_t st);
+dp_status launch_clip_accumulate_fma(const dp_linear_desc* layers, const int* index, int n, dp_dtype dt, int B, int T,
+                                     const float* clip, float* const* outs, const int64_t* ldos, float beta,
+                                     const GtaNoise* noise, cudaStream_t st);
 // partials: [B * ceil(T/16)] floats, example-major
 dp_status launch_cross_term_fma(const int* ids, const void* Ge, int64_t ldge, const void* Al,
                                 int64_t ldal, const void* Gl, int64_t ldgl, dp_dtype dt, int B,

@@ -340,3 +340,29 @@ def test_cross_term_tiles(B, T, d, V):
     bound = 2.0 ** -24 * ((d + 8) * (entry * W.abs()).sum((1, 2)) + 64 * size)
     assert ((cross.double() - want).abs() <= bound).all()
     assert ((sq.double() - 1.0 - 2.0 * want).abs() <= 2.0 * bound + 2.0 ** -22 * (1.0 + size)).all()
+
+
+# ghost norms on the fp32 kernels: tiles of 32 tokens, steps of 32 columns, chunks of 2048 of the wider operand,
+# 64 layers per launch; without a workspace for the partial sums a launch per layer
+@pytest.mark.parametrize("shapes,T", [([(31, 33)], 1), ([(32, 64), (5, 2048), (2049, 7)], 31), ([(40, 60)] * 65, 32),
+                                      ([(33, 4100)], 33), ([(100, 50), (64, 64)], 65)])
+@pytest.mark.parametrize("room", [True, False])
+def test_fp32_gram_norms(shapes, T, room):
+    B = 2
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    layers = [dp.Linear(torch.randn(B, T, d, generator=g, device="cuda"), torch.randn(B, T, p, generator=g, device="cuda"),
+                        d=d, p=p, mode=dp.DP_NORM_GHOST) for d, p in shapes]
+    sq = torch.zeros(B, device="cuda")
+    before = dp.dp_debug_force_fma(True)
+    try:
+        need = dp.dp_ghost_norms_ws_bytes(layers, B, T)
+        dp.dp_ghost_norms(layers, B, T, sq, ws=torch.empty(need if room else 16, dtype=torch.uint8, device="cuda"))
+    finally:
+        dp.dp_debug_force_fma(before)
+    want, size = 0, 0
+    for l in layers:
+        want = want + (torch.einsum("btp,btd->bpd", l.G.double(), l.A.double()) ** 2).sum((1, 2))
+        size = size + (l.A.double() ** 2).sum((1, 2)) * (l.G.double() ** 2).sum((1, 2))
+    # dots in chains of at most 32 + p / 32 terms, then sums over pairs: against |A|^2 |G|^2
+    assert ((sq.double() - want).abs() <= 2.0 ** -24 * 256 * size).all()
