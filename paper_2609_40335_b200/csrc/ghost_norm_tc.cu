@@ -34,13 +34,15 @@ constexpr int kTileBytes = kTile * kKStep * 2;   // 16 KiB
 // pair is diagonal, so stages shrink to one tile and twice as many are kept in flight (the
 // kernel is HBM-bound there: bytes in flight are what counts).  Split operands (fp32 inputs) bring
 // two tiles, high and low terms, for each.
-template <bool kDiagOnly, bool kSplit>
-struct GhostGeo {
-  static constexpr int kTermBytes = (kSplit ? 2 : 1) * kTileBytes;       // one row tile, all its terms
-  static constexpr int kStageBytes = (kDiagOnly ? 1 : 2) * kTermBytes;
-  static constexpr int kStages = 12 * kTileBytes / kStageBytes;
-  static constexpr size_t kSmemBytes = size_t(kStages) * kStageBytes + 1024 /*alignment slack*/ + 512;
-};
+// Up to 64 tokens a stage of 16 KiB took the 550 cycles of its hand-offs for a half or a quarter of the
+// data, the rest zeros.  kBoxes = 2 or 4: tiles of T rounded up to 16 rows, and two or four of them, 64
+// columns each, per stage.  B = 16, T = 64, 48 GPT-2-small layers 87.5 -> 71.9 us, B = 32, T = 48, 24 layers 78.9 ->
+// 61.3, B = 37, T = 35, 12 layers of d = 1024 64.3 -> 47.9, B = 6, T = 16, 24 of d = 512 20.3 -> 14.2.  Above 64 tokens
+// short tiles and sizes known at run time cost more than they save (115 -> 122 us at B = 32, T = 128):
+// kBoxes = 1 has full tiles and everything constant.
+constexpr int kRingBytes = 12 * kTileBytes;
+constexpr int kMaxStages = 32;
+constexpr size_t kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 1024 /*barriers*/;
 constexpr int kThreads = 192;
 constexpr int kTmemCols = 512;                   // 2 buffers x (S_A 128 + S_G 128) columns
 
@@ -50,6 +52,7 @@ struct __align__(64) GhostParams {
   GhostLayerPlan layer[kGhostMaxLayers];
   int n_layers;
   int B, T, nt, ntp;
+  int rows, stages;          // kBoxes > 1: tokens of a tile, stages of the ring
   int total_items;
   int n_per;                 // partial sums per example in the workspace
   float* partials;           // [B][n_per]
@@ -90,21 +93,26 @@ __device__ __forceinline__ Item decode_item(const GhostParams& P, int item, int&
 
 // kSplit: fp32 operands stored as two bf16 planes per example (see split_kernels.cu).  Every Gram
 // tile is then S = hi hi^T + hi lo^T + lo hi^T, three MMAs per K step on tiles loaded once.
-template <bool kDiagOnly, bool kSplit>
+template <bool kDiagOnly, bool kSplit, int kBoxes>
 __global__ void __launch_bounds__(kThreads, 1)
 ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
-  using Geo = GhostGeo<kDiagOnly, kSplit>;
-  constexpr int kStages = Geo::kStages;
-  constexpr int kStageBytes = Geo::kStageBytes;
-  constexpr int kTermBytes = Geo::kTermBytes;
+  static_assert(kBoxes == 1 || kDiagOnly, "several column tiles per stage: diagonal pairs only");
+  // an MMA reads 128 rows of its first operand whatever `rows` is: rows beyond it come from the next
+  // stages (the ring ends a whole tile after its last tile begins) and fill accumulator rows nobody reads
+  constexpr bool kShort = kBoxes > 1;
+  const int rows = kShort ? P.rows : kTile;
+  const uint32_t tile_bytes = uint32_t(rows) * (kKStep * 2);
+  const uint32_t term_bytes = (kSplit ? 2 : 1) * tile_bytes;             // one row tile, all its terms
+  const uint32_t stage_bytes = (kDiagOnly ? kBoxes : 2) * term_bytes;
+  const int n_stages = kShort ? P.stages : kRingBytes / int((kDiagOnly ? 1 : 2) * (kSplit ? 2 : 1) * kTileBytes);
   extern __shared__ uint8_t smem_raw[];
   // 128-byte swizzled tiles need 1024-byte alignment
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                               ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + size_t(kStages) * kStageBytes);
-  uint64_t* full = bars;                   // [kStages]  TMA -> MMA
-  uint64_t* empty = bars + kStages;        // [kStages]  MMA -> TMA
-  uint64_t* acc_full = bars + 2 * kStages; // [2]        MMA -> epilogue
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + kRingBytes);
+  uint64_t* full = bars;                   // [n_stages] TMA -> MMA
+  uint64_t* empty = bars + kMaxStages;     // [n_stages] MMA -> TMA
+  uint64_t* acc_full = bars + 2 * kMaxStages; // [2]     MMA -> epilogue
   uint64_t* acc_empty = acc_full + 2;      // [2]        epilogue -> MMA
   uint64_t* mma_done = acc_empty + 2;      // only used when the MMA issuer gives up
   uint64_t* red_bar = mma_done + 1;        // [4]        epilogue warps -> epilogue warp 0
@@ -116,7 +124,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
   const int lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&empty[s], 1); }
+    for (int s = 0; s < n_stages; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&empty[s], 1); }
     for (int b = 0; b < 2; ++b) { ptx::mbar_init(&acc_full[b], 1); ptx::mbar_init(&acc_empty[b], 4); }
     ptx::mbar_init(mma_done, 1);
     for (int b = 0; b < 4; ++b) ptx::mbar_init(&red_bar[b], 4);
@@ -142,39 +150,45 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
     for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x) {
       const Item it = decode_item(P, item, lay);
       const bool diag = kDiagOnly || (it.ti == it.tj);
-      const uint32_t bytes = diag ? kTermBytes : kStageBytes;
+      const uint32_t bytes = diag ? term_bytes : stage_bytes;
       const int ex = kSplit ? 2 * it.example : it.example;     // (high) plane of the example
       for (int pass = 0; pass < 2 && ok; ++pass) {
         const uint64_t tm = reinterpret_cast<uint64_t>(pass == 0 ? &P.tmA[it.layer] : &P.tmG[it.layer]);
         const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
-        for (int k = k0; k < k1; ++k) {
+        for (int k = k0; k < k1; k += kBoxes) {
           ok = ptx::warp_ok(ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit));
           if (!ok) break;
-          const uint32_t dst = tiles_a + stage * kStageBytes, bar = full_a + 8 * stage;
+          const uint32_t dst = tiles_a + stage * stage_bytes, bar = full_a + 8 * stage;
+          const int nb = kShort ? min(kBoxes, k1 - k) : 1;
           if (ptx::elect_one()) {
-            ptx::mbar_arrive_expect_tx_a(bar, bytes);
-            ptx::tma_load_3d_a(dst, tm, bar, k * kKStep, it.ti * kTile, ex);
-            if (kSplit) ptx::tma_load_3d_a(dst + kTileBytes, tm, bar, k * kKStep, it.ti * kTile, ex + 1);
-            if (!diag) {
-              ptx::tma_load_3d_a(dst + kTermBytes, tm, bar, k * kKStep, it.tj * kTile, ex);
+            ptx::mbar_arrive_expect_tx_a(bar, kShort ? nb * term_bytes : bytes);
+#pragma unroll
+            for (int b = 0; b < kBoxes; ++b) {
+              if (b >= nb) break;
+              ptx::tma_load_3d_a(dst + b * term_bytes, tm, bar, (k + b) * kKStep, it.ti * kTile, ex);
               if (kSplit)
-                ptx::tma_load_3d_a(dst + kTermBytes + kTileBytes, tm, bar, k * kKStep, it.tj * kTile, ex + 1);
+                ptx::tma_load_3d_a(dst + b * term_bytes + tile_bytes, tm, bar, (k + b) * kKStep, it.ti * kTile, ex + 1);
+            }
+            if (!diag) {
+              ptx::tma_load_3d_a(dst + term_bytes, tm, bar, k * kKStep, it.tj * kTile, ex);
+              if (kSplit)
+                ptx::tma_load_3d_a(dst + term_bytes + tile_bytes, tm, bar, k * kKStep, it.tj * kTile, ex + 1);
             }
           }
           __syncwarp();
           ++issued;
-          if (++stage == kStages) { stage = 0; phase ^= 1; }
+          if (++stage == uint32_t(n_stages)) { stage = 0; phase ^= 1; }
         }
       }
     }
     if (!ok && ptx::elect_one()) {
       *abort_flag = 1;
       if (P.dev_status) atomicOr(P.dev_status, DP_DEV_TIMEOUT);
-      ptx::drain_issued_copies(full, kStages, issued);   // copies in flight land before exit
+      ptx::drain_issued_copies(full, n_stages, issued);   // copies in flight land before exit
     }
   } else if (warp == 1) {
     // --------------------------------------------------------------- MMA issuer
-    constexpr uint32_t idesc = ptx::idesc_bf16_f32(kTile, kTile, 0, 0);
+    const uint32_t idesc = ptx::idesc_bf16_f32(kTile, rows, 0, 0);
     // K-major operand, 128-byte swizzle: 8-row groups are 1024 bytes apart; 16 bf16 = 32 bytes
     // further along K inside the swizzle atom
     constexpr uint64_t dbase = ptx::smem_desc_base(16, 1024, ptx::SWIZZLE_128B);
@@ -193,27 +207,32 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
       for (int pass = 0; pass < 2 && ok; ++pass) {
         const uint32_t d_tmem = tmem_base + buf * 256 + pass * 128;
         const int nsteps = pass == 0 ? it.a1 - it.a0 : it.g1 - it.g0;
-        for (int k = 0; k < nsteps; ++k) {
+        for (int k = 0; k < nsteps; k += kBoxes) {
           ok = ptx::warp_ok(ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit));
           if (!ok) break;
           ptx::tc_fence_after();
-          const uint32_t sa = desc_lo0 + stage * (kStageBytes >> 4);
-          const uint32_t sb = diag ? sa : sa + (kTermBytes >> 4);
+          const int nb = kShort ? min(kBoxes, nsteps - k) : 1;
           if (ptx::elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < kKStep / 16; ++kk) {
-              const uint32_t ah = sa + kk * 2, bh = sb + kk * 2, low = kTileBytes >> 4;
-              ptx::mma_bf16_ss_lh(d_tmem, ah, bh, desc_hi, idesc, (k > 0 || kk > 0) ? 1u : 0u);
-              if (kSplit) {
-                ptx::mma_bf16_ss_lh(d_tmem, ah, bh + low, desc_hi, idesc, 1u);
-                ptx::mma_bf16_ss_lh(d_tmem, ah + low, bh, desc_hi, idesc, 1u);
+            for (int b = 0; b < kBoxes; ++b) {
+              if (b >= nb) break;
+              const uint32_t sa = desc_lo0 + ((stage * stage_bytes + b * term_bytes) >> 4);
+              const uint32_t sb = diag ? sa : sa + (term_bytes >> 4);
+#pragma unroll
+              for (int kk = 0; kk < kKStep / 16; ++kk) {
+                const uint32_t ah = sa + kk * 2, bh = sb + kk * 2, low = tile_bytes >> 4;
+                ptx::mma_bf16_ss_lh(d_tmem, ah, bh, desc_hi, idesc, (k + b > 0 || kk > 0) ? 1u : 0u);
+                if (kSplit) {
+                  ptx::mma_bf16_ss_lh(d_tmem, ah, bh + low, desc_hi, idesc, 1u);
+                  ptx::mma_bf16_ss_lh(d_tmem, ah + low, bh, desc_hi, idesc, 1u);
+                }
               }
             }
             ptx::mma_commit_a(empty_a + 8 * stage);      // stage reusable once these MMAs retire
-            if (pass == 1 && k + 1 == nsteps) ptx::mma_commit(&acc_full[buf]);     // both Gram tiles complete
+            if (pass == 1 && k + nb >= nsteps) ptx::mma_commit(&acc_full[buf]);     // both Gram tiles complete
           }
           __syncwarp();
-          if (++stage == kStages) { stage = 0; phase ^= 1; }
+          if (++stage == uint32_t(n_stages)) { stage = 0; phase ^= 1; }
         }
       }
     }
@@ -237,14 +256,23 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
       const uint32_t t0 = tmem_base + (uint32_t(q * 32) << 16) + buf * 256;
       float acc = 0.f;
 #pragma unroll 1
-      for (int c = 0; c < kTile / 32; ++c) {
+      for (int c = 0; c + 32 <= rows; c += 32) {
         uint32_t ra[32], rg[32];
-        ptx::tmem_ld_32x32b_x32(t0 + c * 32, ra);
-        ptx::tmem_ld_32x32b_x32(t0 + 128 + c * 32, rg);
+        ptx::tmem_ld_32x32b_x32(t0 + c, ra);
+        ptx::tmem_ld_32x32b_x32(t0 + 128 + c, rg);
         ptx::tmem_ld_wait();
 #pragma unroll
         for (int j = 0; j < 32; ++j) acc = fmaf(__uint_as_float(ra[j]), __uint_as_float(rg[j]), acc);
       }
+      if (kShort && (rows & 16)) {
+        uint32_t ra[16], rg[16];
+        ptx::tmem_ld_32x32b_x16(t0 + rows - 16, ra);
+        ptx::tmem_ld_32x32b_x16(t0 + 128 + rows - 16, rg);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int j = 0; j < 16; ++j) acc = fmaf(__uint_as_float(ra[j]), __uint_as_float(rg[j]), acc);
+      }
+      if (kShort && q * 32 + lane >= P.T) acc = 0.f;     // a row beyond the tile: whatever lay there
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&acc_empty[buf]);   // accumulators may be overwritten
@@ -308,12 +336,12 @@ dp_status launch_reduce_partials(const float* partials, int n_per, int B, float*
 
 namespace {
 
-template <bool kDiagOnly, bool kSplit>
+template <bool kDiagOnly, bool kSplit, int kBoxes>
 dp_status launch_variant(const GhostParams& P, cudaStream_t st) {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_tc_kernel<kDiagOnly, kSplit>)))
-    DP_CUDA_OK(allow_shared(ghost_norm_tc_kernel<kDiagOnly, kSplit>, GhostGeo<kDiagOnly, kSplit>::kSmemBytes));
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_tc_kernel<kDiagOnly, kSplit, kBoxes>)))
+    DP_CUDA_OK((allow_shared(ghost_norm_tc_kernel<kDiagOnly, kSplit, kBoxes>, kSmemBytes)));
   const int grid = std::min(P.total_items, sm_count());
-  ghost_norm_tc_kernel<kDiagOnly, kSplit><<<grid, kThreads, GhostGeo<kDiagOnly, kSplit>::kSmemBytes, st>>>(P);
+  ghost_norm_tc_kernel<kDiagOnly, kSplit, kBoxes><<<grid, kThreads, kSmemBytes, st>>>(P);
   DP_LAUNCH_OK();
   return DP_OK;
 }
@@ -326,6 +354,9 @@ dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& pl
                                float* partials, int* dev_status, cudaStream_t st, bool split) {
   const int nt = ceil_div(T, kTile);
   const int planes = split ? 2 * B : B;
+  const int boxes = T > 64 ? 1 : T > 32 || split ? 2 : 4;       // split operands: T >= 32
+  const int rows = boxes > 1 ? (T + 15) / 16 * 16 : kTile, tile_bytes = rows * kKStep * 2;
+  const int stages = std::min(kMaxStages, (kRingBytes - (kTileBytes - tile_bytes)) / (boxes * (split ? 2 : 1) * tile_bytes));
   // layers are processed in groups that fit one parameter block
   for (size_t g0 = 0; g0 < plan.ghost_layers.size(); g0 += kGhostMaxLayers) {
     const size_t g1 = std::min(plan.ghost_layers.size(), g0 + kGhostMaxLayers);
@@ -335,9 +366,9 @@ dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& pl
     for (size_t g = g0; g < g1; ++g) {
       const int li = plan.ghost_layers[g];
       const dp_linear_desc& L = layers[li];
-      dp_status s = make_tmap_bf16_3d(&P.tmA[g - g0], L.A, L.lda, L.d, T, planes, kKStep, kTile);
+      dp_status s = make_tmap_bf16_3d(&P.tmA[g - g0], L.A, L.lda, L.d, T, planes, kKStep, rows);
       if (s != DP_OK) return s;
-      s = make_tmap_bf16_3d(&P.tmG[g - g0], L.G, L.ldg, L.p, T, planes, kKStep, kTile);
+      s = make_tmap_bf16_3d(&P.tmG[g - g0], L.G, L.ldg, L.p, T, planes, kKStep, rows);
       if (s != DP_OK) return s;
       GhostLayerPlan lp = plan.layer[li];
       lp.item_begin = items;
@@ -346,13 +377,19 @@ dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& pl
     }
     P.n_layers = int(g1 - g0);
     P.B = B; P.T = T; P.nt = nt; P.ntp = plan.ntp;
+    P.rows = rows; P.stages = stages;
     P.total_items = items;
     P.n_per = plan.n_per;
     P.partials = partials;
     P.dev_status = dev_status;
     P.wait_limit = g_wait_limit;
-    const dp_status s = split ? (nt == 1 ? launch_variant<true, true>(P, st) : launch_variant<false, true>(P, st))
-                              : (nt == 1 ? launch_variant<true, false>(P, st) : launch_variant<false, false>(P, st));
+    dp_status s;
+    if (split)
+      s = nt > 1 ? launch_variant<false, true, 1>(P, st)
+                 : boxes == 1 ? launch_variant<true, true, 1>(P, st) : launch_variant<true, true, 2>(P, st);
+    else if (nt > 1) s = launch_variant<false, false, 1>(P, st);
+    else if (boxes == 1) s = launch_variant<true, false, 1>(P, st);
+    else s = boxes == 2 ? launch_variant<true, false, 2>(P, st) : launch_variant<true, false, 4>(P, st);
     if (s != DP_OK) return s;
   }
   return DP_OK;

@@ -366,3 +366,26 @@ def test_fp32_gram_norms(shapes, T, room):
         size = size + (l.A.double() ** 2).sum((1, 2)) * (l.G.double() ** 2).sum((1, 2))
     # dots in chains of at most 32 + p / 32 terms, then sums over pairs: against |A|^2 |G|^2
     assert ((sq.double() - want).abs() <= 2.0 ** -24 * 256 * size).all()
+
+
+# Gram tiles as tall as the sequence, rounded up to 16 tokens, up to 64 tokens: rings of up to 32 stages of two
+# or four column tiles; bf16 and split fp32
+@pytest.mark.parametrize("T", [1, 15, 16, 17, 31, 32, 33, 48, 49, 64, 65, 77, 127, 128, 129])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_gram_tiles_of_short_sequences(T, dtype):
+    B, shapes = 3, [(64, 72), (300, 64), (136, 2500)]
+    layers = [dp.Linear(bf16((B, T, d), 1.0, k, ld=(d + 7) // 8 * 8), bf16((B, T, p), 0.1, 50 + k, ld=(p + 7) // 8 * 8),
+                        d=d, p=p, mode=dp.DP_NORM_GHOST) for k, (d, p) in enumerate(shapes)]
+    if dtype == "f32":
+        layers = [dp.Linear(l.A[..., :l.d].float().contiguous(), l.G[..., :l.p].float().contiguous(), d=l.d, p=l.p,
+                            mode=dp.DP_NORM_GHOST) for l in layers]
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(2):                                     # the second call finds the first one's shared memory
+        sq = torch.zeros(B, device="cuda")
+        dp.dp_ghost_norms(layers, B, T, sq, dev_status=st)
+    want = np.zeros(B)
+    for l in layers:
+        want += (np.einsum("btp,btd->bpd", f64(l.G, l.p), f64(l.A, l.d)) ** 2).sum((1, 2))
+    # exact products, fp32 sums of at most 2500 terms
+    assert (np.abs(sq.double().cpu().numpy() / want - 1) < 1e-5).all()
+    assert int(st.item()) == 0
