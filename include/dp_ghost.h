@@ -307,7 +307,8 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
  * clipped sums.  sq, clip [dev, B] and norms, cross [dev, B or NULL; cross is needed when tied] are
  * overwritten; side_sq [dev, B], perm / seg and pos_perm / pos_seg [dev, as in dp_embed_sort] are
  * scratch, as are ws (the largest *_ws_bytes of the calls on `stream`, dp_step_ws_bytes if fp32 layers
- * are to be split once instead of for the norms and again for the sums, and
+ * are to be split once instead of for the norms and again for the sums, and the norms of short ones to
+ * take one launch instead of one per layer, and
  * dp_clip_accumulate_embed_ws_bytes when tied) and side_ws (the largest of dp_embed_norms_ws_bytes,
  * dp_embed_sort_ws_bytes and dp_clip_accumulate_embed_ws_bytes over both tables; with
  * dp_embed_norms_ws_bytes more per table one kernel adds up all the norms' partial sums).  events: four

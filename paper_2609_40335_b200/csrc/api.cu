@@ -293,7 +293,7 @@ static size_t f32_norms_bytes(const dp_linear_desc* layers, int n_layers, dp_dty
   return need;
 }
 
-// ... the partial sums of the ghost norms on the fp32 kernels
+// ... where there is room for them, the partial sums of the ghost norms on the fp32 kernels
 static int fma_norms_partials(const dp_linear_desc* layers, int n_layers, dp_dtype dt, int T) {
   int n = 0;
   for (int l = 0; l < n_layers; ++l)
@@ -308,8 +308,7 @@ static size_t fma_norms_bytes(const dp_linear_desc* layers, int n_layers, dp_dty
 size_t dp_ghost_norms_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt,
                                int32_t B, int32_t T) {
   if (!layers || n_layers <= 0 || B <= 0 || T <= 0) return 0;
-  if (dt == DP_F32 || g_force_fma)
-    return f32_norms_bytes(layers, n_layers, dt, B, T) + fma_norms_bytes(layers, n_layers, dt, B, T);
+  if (dt == DP_F32 || g_force_fma) return f32_norms_bytes(layers, n_layers, dt, B, T);
   const GhostPlan plan = plan_ghost_norms(layers, n_layers, B, T, sm_count());
   return align_up(size_t(B) * plan.n_per * sizeof(float), 256);
 }
@@ -914,7 +913,8 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
 
 // ------------------------------------------------------------------------------ whole step
 // Workspace with which fp32 layers are split once per step: the group of all of them, the norms' partial
-// sums, the K-split planes.  Beyond 16 GiB the layers go through less in groups.
+// sums, the K-split planes.  Beyond 16 GiB the layers go through less in groups.  With the partial sums
+// of layers on the fp32 kernels, whose norms then take one launch.
 size_t dp_step_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B, int32_t T) {
   if (!layers || n_layers <= 0 || B <= 0 || T <= 0 || dt != DP_F32) return 0;
   std::vector<dp_linear_desc> on;
@@ -924,9 +924,9 @@ size_t dp_step_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype
       need += f32_norm_bytes(layers[l], B, T, sm_count());
       on.push_back(layers[l]);
     }
-  if (on.empty()) return 0;
-  need += gta_partial_bytes(on.data(), (int)on.size(), B, T, 3, sm_count()) + fma_norms_bytes(layers, n_layers, dt, B, T);
-  return need <= (size_t(16) << 30) ? need : 0;
+  if (!on.empty()) need += gta_partial_bytes(on.data(), (int)on.size(), B, T, 3, sm_count());
+  if (need > (size_t(16) << 30)) need = f32_norms_bytes(layers, n_layers, dt, B, T);
+  return need + fma_norms_bytes(layers, n_layers, dt, B, T);
 }
 
 static dp_status check_step(const dp_step_desc* S) {

@@ -356,8 +356,10 @@ def test_fp32_gram_norms(shapes, T, room):
     sq = torch.zeros(B, device="cuda")
     before = dp.dp_debug_force_fma(True)
     try:
-        need = dp.dp_ghost_norms_ws_bytes(layers, B, T)
-        dp.dp_ghost_norms(layers, B, T, sq, ws=torch.empty(need if room else 16, dtype=torch.uint8, device="cuda"))
+        ws = torch.empty(dp.dp_step_ws_bytes(layers, B, T) if room else 16, dtype=torch.uint8, device="cuda")
+        n0 = dp.dp_kernel_launches()
+        dp.dp_ghost_norms(layers, B, T, sq, ws=ws)
+        assert dp.dp_kernel_launches() - n0 == (-(-len(shapes) // 64) + 1 if room else len(shapes))
     finally:
         dp.dp_debug_force_fma(before)
     want, size = 0, 0
