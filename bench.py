@@ -600,7 +600,7 @@ def run_ours(args):
 
     # dominant kernel: the tensor-core G^T A GEMM of the clipped sums, timed live (see above)
     achieved_tf = counts["acc_flops"] / (gemm_ms_avg * 1e-3) / 1e12
-    roofline = {"kernel": "gemm_gta_kernel<scale, pair> (%s)" % (
+    roofline = {"kernel": "gemm_gta_big_kernel (%s)" % (
                     "dp_clip_accumulate_noise_grouped, Gaussian noise drawn in the epilogue"
                     if fused and not args.prefill else
                     "dp_clip_accumulate_grouped, accumulating onto noise filled beside the norm phase"
