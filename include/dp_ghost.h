@@ -303,8 +303,9 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
  * times pays one call instead of a dozen.  Nothing is kept between calls.
  * layers [host, n_layers; the LM head, if any, is the last one], with outs / ldos / tensor_ids as in
  * dp_clip_accumulate_noise_grouped (tied: the head's out is wte).  vectors, vector_outs, vector_ids
- * as in dp_clip_accumulate_vectors.  pos_ids NULL: no position table.  with_noise 0: the bare
- * clipped sums.  sq, clip [dev, B] and norms, cross [dev, B or NULL; cross is needed when tied] are
+ * as in dp_clip_accumulate_vectors.  layer_dtype, vector_dtype, embed_dtype: the storage types of the
+ * layers' A and G, the vectors' G and X, and G_emb (tied: that of the layers, since the cross term takes
+ * one type).  pos_ids NULL: no position table.  with_noise 0: the bare clipped sums.  sq, clip [dev, B] and norms, cross [dev, B or NULL; cross is needed when tied] are
  * overwritten; side_sq [dev, B], perm / seg and pos_perm / pos_seg [dev, as in dp_embed_sort] are
  * scratch, as are ws (the largest *_ws_bytes of the calls on `stream`, dp_step_ws_bytes if fp32 layers
  * are to be split once instead of for the norms and again for the sums, and the norms of short ones to
@@ -329,7 +330,7 @@ typedef struct {
   void* ws;  size_t ws_bytes;  void* side_ws;  size_t side_ws_bytes;
   int32_t* dev_status;  void* stream;  void* side_stream;  void* events[4];
   uint64_t seed;
-  int32_t n_layers, n_vectors, dtype, B, T, V, d, pos_rows, tied, with_noise;
+  int32_t n_layers, n_vectors, layer_dtype, vector_dtype, embed_dtype, B, T, V, d, pos_rows, tied, with_noise;
   float C, sigma;
   uint32_t step, wte_id, wpe_id;
 } dp_step_desc;

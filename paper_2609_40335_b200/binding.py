@@ -192,6 +192,13 @@ def _rows_ld(t: torch.Tensor) -> int:
     return ld
 
 
+def _one_dtype(tensors, what: str) -> None:
+    """Complains unless the tensors have one storage type, a supported one (a call takes one for all)."""
+    kinds = {t.dtype: _dt(t) for t in tensors}
+    if len(kinds) > 1:
+        raise DpGhostError(1, "marshal", f"{what} of different dtypes: {', '.join(map(str, kinds))}")
+
+
 def _marshal():
     """The native half of the marshalling (csrc/marshal.cpp)."""
     global _native
@@ -237,6 +244,7 @@ def _descs(layers: Sequence[Linear]):
     if buf is None:
         for l in layers:                       # one of these says what is wrong
             _ptr(l.A), _ptr(l.G), _rows_ld(l.A), _rows_ld(l.G)
+        _one_dtype([t for l in layers for t in (l.A, l.G)], "layers with tensors A and G")
         raise DpGhostError(1, "marshal", "layers need tensors A and G of at least two axes")
     return (_LinearDesc * len(layers)).from_buffer(buf)
 
@@ -295,6 +303,7 @@ def _vdescs(params: Sequence[Vector]):
             _ptr(v.G), _rows_ld(v.G)
             if v.X is not None:
                 _ptr(v.X), _rows_ld(v.X)
+        _one_dtype([t for v in params for t in (v.G, v.X) if t is not None], "parameters with tensors G and X")
         raise DpGhostError(1, "marshal", "parameters need tensors of at least two axes")
     return (_VectorDesc * len(params)).from_buffer(buf)
 
@@ -362,6 +371,7 @@ def dp_tied_cross_term(ids, G_emb, A_lm, G_lm, V: int, sq=None, cross=None, d=No
     need = int(L.dp_tied_cross_term_ws_bytes(B, T, d, V))
     dev = G_emb.device
     ws = _ws(need, ws, dev)
+    _one_dtype((G_emb, A_lm, G_lm), "cross term of tensors")
     st = L.dp_tied_cross_term(_ptr(ids), _ptr(G_emb), _rows_ld(G_emb), _ptr(A_lm), _rows_ld(A_lm),
                               _ptr(G_lm), _rows_ld(G_lm), _dt(G_emb), B, T, d, V, _ptr(sq),
                               _ptr(cross), _ptr(ws), ws.numel() * ws.element_size(),
@@ -554,12 +564,18 @@ def dp_step_enqueue(layers, outs, tensor_ids, vectors, vector_outs, vector_ids, 
                side_ws, dev_status)
     st = _marshal().step(
         C.cast(L.dp_step_enqueue, C.c_void_p).value, layers, outs, tensor_ids, vectors, vector_outs, vector_ids, tensors,
-        (None if stream is None else _stream(stream), _stream(side_stream), *events, int(seed), _dt(G_emb), V, d,
+        (None if stream is None else _stream(stream), _stream(side_stream), *events, int(seed), V, d,
          bool(tied), bool(noise), int(step), wte_id, wpe_id, phases), C_, sigma)
     if st is None:                             # one of these says what is wrong
-        _descs(layers), _vdescs(vectors), _outputs(outs), _outputs(vector_outs), _rows_ld(G_emb)
+        _descs(layers), _vdescs(vectors), _outputs(outs), _outputs(vector_outs), _rows_ld(G_emb), _dt(G_emb)
         for t in tensors:
             _ptr(t)
+        for t in (ids, pos_ids, perm, seg, pos_perm, pos_seg, dev_status):
+            if t is not None and t.dtype != torch.int32:
+                raise DpGhostError(1, "marshal", f"ids, sorts and status are int32 tensors, not {t.dtype}")
+        for t in (*outs, *vector_outs, wte, wpe, sq, clip, norms, cross, side_sq):
+            if t is not None and t.dtype != torch.float32:
+                raise DpGhostError(1, "marshal", f"outputs, norms and clip factors are float32 tensors, not {t.dtype}")
         raise DpGhostError(1, "marshal", "dp_step_enqueue: arguments of the wrong kind or number")
     _check(st, "dp_step_enqueue")
 

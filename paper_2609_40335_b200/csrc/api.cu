@@ -937,6 +937,9 @@ static dp_status check_step(const dp_step_desc* S) {
   if (S->n_layers && (!S->layers || !S->outs || !S->ldos || (S->with_noise && !S->tensor_ids)))
     return DP_ERR_INVALID_ARG;
   if (S->tied && (S->n_layers == 0 || !S->cross)) return DP_ERR_INVALID_ARG;
+  auto dtype_ok = [](int32_t t) { return t == DP_F32 || t == DP_BF16; };
+  if (!dtype_ok(S->layer_dtype) || !dtype_ok(S->vector_dtype) || !dtype_ok(S->embed_dtype)) return DP_ERR_INVALID_ARG;
+  if (S->tied && S->embed_dtype != S->layer_dtype) return DP_ERR_INVALID_ARG;      // one type in the cross term
   if (S->pos_ids && (!S->wpe || !S->pos_perm || !S->pos_seg || S->pos_rows <= 0)) return DP_ERR_INVALID_ARG;
   for (int k = 0; k < 4; ++k) if (!S->events[k]) return DP_ERR_INVALID_ARG;
   if (S->with_noise && !noise_args_ok(S->sigma, S->C, 1.f)) return DP_ERR_INVALID_ARG;
@@ -957,7 +960,7 @@ static dp_status start_table(const dp_step_desc* S, float* table, int64_t ld, in
 // events: [0] the step began, [1] embedding norms done, [2] row sums done, [3] clip factors exist
 static dp_status step_norms(const dp_step_desc* S, SplitGroup* kept) {
   cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
-  const dp_dtype dt = (dp_dtype)S->dtype;
+  const dp_dtype embed_dt = (dp_dtype)S->embed_dtype;
   const int B = S->B, T = S->T;
   dp_status s;
   NormSources N;                 // partial sums that the last kernel of this phase adds up
@@ -966,8 +969,8 @@ static dp_status step_norms(const dp_step_desc* S, SplitGroup* kept) {
   char* ws = static_cast<char*>(S->ws);
   DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[0], main));
   if (S->n_layers) {
-    s = ghost_norms_impl(S->layers, S->n_layers, dt, B, T, S->sq, S->ws, S->ws_bytes, S->dev_status, main, true,
-                         &N.src[0], kept);
+    s = ghost_norms_impl(S->layers, S->n_layers, (dp_dtype)S->layer_dtype, B, T, S->sq, S->ws, S->ws_bytes, S->dev_status,
+                         main, true, &N.src[0], kept);
     if (s != DP_OK) return s;
     N.n = 1;
     if (N.src[0].partials != S->sq)
@@ -990,8 +993,8 @@ static dp_status step_norms(const dp_step_desc* S, SplitGroup* kept) {
   for (size_t k = 0; k < tables; ++k) {
     char* w = side_ws;
     if (keep) { side_bytes -= each; w += side_bytes; }
-    s = embed_norms_impl(k ? S->pos_ids : S->ids, S->G_emb, S->ldge, dt, B, T, S->d, k ? T : S->V, S->side_sq, nullptr,
-                         w, keep ? each : S->side_ws_bytes, S->dev_status, side, k == 0, keep ? &embed[k] : nullptr);
+    s = embed_norms_impl(k ? S->pos_ids : S->ids, S->G_emb, S->ldge, embed_dt, B, T, S->d, k ? T : S->V, S->side_sq,
+                         nullptr, w, keep ? each : S->side_ws_bytes, S->dev_status, side, k == 0, keep ? &embed[k] : nullptr);
     if (s != DP_OK) return s;
   }
   if (!keep) embed[0] = NormSource{S->side_sq, 1, 1.f, nullptr};
@@ -1027,7 +1030,8 @@ static dp_status step_norms(const dp_step_desc* S, SplitGroup* kept) {
     const size_t need = dp_vector_norms_ws_bytes(S->vectors, S->n_vectors, B, T);
     s = room(need);
     if (s != DP_OK) return s;
-    s = vector_norms_impl(S->vectors, S->n_vectors, dt, B, T, S->sq, ws + held, S->ws_bytes - held, main, &N.src[N.n]);
+    s = vector_norms_impl(S->vectors, S->n_vectors, (dp_dtype)S->vector_dtype, B, T, S->sq, ws + held, S->ws_bytes - held,
+                          main, &N.src[N.n]);
     if (s != DP_OK) return s;
     ++N.n;
     held += need;
@@ -1036,8 +1040,8 @@ static dp_status step_norms(const dp_step_desc* S, SplitGroup* kept) {
     const dp_linear_desc& lm = S->layers[S->n_layers - 1];
     s = room(dp_tied_cross_term_ws_bytes(B, T, S->d, S->V));
     if (s != DP_OK) return s;
-    s = cross_term_impl(S->ids, S->G_emb, S->ldge, lm.A, lm.lda, lm.G, lm.ldg, dt, B, T, S->d, S->V, S->sq, S->cross,
-                        ws + held, S->ws_bytes - held, S->dev_status, main, &N.src[N.n]);
+    s = cross_term_impl(S->ids, S->G_emb, S->ldge, lm.A, lm.lda, lm.G, lm.ldg, embed_dt, B, T, S->d, S->V, S->sq,
+                        S->cross, ws + held, S->ws_bytes - held, S->dev_status, main, &N.src[N.n]);
     if (s != DP_OK) return s;
     ++N.n;
   }
@@ -1054,14 +1058,14 @@ static dp_status step_norms(const dp_step_desc* S, SplitGroup* kept) {
 static dp_status step_gemm(const dp_step_desc* S, const SplitGroup* kept) {
   if (!S->n_layers) return DP_OK;
   const GtaNoise noise{S->sigma * S->C, 1.f, S->seed, S->step, S->tensor_ids};
-  return clip_accumulate_impl(S->layers, S->n_layers, (dp_dtype)S->dtype, S->B, S->T, nullptr, S->C, S->clip, S->outs,
-                              S->ldos, 0.f, S->with_noise ? &noise : nullptr, S->ws, S->ws_bytes, S->dev_status,
+  return clip_accumulate_impl(S->layers, S->n_layers, (dp_dtype)S->layer_dtype, S->B, S->T, nullptr, S->C, S->clip,
+                              S->outs, S->ldos, 0.f, S->with_noise ? &noise : nullptr, S->ws, S->ws_bytes, S->dev_status,
                               S->stream, kept);
 }
 
 static dp_status step_rest(const dp_step_desc* S) {
   cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
-  const dp_dtype dt = (dp_dtype)S->dtype;
+  const dp_dtype dt = (dp_dtype)S->embed_dtype;
   dp_status s;
   // Row sums of tables that no GEMM writes need the clip factors only: on the side stream they run
   // where the GEMM's last wave leaves SMs idle.
@@ -1087,7 +1091,7 @@ static dp_status step_rest(const dp_step_desc* S) {
     if (s != DP_OK) return s;
   }
   if (S->n_vectors)
-    return dp_clip_accumulate_vectors(S->vectors, S->n_vectors, dt, S->B, S->T, nullptr, S->C, S->clip,
+    return dp_clip_accumulate_vectors(S->vectors, S->n_vectors, (dp_dtype)S->vector_dtype, S->B, S->T, nullptr, S->C, S->clip,
                                       S->vector_outs, 0.f, S->with_noise, S->sigma, 1.f, S->seed,
                                       S->vector_ids, S->step, S->ws, S->ws_bytes, main);
   return DP_OK;
@@ -1098,7 +1102,7 @@ dp_status dp_step_enqueue(const dp_step_desc* S, int32_t phases) {
   if (s != DP_OK) return s;
   // fp32 layers: within one call the sums can use the norms' split operands
   SplitGroup split;
-  SplitGroup* kept = phases == DP_STEP_ALL && S->dtype == DP_F32 ? &split : nullptr;
+  SplitGroup* kept = phases == DP_STEP_ALL && S->layer_dtype == DP_F32 ? &split : nullptr;
   if (phases & DP_STEP_NORMS) { s = step_norms(S, kept); if (s != DP_OK) return s; }
   if (phases & DP_STEP_GEMM) { s = step_gemm(S, kept); if (s != DP_OK) return s; }
   if (phases & DP_STEP_REST) { s = step_rest(S); if (s != DP_OK) return s; }

@@ -17,14 +17,26 @@
 
 namespace {
 
-// base pointer and leading dimension of a (..., ld) CUDA tensor whose leading axes are densely packed;
-// false: the caller's Python check words the complaint
-bool rows(PyObject* o, const void** ptr, int64_t* ld, int64_t* cols) {
+// dp_dtype of a tensor, kOther if it has none; *kind: that of the tensors seen before, kNone at first
+constexpr int32_t kNone = -1, kOther = -2;
+int32_t dtype_of(const at::Tensor& t) {
+  return t.scalar_type() == at::kFloat ? int32_t(DP_F32) : t.scalar_type() == at::kBFloat16 ? int32_t(DP_BF16) : kOther;
+}
+bool same_dtype(const at::Tensor& t, int32_t* kind) {
+  const int32_t k = dtype_of(t);
+  if (k == kOther || (*kind != kNone && *kind != k)) return false;
+  *kind = k;
+  return true;
+}
+
+// base pointer and leading dimension of a (..., ld) CUDA tensor whose leading axes are densely packed and whose
+// type is *kind; false: the caller's Python check words the complaint
+bool rows(PyObject* o, const void** ptr, int64_t* ld, int64_t* cols, int32_t* kind) {
   if (!THPVariable_Check(o)) return false;
   const at::Tensor& t = THPVariable_Unpack(o);
   const auto st = t.strides();
   const size_t n = st.size();
-  if (!t.is_cuda() || n < 2 || st[n - 1] != 1) return false;
+  if (!t.is_cuda() || n < 2 || st[n - 1] != 1 || !same_dtype(t, kind)) return false;
   if (n == 3 && st[0] != t.size(1) * st[1]) return false;
   *ptr = t.const_data_ptr();
   *ld = st[n - 2];
@@ -42,34 +54,35 @@ bool integer(PyObject* o, const char* name, int64_t otherwise, int64_t* out) {
   return true;
 }
 
-bool attr_rows(PyObject* o, const char* name, const void** ptr, int64_t* ld, int64_t* cols) {
+bool attr_rows(PyObject* o, const char* name, const void** ptr, int64_t* ld, int64_t* cols, int32_t* kind) {
   PyObject* v = PyObject_GetAttrString(o, name);
   if (!v) { PyErr_Clear(); return false; }
-  const bool ok = rows(v, ptr, ld, cols);
+  const bool ok = rows(v, ptr, ld, cols, kind);
   Py_DECREF(v);
   return ok;
 }
 
-bool linear_record(dp_linear_desc& L, PyObject* o) {
+bool linear_record(dp_linear_desc& L, PyObject* o, int32_t* kind) {
   int64_t ca = 0, cg = 0, d = 0, p = 0, mode = 0;
-  const bool ok = attr_rows(o, "A", &L.A, &L.lda, &ca) && attr_rows(o, "G", &L.G, &L.ldg, &cg) &&
+  const bool ok = attr_rows(o, "A", &L.A, &L.lda, &ca, kind) && attr_rows(o, "G", &L.G, &L.ldg, &cg, kind) &&
                   integer(o, "d", ca, &d) && integer(o, "p", cg, &p) && integer(o, "mode", 0, &mode);
   L.d = int32_t(d); L.p = int32_t(p); L.mode = int32_t(mode); L.mode_used = -1;
   return ok;
 }
 
-bool vector_record(dp_vector_desc& v, PyObject* o) {
+bool vector_record(dp_vector_desc& v, PyObject* o, int32_t* kind) {
   int64_t cols = 0, other = 0, p = 0;
-  bool ok = attr_rows(o, "G", &v.G, &v.ldg, &cols) && integer(o, "p", cols, &p);
+  bool ok = attr_rows(o, "G", &v.G, &v.ldg, &cols, kind) && integer(o, "p", cols, &p);
   PyObject* x = PyObject_GetAttrString(o, "X");
   if (!x) { PyErr_Clear(); return false; }
-  if (x != Py_None) ok = ok && rows(x, &v.X, &v.ldx, &other);
+  if (x != Py_None) ok = ok && rows(x, &v.X, &v.ldx, &other, kind);
   Py_DECREF(x);
   v.p = int32_t(p);
   return ok;
 }
 
-// f(record, object) over a sequence -> bytearray of records, or None if a tensor is not usable
+// f(record, object, kind) over a sequence -> bytearray of records, or None if a tensor is not usable or the
+// tensors are not all of one type
 template <typename Rec, typename F>
 PyObject* records(PyObject* arg, F f) {
   PyObject* seq = PySequence_Fast(arg, "a sequence");
@@ -80,7 +93,8 @@ PyObject* records(PyObject* arg, F f) {
   auto* rec = reinterpret_cast<Rec*>(PyByteArray_AS_STRING(out));
   memset(static_cast<void*>(rec), 0, size_t(n) * sizeof(Rec));
   bool ok = true;
-  for (Py_ssize_t k = 0; k < n && ok; ++k) ok = f(rec[k], PySequence_Fast_GET_ITEM(seq, k));
+  int32_t kind = kNone;
+  for (Py_ssize_t k = 0; k < n && ok; ++k) ok = f(rec[k], PySequence_Fast_GET_ITEM(seq, k), &kind);
   Py_DECREF(seq);
   if (!ok) { Py_DECREF(out); Py_RETURN_NONE; }
   return out;
@@ -145,7 +159,7 @@ bool output_list(PyObject* arg, Py_ssize_t n, std::vector<float*>& ptr, std::vec
   ptr.resize(size_t(n)); ld.resize(size_t(n));
   return each(arg, n, [&](Py_ssize_t k, PyObject* o) {
     const at::Tensor* t;
-    if (!device_tensor(o, &t) || !t) return false;
+    if (!device_tensor(o, &t) || !t || t->scalar_type() != at::kFloat) return false;
     ptr[size_t(k)] = pointer<float>(t);
     ld[size_t(k)] = t->dim() > 0 ? t->stride(0) : 0;
     return true;
@@ -162,7 +176,7 @@ bool word_list(PyObject* arg, Py_ssize_t n, std::vector<uint32_t>& w) {
 }
 
 // step(address of dp_step_enqueue, layers, outs, ids of outs, vectors, vector outs, their ids,
-//      (17 tensors or None), (stream or None, side stream, 4 events, seed, dtype, V, d, tied, noise, step, wte id,
+//      (17 tensors or None), (stream or None, side stream, 4 events, seed, V, d, tied, noise, step, wte id,
 //      wpe id, phases), C, sigma) -> status, with mode_used set on the layers; None: some argument is not
 // usable and the caller's Python checks say which
 PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t na) {
@@ -178,15 +192,16 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t na) {
   std::vector<int64_t> ldos, unused;
   std::vector<uint32_t> ids, vids;
   const at::Tensor* t[17];
-  int64_t v[16];
+  int64_t v[15];
+  int32_t layer_kind = kNone, vector_kind = kNone, embed_kind = kNone;
   memset(static_cast<void*>(layers.data()), 0, layers.size() * sizeof(dp_linear_desc));
   memset(static_cast<void*>(vectors.data()), 0, vectors.size() * sizeof(dp_vector_desc));
-  bool ok = each(a[1], n, [&](Py_ssize_t k, PyObject* o) { return linear_record(layers[size_t(k)], o); }) &&
+  bool ok = each(a[1], n, [&](Py_ssize_t k, PyObject* o) { return linear_record(layers[size_t(k)], o, &layer_kind); }) &&
             output_list(a[2], n, outs, ldos) && word_list(a[3], n, ids) &&
-            each(a[4], nv, [&](Py_ssize_t k, PyObject* o) { return vector_record(vectors[size_t(k)], o); }) &&
+            each(a[4], nv, [&](Py_ssize_t k, PyObject* o) { return vector_record(vectors[size_t(k)], o, &vector_kind); }) &&
             output_list(a[5], nv, vouts, unused) && word_list(a[6], nv, vids) &&
             each(a[7], 17, [&](Py_ssize_t k, PyObject* o) { return device_tensor(o, &t[k]); }) &&
-            each(a[8], 16, [&](Py_ssize_t k, PyObject* o) {
+            each(a[8], 15, [&](Py_ssize_t k, PyObject* o) {
               if (k == 0 && o == Py_None) v[k] = reinterpret_cast<int64_t>(c10::cuda::getCurrentCUDAStream().stream());
               else v[k] = int64_t(PyLong_AsUnsignedLongLongMask(o));
               if (PyErr_Occurred()) { PyErr_Clear(); return false; }
@@ -196,9 +211,11 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t na) {
   const void* g = nullptr;
   int64_t ldg = 0, cols = 0;
   PyObject* tensors = a[7];
-  ok = ok && PyTuple_Check(tensors) && rows(PyTuple_GET_ITEM(tensors, G_EMB), &g, &ldg, &cols);
+  ok = ok && PyTuple_Check(tensors) && rows(PyTuple_GET_ITEM(tensors, G_EMB), &g, &ldg, &cols, &embed_kind);
   ok = ok && t[IDS] && t[IDS]->dim() == 2 && t[WTE] && t[WTE]->dim() == 2 && (!t[WPE] || t[WPE]->dim() == 2) && t[WS] &&
        t[SIDE_WS];
+  for (int k : {IDS, POS_IDS, PERM, SEG, POS_PERM, POS_SEG, STATUS}) ok = ok && (!t[k] || t[k]->scalar_type() == at::kInt);
+  for (int k : {WTE, WPE, SQ, CLIP, NORMS, CROSS, SIDE_SQ}) ok = ok && (!t[k] || t[k]->scalar_type() == at::kFloat);
   const double C = PyFloat_AsDouble(a[9]), sigma = PyFloat_AsDouble(a[10]);
   if (PyErr_Occurred()) { PyErr_Clear(); ok = false; }
   if (!ok) Py_RETURN_NONE;
@@ -221,13 +238,16 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t na) {
   S.dev_status = pointer<int32_t>(t[STATUS]);
   S.stream = reinterpret_cast<void*>(v[0]); S.side_stream = reinterpret_cast<void*>(v[1]);
   for (int k = 0; k < 4; ++k) S.events[k] = reinterpret_cast<void*>(v[2 + k]);
-  S.seed = uint64_t(v[6]); S.dtype = int32_t(v[7]);
+  S.seed = uint64_t(v[6]);
+  S.layer_dtype = layer_kind == kNone ? embed_kind : layer_kind;           // no layers, no vectors: nothing to read
+  S.vector_dtype = vector_kind == kNone ? embed_kind : vector_kind;
+  S.embed_dtype = embed_kind;
   S.n_layers = int32_t(n); S.n_vectors = int32_t(nv);
-  S.B = int32_t(t[IDS]->size(0)); S.T = int32_t(t[IDS]->size(1)); S.V = int32_t(v[8]); S.d = int32_t(v[9]);
+  S.B = int32_t(t[IDS]->size(0)); S.T = int32_t(t[IDS]->size(1)); S.V = int32_t(v[7]); S.d = int32_t(v[8]);
   S.pos_rows = t[WPE] ? int32_t(t[WPE]->size(0)) : 0;
-  S.tied = int32_t(v[10]); S.with_noise = int32_t(v[11]); S.C = float(C); S.sigma = float(sigma);
-  S.step = uint32_t(v[12]); S.wte_id = uint32_t(v[13]); S.wpe_id = uint32_t(v[14]);
-  const int32_t phases = int32_t(v[15]);
+  S.tied = int32_t(v[9]); S.with_noise = int32_t(v[10]); S.C = float(C); S.sigma = float(sigma);
+  S.step = uint32_t(v[11]); S.wte_id = uint32_t(v[12]); S.wpe_id = uint32_t(v[13]);
+  const int32_t phases = int32_t(v[14]);
   dp_status st;
   Py_BEGIN_ALLOW_THREADS
   st = enqueue(&S, phases);

@@ -1,0 +1,86 @@
+"""The one-call step (pipeline.dp_step, dp_step_enqueue) against the same step call by call."""
+import pytest
+import torch
+
+from paper_2609_40335_b200 import binding as dp, pipeline
+
+pytestmark = pytest.mark.gpu
+
+F32, BF16 = torch.float32, torch.bfloat16
+
+
+def make_step(layers=BF16, vectors=BF16, embed=BF16, *, B=3, T=40, V=700, d=64, tied=False, lm=True, positions=False,
+              pos_ids=None, seed=5):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+
+    def normal(cols, std, dtype, ld=None):
+        return torch.empty(B, T, ld or cols, dtype=dtype, device="cuda").normal_(0.0, std, generator=g)
+
+    linears = [dp.Linear(normal(i, 1.0, layers), normal(o, 0.05, layers), d=i, p=o) for i, o in [(d, 3 * d), (3 * d, d), (d, 72)]]
+    head = dp.Linear(normal(d, 1.0, layers), normal(V, 0.02, layers, ld=(V + 7) // 8 * 8), d=d, p=V) if lm else None
+    per = dict(dtype=F32, device="cuda")
+    if positions and pos_ids is None:
+        pos_ids = torch.arange(T, dtype=torch.int32, device="cuda").repeat(B, 1).contiguous()
+    ds = pipeline.DeviceStep(
+        B=B, T=T, V=V, C=1.0, sigma=0.8, tied=tied, positions=positions, linears=linears, lm=head,
+        ids=torch.randint(0, V, (B, T), generator=g, device="cuda", dtype=torch.int32), pos_ids=pos_ids,
+        G_emb=normal(d, 0.05, embed), d_model=d, sq=torch.zeros(B, **per), clip=torch.zeros(B, **per),
+        norms=torch.zeros(B, **per), cross=torch.zeros(B, **per) if tied else None,
+        dev_status=torch.zeros(1, dtype=torch.int32, device="cuda"))
+    ds.vectors = [dp.Vector(normal(d, 0.05, vectors), normal(d, 1.0, vectors), p=d), dp.Vector(normal(3 * d, 0.05, vectors), None, p=3 * d)]
+    pipeline.allocate(ds)
+    return ds
+
+
+def state(ds):
+    torch.cuda.synchronize()
+    return dict({n: t.clone() for n, t in ds.outs.items()}, sq=ds.sq.clone(), clip=ds.clip.clone())
+
+
+def wipe(ds):
+    for t in ds.outs.values():
+        t.fill_(9.0)
+    ds.sq.fill_(-1.0)
+    ds.clip.fill_(-1.0)
+
+
+def assert_same(got, want, rel=5e-5):
+    """The same products in fp32, summed in another order: 1e-5.  A clip factor that differs by 2^-24 flips the bf16
+    rounding of 2^-16 of the R_i * x, by 2^-8 each: 2^-16 = 1.5e-5 more."""
+    for n, t in want.items():
+        assert float((got[n] - t).norm()) <= rel * float(t.norm()), n
+
+
+@pytest.mark.parametrize("noise", [False, True])
+@pytest.mark.parametrize("layers,vectors,embed", [(BF16, F32, BF16), (F32, BF16, BF16), (BF16, BF16, F32), (BF16, F32, F32),
+                                                  (F32, BF16, F32), (F32, F32, BF16)])
+def test_step_of_mixed_dtypes(layers, vectors, embed, noise):
+    ds = make_step(layers, vectors, embed, positions=True)
+    pipeline.dp_step(ds, seed=3, step=2, noise=noise, overlap=False)
+    want = state(ds)
+    wipe(ds)
+    pipeline.dp_step(ds, seed=3, step=2, noise=noise)
+    assert_same(state(ds), want)
+    assert int(ds.dev_status.item()) == 0
+
+
+def test_unsupported_and_clashing_dtypes_are_refused():
+    for change in ("half_vector", "mixed_vector", "mixed_layer", "ids", "out", "tied"):
+        ds = make_step(tied=change == "tied")
+        if change == "half_vector":
+            ds.vectors[1].G = ds.vectors[1].G.half()
+        elif change == "mixed_vector":
+            ds.vectors[0].X = ds.vectors[0].X.float()
+        elif change == "mixed_layer":
+            ds.linears[1].G = ds.linears[1].G.float()
+        elif change == "ids":
+            ds.ids = ds.ids.long()
+        elif change == "out":
+            ds.outs["linear1"] = ds.outs["linear1"].bfloat16()
+        else:
+            ds.G_emb = ds.G_emb.float()
+        with pytest.raises(dp.DpGhostError) as e:
+            pipeline.dp_step(ds)
+        assert e.value.status == 1
+        torch.cuda.synchronize()
