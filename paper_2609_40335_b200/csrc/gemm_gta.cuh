@@ -34,6 +34,33 @@ struct GtaNoise {
 
 // terms = 3: the operands are (2B, T, .) planes of high and low bf16 terms (fp32 inputs) and a product
 // takes three K steps per 64 tokens; terms = 1: plain bf16 operands.
+//
+// Order of a contraction's K steps.  With three terms, first lo hi' and hi lo' of all its 64-token blocks, then
+// hi hi' of all: an MMA rounds its sum towards zero, by as much as the sum is large, and while the small products
+// are added the sum is 2^-8 of its final size.  Block by block, every product of the three rounded the whole sum: error of
+// 25 layers of DistilGPT2's shapes against 64 bits 9.1e-6 at 2048 tokens, 2.8e-5 at 16384; in this order 5.1e-6 and 1.0e-5 (4.5e-6
+// is the operands' own).  The fp32 step of DistilGPT2 at B = 8, T = 128 takes 876 us in this order, 868 in the other.
+struct GtaWalk {
+  int ex, ts, term;                    // example, block in it, which product
+  int ex0, ts0, left, tblocks, terms;  // where the contraction starts, blocks left in this round, blocks per example
+
+  // blocks [b0, b1), counted from example `first`
+  __device__ __forceinline__ GtaWalk(int first, int b0, int b1, int tblocks_, int terms_)
+      : term(0), left(b1 - b0), tblocks(tblocks_), terms(terms_) {
+    ex = ex0 = first + b0 / tblocks;
+    ts = ts0 = b0 % tblocks;
+  }
+  __device__ __forceinline__ void next() {
+    if (terms > 1 && term == 0) { term = 1; return; }
+    if (++ts == tblocks) { ts = 0; ++ex; }
+    if (term != 1) return;
+    term = 0;
+    if (--left == 0) { ex = ex0; ts = ts0; term = 2; }
+  }
+  // plane of the A or G operand
+  __device__ __forceinline__ int plane(bool is_a) const { return terms > 1 ? 2 * ex + (term == (is_a ? 0 : 1)) : ex; }
+};
+
 long long gta_tiles(const dp_linear_desc& L);           // output tiles of one layer
 int gta_choose_nsplit(long long tiles, int B, int T, int terms, int sms);
 // scratch of a grouped call behind the clip factors: K-split planes (if any) and, terms = 1, the

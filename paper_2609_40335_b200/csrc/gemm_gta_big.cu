@@ -215,14 +215,13 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
       const int skew = it.nsub == 2 ? P.skew : 0, steps = P.ksteps + skew;
       // the steps in which this warp's part takes part
       const int from = sub ? skew : 0, to = is_x || sub ? steps : P.ksteps;
-      int ex = 0, ts = 0, term = 0;
-      const int terms = P.terms, low_term = is_g ? 2 : 1, tblocks = P.tsteps / terms;
+      const GtaWalk start(0, 0, P.ksteps / P.terms, P.tsteps / P.terms, P.terms);
+      GtaWalk at = start;
       for (int j = 0; j < steps; ++j) {
-        if (j == P.ksteps) { ex = 0; ts = 0; term = 0; }
+        if (j == P.ksteps) at = start;
         ok = ptx::warp_ok(ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit));
         if (!ok) break;
         const uint32_t bar = full_a + 8 * stage;
-        const int plane = terms > 1 ? 2 * ex + (term == low_term) : ex;
         const uint32_t dst = dst0 + stage * kStageBytes;
         const bool go = loads && j >= from && j < to;
         if (ptx::elect_one()) {
@@ -230,14 +229,11 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
           if (go)
 #pragma unroll
             for (int b = 0; b < kHalf / 64; ++b)
-              ptx::tma_load_3d_a(dst + b * kBoxBytes, tm, bar, c0 + b * 64, ts * kBK, plane);
+              ptx::tma_load_3d_a(dst + b * kBoxBytes, tm, bar, c0 + b * 64, at.ts * kBK, at.plane(!is_g));
         }
         __syncwarp();
         ++issued;
-        if (++term == terms) {
-          term = 0;
-          if (++ts == tblocks) { ts = 0; ++ex; }
-        }
+        at.next();
         if (++stage == kStages) { stage = 0; phase ^= 1; }
       }
     }

@@ -74,8 +74,8 @@ struct __align__(64) GtaParams {
   GtaLayer layer[kGtaMaxLayers];
   int n_layers;
   int B, T, tsteps;          // tsteps = terms * ceil(T / 64) K steps per example
-  int terms;                 // 3: split fp32 operands (hi hi, hi lo, lo hi per 64 tokens), else 1
-  int nsplit, ksteps_per_split;   // K splits, the same for all layers of a call
+  int terms;                 // 3: split fp32 operands (three products per 64 tokens), else 1
+  int nsplit, ksteps_per_split;   // K splits, the same for all layers of a call; multiples of `terms` steps
   float beta;
   int total_items;
   const float* clip;         // [B] R_i (scale mode)
@@ -197,23 +197,16 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
         // first column of this CTA's part of the tile: its G rows, or its share of the A columns
         const int c0 = is_a ? it.tn * kBN + int(rank) * Geo<kPair>::kAColsPerCta
                             : it.tm * kTileM + int(rank) * kBM;
-        // K step -> example, token block and (split operands) which of the three products
-        int ex = it.k0 / P.tsteps, ts = it.k0 - ex * P.tsteps, term = 0;
-        const int terms = P.terms, low_term = is_a ? 1 : 2, tblocks = P.tsteps / terms;
-        if (terms > 1) { term = ts % terms; ts /= terms; }
+        GtaWalk at(0, it.k0 / P.terms, it.k1 / P.terms, P.tsteps / P.terms, P.terms);
         for (int ks = it.k0; ks < it.k1; ++ks) {
           if (!ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
           const uint32_t bar = full_a + 8 * stage;
           const uint32_t dst = tiles_a + stage * kStageBytes + (is_a ? kGBytes : 0);
           ptx::mbar_arrive_expect_tx_a(bar, my_bytes);
           for (int j = 0; j < nbox; ++j)
-            ptx::tma_load_3d_a(dst + j * kBoxBytes, tm, bar, c0 + j * 64, ts * kBK,
-                               terms > 1 ? 2 * ex + (term == low_term) : ex);
+            ptx::tma_load_3d_a(dst + j * kBoxBytes, tm, bar, c0 + j * 64, at.ts * kBK, at.plane(is_a));
           ++issued;
-          if (++term == terms) {
-            term = 0;
-            if (++ts == tblocks) { ts = 0; ++ex; }
-          }
+          at.next();
           if (++stage == kStages) { stage = 0; phase ^= 1; }
         }
       }
@@ -696,7 +689,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
   const int tsteps = terms * ceil_div(T, kBK), planes = terms > 1 ? 2 * B : B;
   const int ksteps = B * tsteps;
   int nsplit = gta_choose_nsplit(gta_tiles(layers, n_layers), B, T, terms, sms);
-  const int kps = ceil_div(ksteps, nsplit);
+  const int kps = terms * ceil_div(ksteps / terms, nsplit);   // whole 64-token blocks
   nsplit = ceil_div(ksteps, kps);                       // drop empty trailing splits
   // Two tiles per item need the tiles for it: at least two per CTA pair (the bound below which K is split;
   // with fewer, one-tile items spread over more SMs).
