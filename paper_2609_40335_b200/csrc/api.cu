@@ -59,10 +59,9 @@ bool first_use_on_this_device(const void* key) {
 }
 
 // ---- planning of dp_ghost_norms ------------------------------------------------------------
-GhostPlan plan_ghost_norms(const dp_linear_desc* layers, int n_layers, int B, int T, int sms,
-                           bool allow_pair) {
+GhostPlan plan_ghost_norms(const dp_linear_desc* layers, int n_layers, int B, int T, int sms, bool split) {
   GhostPlan plan;
-  plan.pair = allow_pair && T > 128 && !g_ghost_single;
+  plan.pair = !split && T > 128 && !g_ghost_single;
   const int nt = ceil_div(T, plan.pair ? 256 : 128);
   const int slots = plan.pair ? 2 : 1;           // partial sums per work item
   const int units = plan.pair ? sms / 2 : sms;   // persistent CTAs or CTA pairs
@@ -78,8 +77,10 @@ GhostPlan plan_ghost_norms(const dp_linear_desc* layers, int n_layers, int B, in
     (mode == DP_NORM_GHOST ? plan.ghost_layers : plan.direct_layers).push_back(l);
   }
   // Column chunking of wide operands.  The per-item step budget shrinks until there are at
-  // least two items per SM (or the budget bottoms out).
-  int budget = 64;
+  // least two items per SM (or the budget bottoms out).  Split operands have sums no longer than those of layers
+  // planned one by one on widened operands (24 steps at d = 768, with 2.4 times the error per step): see
+  // ghost_norm_tc_kernel.
+  int budget = split ? 48 : 64;
   for (;;) {
     long long items = 0;
     for (int l : plan.ghost_layers) {
@@ -186,7 +187,7 @@ static size_t split_layer_bytes(const dp_linear_desc& L, int B, int T) {
 static size_t f32_norm_bytes(const dp_linear_desc& L, int B, int T, int sms) {
   dp_linear_desc one = L;
   one.mode = resolve_mode(L, T);
-  const GhostPlan plan = plan_ghost_norms(&one, 1, B, T, sms, false);
+  const GhostPlan plan = plan_ghost_norms(&one, 1, B, T, sms, true);
   return split_layer_bytes(L, B, T) + align_up(size_t(B) * plan.n_per * sizeof(float), 256);
 }
 
@@ -194,7 +195,7 @@ static size_t f32_norm_bytes(const dp_linear_desc& L, int B, int T, int sms) {
 // the place of the partial sums)
 static dp_status f32_norm_group(const SplitGroup& g, int B, int T, float* sq, char* ws, int* dev_status,
                                 cudaStream_t st, bool overwrite, NormSource* left) {
-  const GhostPlan plan = plan_ghost_norms(g.desc.data(), (int)g.desc.size(), B, T, sm_count(), false);
+  const GhostPlan plan = plan_ghost_norms(g.desc.data(), (int)g.desc.size(), B, T, sm_count(), true);
   float* partials = reinterpret_cast<float*>(ws + g.bytes);
   dp_status s = launch_split(g.jobs.data(), (int)g.jobs.size(), B, T, nullptr, st);
   if (s != DP_OK) return s;

@@ -44,7 +44,7 @@ constexpr int kRingBytes = 12 * kTileBytes;
 constexpr int kMaxStages = 32;
 constexpr size_t kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 1024 /*barriers*/;
 constexpr int kThreads = 192;
-constexpr int kTmemCols = 512;                   // 2 buffers x (S_A 128 + S_G 128) columns
+constexpr int kTmemCols = 512;                   // 2 buffers x (S_A 128 + S_G 128) columns; split: hi hi, small products
 
 struct __align__(64) GhostParams {
   CUtensorMap tmA[kGhostMaxLayers];
@@ -91,8 +91,17 @@ __device__ __forceinline__ Item decode_item(const GhostParams& P, int item, int&
   return it;
 }
 
+__device__ __forceinline__ uint32_t add_f32(uint32_t a, uint32_t b) {
+  return __float_as_uint(__uint_as_float(a) + __uint_as_float(b));
+}
+
 // kSplit: fp32 operands stored as two bf16 planes per example (see split_kernels.cu).  Every Gram
-// tile is then S = hi hi^T + hi lo^T + lo hi^T, three MMAs per K step on tiles loaded once.
+// tile is then S = hi hi^T + hi lo^T + lo hi^T, three MMAs per K step on tiles loaded once.  An MMA rounds its sum
+// towards zero, by as much as the sum is large, and the diagonal of S is a sum of positive terms: the two small
+// products have an accumulator of their own, the second buffer's, which leaves a third of the roundings.
+// 25 layers of DistilGPT2's shapes at B = 64, T = 256, error against 64 bits: 2.2e-5 with all three in one, now
+// 1.4e-5.  The epilogue no longer overlaps the next item's MMAs; fewer chunks of wide operands make up for it (the fp32
+// step of DistilGPT2 at B = 8, T = 128: no difference beyond 0.5 %).
 template <bool kDiagOnly, bool kSplit, int kBoxes>
 __global__ void __launch_bounds__(kThreads, 1)
 ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
@@ -200,7 +209,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
     for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x, ++n_item) {
       const Item it = decode_item(P, item, lay);
       const bool diag = kDiagOnly || (it.ti == it.tj);
-      const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
+      const uint32_t buf = kSplit ? 0 : n_item & 1, acc_phase = (kSplit ? n_item : n_item >> 1) & 1;
       ok = ptx::warp_ok(ptx::mbar_wait(&acc_empty[buf], acc_phase ^ 1, abort_flag, P.wait_limit));
       if (!ok) break;
       ptx::tc_fence_after();
@@ -223,8 +232,8 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
                 const uint32_t ah = sa + kk * 2, bh = sb + kk * 2, low = tile_bytes >> 4;
                 ptx::mma_bf16_ss_lh(d_tmem, ah, bh, desc_hi, idesc, (k + b > 0 || kk > 0) ? 1u : 0u);
                 if (kSplit) {
-                  ptx::mma_bf16_ss_lh(d_tmem, ah, bh + low, desc_hi, idesc, 1u);
-                  ptx::mma_bf16_ss_lh(d_tmem, ah + low, bh, desc_hi, idesc, 1u);
+                  ptx::mma_bf16_ss_lh(d_tmem + 256, ah, bh + low, desc_hi, idesc, (k + b > 0 || kk > 0) ? 1u : 0u);
+                  ptx::mma_bf16_ss_lh(d_tmem + 256, ah + low, bh, desc_hi, idesc, 1u);
                 }
               }
             }
@@ -250,7 +259,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
     bool ok = true;
     for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x, ++n_item) {
       const Item it = decode_item(P, item, lay);
-      const uint32_t buf = n_item & 1, acc_phase = (n_item >> 1) & 1;
+      const uint32_t buf = kSplit ? 0 : n_item & 1, acc_phase = (kSplit ? n_item : n_item >> 1) & 1;
       if (!ptx::mbar_wait_relaxed(&acc_full[buf], acc_phase, abort_flag, P.wait_limit)) { ok = false; break; }
       ptx::tc_fence_after();
       const uint32_t t0 = tmem_base + (uint32_t(q * 32) << 16) + buf * 256;
@@ -260,7 +269,16 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
         uint32_t ra[32], rg[32];
         ptx::tmem_ld_32x32b_x32(t0 + c, ra);
         ptx::tmem_ld_32x32b_x32(t0 + 128 + c, rg);
-        ptx::tmem_ld_wait();
+        if (kSplit) {
+          uint32_t sa[32], sg[32];
+          ptx::tmem_ld_32x32b_x32(t0 + 256 + c, sa);
+          ptx::tmem_ld_32x32b_x32(t0 + 384 + c, sg);
+          ptx::tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) { ra[j] = add_f32(ra[j], sa[j]); rg[j] = add_f32(rg[j], sg[j]); }
+        } else {
+          ptx::tmem_ld_wait();
+        }
 #pragma unroll
         for (int j = 0; j < 32; ++j) acc = fmaf(__uint_as_float(ra[j]), __uint_as_float(rg[j]), acc);
       }
@@ -268,7 +286,16 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
         uint32_t ra[16], rg[16];
         ptx::tmem_ld_32x32b_x16(t0 + rows - 16, ra);
         ptx::tmem_ld_32x32b_x16(t0 + 128 + rows - 16, rg);
-        ptx::tmem_ld_wait();
+        if (kSplit) {
+          uint32_t sa[16], sg[16];
+          ptx::tmem_ld_32x32b_x16(t0 + 256 + rows - 16, sa);
+          ptx::tmem_ld_32x32b_x16(t0 + 384 + rows - 16, sg);
+          ptx::tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) { ra[j] = add_f32(ra[j], sa[j]); rg[j] = add_f32(rg[j], sg[j]); }
+        } else {
+          ptx::tmem_ld_wait();
+        }
 #pragma unroll
         for (int j = 0; j < 16; ++j) acc = fmaf(__uint_as_float(ra[j]), __uint_as_float(rg[j]), acc);
       }

@@ -40,9 +40,9 @@ struct GhostPlan {
 };
 
 // T*T > d*p selects DIRECT under AUTO (strict), otherwise GHOST.
-// allow_pair = false keeps the single-CTA Gram kernel whatever T is.
+// split: fp32 layers on their two bf16 planes, which stay on the single-CTA Gram kernel whatever T is.
 GhostPlan plan_ghost_norms(const dp_linear_desc* layers, int n_layers, int B, int T, int sms,
-                           bool allow_pair = true);
+                           bool split = false);
 
 dp_status launch_ghost_norm_pair(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
                                  float* partials, int* dev_status, cudaStream_t st);

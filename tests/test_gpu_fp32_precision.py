@@ -29,3 +29,22 @@ def test_clipped_sums_over_many_tokens(n_layers):
     bound = 4.5e-6 + 2 / 3 * 1024 * 2.0 ** -24
     for o in (outs[0], outs[-1]):
         assert float((o.double() - want).norm() / want.norm()) < bound
+
+
+# many examples: work items enough without cutting wide operands
+@pytest.mark.parametrize("B,T", [(64, 256), (128, 64)])
+@pytest.mark.parametrize("shapes", [[(768, 2304), (768, 768), (768, 3072), (3072, 768)], [(66, 2000)], [(128, 5000), (64, 2304)]])
+def test_norms_of_many_examples(shapes, B, T):
+    layers = [dp.Linear(normal(B, T, d, seed=k), normal(B, T, p, std=1e-2, seed=50 + k), d=d, p=p, mode=dp.DP_NORM_GHOST)
+              for k, (d, p) in enumerate(shapes)]
+    sq = torch.zeros(B, device="cuda")
+    ws = torch.empty(1 << 32, dtype=torch.uint8, device="cuda")
+    dp.dp_ghost_norms(layers, B, T, sq, ws=ws)
+    want = 0
+    for l in layers:
+        a, g = l.A.double(), l.G.double()
+        want = want + (torch.bmm(a, a.transpose(1, 2)) * torch.bmm(g, g.transpose(1, 2))).sum((1, 2))
+    # A Gram entry's diagonal is a sum of positive terms: an MMA of full size, four per 64 columns, takes 2^-24 of its
+    # final size from it (measured: 0.7 of that).  Narrow and wide part of an item are 60 steps together.  lo lo' is left
+    # out: |lo| <= 2^-8 of a value's power of two, 2.6e-6 of the sum of squares, for either operand.
+    assert float(((sq.double() - want) / want).norm() / B ** 0.5) < 60 * 4 * 2.0 ** -24 + 2 * 2.6e-6
