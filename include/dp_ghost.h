@@ -18,7 +18,9 @@
  *     caller; [host] is ordinary host memory.  The library never allocates, frees or
  *     synchronises: work is enqueued on `stream` (a cudaStream_t passed as void*) and the
  *     call returns.  Scratch comes from a caller-provided [dev] workspace whose minimum
- *     size the matching *_ws_bytes function reports (0 means none is needed).
+ *     size the matching *_ws_bytes function reports (0 means none is needed).  It lies on a 4-byte
+ *     boundary at least, a 16-byte one where operands are copied into it for TMA (DP_F32 layers on the tensor
+ *     cores, clipped sums of layers like an LM head): else DP_ERR_ALIGNMENT, from the norms DP_ERR_WORKSPACE.
  *   - Tensors are row-major with an explicit leading dimension (elements between rows).
  *     Activations A are (B*T, d), output gradients G are (B*T, p); example i owns rows
  *     i*T .. i*T+T-1.  dp_dtype names the storage type of A / G; accumulation is fp32.

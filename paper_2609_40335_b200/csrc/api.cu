@@ -618,6 +618,8 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
   }
   if (!ws || ws_bytes < dp_clip_accumulate_grouped_ws_bytes(layers, n_layers, dt, B, T))
     return DP_ERR_WORKSPACE;
+  for (int l = 0; l < n_layers && !aligned16(ws); ++l)     // operands that TMA reads from there
+    if (tc ? gta_prescales(layers[l]) : dt == DP_F32 && f32_on_tensor_cores(layers[l], T)) return DP_ERR_ALIGNMENT;
   cudaStream_t st = (cudaStream_t)stream;
   float* clip_ws = static_cast<float*>(ws);
   dp_status s = resolve_clip(sq, B, C, clip, &clip_ws, st);

@@ -407,11 +407,15 @@ sort_scan_kernel(const int* __restrict__ totals, int V, int* __restrict__ seg) {
   __shared__ int wsum[kWarps], wbase[kWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int base = 0;
-  const int4* t4 = reinterpret_cast<const int4*>(totals);
+  if ((reinterpret_cast<uintptr_t>(totals) & 15) == 0) {
+    const int4* t4 = reinterpret_cast<const int4*>(totals);
 #pragma unroll 4
-  for (int v = threadIdx.x; v < blockIdx.x * 256; v += kSideThreads) {
-    const int4 y = t4[v];
-    base += (y.x + y.y) + (y.z + y.w);
+    for (int v = threadIdx.x; v < blockIdx.x * 256; v += kSideThreads) {
+      const int4 y = t4[v];
+      base += (y.x + y.y) + (y.z + y.w);
+    }
+  } else {                                             // a workspace on any 4-byte boundary will do
+    for (int v = threadIdx.x; v < blockIdx.x * 1024; v += kSideThreads) base += totals[v];
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) base += __shfl_xor_sync(0xffffffffu, base, o);

@@ -62,6 +62,7 @@ struct GtaWalk {
 };
 
 long long gta_tiles(const dp_linear_desc& L);           // output tiles of one layer
+bool gta_prescales(const dp_linear_desc& L);            // terms = 1: a scaled copy goes into the scratch, for TMA to read
 int gta_choose_nsplit(long long tiles, int B, int T, int terms, int sms);
 // scratch of a grouped call behind the clip factors: K-split planes (if any) and, terms = 1, the
 // pre-scaled copies of very narrow operands

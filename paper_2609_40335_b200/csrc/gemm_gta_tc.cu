@@ -528,7 +528,7 @@ splitk_reduce_kernel(const __grid_constant__ ReduceParams P) {
   }
   const ReduceLayer& L = P.layer[lo];
   const size_t total = size_t(L.M) * L.N;
-  const bool vec = (total & 3) == 0;                 // planes are 256-byte aligned
+  const bool vec = (total & 3) == 0 && (reinterpret_cast<uintptr_t>(L.partial) & 15) == 0;
   const bool ovec = (L.N & 3) == 0 && (L.ldo & 3) == 0 && (reinterpret_cast<uintptr_t>(L.out) & 15) == 0;
   const uint32_t step = effective_step(P.step, P.step_dev);
 #pragma unroll
@@ -659,6 +659,8 @@ static long long gta_tiles(const dp_linear_desc* layers, int n_layers) {
   for (int l = 0; l < n_layers; ++l) tiles += gta_tiles(layers[l]);
   return tiles;
 }
+
+bool gta_prescales(const dp_linear_desc& L) { return prescale_layer(L); }
 
 int gta_choose_nsplit(long long tiles, int B, int T, int terms, int sms) {
   const int ksteps = B * terms * ceil_div(T, kBK);
