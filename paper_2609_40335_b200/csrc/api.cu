@@ -314,25 +314,35 @@ size_t dp_ghost_norms_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, d
   return align_up(size_t(B) * plan.n_per * sizeof(float), 256);
 }
 
-// overwrite: sq is written instead of added to (its first contribution of a step)
-static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B,
+// all that can be wrong with a call, before anything is enqueued; and its plan
+static dp_status ghost_norms_check(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B, int32_t T,
+                                   const float* sq, const void* ws, size_t ws_bytes, GhostPlan* plan) {
+  if (!layers || n_layers <= 0 || B <= 0 || T <= 0 || !sq) return DP_ERR_INVALID_ARG;
+  if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
+  const bool tc = (dt == DP_BF16) && !g_force_fma;
+  bool split = false;
+  for (int l = 0; l < n_layers; ++l) {
+    const dp_status s = check_linear(layers[l], dt, tc);
+    if (s != DP_OK) return s;
+    split = split || (dt == DP_F32 && f32_on_tensor_cores(layers[l], T));
+  }
+  *plan = plan_ghost_norms(layers, n_layers, B, T, sm_count());
+  const size_t need = tc ? align_up(size_t(B) * plan->n_per * sizeof(float), 256) : f32_norms_bytes(layers, n_layers, dt, B, T);
+  if (ws_bytes < need || ((tc || split) && !ws) || (split && !aligned16(ws))) return DP_ERR_WORKSPACE;
+  return DP_OK;
+}
+
+// overwrite: sq is written instead of added to (its first contribution of a step); the call has been checked
+static dp_status ghost_norms_impl(const GhostPlan& plan, dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B,
                                   int32_t T, float* sq, void* ws, size_t ws_bytes, int32_t* dev_status,
                                   void* stream, bool overwrite, NormSource* left = nullptr,
                                   SplitGroup* kept = nullptr) {
   // left: the last reduction is not done; *left says where its partial sums are (or sq itself)
   // kept: the split operands of fp32 layers, where they stay in ws all together; empty if they do not
-  if (!layers || n_layers <= 0 || B <= 0 || T <= 0 || !sq) return DP_ERR_INVALID_ARG;
-  if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const bool tc = (dt == DP_BF16) && !g_force_fma;
-  for (int l = 0; l < n_layers; ++l) {
-    const dp_status s = check_linear(layers[l], dt, tc);
-    if (s != DP_OK) return s;
-  }
-  const GhostPlan plan = plan_ghost_norms(layers, n_layers, B, T, sm_count());
   if (!tc) {
     const size_t split_need = f32_norms_bytes(layers, n_layers, dt, B, T);
-    if (split_need > ws_bytes) return DP_ERR_WORKSPACE;
     SplitGroup group;
     char* base = static_cast<char*>(ws);
     if (left) *left = NormSource{sq, 1, 1.f, nullptr};
@@ -376,7 +386,6 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
       dp_status s = DP_OK;
       if (together && !on_tensor_cores(layers[l], dt, T) && plan.mode_used[l] == DP_NORM_GHOST) continue;
       if (dt == DP_F32 && f32_on_tensor_cores(layers[l], T)) {
-        if (!ws || !aligned16(ws)) return DP_ERR_WORKSPACE;
         const size_t more = f32_norm_bytes(layers[l], B, T, sm_count());
         if (group.bound + more > ws_bytes) s = flush();
         if (s != DP_OK) return s;
@@ -391,8 +400,6 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
     }
     return flush();
   }
-  const size_t need = align_up(size_t(B) * plan.n_per * sizeof(float), 256);
-  if (!ws || ws_bytes < need) return DP_ERR_WORKSPACE;
   float* partials = static_cast<float*>(ws);
   dp_status s = DP_OK;
   if (!plan.ghost_layers.empty()) {
@@ -414,7 +421,9 @@ static dp_status ghost_norms_impl(dp_linear_desc* layers, int32_t n_layers, dp_d
 dp_status dp_ghost_norms(dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B,
                          int32_t T, float* sq, void* ws, size_t ws_bytes, int32_t* dev_status,
                          void* stream) {
-  return ghost_norms_impl(layers, n_layers, dt, B, T, sq, ws, ws_bytes, dev_status, stream, false);
+  GhostPlan plan;
+  const dp_status s = ghost_norms_check(layers, n_layers, dt, B, T, sq, ws, ws_bytes, &plan);
+  return s != DP_OK ? s : ghost_norms_impl(plan, layers, n_layers, dt, B, T, sq, ws, ws_bytes, dev_status, stream, false);
 }
 
 // ------------------------------------------------------------------------ embedding norms
@@ -456,21 +465,28 @@ size_t dp_tied_cross_term_ws_bytes(int32_t B, int32_t T, int32_t d, int32_t V) {
   return align_up(size_t(B) * per * sizeof(float), 256);
 }
 
-static dp_status cross_term_impl(const int32_t* ids, const void* G_emb, int64_t ldge, const void* A_lm,
-                                 int64_t ldal, const void* G_lm, int64_t ldgl, dp_dtype dt, int32_t B,
-                                 int32_t T, int32_t d, int32_t V, float* sq, float* cross, void* ws,
-                                 size_t ws_bytes, int32_t* dev_status, void* stream, NormSource* left) {
+static dp_status cross_term_check(const int32_t* ids, const void* G_emb, int64_t ldge, const void* A_lm, int64_t ldal,
+                                  const void* G_lm, int64_t ldgl, dp_dtype dt, int32_t B, int32_t T, int32_t d, int32_t V,
+                                  const void* ws, size_t ws_bytes) {
   if (!ids || !G_emb || !A_lm || !G_lm || B <= 0 || T <= 0 || d <= 0 || V <= 0)
     return DP_ERR_INVALID_ARG;
-  if (!sq && !cross) return DP_ERR_INVALID_ARG;
   if (ldge < d || ldal < d || ldgl < V) return DP_ERR_INVALID_ARG;
   if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
   const bool tc = (dt == DP_BF16) && !g_force_fma;
   if (tc && (!aligned16(G_emb) || !aligned16(A_lm) || (ldge % 8) || (ldal % 8))) return DP_ERR_ALIGNMENT;
-  if (!ws || ws_bytes < dp_tied_cross_term_ws_bytes(B, T, d, V)) return DP_ERR_WORKSPACE;
+  return !ws || ws_bytes < dp_tied_cross_term_ws_bytes(B, T, d, V) ? DP_ERR_WORKSPACE : DP_OK;
+}
+
+static dp_status cross_term_impl(const int32_t* ids, const void* G_emb, int64_t ldge, const void* A_lm,
+                                 int64_t ldal, const void* G_lm, int64_t ldgl, dp_dtype dt, int32_t B,
+                                 int32_t T, int32_t d, int32_t V, float* sq, float* cross, void* ws,
+                                 size_t ws_bytes, int32_t* dev_status, void* stream, NormSource* left) {
+  if (!sq && !cross) return DP_ERR_INVALID_ARG;
+  dp_status s = cross_term_check(ids, G_emb, ldge, A_lm, ldal, G_lm, ldgl, dt, B, T, d, V, ws, ws_bytes);
+  if (s != DP_OK) return s;
+  const bool tc = (dt == DP_BF16) && !g_force_fma;
   cudaStream_t st = (cudaStream_t)stream;
   float* partials = static_cast<float*>(ws);
-  dp_status s;
   int per;
   if (tc) {
     s = launch_cross_term_tc(ids, G_emb, ldge, A_lm, ldal, G_lm, ldgl, B, T, d, V, partials,
@@ -600,12 +616,10 @@ size_t dp_clip_accumulate_grouped_ws_bytes(const dp_linear_desc* layers, int32_t
   return n;
 }
 
-static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt,
-                                      int32_t B, int32_t T, const float* sq, float C, float* clip,
-                                      float* const* outs, const int64_t* ldos, float beta,
-                                      const GtaNoise* noise, void* ws, size_t ws_bytes,
-                                      int32_t* dev_status, void* stream, const SplitGroup* kept = nullptr) {
-  if (!layers || n_layers <= 0 || !outs || !ldos || (!sq && !clip) || B <= 0 || T <= 0) return DP_ERR_INVALID_ARG;
+static dp_status clip_accumulate_check(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B, int32_t T,
+                                       float* const* outs, const int64_t* ldos, float beta, float C, const void* ws,
+                                       size_t ws_bytes) {
+  if (!layers || n_layers <= 0 || !outs || !ldos || B <= 0 || T <= 0) return DP_ERR_INVALID_ARG;
   if (dt != DP_F32 && dt != DP_BF16) return DP_ERR_INVALID_ARG;
   if (!(beta == 0.f || beta == 1.f) || !finite_pos(C)) return DP_ERR_INVALID_ARG;
   const bool tc = (dt == DP_BF16) && !g_force_fma;
@@ -620,6 +634,16 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
     return DP_ERR_WORKSPACE;
   for (int l = 0; l < n_layers && !aligned16(ws); ++l)     // operands that TMA reads from there
     if (tc ? gta_prescales(layers[l]) : dt == DP_F32 && f32_on_tensor_cores(layers[l], T)) return DP_ERR_ALIGNMENT;
+  return DP_OK;
+}
+
+// the call has been checked
+static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt,
+                                      int32_t B, int32_t T, const float* sq, float C, float* clip,
+                                      float* const* outs, const int64_t* ldos, float beta,
+                                      const GtaNoise* noise, void* ws, size_t ws_bytes,
+                                      int32_t* dev_status, void* stream, const SplitGroup* kept = nullptr) {
+  const bool tc = (dt == DP_BF16) && !g_force_fma;
   cudaStream_t st = (cudaStream_t)stream;
   float* clip_ws = static_cast<float*>(ws);
   dp_status s = resolve_clip(sq, B, C, clip, &clip_ws, st);
@@ -694,8 +718,10 @@ dp_status dp_clip_accumulate_grouped(const dp_linear_desc* layers, int32_t n_lay
                                      int32_t B, int32_t T, const float* sq, float C, float* clip,
                                      float* const* outs, const int64_t* ldos, float beta, void* ws,
                                      size_t ws_bytes, int32_t* dev_status, void* stream) {
-  return clip_accumulate_impl(layers, n_layers, dt, B, T, sq, C, clip, outs, ldos, beta, nullptr, ws,
-                              ws_bytes, dev_status, stream);
+  if (!sq && !clip) return DP_ERR_INVALID_ARG;
+  const dp_status s = clip_accumulate_check(layers, n_layers, dt, B, T, outs, ldos, beta, C, ws, ws_bytes);
+  return s != DP_OK ? s : clip_accumulate_impl(layers, n_layers, dt, B, T, sq, C, clip, outs, ldos, beta, nullptr, ws,
+                                               ws_bytes, dev_status, stream);
 }
 
 static bool noise_args_ok(float sigma, float C, float scale) {
@@ -709,7 +735,9 @@ dp_status dp_clip_accumulate_noise_grouped(const dp_linear_desc* layers, int32_t
                                            uint64_t seed, const uint32_t* tensor_ids, uint32_t step,
                                            void* ws, size_t ws_bytes, int32_t* dev_status,
                                            void* stream) {
-  if (!tensor_ids || !noise_args_ok(sigma, C, scale)) return DP_ERR_INVALID_ARG;
+  if (!tensor_ids || !noise_args_ok(sigma, C, scale) || (!sq && !clip)) return DP_ERR_INVALID_ARG;
+  const dp_status s = clip_accumulate_check(layers, n_layers, dt, B, T, outs, ldos, beta, C, ws, ws_bytes);
+  if (s != DP_OK) return s;
   const GtaNoise noise{sigma * C, scale, seed, step, tensor_ids};
   return clip_accumulate_impl(layers, n_layers, dt, B, T, sq, C, clip, outs, ldos, beta, &noise, ws,
                               ws_bytes, dev_status, stream);
@@ -932,7 +960,9 @@ size_t dp_step_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype
   return need + fma_norms_bytes(layers, n_layers, dt, B, T);
 }
 
-static dp_status check_step(const dp_step_desc* S) {
+// All that can be wrong with a step, before anything is enqueued: an error found halfway would leave work on two
+// streams.  Workspaces as the requested phases use them; plan: of the layers' norms, if those are among them.
+static dp_status check_step(const dp_step_desc* S, int32_t phases, GhostPlan* plan) {
   if (!S || S->B <= 0 || S->T <= 0 || S->V <= 0 || S->d <= 0 || S->n_layers < 0 || S->n_vectors < 0)
     return DP_ERR_INVALID_ARG;
   if (!S->ids || !S->G_emb || !S->wte || !S->sq || !S->clip || !S->side_sq || !S->perm || !S->seg)
@@ -945,7 +975,46 @@ static dp_status check_step(const dp_step_desc* S) {
   if (S->tied && S->embed_dtype != S->layer_dtype) return DP_ERR_INVALID_ARG;      // one type in the cross term
   if (S->pos_ids && (!S->wpe || !S->pos_perm || !S->pos_seg || S->pos_rows <= 0)) return DP_ERR_INVALID_ARG;
   for (int k = 0; k < 4; ++k) if (!S->events[k]) return DP_ERR_INVALID_ARG;
-  if (S->with_noise && !noise_args_ok(S->sigma, S->C, 1.f)) return DP_ERR_INVALID_ARG;
+  if (!finite_pos(S->C) || (S->with_noise && !noise_args_ok(S->sigma, S->C, 1.f))) return DP_ERR_INVALID_ARG;
+  if (S->ldge < S->d || S->ld_wte < S->d || (S->pos_ids && S->ld_wpe < S->d)) return DP_ERR_INVALID_ARG;
+  const int B = S->B, T = S->T, d = S->d;
+  if (S->n_vectors) {
+    const dp_status s = check_vectors(S->vectors, S->n_vectors, B, T);
+    if (s != DP_OK) return s;
+    if (!S->vector_outs || (S->with_noise && !S->vector_ids)) return DP_ERR_INVALID_ARG;
+    for (int k = 0; k < S->n_vectors; ++k) if (!S->vector_outs[k]) return DP_ERR_INVALID_ARG;
+  }
+  if (T > kEmbedMaxT || (long long)B * T > 0x7fffffffLL) return DP_ERR_UNSUPPORTED;
+  const int32_t rows[2] = {S->V, S->pos_ids ? S->pos_rows : 0};              // of the tables
+  size_t ws = 0, side = 0;
+  if (phases & DP_STEP_NORMS) {
+    if (S->n_layers) {
+      const dp_status s = ghost_norms_check(S->layers, S->n_layers, (dp_dtype)S->layer_dtype, B, T, S->sq, S->ws, S->ws_bytes, plan);
+      if (s != DP_OK) return s;
+    }
+    if (S->n_vectors) ws = std::max(ws, dp_vector_norms_ws_bytes(S->vectors, S->n_vectors, B, T));
+    if (S->tied) {
+      const dp_linear_desc& lm = S->layers[S->n_layers - 1];
+      const dp_status s = cross_term_check(S->ids, S->G_emb, S->ldge, lm.A, lm.lda, lm.G, lm.ldg, (dp_dtype)S->embed_dtype, B, T,
+                                           d, S->V, S->ws, S->ws_bytes);
+      if (s != DP_OK) return s;
+    }
+    side = dp_embed_norms_ws_bytes(B, T, d);
+    for (int32_t r : rows) side = std::max(side, dp_embed_sort_ws_bytes(B, T, r));
+  }
+  if ((phases & DP_STEP_GEMM) && S->n_layers) {
+    const dp_status s = clip_accumulate_check(S->layers, S->n_layers, (dp_dtype)S->layer_dtype, B, T, S->outs, S->ldos, 0.f, S->C,
+                                              S->ws, S->ws_bytes);
+    if (s != DP_OK) return s;
+  }
+  if (phases & DP_STEP_REST) {
+    for (int k = 0; k < 2; ++k) {
+      size_t& w = k == 0 && S->tied ? ws : side;
+      w = std::max(w, dp_clip_accumulate_embed_ws_bytes(B, T, d, rows[k]));
+    }
+    if (S->n_vectors) ws = std::max(ws, dp_clip_accumulate_vectors_ws_bytes(S->vectors, S->n_vectors, B, T));
+  }
+  if (S->ws_bytes < ws || (ws && !S->ws) || S->side_ws_bytes < side || (side && !S->side_ws)) return DP_ERR_WORKSPACE;
   return DP_OK;
 }
 
@@ -961,7 +1030,7 @@ static dp_status start_table(const dp_step_desc* S, float* table, int64_t ld, in
 }
 
 // events: [0] the step began, [1] embedding norms done, [2] row sums done, [3] clip factors exist
-static dp_status step_norms(const dp_step_desc* S, SplitGroup* kept) {
+static dp_status step_norms(const dp_step_desc* S, const GhostPlan& plan, SplitGroup* kept) {
   cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
   const dp_dtype embed_dt = (dp_dtype)S->embed_dtype;
   const int B = S->B, T = S->T;
@@ -972,8 +1041,8 @@ static dp_status step_norms(const dp_step_desc* S, SplitGroup* kept) {
   char* ws = static_cast<char*>(S->ws);
   DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[0], main));
   if (S->n_layers) {
-    s = ghost_norms_impl(S->layers, S->n_layers, (dp_dtype)S->layer_dtype, B, T, S->sq, S->ws, S->ws_bytes, S->dev_status,
-                         main, true, &N.src[0], kept);
+    s = ghost_norms_impl(plan, S->layers, S->n_layers, (dp_dtype)S->layer_dtype, B, T, S->sq, S->ws, S->ws_bytes,
+                         S->dev_status, main, true, &N.src[0], kept);
     if (s != DP_OK) return s;
     N.n = 1;
     if (N.src[0].partials != S->sq)
@@ -1101,15 +1170,24 @@ static dp_status step_rest(const dp_step_desc* S) {
 }
 
 dp_status dp_step_enqueue(const dp_step_desc* S, int32_t phases) {
-  dp_status s = check_step(S);
+  GhostPlan plan;
+  dp_status s = check_step(S, phases, &plan);
   if (s != DP_OK) return s;
   // fp32 layers: within one call the sums can use the norms' split operands
   SplitGroup split;
   SplitGroup* kept = phases == DP_STEP_ALL && S->layer_dtype == DP_F32 ? &split : nullptr;
-  if (phases & DP_STEP_NORMS) { s = step_norms(S, kept); if (s != DP_OK) return s; }
-  if (phases & DP_STEP_GEMM) { s = step_gemm(S, kept); if (s != DP_OK) return s; }
-  if (phases & DP_STEP_REST) { s = step_rest(S); if (s != DP_OK) return s; }
-  return DP_OK;
+  if (phases & DP_STEP_NORMS) s = step_norms(S, plan, kept);
+  if (s == DP_OK && (phases & DP_STEP_GEMM)) s = step_gemm(S, kept);
+  if (s == DP_OK && (phases & DP_STEP_REST)) s = step_rest(S);
+  if (s != DP_OK) {
+    // a launch failed: whatever the side stream still does to the caller's tensors, `stream` waits for it
+    const int error = g_last_cuda_error;
+    if (cudaEventRecord((cudaEvent_t)S->events[2], (cudaStream_t)S->side_stream) == cudaSuccess)
+      (void)cudaStreamWaitEvent((cudaStream_t)S->stream, (cudaEvent_t)S->events[2], 0);
+    (void)cudaGetLastError();
+    g_last_cuda_error = error;
+  }
+  return s;
 }
 
 }  // extern "C"
