@@ -1065,7 +1065,7 @@ static dp_status step_norms(const dp_step_desc* S, const GhostPlan& plan, SplitG
   for (size_t k = 0; k < tables; ++k) {
     char* w = side_ws;
     if (keep) { side_bytes -= each; w += side_bytes; }
-    s = embed_norms_impl(k ? S->pos_ids : S->ids, S->G_emb, S->ldge, embed_dt, B, T, S->d, k ? T : S->V, S->side_sq,
+    s = embed_norms_impl(k ? S->pos_ids : S->ids, S->G_emb, S->ldge, embed_dt, B, T, S->d, k ? S->pos_rows : S->V, S->side_sq,
                          nullptr, w, keep ? each : S->side_ws_bytes, S->dev_status, side, k == 0, keep ? &embed[k] : nullptr);
     if (s != DP_OK) return s;
   }

@@ -187,7 +187,7 @@ def norms_phase(ds: DeviceStep, stream=None, after_first_launch=None) -> None:
         dp.dp_vector_norms(ds.vectors, ds.B, ds.T, ds.sq, ws=ds.ws, stream=stream)
     dp.dp_embed_norms(ds.ids, ds.G_emb, ds.V, ds.sq, ws=ds.ws, dev_status=ds.dev_status, stream=stream)
     if ds.positions:
-        dp.dp_embed_norms(ds.pos_ids, ds.G_emb, ds.T, ds.sq, ws=ds.ws, dev_status=ds.dev_status,
+        dp.dp_embed_norms(ds.pos_ids, ds.G_emb, WPE_ROWS, ds.sq, ws=ds.ws, dev_status=ds.dev_status,
                           stream=stream)
     if ds.tied:
         dp.dp_tied_cross_term(ds.ids, ds.G_emb, ds.lm.A, ds.lm.G, ds.V, sq=ds.sq, cross=ds.cross,

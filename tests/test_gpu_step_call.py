@@ -84,3 +84,38 @@ def test_unsupported_and_clashing_dtypes_are_refused():
             pipeline.dp_step(ds)
         assert e.value.status == 1
         torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("overlap", [False, True])
+def test_positions_beyond_the_sequence_length_count_in_the_norm(overlap):
+    """Offset (packed, left-padded) positions: rows of the table that the sum receives belong to the norm as well."""
+    B, T, d = 3, 40, 64
+    first = torch.tensor([0, 100, 1024 - T], dtype=torch.int32, device="cuda")
+    pos = (first[:, None] + torch.arange(T, dtype=torch.int32, device="cuda")).contiguous()
+    ds = make_step(B=B, T=T, d=d, positions=True, pos_ids=pos)
+    plain = make_step(B=B, T=T, d=d)                  # the same inputs without the position table
+    pipeline.dp_step(plain, noise=False, overlap=False)
+    pipeline.dp_step(ds, noise=False, overlap=overlap)
+    torch.cuda.synchronize()
+    assert int(ds.dev_status.item()) == 0
+    rows = ds.G_emb.double()                          # every position is its own row: the norm of its gradient
+    want = plain.sq.double() + (rows ** 2).sum((1, 2))
+    assert ((ds.sq.double() / want - 1).abs() < 1e-5).all()
+    table = torch.zeros(1024, d, dtype=torch.float64, device="cuda")
+    table.index_add_(0, pos.flatten().long(), (rows * ds.clip.double()[:, None, None]).reshape(-1, d))
+    assert float((ds.outs["wpe"].double() - table).norm() / table.norm()) < 1e-6
+
+
+def test_position_outside_the_table_is_flagged_and_skipped_by_both():
+    pos = torch.arange(40, dtype=torch.int32, device="cuda").repeat(3, 1).contiguous()
+    pos[1, 7], pos[2, 0] = 1024, -1
+    ds = make_step(positions=True, pos_ids=pos)
+    plain = make_step()
+    pipeline.dp_step(plain, noise=False)
+    pipeline.dp_step(ds, noise=False)
+    torch.cuda.synchronize()
+    assert int(ds.dev_status.item()) == dp.DP_DEV_BAD_ID
+    rows = ds.G_emb.double()
+    inside = ((pos >= 0) & (pos < 1024)).double()
+    want = plain.sq.double() + (rows ** 2 * inside[:, :, None]).sum((1, 2))
+    assert ((ds.sq.double() / want - 1).abs() < 1e-5).all()
