@@ -11,11 +11,17 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <cstring>
+#include <exception>
+#include <memory>
 #include <vector>
 
 #include "../../include/dp_ghost.h"
 
 namespace {
+
+// an owned reference, released also where torch throws
+struct Decref { void operator()(PyObject* o) const { Py_DECREF(o); } };
+using Ref = std::unique_ptr<PyObject, Decref>;
 
 // dp_dtype of a tensor, kOther if it has none; *kind: that of the tensors seen before, kNone at first
 constexpr int32_t kNone = -1, kOther = -2;
@@ -46,20 +52,17 @@ bool rows(PyObject* o, const void** ptr, int64_t* ld, int64_t* cols, int32_t* ki
 
 // integer attribute; None gives `otherwise`
 bool integer(PyObject* o, const char* name, int64_t otherwise, int64_t* out) {
-  PyObject* v = PyObject_GetAttrString(o, name);
+  const Ref v(PyObject_GetAttrString(o, name));
   if (!v) { PyErr_Clear(); return false; }
-  *out = v == Py_None ? otherwise : PyLong_AsLongLong(v);
-  Py_DECREF(v);
+  *out = v.get() == Py_None ? otherwise : PyLong_AsLongLong(v.get());
   if (PyErr_Occurred()) { PyErr_Clear(); return false; }
   return true;
 }
 
 bool attr_rows(PyObject* o, const char* name, const void** ptr, int64_t* ld, int64_t* cols, int32_t* kind) {
-  PyObject* v = PyObject_GetAttrString(o, name);
+  const Ref v(PyObject_GetAttrString(o, name));
   if (!v) { PyErr_Clear(); return false; }
-  const bool ok = rows(v, ptr, ld, cols, kind);
-  Py_DECREF(v);
-  return ok;
+  return rows(v.get(), ptr, ld, cols, kind);
 }
 
 bool linear_record(dp_linear_desc& L, PyObject* o, int32_t* kind) {
@@ -73,10 +76,9 @@ bool linear_record(dp_linear_desc& L, PyObject* o, int32_t* kind) {
 bool vector_record(dp_vector_desc& v, PyObject* o, int32_t* kind) {
   int64_t cols = 0, other = 0, p = 0;
   bool ok = attr_rows(o, "G", &v.G, &v.ldg, &cols, kind) && integer(o, "p", cols, &p);
-  PyObject* x = PyObject_GetAttrString(o, "X");
+  const Ref x(PyObject_GetAttrString(o, "X"));
   if (!x) { PyErr_Clear(); return false; }
-  if (x != Py_None) ok = ok && rows(x, &v.X, &v.ldx, &other, kind);
-  Py_DECREF(x);
+  if (x.get() != Py_None) ok = ok && rows(x.get(), &v.X, &v.ldx, &other, kind);
   v.p = int32_t(p);
   return ok;
 }
@@ -85,19 +87,18 @@ bool vector_record(dp_vector_desc& v, PyObject* o, int32_t* kind) {
 // tensors are not all of one type
 template <typename Rec, typename F>
 PyObject* records(PyObject* arg, F f) {
-  PyObject* seq = PySequence_Fast(arg, "a sequence");
+  const Ref seq(PySequence_Fast(arg, "a sequence"));
   if (!seq) return nullptr;
-  const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);
-  PyObject* out = PyByteArray_FromStringAndSize(nullptr, n * Py_ssize_t(sizeof(Rec)));
-  if (!out) { Py_DECREF(seq); return nullptr; }
-  auto* rec = reinterpret_cast<Rec*>(PyByteArray_AS_STRING(out));
+  const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq.get());
+  Ref out(PyByteArray_FromStringAndSize(nullptr, n * Py_ssize_t(sizeof(Rec))));
+  if (!out) return nullptr;
+  auto* rec = reinterpret_cast<Rec*>(PyByteArray_AS_STRING(out.get()));
   memset(static_cast<void*>(rec), 0, size_t(n) * sizeof(Rec));
   bool ok = true;
   int32_t kind = kNone;
-  for (Py_ssize_t k = 0; k < n && ok; ++k) ok = f(rec[k], PySequence_Fast_GET_ITEM(seq, k), &kind);
-  Py_DECREF(seq);
-  if (!ok) { Py_DECREF(out); Py_RETURN_NONE; }
-  return out;
+  for (Py_ssize_t k = 0; k < n && ok; ++k) ok = f(rec[k], PySequence_Fast_GET_ITEM(seq.get(), k), &kind);
+  if (!ok) Py_RETURN_NONE;
+  return out.release();
 }
 
 // linears(sequence of Linear) -> dp_linear_desc[]
@@ -112,34 +113,29 @@ PyObject* vectors(PyObject*, PyObject* arg) {
 
 // outputs(sequence of CUDA tensors) -> bytearray: n pointers, then n leading strides; or None
 PyObject* outputs(PyObject*, PyObject* arg) {
-  PyObject* seq = PySequence_Fast(arg, "a sequence of tensors");
+  const Ref seq(PySequence_Fast(arg, "a sequence of tensors"));
   if (!seq) return nullptr;
-  const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);
-  PyObject* out = PyByteArray_FromStringAndSize(nullptr, 16 * n);
-  if (!out) { Py_DECREF(seq); return nullptr; }
-  auto* w = reinterpret_cast<int64_t*>(PyByteArray_AS_STRING(out));
-  bool ok = true;
+  const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq.get());
+  Ref out(PyByteArray_FromStringAndSize(nullptr, 16 * n));
+  if (!out) return nullptr;
+  auto* w = reinterpret_cast<int64_t*>(PyByteArray_AS_STRING(out.get()));
   for (Py_ssize_t k = 0; k < n; ++k) {
-    PyObject* o = PySequence_Fast_GET_ITEM(seq, k);
-    ok = THPVariable_Check(o) && THPVariable_Unpack(o).is_cuda();
-    if (!ok) break;
+    PyObject* o = PySequence_Fast_GET_ITEM(seq.get(), k);
+    if (!THPVariable_Check(o) || !THPVariable_Unpack(o).is_cuda()) Py_RETURN_NONE;
     const at::Tensor& t = THPVariable_Unpack(o);
     w[k] = reinterpret_cast<int64_t>(t.const_data_ptr());
     w[n + k] = t.dim() > 0 ? t.stride(0) : 0;
   }
-  Py_DECREF(seq);
-  if (!ok) { Py_DECREF(out); Py_RETURN_NONE; }
-  return out;
+  return out.release();
 }
 
 // f(index, object) over a sequence; false: it said no, or it is no sequence of n objects
 template <typename F>
 bool each(PyObject* arg, Py_ssize_t n, F f) {
-  PyObject* seq = PySequence_Fast(arg, "a sequence");
+  const Ref seq(PySequence_Fast(arg, "a sequence"));
   if (!seq) { PyErr_Clear(); return false; }
-  bool ok = PySequence_Fast_GET_SIZE(seq) == n;
-  for (Py_ssize_t k = 0; k < n && ok; ++k) ok = f(k, PySequence_Fast_GET_ITEM(seq, k));
-  Py_DECREF(seq);
+  bool ok = PySequence_Fast_GET_SIZE(seq.get()) == n;
+  for (Py_ssize_t k = 0; k < n && ok; ++k) ok = f(k, PySequence_Fast_GET_ITEM(seq.get(), k));
   return ok;
 }
 
@@ -249,9 +245,13 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t na) {
   S.step = uint32_t(v[11]); S.wte_id = uint32_t(v[12]); S.wpe_id = uint32_t(v[13]);
   const int32_t phases = int32_t(v[14]);
   dp_status st;
-  Py_BEGIN_ALLOW_THREADS
-  st = enqueue(&S, phases);
-  Py_END_ALLOW_THREADS
+  {
+    struct Unlocked {
+      PyThreadState* state = PyEval_SaveThread();
+      ~Unlocked() { PyEval_RestoreThread(state); }
+    } unlocked;
+    st = enqueue(&S, phases);
+  }
   if (st == DP_OK && (phases & DP_STEP_NORMS))
     each(a[1], n, [&](Py_ssize_t k, PyObject* o) {
       PyObject* m = PyLong_FromLong(layers[size_t(k)].mode_used);
@@ -263,10 +263,30 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t na) {
   return PyLong_FromLong(long(st));
 }
 
-PyMethodDef methods[] = {{"step", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(step)), METH_FASTCALL, nullptr},
-                         {"linears", linears, METH_O, nullptr},
-                         {"vectors", vectors, METH_O, nullptr},
-                         {"outputs", outputs, METH_O, nullptr},
+// What torch throws for tensors without strides or memory of their own (nested ones, those inside vmap) becomes a
+// Python exception: past the C entry it would end the process.
+template <PyObject* (*F)(PyObject*, PyObject*)>
+PyObject* guarded(PyObject* self, PyObject* arg) {
+  try {
+    return F(self, arg);
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+}
+PyObject* guarded_step(PyObject* self, PyObject* const* a, Py_ssize_t na) {
+  try {
+    return step(self, a, na);
+  } catch (const std::exception& e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
+  }
+}
+
+PyMethodDef methods[] = {{"step", reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded_step)), METH_FASTCALL, nullptr},
+                         {"linears", guarded<linears>, METH_O, nullptr},
+                         {"vectors", guarded<vectors>, METH_O, nullptr},
+                         {"outputs", guarded<outputs>, METH_O, nullptr},
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
