@@ -13,6 +13,7 @@
 #include <cstring>
 #include <exception>
 #include <memory>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/dp_ghost.h"
@@ -123,7 +124,7 @@ PyObject* outputs(PyObject*, PyObject* arg) {
     PyObject* o = PySequence_Fast_GET_ITEM(seq.get(), k);
     if (!THPVariable_Check(o) || !THPVariable_Unpack(o).is_cuda()) Py_RETURN_NONE;
     const at::Tensor& t = THPVariable_Unpack(o);
-    w[k] = reinterpret_cast<int64_t>(t.const_data_ptr());
+    w[k] = reinterpret_cast<int64_t>(t.mutable_data_ptr());
     w[n + k] = t.dim() > 0 ? t.stride(0) : 0;
   }
   return out.release();
@@ -148,8 +149,14 @@ bool device_tensor(PyObject* o, const at::Tensor** t) {
   return (*t)->is_cuda();
 }
 
+// address to read from (P const) or to write to: a tensor that shares its memory until it is written to
+// (copy-on-write) gets its own first
 template <typename P>
-P* pointer(const at::Tensor* t) { return t ? const_cast<P*>(static_cast<const P*>(t->const_data_ptr())) : nullptr; }
+P* pointer(const at::Tensor* t) {
+  if (!t) return nullptr;
+  if constexpr (std::is_const_v<P>) return static_cast<P*>(t->const_data_ptr());
+  else return static_cast<P*>(t->mutable_data_ptr());
+}
 
 bool output_list(PyObject* arg, Py_ssize_t n, std::vector<float*>& ptr, std::vector<int64_t>& ld) {
   ptr.resize(size_t(n)); ld.resize(size_t(n));
@@ -221,8 +228,8 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t na) {
   S.tensor_ids = ids.data();
   if (nv) { S.vectors = vectors.data(); S.vector_outs = vouts.data(); }
   S.vector_ids = vids.data();
-  S.ids = pointer<int32_t>(t[IDS]); S.G_emb = g; S.ldge = ldg;
-  S.pos_ids = pointer<int32_t>(t[POS_IDS]);
+  S.ids = pointer<const int32_t>(t[IDS]); S.G_emb = g; S.ldge = ldg;
+  S.pos_ids = pointer<const int32_t>(t[POS_IDS]);
   S.wte = pointer<float>(t[WTE]); S.ld_wte = t[WTE]->stride(0);
   S.wpe = pointer<float>(t[WPE]); S.ld_wpe = t[WPE] ? t[WPE]->stride(0) : 0;
   S.sq = pointer<float>(t[SQ]); S.clip = pointer<float>(t[CLIP]); S.norms = pointer<float>(t[NORMS]);

@@ -119,3 +119,24 @@ def test_position_outside_the_table_is_flagged_and_skipped_by_both():
     inside = ((pos >= 0) & (pos < 1024)).double()
     want = plain.sq.double() + (rows ** 2 * inside[:, :, None]).sum((1, 2))
     assert ((ds.sq.double() / want - 1).abs() < 1e-5).all()
+
+
+def test_copy_on_write_outputs_are_written_apart():
+    """A lazy clone shares memory until it is written to; the library's writes count."""
+    ds = make_step()
+    pipeline.dp_step(ds, noise=False)
+    want = state(ds)
+    wipe(ds)
+    kept = {n: ds.outs[n] for n in ("linear0", "wte", "vector0")}
+    for n, t in kept.items():
+        ds.outs[n] = torch._lazy_clone(t)
+    pipeline.dp_step(ds, noise=False)
+    assert_same(state(ds), want)
+    for n, t in kept.items():
+        assert (t == 9.0).all(), n
+    for n, t in kept.items():
+        ds.outs[n] = torch._lazy_clone(t)
+    pipeline.dp_step(ds, noise=False, overlap=False)      # call by call: lists of outputs
+    assert_same(state(ds), want)
+    for n, t in kept.items():
+        assert (t == 9.0).all(), n
