@@ -317,7 +317,7 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
  * dp_embed_norms_ws_bytes more per table one kernel adds up all the norms' partial sums).  events: four
  * cudaEvent_t of the caller that order the two streams; `stream` has waited for `side_stream` at the
  * end.  phases: DP_STEP_ALL, or the three phases one after the other with the same descriptor (so
- * that a caller can time them). */
+ * that a caller can time them, or change the clip factors on `stream` before the second). */
 size_t dp_step_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B, int32_t T);
 enum { DP_STEP_NORMS = 1, DP_STEP_GEMM = 2, DP_STEP_REST = 4, DP_STEP_ALL = 7 };
 typedef struct {

@@ -1029,7 +1029,8 @@ static dp_status start_table(const dp_step_desc* S, float* table, int64_t ld, in
   return DP_OK;
 }
 
-// events: [0] the step began, [1] embedding norms done, [2] row sums done, [3] clip factors exist
+// events: [0] the step began, [1] embedding norms done, [2] row sums done, [3] clip factors exist (as the clipped sums
+// take them)
 static dp_status step_norms(const dp_step_desc* S, const GhostPlan& plan, SplitGroup* kept) {
   cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
   const dp_dtype embed_dt = (dp_dtype)S->embed_dtype;
@@ -1177,6 +1178,9 @@ dp_status dp_step_enqueue(const dp_step_desc* S, int32_t phases) {
   SplitGroup split;
   SplitGroup* kept = phases == DP_STEP_ALL && S->layer_dtype == DP_F32 ? &split : nullptr;
   if (phases & DP_STEP_NORMS) s = step_norms(S, plan, kept);
+  // a call of its own: what `stream` did in between (other clip factors, say) comes before the row sums as well
+  if ((phases & (DP_STEP_NORMS | DP_STEP_GEMM)) == DP_STEP_GEMM)
+    DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[3], (cudaStream_t)S->stream));
   if (s == DP_OK && (phases & DP_STEP_GEMM)) s = step_gemm(S, kept);
   if (s == DP_OK && (phases & DP_STEP_REST)) s = step_rest(S);
   if (s != DP_OK) {

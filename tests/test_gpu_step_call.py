@@ -140,3 +140,21 @@ def test_copy_on_write_outputs_are_written_apart():
     assert_same(state(ds), want)
     for n, t in kept.items():
         assert (t == 9.0).all(), n
+
+
+def test_clip_factors_changed_between_the_phases_reach_the_row_sums():
+    """Work on the caller's stream between the norms and the sums is ordered before all sums, those of the side stream
+    too: here the factors change 50 ms later."""
+    ds = make_step(positions=True)
+    step = dict(seed=3, step=2)
+    pipeline.clip_after_prefill(ds, **step, filled=pipeline.overlapped_norms(ds, **step))     # a kernel's first launch waits
+    filled = pipeline.overlapped_norms(ds, **step)
+    torch.cuda._sleep(100_000_000)
+    ds.clip.fill_(0.25)
+    pipeline.clip_after_prefill(ds, **step, filled=filled)
+    torch.cuda.synchronize()
+    for name, ids in (("wte", ds.ids), ("wpe", ds.pos_ids)):
+        noise = torch.empty_like(ds.outs[name])
+        dp.dp_fill_noise(noise, ds.sigma, ds.C, 1.0, 3, pipeline.tensor_ids(ds)[name], 2)
+        want = noise.double().index_add_(0, ids.flatten().long(), 0.25 * ds.G_emb.double().reshape(-1, ds.d_model))
+        assert float((ds.outs[name].double() - want).norm() / want.norm()) < 1e-6, name
