@@ -393,10 +393,13 @@ def _enqueue(ds: DeviceStep, seed: int, step: int, phases: int, noise: bool = Tr
 def overlapped_norms(ds: DeviceStep, seed: int, step: int) -> torch.cuda.Event:
     """Norm phase with everything that does not need the big norm kernel running BESIDE it on a
     side stream: the embedding norms, the token sorts of the scatter (they need only the ids) and
-    the embedding tables' noise (ALU-bound, depends on no gradient).  clip_after_prefill completes
-    the step; it takes the returned event (the clip factors exist)."""
+    the embedding tables' noise (ALU-bound, depends on no gradient).  The clip factors exist on the
+    current stream.  Returns the event after which the tables hold their noise and the sorts exist;
+    clip_after_prefill completes the step with it."""
     _enqueue(ds, seed, step, dp.STEP_NORMS)
-    return ds.side["events"][3]
+    filled = torch.cuda.Event()
+    filled.record(ds.side_stream)
+    return filled
 
 
 def clip_after_prefill(ds: DeviceStep, seed: int, step: int, filled: torch.cuda.Event,
@@ -406,12 +409,13 @@ def clip_after_prefill(ds: DeviceStep, seed: int, step: int, filled: torch.cuda.
     if scale != 1.0:
         raise ValueError("the overlapped step draws its noise at scale 1")
     cur = torch.cuda.current_stream()
-    cur.wait_event(filled)
     if gemm_events:
         gemm_events[0].record(cur)
     _enqueue(ds, seed, step, dp.STEP_GEMM)
     if gemm_events:
         gemm_events[1].record(cur)
+    cur.wait_event(filled)                   # the GEMM need not wait for the tables, their row sums do
+    ds.side_stream.wait_event(filled)
     _enqueue(ds, seed, step, dp.STEP_REST)
 
 

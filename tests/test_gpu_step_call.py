@@ -158,3 +158,33 @@ def test_clip_factors_changed_between_the_phases_reach_the_row_sums():
         dp.dp_fill_noise(noise, ds.sigma, ds.C, 1.0, 3, pipeline.tensor_ids(ds)[name], 2)
         want = noise.double().index_add_(0, ids.flatten().long(), 0.25 * ds.G_emb.double().reshape(-1, ds.d_model))
         assert float((ds.outs[name].double() - want).norm() / want.norm()) < 1e-6, name
+
+
+def test_event_of_the_overlapped_norms_orders_the_tables_and_sorts():
+    """A third stream that waits for it sees the table's noise and the sort, not what was there before."""
+    ds = make_step(V=200000, d=768, B=4, lm=False)        # the fill outlasts the norms
+    step = dict(seed=3, step=2)
+    pipeline.clip_after_prefill(ds, **step, filled=pipeline.overlapped_norms(ds, **step))
+    want = state(ds)
+    noise = torch.empty_like(ds.outs["wte"])
+    dp.dp_fill_noise(noise, ds.sigma, ds.C, 1.0, 3, pipeline.tensor_ids(ds)["wte"], 2)
+    parts = [ds.side["perm"], ds.side["seg"], ds.outs["wte"][-20000:]]       # the fill's last rows
+    expected = [parts[0].cpu(), parts[1].cpu(), noise[-20000:].cpu()]
+    seen = [torch.empty(p.shape, dtype=p.dtype, pin_memory=True) for p in parts]
+    other = torch.cuda.Stream()
+    for _ in range(5):
+        wipe(ds)
+        for p in parts[:2]:
+            p.fill_(-1)
+        torch.cuda.synchronize()
+        filled = pipeline.overlapped_norms(ds, **step)
+        other.wait_event(filled)
+        with torch.cuda.stream(other):
+            for s, p in zip(reversed(seen), reversed(parts)):    # the copy engine's work: no kernel, which would have to
+                s.copy_(p, non_blocking=True)                    # wait until the fill leaves it room
+        torch.cuda.current_stream().wait_stream(other)
+        pipeline.clip_after_prefill(ds, **step, filled=filled)
+        torch.cuda.synchronize()
+        for s, e in zip(seen, expected):
+            assert torch.equal(s, e)
+        assert_same(state(ds), want)
