@@ -308,6 +308,29 @@ def clip_noise_phase(ds: DeviceStep, seed: int, step: int, scale: float = 1.0, s
     _clip_vectors(ds, 0.0, noise=(seed, step, scale), stream=stream)
 
 
+def prefill_embedding_noise(ds: DeviceStep, seed: int, step: int, scale: float = 1.0,
+                            after: Optional[torch.cuda.Event] = None) -> torch.cuda.Event:
+    """Start the noise fill of the embedding tables on the side stream; returns the event to wait for.
+    (overlapped_norms starts it by itself, at scale 1.)
+    after: event that orders the fill behind the previous users of the tables (default: all
+    work enqueued so far on the current stream)."""
+    if ds.side_stream is None:
+        ds.side_stream = torch.cuda.Stream(device=ds.sq.device)
+    side, tid = ds.side_stream, tensor_ids(ds)
+    if after is not None:
+        side.wait_event(after)
+    else:
+        side.wait_stream(torch.cuda.current_stream())
+    names = ["wpe"] if ds.positions else []
+    if not (ds.tied and ds.lm is not None):
+        names.append("wte")                      # tied: the head GEMM writes the table first
+    for name in names:
+        dp.dp_fill_noise(ds.outs[name], ds.sigma, ds.C, scale, seed, tid[name], step, stream=side)
+    ev = torch.cuda.Event()
+    ev.record(side)
+    return ev
+
+
 def prefill_all_noise(ds: DeviceStep, seed: int, step: int) -> torch.cuda.Event:
     """Fill EVERY output tensor with its noise on the side stream (scale 1).  The fills are
     ALU-bound and depend on no gradient, the norm phase is HBM-bound: they share the SMs."""
@@ -405,10 +428,12 @@ def overlapped_norms(ds: DeviceStep, seed: int, step: int) -> torch.cuda.Event:
 def clip_after_prefill(ds: DeviceStep, seed: int, step: int, filled: torch.cuda.Event,
                        scale: float = 1.0, gemm_events=None) -> None:
     """Clipped sums after overlapped_norms (the tables hold their noise, the sorts exist).
+    scale: of the layers' and vectors' sums and noise; rows are added to the tables as they are.
     gemm_events: optional (start, stop) CUDA events recorded around the grouped GEMM call."""
-    if scale != 1.0:
-        raise ValueError("the overlapped step draws its noise at scale 1")
     cur = torch.cuda.current_stream()
+    if scale != 1.0:
+        _clip_after_prefill_scaled(ds, seed, step, filled, scale, gemm_events)
+        return
     if gemm_events:
         gemm_events[0].record(cur)
     _enqueue(ds, seed, step, dp.STEP_GEMM)
@@ -417,6 +442,30 @@ def clip_after_prefill(ds: DeviceStep, seed: int, step: int, filled: torch.cuda.
     cur.wait_event(filled)                   # the GEMM need not wait for the tables, their row sums do
     ds.side_stream.wait_event(filled)
     _enqueue(ds, seed, step, dp.STEP_REST)
+
+
+def _clip_after_prefill_scaled(ds: DeviceStep, seed: int, step: int, filled, scale: float, gemm_events) -> None:
+    """The same call by call: the one-call form draws its noise at scale 1."""
+    cur, sb, tid = torch.cuda.current_stream(), _side_buffers(ds), tensor_ids(ds)
+    kw = dict(ws=ds.ws, dev_status=ds.dev_status, clip=ds.clip)
+    layers = ds.linears + ([ds.lm] if ds.lm is not None else [])
+    names = [f"linear{k}" for k in range(len(ds.linears))]
+    if ds.lm is not None:
+        names.append("wte" if ds.tied else "lm_head")
+    if layers:
+        if gemm_events:
+            gemm_events[0].record(cur)
+        dp.dp_clip_accumulate_noise_grouped(layers, ds.B, ds.T, None, ds.C, [ds.outs[n] for n in names], ds.sigma,
+                                            scale, seed, [tid[n] for n in names], step, beta=0.0, **kw)
+        if gemm_events:
+            gemm_events[1].record(cur)
+    cur.wait_event(filled)
+    dp.dp_clip_accumulate_embed_sorted(ds.ids, ds.G_emb, ds.V, None, ds.C, ds.outs["wte"], sb["perm"], sb["seg"],
+                                       beta=1.0, d=ds.d_model, **kw)
+    if ds.positions:
+        dp.dp_clip_accumulate_embed_sorted(ds.pos_ids, ds.G_emb, WPE_ROWS, None, ds.C, ds.outs["wpe"], sb["pos_perm"],
+                                           sb["pos_seg"], beta=1.0, d=ds.d_model, **kw)
+    _clip_vectors(ds, 0.0, noise=(seed, step, scale), factors=True)
 
 
 def dp_step(ds: DeviceStep, seed: int = 0, step: int = 0, noise: bool = True, fused: bool = True,

@@ -188,3 +188,33 @@ def test_event_of_the_overlapped_norms_orders_the_tables_and_sorts():
         for s, e in zip(seen, expected):
             assert torch.equal(s, e)
         assert_same(state(ds), want)
+
+
+@pytest.mark.parametrize("tied", [False, True])
+def test_prefill_and_scale_of_the_overlapped_step(tied):
+    """Tables filled at a scale of the caller's; layers and vectors scaled by clip_after_prefill."""
+    step, scale = dict(seed=3, step=2), 0.25
+    ds = make_step(tied=tied, positions=True)
+    tid = pipeline.tensor_ids(ds)
+    pipeline.dp_step(ds, **step, noise=False)
+    sums = state(ds)
+    rows = torch.zeros_like(ds.outs["wte"])
+    dp.dp_clip_accumulate_embed(ds.ids, ds.G_emb, ds.V, None, ds.C, rows, d=ds.d_model, clip=ds.clip)
+    wipe(ds)
+    pipeline.overlapped_norms(ds, **step)
+    filled = pipeline.prefill_embedding_noise(ds, **step, scale=scale)
+    pipeline.clip_after_prefill(ds, **step, filled=filled, scale=scale)
+    got = state(ds)
+    for name in ds.outs:
+        want = torch.zeros_like(got[name])
+        if name in ("wte", "wpe") and not (tied and name == "wte"):
+            dp.dp_fill_noise(want, ds.sigma, ds.C, scale, 3, tid[name], 2)
+            want += sums[name]
+        elif name == "wte":                              # head's sum and noise, scaled; the rows as they are
+            want = sums[name] - rows
+            dp.dp_add_noise(want, ds.sigma, ds.C, scale, 3, tid[name], 2)
+            want += rows
+        else:
+            want = sums[name].clone()
+            dp.dp_add_noise(want, ds.sigma, ds.C, scale, 3, tid[name], 2)
+        assert float((got[name] - want).norm()) < 1e-5 * float(want.norm()), name
