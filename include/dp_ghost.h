@@ -307,7 +307,7 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
  * dp_clip_accumulate_noise_grouped (tied: the head's out is wte).  vectors, vector_outs, vector_ids
  * as in dp_clip_accumulate_vectors.  layer_dtype, vector_dtype, embed_dtype: the storage types of the
  * layers' A and G, the vectors' G and X, and G_emb (tied: that of the layers, since the cross term takes
- * one type).  pos_ids [dev, (B, T)]: rows of wpe, below pos_rows; NULL: no position table.  with_noise 0: the bare clipped sums.  sq, clip [dev, B] and norms, cross [dev, B or NULL; cross is needed when tied] are
+ * one type).  pos_ids [dev, (B, T)]: rows of wpe, below pos_rows; NULL: no position table.  with_noise 0: the bare clipped sums.  sq, clip [dev, B] and norms, cross [dev, B or NULL] are
  * overwritten; side_sq [dev, B], perm / seg and pos_perm / pos_seg [dev, as in dp_embed_sort] are
  * scratch, as are ws (the largest *_ws_bytes of the calls on `stream`, dp_step_ws_bytes if fp32 layers
  * are to be split once instead of for the norms and again for the sums, and the norms of short ones to

@@ -969,7 +969,7 @@ static dp_status check_step(const dp_step_desc* S, int32_t phases, GhostPlan* pl
     return DP_ERR_INVALID_ARG;
   if (S->n_layers && (!S->layers || !S->outs || !S->ldos || (S->with_noise && !S->tensor_ids)))
     return DP_ERR_INVALID_ARG;
-  if (S->tied && (S->n_layers == 0 || !S->cross)) return DP_ERR_INVALID_ARG;
+  if (S->tied && S->n_layers == 0) return DP_ERR_INVALID_ARG;
   auto dtype_ok = [](int32_t t) { return t == DP_F32 || t == DP_BF16; };
   if (!dtype_ok(S->layer_dtype) || !dtype_ok(S->vector_dtype) || !dtype_ok(S->embed_dtype)) return DP_ERR_INVALID_ARG;
   if (S->tied && S->embed_dtype != S->layer_dtype) return DP_ERR_INVALID_ARG;      // one type in the cross term

@@ -218,3 +218,15 @@ def test_prefill_and_scale_of_the_overlapped_step(tied):
             want = sums[name].clone()
             dp.dp_add_noise(want, ds.sigma, ds.C, scale, 3, tid[name], 2)
         assert float((got[name] - want).norm()) < 1e-5 * float(want.norm()), name
+
+
+def test_tied_step_without_a_place_for_the_cross_term():
+    ds = make_step(tied=True)
+    pipeline.dp_step(ds, noise=False)
+    want = state(ds)
+    ds.cross = ds.norms = None
+    wipe(ds)
+    pipeline.dp_step(ds, noise=False)
+    got = state(ds)
+    for n, t in want.items():
+        assert torch.equal(got[n], t), n

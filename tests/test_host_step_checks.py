@@ -70,6 +70,14 @@ def test_a_sound_step_reaches_the_runtime(lib):
             assert call(lib, desc(dtype, tied=tied)) == CUDA
 
 
+def test_what_may_be_left_out(lib):
+    S = desc(tied=True)
+    S.norms = S.cross = S.dev_status = S.pos_ids = S.wpe = S.pos_perm = S.pos_seg = None
+    S.n_vectors, S.vectors, S.vector_outs, S.vector_ids = 0, None, None, None
+    S.with_noise, S.tensor_ids = 0, None
+    assert call(lib, S) == CUDA
+
+
 def spoil(S, what):
     if what == "T":
         S.T = 4097
