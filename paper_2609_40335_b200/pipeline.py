@@ -146,8 +146,12 @@ def allocate(ds: DeviceStep) -> None:
         ds.outs["wpe"] = torch.empty(WPE_ROWS, ds.d_model, **f32)
     for k, v in enumerate(ds.vectors):
         ds.outs[f"vector{k}"] = torch.empty(v.p, **f32)
+    ds.ws = torch.empty(_ws_bytes(ds), dtype=torch.uint8, device=dev)
+
+
+def _ws_bytes(ds: DeviceStep) -> int:
+    """Workspace large enough for every call of a step."""
     every = ds.linears + ([ds.lm] if ds.lm else [])
-    dt = dp._dt(every[0].A) if every else dp._dt(ds.G_emb)
     need = 256
     if every:
         need = max(need, dp.dp_ghost_norms_ws_bytes(every, ds.B, ds.T))
@@ -170,7 +174,7 @@ def allocate(ds: DeviceStep) -> None:
             if ds.tied:
                 once += int(L.dp_tied_cross_term_ws_bytes(ds.B, ds.T, ds.d_model, ds.V))
         need = max(need, once)
-    ds.ws = torch.empty(need, dtype=torch.uint8, device=dev)
+    return need
 
 
 def norms_phase(ds: DeviceStep, stream=None, after_first_launch=None) -> None:
@@ -402,12 +406,15 @@ def _enqueue(ds: DeviceStep, seed: int, step: int, phases: int, noise: bool = Tr
         layers = layers + [ds.lm]
         names.append("wte" if ds.tied else "lm_head")
     tid = tensor_ids(ds)
+    ws = ds.ws
+    if ws is None:                       # none allocated: one for this call (it is used on the current stream only)
+        ws = torch.empty(_ws_bytes(ds), dtype=torch.uint8, device=ds.sq.device)
     dp.dp_step_enqueue(
         layers, [outs[n] for n in names], [tid[n] for n in names], ds.vectors, [outs[n] for n in vnames],
         [tid[n] for n in vnames], ids=ds.ids, G_emb=ds.G_emb, pos_ids=ds.pos_ids if ds.positions else None,
         wte=outs["wte"], wpe=outs["wpe"] if ds.positions else None, sq=ds.sq, clip=ds.clip, norms=ds.norms,
         cross=ds.cross, side_sq=sb["sq"], perm=sb["perm"], seg=sb["seg"], pos_perm=sb["pos_perm"],
-        pos_seg=sb["pos_seg"], ws=ds.ws, side_ws=sb["ws"], dev_status=ds.dev_status, stream=None,
+        pos_seg=sb["pos_seg"], ws=ws, side_ws=sb["ws"], dev_status=ds.dev_status, stream=None,
         side_stream=ds.side_stream, events=[e.cuda_event for e in sb["events"]], V=ds.V, d=ds.d_model,
         tied=ds.tied and ds.lm is not None, noise=noise, C_=ds.C, sigma=ds.sigma, seed=seed, step=step,
         wte_id=tid["wte"], wpe_id=tid["wpe"] if ds.positions else 0, phases=phases)

@@ -230,3 +230,20 @@ def test_tied_step_without_a_place_for_the_cross_term():
     got = state(ds)
     for n, t in want.items():
         assert torch.equal(got[n], t), n
+
+
+@pytest.mark.parametrize("dtype", [BF16, F32])
+def test_step_without_a_workspace_of_its_own(dtype):
+    """A DeviceStep whose user gave it outputs but no workspace."""
+    ds = make_step(dtype, dtype, dtype, tied=True, positions=True)
+    pipeline.dp_step(ds, seed=3, step=2)
+    want = state(ds)
+    ds.ws = None
+    for by_phases in (False, True):
+        wipe(ds)
+        if by_phases:
+            pipeline.clip_after_prefill(ds, seed=3, step=2, filled=pipeline.overlapped_norms(ds, seed=3, step=2))
+        else:
+            pipeline.dp_step(ds, seed=3, step=2)
+        assert_same(state(ds), want)
+        assert ds.ws is None
