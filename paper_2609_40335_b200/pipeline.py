@@ -133,8 +133,11 @@ def synthesize_on_device(name: str, B: int, T: int, d_model: int, n_blocks: int,
     return ds
 
 
-def allocate(ds: DeviceStep) -> None:
-    """Output tensors (one per parameter tensor) and one workspace large enough for every call."""
+def allocate(ds: DeviceStep, split_once: bool = True) -> None:
+    """Output tensors (one per parameter tensor) and one workspace large enough for every call.
+    split_once: of fp32 layers, room for the split operands of all of them (as large as the inputs, up to
+    16 GiB), so that a step splits them once; without it, or where that much is not free, for those of the
+    largest layer three times over."""
     dev = ds.sq.device
     f32 = dict(dtype=torch.float32, device=dev)
     for k, l in enumerate(ds.linears):
@@ -146,11 +149,17 @@ def allocate(ds: DeviceStep) -> None:
         ds.outs["wpe"] = torch.empty(WPE_ROWS, ds.d_model, **f32)
     for k, v in enumerate(ds.vectors):
         ds.outs[f"vector{k}"] = torch.empty(v.p, **f32)
-    ds.ws = torch.empty(_ws_bytes(ds), dtype=torch.uint8, device=dev)
+    least, need = _ws_bytes(ds, False), _ws_bytes(ds, split_once)
+    try:
+        ds.ws = torch.empty(need, dtype=torch.uint8, device=dev)
+    except torch.cuda.OutOfMemoryError:
+        if need == least:
+            raise
+        ds.ws = torch.empty(least, dtype=torch.uint8, device=dev)
 
 
-def _ws_bytes(ds: DeviceStep) -> int:
-    """Workspace large enough for every call of a step."""
+def _ws_bytes(ds: DeviceStep, split_once: bool) -> int:
+    """Workspace large enough for every call of a step (split_once: see allocate)."""
     every = ds.linears + ([ds.lm] if ds.lm else [])
     need = 256
     if every:
@@ -166,7 +175,7 @@ def _ws_bytes(ds: DeviceStep) -> int:
         need = max(need, int(L.dp_clip_accumulate_embed_ws_bytes(ds.B, ds.T, ds.d_model, WPE_ROWS)))
     if ds.tied:
         need = max(need, int(L.dp_tied_cross_term_ws_bytes(ds.B, ds.T, ds.d_model, ds.V)))
-    if every:
+    if every and split_once:
         once = dp.dp_step_ws_bytes(every, ds.B, ds.T)
         if once:                      # the norms' partial sums of vectors and cross term lie behind it
             if ds.vectors:
@@ -408,7 +417,7 @@ def _enqueue(ds: DeviceStep, seed: int, step: int, phases: int, noise: bool = Tr
     tid = tensor_ids(ds)
     ws = ds.ws
     if ws is None:                       # none allocated: one for this call (it is used on the current stream only)
-        ws = torch.empty(_ws_bytes(ds), dtype=torch.uint8, device=ds.sq.device)
+        ws = torch.empty(_ws_bytes(ds, False), dtype=torch.uint8, device=ds.sq.device)
     dp.dp_step_enqueue(
         layers, [outs[n] for n in names], [tid[n] for n in names], ds.vectors, [outs[n] for n in vnames],
         [tid[n] for n in vnames], ids=ds.ids, G_emb=ds.G_emb, pos_ids=ds.pos_ids if ds.positions else None,

@@ -247,3 +247,28 @@ def test_step_without_a_workspace_of_its_own(dtype):
             pipeline.dp_step(ds, seed=3, step=2)
         assert_same(state(ds), want)
         assert ds.ws is None
+
+
+def test_fp32_step_in_the_least_memory(monkeypatch):
+    """By request, and where the large workspace does not fit."""
+    ds = make_step(F32, F32, F32)
+    pipeline.dp_step(ds, noise=False)
+    want, large = state(ds), ds.ws.numel()
+    every = ds.linears + [ds.lm]
+    pipeline.allocate(ds, split_once=False)
+    small = ds.ws.numel()
+    lib = dp.load()
+    assert small == max(dp.dp_ghost_norms_ws_bytes(every, ds.B, ds.T), dp.dp_clip_accumulate_grouped_ws_bytes(every, ds.B, ds.T),
+                        int(lib.dp_clip_accumulate_embed_ws_bytes(ds.B, ds.T, ds.d_model, ds.V))) < large
+    pipeline.dp_step(ds, noise=False)
+    assert_same(state(ds), want)
+    empty = torch.empty
+
+    def full(*size, **kw):
+        if kw.get("dtype") == torch.uint8 and size[0] > small:
+            raise torch.cuda.OutOfMemoryError("no room")
+        return empty(*size, **kw)
+
+    monkeypatch.setattr(torch, "empty", full)
+    pipeline.allocate(ds)
+    assert ds.ws.numel() == small
