@@ -207,6 +207,9 @@ def _marshal():
             from . import _marshal as m
         except ImportError as e:
             raise DpGhostError(-1, "load", f"{e}: build the package first; there is no fallback") from e
+        if m.torch_version != torch.__version__:           # another C++ interface: tensors would be misread
+            raise DpGhostError(-1, "load", f"_marshal.so was built for torch {m.torch_version}, this is {torch.__version__}: "
+                                           "build the package again")
         _native = m
     return _native
 

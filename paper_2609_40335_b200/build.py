@@ -23,6 +23,7 @@ OBJ_DIR = os.path.join(HERE, "build")
 LIB_PATH = os.path.join(HERE, "libdp_ghost.so")
 CHECK_LIB_PATH = os.path.join(HERE, "libdp_ghost_check.so")
 MARSHAL_PATH = os.path.join(HERE, "_marshal.so")
+MARSHAL_STAMP = os.path.join(OBJ_DIR, "marshal.stamp")       # what _marshal.so was compiled with
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC"]
 
@@ -86,24 +87,32 @@ def build(force: bool = False, verbose: bool = False, check: bool = False) -> st
 
 
 def build_marshal(force: bool = False) -> str:
-    """Compile the extension that reads the tensors of a call (see csrc/marshal.cpp)."""
+    """Compile the extension that reads the tensors of a call (see csrc/marshal.cpp).  It belongs to the torch and
+    the Python it was compiled against: another one of either, or another command, makes it stale as well."""
     import sysconfig
 
     import torch
     root = os.path.dirname(torch.__file__)
     src = os.path.join(CSRC, "marshal.cpp")
     header = os.path.join(os.path.dirname(HERE), "include", "dp_ghost.h")
-    if force or _stale(MARSHAL_PATH, [src, header]):
-        lib = os.path.join(root, "lib")
-        cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
-               f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
-               "-I" + os.path.join(root, "include"), "-I" + sysconfig.get_paths()["include"],
-               "-I" + os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"), src, "-o", MARSHAL_PATH,
-               "-L" + lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath," + lib]
-        r = subprocess.run(cmd, capture_output=True, text=True)
-        if r.returncode != 0:
-            sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
-            raise RuntimeError("compiling marshal.cpp failed")
+    lib = os.path.join(root, "lib")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DDP_TORCH_VERSION="{torch.__version__}"',
+           "-I" + os.path.join(root, "include"), "-I" + sysconfig.get_paths()["include"],
+           "-I" + os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"), src, "-o", MARSHAL_PATH,
+           "-L" + lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-Wl,-rpath," + lib]
+    made_by = "\n".join([sys.version, torch.__version__, *cmd])
+    if not force and not _stale(MARSHAL_PATH, [src, header]) and os.path.exists(MARSHAL_STAMP):
+        with open(MARSHAL_STAMP) as f:
+            if f.read() == made_by:
+                return MARSHAL_PATH
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
+        raise RuntimeError("compiling marshal.cpp failed")
+    os.makedirs(os.path.dirname(MARSHAL_STAMP), exist_ok=True)
+    with open(MARSHAL_STAMP, "w") as f:
+        f.write(made_by)
     return MARSHAL_PATH
 
 

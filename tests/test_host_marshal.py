@@ -3,6 +3,12 @@ the process.  They run in a process of their own, so that an abort is a failed t
 import os
 import subprocess
 import sys
+import types
+
+import pytest
+import torch
+
+from paper_2609_40335_b200 import binding, build
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -51,3 +57,30 @@ def test_tensors_without_memory_are_refused():
     r = subprocess.run([sys.executable, "-c", HEAD + CASES], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, (r.returncode, r.stdout[-500:], r.stderr[-800:])
     assert r.stdout.count("refused:") == 9
+
+
+def test_extension_of_another_torch_is_built_again_and_never_used(tmp_path, monkeypatch):
+    commands = []
+
+    def compile_(cmd, **kw):
+        commands.append(cmd)
+        open(build.MARSHAL_PATH, "w").close()
+        return types.SimpleNamespace(returncode=0, stdout="", stderr="")
+
+    monkeypatch.setattr(build, "MARSHAL_PATH", str(tmp_path / "_marshal.so"))
+    monkeypatch.setattr(build, "MARSHAL_STAMP", str(tmp_path / "build" / "marshal.stamp"))
+    monkeypatch.setattr(build.subprocess, "run", compile_)
+    for expected in (1, 1):
+        build.build_marshal()
+        assert len(commands) == expected
+    version = torch.__version__
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    build.build_marshal()
+    assert len(commands) == 2
+    monkeypatch.setattr(torch, "__version__", version)
+    monkeypatch.setattr(binding, "_native", None)
+    assert binding._marshal().torch_version == version
+    monkeypatch.setattr(binding, "_native", None)
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    with pytest.raises(binding.DpGhostError, match="built for torch"):
+        binding._marshal()
