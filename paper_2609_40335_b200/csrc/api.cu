@@ -770,10 +770,10 @@ dp_status dp_clip_accumulate(const void* A, int64_t lda, const void* G, int64_t 
 }
 
 // ------------------------------------------------------------------ clip accumulate, embedding
-// scratch of the sort: counts per id, overall and per chunk, and the ranks
+// scratch of the sort: counts per id, per 1024 ids, and per chunk and id
 static size_t sort_totals_bytes(size_t n, int V) {
   const size_t chunks = (n + kSortChunk - 1) / kSortChunk;
-  return align_up((chunks + 1) * V * sizeof(int), 256);
+  return align_up(((chunks + 1) * V + ceil_div(V, 1024)) * sizeof(int), 256);
 }
 
 static void embed_ws_layout(int B, int T, int d, int V, size_t* off_clip, size_t* off_totals,

@@ -303,16 +303,19 @@ __global__ void __launch_bounds__(kSideThreads, 16) clear_kernel(uint4* __restri
 // ------------------------------------------------------------------ sort kernels
 // Stable counting sort of the token ids: perm lists the positions by (id, position), seg[v] = number
 // of positions with id < v.
-//   up to kSortOneBlock tokens and kSortOneBlockIds ids: one kernel of one block (grouping, counts into seg, scan over V, placing);
+//   few tokens and ids (sort_in_one_block): one kernel of one block (grouping, counts into seg, scan over V, placing);
 //   more: the tokens are cut into chunks, one block each --
 //     sort_rank_kernel   groups a chunk: rank of every token inside its chunk, counts[chunk][id],
-//                        and the total of every id (integer atomics)
+//                        the total of every id and of every 1024 ids (integer atomics)
 //     sort_scan_kernel   exclusive scan of the totals -> seg
 //     sort_place_kernel  perm[seg[id] + counts of the chunks before + rank] = position
+//   with more than kSortWalk chunks sort_prefix_kernel first turns counts[chunk][id] into those of the chunks
+//   before, so that placing a token stays one read.
 // Latency again: four short dependent launches.  Against histogram, prefix over the chunks, scan and a
-// placing kernel that compared a token with all earlier ones of its chunk (V = 50257): 23.2 -> 15.9 us
-// at n = 4096, 32.8 -> 19.5 at 16384, 121 -> 41 at 131072.
+// placing kernel that compared a token with all earlier ones of its chunk (V = 50257, Zipf ids, replayed as a graph): 9.5 ->
+// 7.9 us at n = 8, 24.7 -> 18.6 at 4096, 33 -> 21 at 16384, 115 -> 34 at 131072, 6.1 -> 0.67 ms at 4 194 304.
 constexpr int kSortThreads = 1024;
+constexpr int kSortBlocksShared = 256;     // blocks of 1024 ids that a chunk counts in shared memory
 
 __device__ __forceinline__ void load_ids(const int* ids, int n, int V, int* out, int* dev_status) {
   for (int t = threadIdx.x; t < n; t += blockDim.x) {
@@ -381,7 +384,8 @@ sort_one_block_kernel(const int* __restrict__ ids, int n, int V, int* __restrict
 template <int kThreads>
 __global__ void __launch_bounds__(kThreads, 2048 / kThreads)
 sort_rank_kernel(const int* __restrict__ ids, int n, int V, int chunk_len, int* __restrict__ counts,
-                 int* __restrict__ totals, int* __restrict__ rank, int* __restrict__ dev_status) {
+                 int* __restrict__ totals, int* __restrict__ blocks, int* __restrict__ rank,
+                 int* __restrict__ dev_status) {
   extern __shared__ __align__(16) int sm_i[];
   const int chunk = blockIdx.x, j0 = chunk * chunk_len, m = min(chunk_len, n - j0);
   const int n32 = (m + 31) & ~31, slots = group_slots(m);
@@ -389,34 +393,58 @@ sort_rank_kernel(const int* __restrict__ ids, int n, int V, int chunk_len, int* 
   const TokenGroups g{sm_i, sm_i + n32, sm_i + 2 * n32, keys, keys + slots};
   load_ids(ids + j0, m, V, g.id, dev_status);
   group_tokens(g, keys, keys + slots, slots, m);
+  // tokens per 1024 ids, added up for the chunk first (ids below 1024 are the most frequent)
+  __shared__ int s_blocks[kSortBlocksShared];
+  const int n_blocks = (V + 1023) >> 10;
+  const bool shared = n_blocks <= kSortBlocksShared;
+  if (shared) {
+    for (int b = threadIdx.x; b < n_blocks; b += kThreads) s_blocks[b] = 0;
+    __syncthreads();
+  }
   for (int t = threadIdx.x; t < m; t += kThreads) {
     rank[j0 + t] = g.rank[t];
     const int id = g.id[t];
     if (id >= 0 && g.size[t] > 0) {
       counts[size_t(chunk) * V + id] = g.size[t];
       atomicAdd(&totals[id], g.size[t]);
+      atomicAdd(shared ? &s_blocks[id >> 10] : &blocks[id >> 10], g.size[t]);
+    }
+  }
+  if (shared) {
+    __syncthreads();
+    for (int b = threadIdx.x; b < n_blocks; b += kThreads)
+      if (s_blocks[b]) atomicAdd(&blocks[b], s_blocks[b]);
+  }
+}
+
+// counts[chunk][id] -> tokens of the id in earlier chunks
+__global__ void __launch_bounds__(kSideThreads, 16)
+sort_prefix_kernel(int* __restrict__ counts, int chunks, int V) {
+  const int v = blockIdx.x * kSideThreads + threadIdx.x;
+  if (v >= V) return;
+  int run = 0;
+  for (int c0 = 0; c0 < chunks; c0 += 8) {             // eight reads in flight
+    int x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) x[k] = c0 + k < chunks ? counts[size_t(c0 + k) * V + v] : 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (c0 + k < chunks) counts[size_t(c0 + k) * V + v] = run;
+      run += x[k];
     }
   }
 }
 
-// exclusive scan of the totals: block b adds up the totals before its 1024 entries itself (L2 reads)
+// exclusive scan of the totals: block b adds up those of the blocks before its 1024 entries.  (Reading all totals
+// before them instead was a chain of loads of 10 us at V = 50257.)
 __global__ void __launch_bounds__(kSideThreads, 16)
-sort_scan_kernel(const int* __restrict__ totals, int V, int* __restrict__ seg) {
+sort_scan_kernel(const int* __restrict__ totals, const int* __restrict__ blocks, int V, int* __restrict__ seg) {
   constexpr int kWarps = kSideThreads / 32;
   static_assert(kSideThreads * 8 == 1024, "eight entries per thread");
   __shared__ int wsum[kWarps], wbase[kWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int base = 0;
-  if ((reinterpret_cast<uintptr_t>(totals) & 15) == 0) {
-    const int4* t4 = reinterpret_cast<const int4*>(totals);
-#pragma unroll 4
-    for (int v = threadIdx.x; v < blockIdx.x * 256; v += kSideThreads) {
-      const int4 y = t4[v];
-      base += (y.x + y.y) + (y.z + y.w);
-    }
-  } else {                                             // a workspace on any 4-byte boundary will do
-    for (int v = threadIdx.x; v < blockIdx.x * 1024; v += kSideThreads) base += totals[v];
-  }
+  for (int b = threadIdx.x; b < int(blockIdx.x); b += kSideThreads) base += blocks[b];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) base += __shfl_xor_sync(0xffffffffu, base, o);
   const int v0 = blockIdx.x * 1024 + 8 * threadIdx.x;
@@ -444,15 +472,19 @@ sort_scan_kernel(const int* __restrict__ totals, int V, int* __restrict__ seg) {
 __global__ void __launch_bounds__(kSideThreads, 16)
 sort_place_kernel(const int* __restrict__ ids, int n, int V, int chunk_len, const int* __restrict__ counts,
                   const int* __restrict__ rank, const int* __restrict__ seg, int* __restrict__ perm,
-                  int* __restrict__ dev_status) {
+                  int prefixed, int* __restrict__ dev_status) {
   const int j = blockIdx.x * kSideThreads + threadIdx.x;
   if (j >= n) return;
   const int id = ids[j];
   if (id < 0 || id >= V) return;
   int dst = seg[id] + rank[j];
   const int chunk = j / chunk_len;
+  if (prefixed) {
+    dst += counts[size_t(chunk) * V + id];
+  } else {
 #pragma unroll 8
-  for (int c = 0; c < chunk; ++c) dst += counts[size_t(c) * V + id];
+    for (int c = 0; c < chunk; ++c) dst += counts[size_t(c) * V + id];
+  }
   if (dp_in_range(dst, n, dev_status)) perm[dst] = j;
 }
 
@@ -735,9 +767,10 @@ dp_status launch_embed_sort(const int* ids, int n, int V, const EmbedSortWs& ws,
     DP_CUDA_OK(allow_shared(sort_rank_kernel<4 * kSideThreads>, group_smem_bytes(4 * kSortChunk)));
     DP_CUDA_OK(prefer_max_shared(sort_one_block_kernel));
     DP_CUDA_OK(prefer_max_shared(sort_scan_kernel));
+    DP_CUDA_OK(prefer_max_shared(sort_prefix_kernel));
     DP_CUDA_OK(prefer_max_shared(sort_place_kernel));
   }
-  if (n <= kSortOneBlock && V <= kSortOneBlockIds) {
+  if (sort_in_one_block(n, V)) {
     sort_one_block_kernel<<<1, kSortThreads, group_smem_bytes(n), st>>>(ids, n, V, ws.seg, ws.perm, dev_status);
     DP_LAUNCH_OK();
     return DP_OK;
@@ -746,20 +779,27 @@ dp_status launch_embed_sort(const int* ids, int n, int V, const EmbedSortWs& ws,
   // counts of the chunks before a token few
   const int chunk_len = n <= 32 * kSortChunk ? kSortChunk : 4 * kSortChunk;
   const int chunks = ceil_div(n, chunk_len);
-  int* counts = ws.totals + V;
-  dp_status s = launch_clear(ws.totals, align_up((size_t(V) + size_t(chunks) * V) * sizeof(int), 16), st);
+  const int blocks = ceil_div(V, 1024);
+  int* block_totals = ws.totals + V;
+  int* counts = block_totals + blocks;
+  dp_status s = launch_clear(ws.totals, align_up((size_t(V) + blocks + size_t(chunks) * V) * sizeof(int), 16), st);
   if (s != DP_OK) return s;
   if (chunk_len == kSortChunk)
     sort_rank_kernel<kSideThreads><<<chunks, kSideThreads, group_smem_bytes(chunk_len), st>>>(
-        ids, n, V, chunk_len, counts, ws.totals, ws.rank, dev_status);
+        ids, n, V, chunk_len, counts, ws.totals, block_totals, ws.rank, dev_status);
   else
     sort_rank_kernel<4 * kSideThreads><<<chunks, 4 * kSideThreads, group_smem_bytes(chunk_len), st>>>(
-        ids, n, V, chunk_len, counts, ws.totals, ws.rank, dev_status);
+        ids, n, V, chunk_len, counts, ws.totals, block_totals, ws.rank, dev_status);
   DP_LAUNCH_OK();
-  sort_scan_kernel<<<ceil_div(V + 1, 1024), kSideThreads, 0, st>>>(ws.totals, V, ws.seg);
+  const bool prefix = chunks > kSortWalk;
+  if (prefix) {
+    sort_prefix_kernel<<<ceil_div(V, kSideThreads), kSideThreads, 0, st>>>(counts, chunks, V);
+    DP_LAUNCH_OK();
+  }
+  sort_scan_kernel<<<ceil_div(V + 1, 1024), kSideThreads, 0, st>>>(ws.totals, block_totals, V, ws.seg);
   DP_LAUNCH_OK();
   sort_place_kernel<<<ceil_div(n, kSideThreads), kSideThreads, 0, st>>>(ids, n, V, chunk_len, counts, ws.rank,
-                                                                       ws.seg, ws.perm, dev_status);
+                                                                       ws.seg, ws.perm, prefix ? 1 : 0, dev_status);
   DP_LAUNCH_OK();
   return DP_OK;
 }

@@ -42,15 +42,20 @@ dp_status launch_embed_norms(const int* ids, const void* G, int64_t ldg, dp_dtyp
                              int* dev_status, cudaStream_t st);
 int embed_norm_parts(int B, int T, int d);      // partial sums per (example, 256-column slab)
 struct EmbedSortWs {
-  int* totals;      // [V] followed by [chunks][V]: tokens per id, overall and per chunk
+  int* totals;      // [V], [ceil(V / 1024)] and [chunks][V]: tokens per id, per 1024 ids, per chunk and id
   int* seg;         // [V+1]
   int* perm;        // [B*T]
   int* rank;        // [B*T]  rank of a token among the equal ids of its chunk
 };
 constexpr int kSortChunk = 1024;
-// Most tokens and ids that one block sorts by itself: one launch instead of four (10.4 -> 4.5 us at 64
-// tokens, 1000 ids); its scan over 50 257 ids by one SM would take 40 us.
-constexpr int kSortOneBlock = 4096, kSortOneBlockIds = 8192;
+// One block sorts by itself in one launch instead of four, but its walk over the tokens and its scan over the ids are
+// serial.  One block and chunks, Zipf ids: 5.8 and 8.5 us at 64 tokens and 1000 ids, 14.7 and 16.4 at 2048 and 4000; 18.3 and
+// 16.7 at 3072 and 4000, 18.9 and 16.8 at 2048 and 8192, 11.2 and 8.2 at 64 and 8192.
+constexpr int kSortOneBlock = 2048, kSortOneBlockIds = 4096;
+inline bool sort_in_one_block(int n, int V) { return n <= kSortOneBlock && V <= kSortOneBlockIds; }
+// Chunks whose counts a token adds up when it is placed; with more, sort_prefix_kernel adds them up once: 22.7 us with it
+// against 21.9 at 4 chunks, 24.9 against 25.4 at 16, 55 against 77 at 64, 0.84 against 14.7 ms at 1024 (V = 50257).
+constexpr int kSortWalk = 8;
 dp_status launch_clear(void* p, size_t bytes, cudaStream_t st);
 dp_status launch_embed_sort(const int* ids, int n, int V, const EmbedSortWs& ws, int* dev_status,
                             cudaStream_t st);

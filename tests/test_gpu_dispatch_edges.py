@@ -50,7 +50,7 @@ def reference_sort(ids, V):
     return perm, np.concatenate([[0], np.cumsum(np.bincount(flat[ok], minlength=V))])
 
 
-# one block up to 4096 tokens and 8192 ids; chunks of 1024 up to 32768 tokens, of 4096 beyond
+# one block or chunks of 1024 tokens, of 4096 beyond 32768 tokens
 @pytest.mark.parametrize("B,T,V", [(1, 1, 1), (1, 31, 5), (2, 2048, 8192), (1, 4097, 100), (3, 1365, 8193),
                                    (8, 4096, 300), (1, 32769, 70000), (3, 13107, 9)])
 def test_token_sort_at_the_edges_of_its_variants(B, T, V):
@@ -67,6 +67,14 @@ def test_token_sort_at_the_edges_of_its_variants(B, T, V):
     got = perm.cpu().numpy()
     assert np.array_equal(got[:len(want_perm)], want_perm)
     assert (got[len(want_perm):] == -7).all()
+
+
+# one block up to 2048 tokens and 4096 ids; counts of up to 8 chunks are added up token by token, of more once for
+# all; tokens per 1024 ids are counted in shared memory up to 262144 ids
+@pytest.mark.parametrize("B,T,V", [(1, 2048, 4096), (1, 2049, 4096), (1, 64, 4097), (2, 4096, 6000),
+                                   (1, 8193, 6000), (9, 4096, 1025), (8, 4097, 262144), (2, 4096, 262145), (300, 2048, 5000)])
+def test_token_sort_at_the_lines_of_its_rules(B, T, V):
+    test_token_sort_at_the_edges_of_its_variants(B, T, V)
 
 
 # 48 rows of one id are summed by one warp, 49 by eight; rows are cut into parts of at least 64
