@@ -352,7 +352,8 @@ static dp_status ghost_norms_impl(const GhostPlan& plan, dp_linear_desc* layers,
     for (int l = 0; l < n_layers; ++l)
       if (!on_tensor_cores(layers[l], dt, T) && plan.mode_used[l] == DP_NORM_GHOST) fma.push_back(l);
     const size_t fma_need = fma_norms_bytes(layers, n_layers, dt, B, T);
-    const bool together = !fma.empty() && ws && aligned16(ws) && split_need + fma_need <= ws_bytes;
+    const bool together = !fma.empty() && ws && aligned16(ws) && split_need + fma_need <= ws_bytes &&
+                          !(fma.size() == 1 && gram_alone_fma(layers[fma[0]], T));
     if (together) {
       char* at = base;
       if (split_need) {

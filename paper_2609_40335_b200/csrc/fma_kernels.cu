@@ -18,16 +18,11 @@ namespace {
 // reductions: 1024 threads against 256 at B = 4, T = 16, d = p = 64: 15.1 -> 7.5 us.
 constexpr int kNormThreads = 1024;
 
+// sum over the pairs of tokens of one example of (a_t.a_s over columns [a0, a1)) * (g_t.g_s over [g0, g1)); in thread 0
 template <typename T>
-__global__ void __launch_bounds__(kNormThreads)
-ghost_norm_fma_kernel(const T* __restrict__ A, long long lda, int d,
-                                      const T* __restrict__ G, long long ldg, int p, int Tn,
-                                      float* __restrict__ sq, int overwrite) {
-  __shared__ float red[32];
-  const int i = blockIdx.x;
+__device__ __forceinline__ float pairs_sum(const T* Ai, long long lda, int a0, int a1, const T* Gi, long long ldg, int g0, int g1,
+                                           int Tn, float* red) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const T* Ai = A + size_t(i) * Tn * lda;
-  const T* Gi = G + size_t(i) * Tn * ldg;
   const long long npairs = (long long)Tn * (Tn + 1) / 2;
   float acc = 0.f;
   int t = 0, s = 0;                       // pair index -> (t, s), s >= t, walked incrementally
@@ -41,14 +36,24 @@ ghost_norm_fma_kernel(const T* __restrict__ A, long long lda, int d,
     }
     float da = 0.f, dg = 0.f;
 #pragma unroll 4
-    for (int k = lane; k < d; k += 32) da = fmaf(to_f32(Ai[t * lda + k]), to_f32(Ai[s * lda + k]), da);
+    for (int k = a0 + lane; k < a1; k += 32) da = fmaf(to_f32(Ai[t * lda + k]), to_f32(Ai[s * lda + k]), da);
 #pragma unroll 4
-    for (int k = lane; k < p; k += 32) dg = fmaf(to_f32(Gi[t * ldg + k]), to_f32(Gi[s * ldg + k]), dg);
+    for (int k = g0 + lane; k < g1; k += 32) dg = fmaf(to_f32(Gi[t * ldg + k]), to_f32(Gi[s * ldg + k]), dg);
     da = warp_sum(da);
     dg = warp_sum(dg);
     acc += (t == s ? 1.f : 2.f) * da * dg;
   }
-  const float tot = block_sum(lane == 0 ? acc : 0.f, red);
+  return block_sum(lane == 0 ? acc : 0.f, red);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kNormThreads)
+ghost_norm_fma_kernel(const T* __restrict__ A, long long lda, int d,
+                                      const T* __restrict__ G, long long ldg, int p, int Tn,
+                                      float* __restrict__ sq, int overwrite) {
+  __shared__ float red[32];
+  const int i = blockIdx.x;
+  const float tot = pairs_sum(A + size_t(i) * Tn * lda, lda, 0, d, G + size_t(i) * Tn * ldg, ldg, 0, p, Tn, red);
   if (threadIdx.x == 0) sq[i] = (overwrite ? 0.f : sq[i]) + tot;
 }
 
@@ -204,6 +209,9 @@ clip_accumulate_fma_kernel(const __grid_constant__ FmaSumParams P) {
 // step of three blocks of d = 64 with V = 8064 at B = 2, T = 29 took 616 us, now 72; five of d = 640 at B = 16, T = 26
 // 2918, now 1010 (most of it the sums' FMAs).  Those kernels remain for a workspace without room for the
 // partial sums.
+// Very short sequences (gram_by_pairs) fill little of a tile, whose walk over the columns takes as long as ever: there an
+// item is all pairs of tokens, a warp each (gram_pairs_fma_kernel): one layer of 768 -> 3072 at B = 4, T = 16 67 -> 23 us, 24 layers of
+// DistilGPT2 at B = 32, T = 16 364 -> 194 (829 with a launch per layer).
 constexpr int kGramTile = 32, kGramChunk = 2048;     // tokens per tile; columns per item of the wider operand
 struct FmaNormLayer {
   const void *A, *G;
@@ -284,6 +292,19 @@ gram_norm_fma_kernel(const __grid_constant__ FmaNormParams P) {
   for (int e = 0; e < 4; ++e) acc = fmaf(sa[e >> 1][e & 1], sg[e >> 1][e & 1], acc);
   const float tot = block_sum(acc, red);
   if (threadIdx.x == 0) P.partials[size_t(i) * P.n_per + L.col_begin + tp * L.nsplit + sp] = ri == rj ? tot : 2.f * tot;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kNormThreads)
+gram_pairs_fma_kernel(const __grid_constant__ FmaNormParams P) {
+  __shared__ float red[32];
+  const FmaNormLayer& L = find_layer(P.layer, P.n, int(blockIdx.x), [](const FmaNormLayer& x) { return x.item_begin; });
+  const int local = int(blockIdx.x) - L.item_begin, sp = local % L.nsplit, i = local / L.nsplit;
+  const bool wide_g = L.p >= L.d;
+  const int lo = sp * kGramChunk, hi = min(wide_g ? L.p : L.d, lo + kGramChunk);
+  const float tot = pairs_sum(static_cast<const T*>(L.A) + size_t(i) * P.T * L.lda, L.lda, wide_g ? 0 : lo, wide_g ? L.d : hi,
+                              static_cast<const T*>(L.G) + size_t(i) * P.T * L.ldg, L.ldg, wide_g ? lo : 0, wide_g ? hi : L.p, P.T, red);
+  if (threadIdx.x == 0) P.partials[size_t(i) * P.n_per + L.col_begin + sp] = tot;
 }
 
 // <g_in_i, g_out_i> = sum_{t,s} G_lm[i,s,id_t] * (g_emb_t . a_lm_s)   (expansion of Eq. 11's
@@ -425,9 +446,17 @@ int gram_fma_partials(const dp_linear_desc& L, int T) {
   return nt * (nt + 1) / 2 * ceil_div(std::max(L.d, L.p), kGramChunk);
 }
 
+// All pairs of tokens per item, or tiles.  A tile takes about as long whatever the tokens, pairs do not (d = p = 64: 6.4 and 7.6 us at 8
+// tokens, 7.8 and 7.7 at 12; 24 layers of DistilGPT2 at B = 32: 255 and 370 at 20, about 340 and 374 at 24).
+static bool gram_by_pairs(int T, int widest) { return T <= (widest >= 512 ? 24 : 12); }
+
+bool gram_alone_fma(const dp_linear_desc& L, int T) { return std::max(L.d, L.p) >= 512 && gram_fma_partials(L, T) == 1; }
+
 dp_status launch_gram_norms_fma(const dp_linear_desc* layers, const int* index, int n, dp_dtype dt, int B, int T,
                                 float* partials, int n_per, cudaStream_t st) {
-  int col = 0;
+  int col = 0, widest = 0;
+  for (int k = 0; k < n; ++k) widest = std::max(widest, std::max(layers[index[k]].d, layers[index[k]].p));
+  const bool pairs = gram_by_pairs(T, widest);
   for (int k0 = 0; k0 < n; k0 += kFmaMaxLayers) {
     FmaNormParams P;
     P.n = std::min(n - k0, kFmaMaxLayers);
@@ -442,8 +471,13 @@ dp_status launch_gram_norms_fma(const dp_linear_desc* layers, const int* index, 
       col += P.ntp * nsplit;
     }
     if (items > 0x7fffffffLL) return DP_ERR_UNSUPPORTED;
-    if (dt == DP_F32) gram_norm_fma_kernel<float><<<(unsigned)items, 256, 0, st>>>(P);
-    else gram_norm_fma_kernel<__nv_bfloat16><<<(unsigned)items, 256, 0, st>>>(P);
+    if (pairs) {
+      if (dt == DP_F32) gram_pairs_fma_kernel<float><<<(unsigned)items, kNormThreads, 0, st>>>(P);
+      else gram_pairs_fma_kernel<__nv_bfloat16><<<(unsigned)items, kNormThreads, 0, st>>>(P);
+    } else {
+      if (dt == DP_F32) gram_norm_fma_kernel<float><<<(unsigned)items, 256, 0, st>>>(P);
+      else gram_norm_fma_kernel<__nv_bfloat16><<<(unsigned)items, 256, 0, st>>>(P);
+    }
     DP_LAUNCH_OK();
   }
   return DP_OK;

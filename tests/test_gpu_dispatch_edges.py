@@ -378,6 +378,33 @@ def test_fp32_gram_norms(shapes, T, room):
     assert ((sq.double() - want).abs() <= 2.0 ** -24 * 256 * size).all()
 
 
+# very short sequences: a warp per pair of tokens, up to 12 tokens, or 24 where some operand has 512 columns
+@pytest.mark.parametrize("T", [1, 2, 11, 12, 13, 24, 25])
+@pytest.mark.parametrize("shapes", [[(32, 511), (5, 70)], [(32, 512), (5, 70)], [(40, 60)] * 65, [(33, 4100), (2049, 2048)],
+                                    [(33, 4100)]])     # 4100: three chunks
+def test_fp32_gram_norms_of_very_short_sequences(shapes, T):
+    test_fp32_gram_norms(shapes, T, True)
+
+
+@pytest.mark.parametrize("d,p,T", [(511, 30, 31), (512, 30, 31), (700, 2048, 1), (700, 2049, 1), (64, 600, 33)])
+def test_fp32_gram_norm_of_one_layer(d, p, T):
+    """A layer of 512 columns or more by itself: one kernel, if its partial sums are one per example."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    layer = dp.Linear(torch.randn(2, T, d, generator=g, device="cuda"), torch.randn(2, T, p, generator=g, device="cuda"), d=d, p=p)
+    sq = torch.ones(2, device="cuda")
+    before = dp.dp_debug_force_fma(True)
+    try:
+        n0 = dp.dp_kernel_launches()
+        dp.dp_ghost_norms([layer], 2, T, sq, ws=torch.empty(dp.dp_step_ws_bytes([layer], 2, T), dtype=torch.uint8, device="cuda"))
+        assert dp.dp_kernel_launches() - n0 == (1 if max(d, p) >= 512 and p <= 2048 and T <= 32 else 2)
+    finally:
+        dp.dp_debug_force_fma(before)
+    want = (torch.einsum("btp,btd->bpd", layer.G.double(), layer.A.double()) ** 2).sum((1, 2))
+    size = (layer.A.double() ** 2).sum((1, 2)) * (layer.G.double() ** 2).sum((1, 2))
+    assert ((sq.double() - 1.0 - want).abs() <= 2.0 ** -24 * 256 * size).all()
+
+
 # Gram tiles as tall as the sequence, rounded up to 16 tokens, up to 64 tokens: rings of up to 32 stages of two
 # or four column tiles; bf16 and split fp32
 @pytest.mark.parametrize("T", [1, 15, 16, 17, 31, 32, 33, 48, 49, 64, 65, 77, 127, 128, 129])
