@@ -517,9 +517,11 @@ struct ReduceParams {
   uint32_t step;
   const uint32_t* step_dev;
 };
-constexpr int kReduceQuads = 512;                    // quads per block of 256 threads
-
-__global__ void __launch_bounds__(256)
+// Two quads per thread of 256-thread blocks, four planes in flight each; where that leaves SMs idle one quad per thread of 64,
+// eight planes in flight: with its GEMM, one 64 x 64 layer of 148 planes (bf16, B = 16, T = 512) 18.4 -> 13.5 us, fp32 38 -> 19; one of
+// 768 x 768 and 16 planes would go from 16.2 to 17.7 in that form.
+template <int kThreads, int kPerThread, int kPlanes>
+__global__ void __launch_bounds__(kThreads)
 splitk_reduce_kernel(const __grid_constant__ ReduceParams P) {
   int lo = 0, hi = P.n_layers - 1;                   // the layer this block belongs to
   while (lo < hi) {
@@ -532,14 +534,14 @@ splitk_reduce_kernel(const __grid_constant__ ReduceParams P) {
   const bool ovec = (L.N & 3) == 0 && (L.ldo & 3) == 0 && (reinterpret_cast<uintptr_t>(L.out) & 15) == 0;
   const uint32_t step = effective_step(P.step, P.step_dev);
 #pragma unroll
-  for (int k = 0; k < kReduceQuads / 256; ++k) {
-    const size_t q = size_t(int(blockIdx.x) - L.block_begin) * kReduceQuads + k * 256 + threadIdx.x;
+  for (int k = 0; k < kPerThread; ++k) {
+    const size_t q = (size_t(int(blockIdx.x) - L.block_begin) * kPerThread + k) * kThreads + threadIdx.x;
     const size_t e0 = 4 * q;
     if (e0 >= total) break;
     float v[4] = {0.f, 0.f, 0.f, 0.f};
     if (vec) {
       const float* src = L.partial + e0;
-#pragma unroll 4
+#pragma unroll kPlanes
       for (int s = 0; s < P.nsplit; ++s) {
         const float4 x = __ldcs(reinterpret_cast<const float4*>(src + size_t(s) * total));
         v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
@@ -772,13 +774,17 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
       R.amp = noise ? noise->amp : 0.f; R.scale = noise ? noise->scale : 1.f;
       R.keys = expand_noise_keys(noise ? noise->seed : 0);
       R.step = noise ? noise->step : 0; R.step_dev = noise ? g_step_dev : nullptr;
-      long long blocks = 0;
+      long long quads = 0, blocks = 0;
+      for (int k = 0; k < P.n_layers; ++k) quads += ((long long)P.layer[k].M * P.layer[k].N + 3) / 4;
+      const bool few = quads < (long long)sms * 512;
+      const int per_block = few ? 64 : 512;
       for (int k = 0; k < P.n_layers; ++k) {
         const GtaLayer& L = P.layer[k];
         R.layer[k] = {L.out, L.partial, L.ldo, L.M, L.N, int(blocks), L.tensor_id};
-        blocks += ((long long)L.M * L.N + 4 * kReduceQuads - 1) / (4 * kReduceQuads);
+        blocks += ((long long)L.M * L.N + 4LL * per_block - 1) / (4LL * per_block);
       }
-      splitk_reduce_kernel<<<(unsigned)blocks, 256, 0, st>>>(R);
+      if (few) splitk_reduce_kernel<64, 1, 8><<<(unsigned)blocks, 64, 0, st>>>(R);
+      else splitk_reduce_kernel<256, 2, 4><<<(unsigned)blocks, 256, 0, st>>>(R);
       DP_LAUNCH_OK();
       continue;
     }

@@ -133,7 +133,7 @@ def test_fp32_layers_in_groups(extra, T):
 
 
 # one reduction for the K-split planes of all layers: widths that are and are not multiples of 4
-@pytest.mark.parametrize("shapes", [[(64, 64), (256, 300)], [(50, 70), (33, 41), (3, 5)]])
+@pytest.mark.parametrize("shapes", [[(64, 64), (256, 300)], [(50, 70), (33, 41), (3, 5)], [(512, 592)], [(512, 591), (4, 1)]])
 @pytest.mark.parametrize("noise", [False, True])
 def test_k_split_planes_of_several_layers(shapes, noise):
     B, T = 16, 64
