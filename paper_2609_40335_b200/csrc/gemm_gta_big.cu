@@ -79,7 +79,7 @@ struct __align__(64) BigParams {
   CUtensorMap tmA[kGtaMaxLayers];
   BigLayer layer[kGtaMaxLayers];
   int n_layers;
-  int tsteps, terms, ksteps; // K steps per example, products per 64 tokens (split fp32), K steps in all
+  int tsteps, ksteps;        // K steps per example (split fp32: three per 64 tokens), K steps in all
   int skew;                  // K steps that sub-tile 1 of an item lags behind
   int n_big, n_big_total;    // two-tile items run as such, and in all (the rest as two singles each)
   int total_items;
@@ -152,6 +152,7 @@ struct Slots {
   }
 };
 
+template <bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
   const uint32_t rank = ptx::cluster_ctarank();
@@ -215,10 +216,10 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
       const int skew = it.nsub == 2 ? P.skew : 0, steps = P.ksteps + skew;
       // the steps in which this warp's part takes part
       const int from = sub ? skew : 0, to = is_x || sub ? steps : P.ksteps;
-      const GtaWalk start(0, 0, P.ksteps / P.terms, P.tsteps / P.terms, P.terms);
-      GtaWalk at = start;
+      constexpr int kTerms = kSplit ? 3 : 1;
+      GtaWalk<kSplit> at(0, 0, P.ksteps / kTerms, P.tsteps / kTerms);
       for (int j = 0; j < steps; ++j) {
-        if (j == P.ksteps) at = start;
+        if (j == P.ksteps) at = GtaWalk<kSplit>(0, 0, P.ksteps / kTerms, P.tsteps / kTerms);
         ok = ptx::warp_ok(ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit));
         if (!ok) break;
         const uint32_t bar = full_a + 8 * stage;
@@ -471,11 +472,27 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
 
 }  // namespace
 
+template <bool kSplit>
+static dp_status launch_big(const BigParams& P, int units, cudaStream_t st) {
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_big_kernel<kSplit>)))
+    DP_CUDA_OK(allow_shared(gemm_gta_big_kernel<kSplit>, kSmemBytes));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * units, 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  DP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_gta_big_kernel<kSplit>, P));
+  ++g_kernel_launches;
+  return DP_OK;
+}
+
 // One launch over at most kGtaMaxLayers layers without a K split.
 dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, const float* clip, float beta,
                          const GtaNoise* noise, int* dev_status, cudaStream_t st) {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_big_kernel)))
-    DP_CUDA_OK(allow_shared(gemm_gta_big_kernel, kSmemBytes));
   BigParams P;
   memset(&P, 0, sizeof(P));
   const int planes = terms > 1 ? 2 * B : B;
@@ -507,7 +524,7 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
   P.n_big = (rest && convert < keep) ? bigs - rest : bigs;
   P.total_items = P.n_big + 2 * (bigs - P.n_big) + singles;
   P.n_layers = n;
-  P.terms = terms; P.tsteps = terms * ceil_div(T, kBK); P.ksteps = B * P.tsteps;
+  P.tsteps = terms * ceil_div(T, kBK); P.ksteps = B * P.tsteps;
   // Long enough to read one accumulator, and to draw its noise, while the other is fed: with noise 4, 6, 8,
   // 10, 12, 24 and 40 steps gave 2341, 2278, 2252, 2265, 2283, 2407 and 2513 us (B = 16, T = 512).  The same
   // without noise, which would do with 2 or none, so that a sum does not depend on whether noise is fused.
@@ -524,18 +541,7 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
   P.dev_status = dev_status;
   P.wait_limit = g_wait_limit;
   const int units = std::min(P.total_items, pairs);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * units, 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = kSmemBytes;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  DP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_gta_big_kernel, P));
-  ++g_kernel_launches;
-  return DP_OK;
+  return terms > 1 ? launch_big<true>(P, units, st) : launch_big<false>(P, units, st);
 }
 
 }  // namespace dpg

@@ -74,7 +74,6 @@ struct __align__(64) GtaParams {
   GtaLayer layer[kGtaMaxLayers];
   int n_layers;
   int B, T, tsteps;          // tsteps = terms * ceil(T / 64) K steps per example
-  int terms;                 // 3: split fp32 operands (three products per 64 tokens), else 1
   int nsplit, ksteps_per_split;   // K splits, the same for all layers of a call; multiples of `terms` steps
   float beta;
   int total_items;
@@ -118,7 +117,7 @@ __device__ __forceinline__ Item decode_item(const GtaParams& P, int item, int& l
   return it;
 }
 
-template <bool kScale, bool kSqsum, bool kPair>
+template <bool kScale, bool kSqsum, bool kPair, bool kSplit>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_gta_kernel(const __grid_constant__ GtaParams P) {
   static_assert(kScale || !kPair, "CTA pairs need the scaler warps' cross-CTA stage hand-off");
@@ -197,7 +196,8 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
         // first column of this CTA's part of the tile: its G rows, or its share of the A columns
         const int c0 = is_a ? it.tn * kBN + int(rank) * Geo<kPair>::kAColsPerCta
                             : it.tm * kTileM + int(rank) * kBM;
-        GtaWalk at(0, it.k0 / P.terms, it.k1 / P.terms, P.tsteps / P.terms, P.terms);
+        constexpr int kTerms = kSplit ? 3 : 1;
+        GtaWalk<kSplit> at(0, it.k0 / kTerms, it.k1 / kTerms, P.tsteps / kTerms);
         for (int ks = it.k0; ks < it.k1; ++ks) {
           if (!ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
           const uint32_t bar = full_a + 8 * stage;
@@ -621,16 +621,11 @@ constexpr bool kClipScale = true;
 
 constexpr bool kUsePair = true;
 
-template <bool kScale, bool kSqsum, bool kPair>
-dp_status set_attr_once() {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_kernel<kScale, kSqsum, kPair>)))
-    DP_CUDA_OK(allow_shared(gemm_gta_kernel<kScale, kSqsum, kPair>, Geo<kPair>::kSmemBytes));
-  return DP_OK;
-}
-
 // Launch on `units` persistent CTAs (single) or CTA pairs (cluster of 2).
-template <bool kScale, bool kSqsum, bool kPair>
+template <bool kScale, bool kSqsum, bool kPair, bool kSplit>
 dp_status launch_gta(const GtaParams& P, int units, cudaStream_t st) {
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_kernel<kScale, kSqsum, kPair, kSplit>)))
+    DP_CUDA_OK(allow_shared(gemm_gta_kernel<kScale, kSqsum, kPair, kSplit>, Geo<kPair>::kSmemBytes));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kPair ? 2 * units : units, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -643,7 +638,7 @@ dp_status launch_gta(const GtaParams& P, int units, cudaStream_t st) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  DP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_gta_kernel<kScale, kSqsum, kPair>, P));
+  DP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_gta_kernel<kScale, kSqsum, kPair, kSplit>, P));
   ++g_kernel_launches;
   return DP_OK;
 }
@@ -687,8 +682,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
                                     const float* clip, float* const* outs, const int64_t* ldos,
                                     float beta, const GtaNoise* noise, float* partial_ws,
                                     int* dev_status, cudaStream_t st) {
-  dp_status s = set_attr_once<kClipScale, false, kUsePair>();
-  if (s != DP_OK) return s;
+  dp_status s = DP_OK;
   const int sms = sm_count();
   const int tsteps = terms * ceil_div(T, kBK), planes = terms > 1 ? 2 * B : B;
   const int ksteps = B * tsteps;
@@ -758,7 +752,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
       P.noise_step = noise->step; P.noise_scale = noise->scale;
       P.step_dev = g_step_dev;
     }
-    P.n_layers = g1 - g0; P.B = B; P.T = T; P.tsteps = tsteps; P.terms = terms;
+    P.n_layers = g1 - g0; P.B = B; P.T = T; P.tsteps = tsteps;
     P.total_items = items;
     P.nsplit = nsplit; P.ksteps_per_split = kps; P.beta = beta;
     P.clip = clip;
@@ -766,7 +760,8 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
     P.wait_limit = g_wait_limit;
     const int units = std::min(items, kUsePair ? sms / 2 : sms);
     s = use_big ? launch_gta_big(big.data(), (int)big.size(), B, T, terms, clip, beta, noise, dev_status, st)
-                : launch_gta<kClipScale, false, kUsePair>(P, units, st);
+        : terms > 1 ? launch_gta<kClipScale, false, kUsePair, true>(P, units, st)
+                    : launch_gta<kClipScale, false, kUsePair, false>(P, units, st);
     if (s != DP_OK) return s;
     if (nsplit > 1) {
       ReduceParams R;
@@ -804,8 +799,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
 
 dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T, int terms,
                                 float* partials, int* dev_status, cudaStream_t st) {
-  dp_status s = set_attr_once<false, true, false>();
-  if (s != DP_OK) return s;
+  dp_status s = DP_OK;
   const int sms = sm_count(), planes = terms > 1 ? 2 * B : B;
   for (size_t g0 = 0; g0 < plan.direct_layers.size(); g0 += kGtaMaxLayers) {
     const size_t g1 = std::min(plan.direct_layers.size(), g0 + kGtaMaxLayers);
@@ -826,13 +820,14 @@ dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& p
       items += B * plan.direct[li].tiles_m * plan.direct[li].tiles_n;
     }
     P.n_layers = int(g1 - g0);
-    P.B = B; P.T = T; P.tsteps = terms * ceil_div(T, kBK); P.terms = terms;
+    P.B = B; P.T = T; P.tsteps = terms * ceil_div(T, kBK);
     P.total_items = items;
     P.nsplit = 1;
     P.sq_partials = partials; P.n_per = plan.n_per;
     P.dev_status = dev_status;
     P.wait_limit = g_wait_limit;
-    s = launch_gta<false, true, false>(P, std::min(items, sms), st);
+    s = terms > 1 ? launch_gta<false, true, false, true>(P, std::min(items, sms), st)
+                  : launch_gta<false, true, false, false>(P, std::min(items, sms), st);
     if (s != DP_OK) return s;
   }
   return DP_OK;
