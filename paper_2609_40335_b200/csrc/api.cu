@@ -590,8 +590,7 @@ dp_status dp_clip_accumulate_vectors(const dp_vector_desc* prm, int32_t n, dp_dt
 dp_status dp_clip_factors_sum(float* sq, const float* sq_extra, int32_t B, float C, float* clip,
                               float* norms, void* stream) {
   if (!sq || !sq_extra || B <= 0 || !finite_pos(C)) return DP_ERR_INVALID_ARG;
-  const NormSources N{{{sq, 1, 1.f, nullptr}, {sq_extra, 1, 1.f, nullptr}}, 1, 2};
-  return launch_finish_norms(N, B, C, sq, clip, norms, (cudaStream_t)stream);
+  return launch_clip_factors(sq, B, C, clip, norms, (cudaStream_t)stream, sq_extra, sq);
 }
 
 dp_status dp_clip_factors(const float* sq, int32_t B, float C, float* clip, float* norms,

@@ -26,8 +26,9 @@ dp_status launch_cross_term_fma(const int* ids, const void* Ge, int64_t ldge, co
                                 int64_t ldal, const void* Gl, int64_t ldgl, dp_dtype dt, int B,
                                 int T, int d, int V, float* partials, int* dev_status,
                                 cudaStream_t st);
+// extra: added to sq first, the sum written to `sum` (which may be sq)
 dp_status launch_clip_factors(const float* sq, int B, float C, float* clip, float* norms,
-                              cudaStream_t st);
+                              cudaStream_t st, const float* extra = nullptr, float* sum = nullptr);
 // Partial sums of squared norms that a step has left in workspaces: [B][n_per] floats each.
 struct NormSource { const float* partials; int n_per; float factor; float* plain_out; };
 struct NormSources {
