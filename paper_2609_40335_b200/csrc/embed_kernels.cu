@@ -38,6 +38,22 @@ __host__ __device__ __forceinline__ size_t group_smem_bytes(int n) {
 
 // fills g; g.id must hold the n ids already (the function synchronises first and last)
 __device__ __forceinline__ void group_tokens(const TokenGroups& g, int* keys, int* first, int slots, int n) {
+  if (n <= 32) {                                         // one window: no table (7.3 -> 6.9 us for the norm at B = 1, T = 8, d = 768)
+    __syncthreads();
+    const int lane = threadIdx.x;
+    if (lane < 32) {
+      const int id = lane < n ? g.id[lane] : -1;
+      const unsigned peers = __match_any_sync(0xffffffffu, id >= 0 ? id : int(0x80000000u | unsigned(lane)));
+      if (lane < n) {
+        const int fo = __ffs(peers) - 1;
+        g.fo[lane] = fo;
+        g.rank[lane] = __popc(peers & ((1u << lane) - 1u));
+        g.size[lane] = lane == fo ? __popc(peers) : 0;
+      }
+    }
+    __syncthreads();
+    return;
+  }
   constexpr int kEmpty = int(0x80000000);
   const int shift = __clz(slots) + 1;                    // top log2(slots) bits of the product
   for (int h = threadIdx.x; h < slots; h += blockDim.x) { keys[h] = kEmpty; first[h] = 0x7fffffff; }
@@ -145,7 +161,7 @@ embed_norm_kernel(const int* __restrict__ ids, const T* __restrict__ G, long lon
   __shared__ int wsum[33];
   __shared__ int s_long[kEmbedMaxT / kEmbedLong + 1], s_nlong;
   __shared__ float s_part[8][kEmbedColsPerBlock];
-  constexpr int kBatch = sizeof(T) == 2 ? 8 : 4;
+  constexpr int kBatch = sizeof(T) == 2 ? 8 : 4, kLongBatch = kBatch;
   constexpr int kWarps = kEmbedNormThreads / 32;
   const int part = blockIdx.x % parts, slab = (blockIdx.x / parts) % slabs, i = blockIdx.x / (parts * slabs);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -253,16 +269,16 @@ embed_norm_kernel(const int* __restrict__ ids, const T* __restrict__ G, long lon
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
     if (nvalid > 0) {
-      for (int r0 = a + warp; r0 < b; r0 += kWarps * 8) {
-        Raw8<T> v[8];
+      for (int r0 = a + warp; r0 < b; r0 += kWarps * kLongBatch) {
+        Raw8<T> v[kLongBatch];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < kLongBatch; ++j) {
           const int r = r0 + kWarps * j;
           if (r < b) v[j].load(Gi + size_t(s_ord[r] & 0x7fffffff) * ldg, nvalid, vec);
           else v[j].zero();
         }
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < kLongBatch; ++j) {
           float x[8];
           v[j].unpack(x);
 #pragma unroll
@@ -560,23 +576,21 @@ embed_scatter_kernel(const int* __restrict__ ids, const T* __restrict__ G, long 
   //      classify the chunk's positions (warp 0)
   {
     const int k = kc + threadIdx.x;
-    int pos = 0;
+    int pos = 0, v = -1;
     const bool staged = threadIdx.x < kScatChunk + kScatShort;
     if (staged && k < n_valid) {
       pos = perm[k];
       if (!dp_in_range(pos, n_rows, dev_status)) pos = 0;   // checked build: flagged, row 0 stands in
+      if (w == 0) v = ids[pos];                             // on its way while the factor is waited for
       s_pos[threadIdx.x] = pos;
       s_r[threadIdx.x] = clip[pos / Tn];
     }
     if (staged) s_end[threadIdx.x] = -1;
     if (w == 0) {
-      int v = -1, n = 0, s0 = 0;
-      if (k < n_valid) {
-        v = ids[pos];
-        if (dp_in_range(v, V, dev_status)) {
-          s0 = seg[v];
-          n = seg[v + 1] - s0;
-        }
+      int n = 0, s0 = 0;
+      if (k < n_valid && dp_in_range(v, V, dev_status)) {
+        s0 = seg[v];
+        n = seg[v + 1] - s0;
       }
       const bool head = n > 0 && s0 == k, is_long = n > kScatShort;
       const unsigned sh = __ballot_sync(0xffffffffu, head && !is_long);
@@ -587,7 +601,7 @@ embed_scatter_kernel(const int* __restrict__ ids, const T* __restrict__ G, long 
       __syncwarp();
     }
     __syncthreads();
-    if (w == 0 && ((s_short >> lane) & 1u)) s_end[lane + s_n[lane] - 1] = ids[pos];   // id at a segment's last row
+    if (w == 0 && ((s_short >> lane) & 1u)) s_end[lane + s_n[lane] - 1] = v;   // id at a segment's last row
   }
   __syncthreads();
 
@@ -845,6 +859,7 @@ dp_status launch_embed_scatter(const int* ids, const void* G, int64_t ldg, dp_dt
                                                              d, clip, perm, seg, V, out, ldo, 1.f,
                                                              scale, long_part, n, dev_status);
   DP_LAUNCH_OK();
+  if (n <= kScatShort) return DP_OK;                     // no segment is long
   embed_scatter_combine_kernel<<<grid, kSideThreads, 0, st>>>(ids, perm, seg, V, d, long_part, out, ldo, 1.f,
                                                      scale, n, dev_status);
   DP_LAUNCH_OK();

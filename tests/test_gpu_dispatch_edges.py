@@ -250,6 +250,29 @@ def test_row_sums_at_the_edges(dtype, d, ldo, ldg):
         assert (out[:, d:] == 5.0).all()
 
 
+# up to 32 rows no segment is long, and there is no second pass; a single window of tokens is grouped by one warp
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("T", [1, 2, 31, 32, 33, 34])
+@pytest.mark.parametrize("kind", ["same", "distinct", "mixed", "out"])
+def test_embedding_of_few_tokens(dtype, T, kind):
+    d, V = 70, 50
+    ids = {"same": torch.full((T,), 7), "distinct": torch.arange(T), "mixed": torch.arange(T) * 7 % 5,
+           "out": torch.arange(T) % 3 * 30 - 1}[kind].to(torch.int32).view(1, T).cuda()      # -1, 29, 59
+    G = torch.randn(1, T, d, generator=torch.Generator().manual_seed(T)).to(torch.float32 if dtype == "f32" else torch.bfloat16).cuda()
+    sq, out, st = torch.zeros(1, device="cuda"), torch.empty(V, d, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    first = torch.empty(1, T, dtype=torch.int32, device="cuda")
+    dp.dp_embed_norms(ids, G, V, sq, first_occ=first, dev_status=st)
+    dp.dp_clip_accumulate_embed(ids, G, V, None, 1.0, out, d=d, clip=torch.full((1,), 0.5, device="cuda"), dev_status=st)
+    rows, inside = ids.flatten().long(), (ids.flatten() >= 0) & (ids.flatten() < V)
+    table = torch.zeros(V, d, dtype=torch.float64, device="cuda").index_add_(0, rows[inside], G[0].double()[inside])
+    assert abs(float(sq) - float((table ** 2).sum())) <= 1e-5 * float((table ** 2).sum())
+    assert float((out.double() - 0.5 * table).norm()) <= 1e-6 * float(table.norm())
+    assert int(st.item()) == (0 if bool(inside.all()) else dp.DP_DEV_BAD_ID)
+    for t in range(T):                                     # a token out of range is a group of its own
+        want = t if not inside[t] else int((rows == rows[t]).nonzero()[0])
+        assert int(first[0, t]) == want
+
+
 # layers that stay on the fp32 kernels: tiles of 32 or 64 outputs (64 from 148 of them on), noise inside the
 # kernel where d is a multiple of 4; sums and noise are the same bits as in two calls
 @pytest.mark.parametrize("d,p,B,T", [(64, 64, 4, 16), (32, 33, 1, 1), (4, 7, 3, 5), (30, 40, 2, 31), (62, 70, 1, 33),
