@@ -32,8 +32,8 @@ METRIC = "dp_sgd_examples_per_sec"
 UNIT = "examples/s"
 
 # DRAM bytes of the clipped-sum GEMM (dram__bytes_read.sum + dram__bytes_write.sum, one ncu capture
-# of a three-wave launch of the same kernel) divided by that launch's algorithmic bytes (inputs
-# read once + fp32 outputs written once).  `roofline.traffic` of a workload is this ratio times
+# of a three-wave, head-like launch each of gemm_gta_big_kernel and gemm_gta_kernel, 0.97 for both) divided
+# by that launch's algorithmic bytes (inputs read once + fp32 outputs written once).  `roofline.traffic` of a workload is this ratio times
 # the algorithmic bytes of its own grouped launch: the kernel reads every operand tile from DRAM
 # once whatever the layer list, so traffic grows in proportion to the bytes.
 GEMM_DRAM_OVER_ALGORITHMIC = 0.97
@@ -49,6 +49,15 @@ def measured_peaks():
                 "source": "measured"}
     return {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0,
             "source": "fallback"}
+
+
+def gemm_kernel_name(ds, reserved_sms):
+    """The kernel behind the grouped clipped sums: items of two 256 x 256 tiles where every CTA pair gets two tiles."""
+    import torch
+    sms = torch.cuda.get_device_properties(ds.sq.device).multi_processor_count - reserved_sms
+    layers = ds.linears + ([ds.lm] if ds.lm else [])
+    tiles = sum(-(-l.p // 256) * -(-l.d // 256) for l in layers)
+    return "gemm_gta_big_kernel" if tiles >= 2 * (sms // 2) else "gemm_gta_kernel<scale, pair>"
 
 
 # ------------------------------------------------------------------------------- clocks
@@ -600,7 +609,8 @@ def run_ours(args):
 
     # dominant kernel: the tensor-core G^T A GEMM of the clipped sums, timed live (see above)
     achieved_tf = counts["acc_flops"] / (gemm_ms_avg * 1e-3) / 1e12
-    roofline = {"kernel": "gemm_gta_big_kernel (%s)" % (
+    roofline = {"kernel": "%s (%s)" % (
+                    gemm_kernel_name(ds, reserve),
                     "dp_clip_accumulate_noise_grouped, Gaussian noise drawn in the epilogue"
                     if fused and not args.prefill else
                     "dp_clip_accumulate_grouped, accumulating onto noise filled beside the norm phase"
@@ -622,7 +632,7 @@ def run_ours(args):
                 "flops_per_launch": counts["acc_flops"],
                 "traffic": int(GEMM_DRAM_OVER_ALGORITHMIC * counts["acc_bytes"]),
                 "traffic_how": ("%.2f x the launch's algorithmic bytes (%d): DRAM read + write of one ncu "
-                                "capture of a three-wave launch of this kernel, scaled by bytes"
+                                "capture of a three-wave, head-like launch of this kernel, scaled by bytes"
                                 % (GEMM_DRAM_OVER_ALGORITHMIC, counts["acc_bytes"]))}
     ghost = ghost_norm_alone(dp, ds, peaks, peak_tf, counts)
     big = ds.outs["wte"]
@@ -636,7 +646,7 @@ def run_ours(args):
     others = {
         "%s (dp_ghost_norms)" % ghost["kernel"]: ghost,
         "add_noise_kernel (dp_add_noise, %d elements)" % noise_n: {
-            "bound": "hbm", "note": "bound by instruction issue in practice (about 61 per element)",
+            "bound": "hbm", "note": "bound by instruction issue in practice (about 39 per element)",
             "ms": noise_ms,
             "achieved_GBs": 8 * noise_n / (noise_ms * 1e-3) / 1e9,
             "peak_GBs": peaks["hbm_gbs"], "frac": 8 * noise_n / (noise_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],

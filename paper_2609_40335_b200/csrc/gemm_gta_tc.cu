@@ -13,8 +13,8 @@
 // (packed bf16 FMAs with R_i split into two bf16 parts) between the TMA-full and MMA-ready
 // barriers; four such warps work on four consecutive stages at once.
 //
-// Roles per CTA (704 threads): warp 0 TMA producer, warp 1 MMA issuer, warps 2-5 scalers,
-// warps 6-21 epilogue (four per TMEM lane quarter, two 32-column chunks each; they also draw
+// Roles per CTA (736 threads): warps 0 and 2 TMA producers (G and A), warp 1 MMA issuer, warps 3-6 scalers,
+// warps 7-22 epilogue (four per TMEM lane quarter, two 32-column chunks each; they also draw
 // the fused Gaussian noise, which is latency-bound per warp -- hence so many); two TMEM
 // accumulators overlap the epilogue with the next tile.
 //
@@ -22,7 +22,7 @@
 // in gemm_gta_big.cu): a 256 x 256 output tile per pair,
 // each CTA loading its own 128 G rows and half of the A tile's columns, rank 0 issuing the MMAs
 // for both, stage-free and accumulator-ready signals multicast to both CTAs by tcgen05.commit,
-// scaler and epilogue warps of rank 1 arriving on rank 0's barriers.  The DIRECT-norm variant
+// scaler and epilogue warps of rank 1 signalling rank 0's barriers by asynchronous stores.  The DIRECT-norm variant
 // stays on single CTAs.
 #include <cuda.h>
 #include <cuda_bf16.h>

@@ -67,8 +67,8 @@ def test_workspace_sizes_follow_the_plan(lib):
     # one partial per (example, layer, column chunk): the head is split into several chunks
     assert n >= B * (1 + 8) * 4 and n % 256 == 0
     # fp32 layers of this size run on the tensor cores with their operands split into two bf16
-    # terms: the widened operands of the LARGEST layer (two sides, three column blocks, 2 bytes)
-    # plus its partial sums; layers too small for a tensor-core tile need nothing
+    # terms: three times the planes of the LARGEST layer (two terms, 2 bytes each) plus its
+    # partial sums; layers too small for a tensor-core tile need nothing
     f32 = lib.dp_ghost_norms_ws_bytes(d, 2, 0, B, T)
     widened = 2 * 3 * B * T * (768 + 50264) * 2
     assert widened <= f32 <= widened + (1 << 20) and f32 % 256 == 0
