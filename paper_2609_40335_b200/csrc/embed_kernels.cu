@@ -25,7 +25,6 @@ struct TokenGroups {
   int* fo;      // [n]  first occurrence
   int* rank;    // [n]  number of earlier tokens of the same group
   int* size;    // [n]  group size, at the first occurrence (0 elsewhere)
-  int* spare;   // [2n rounded up] free once the groups are known
 };
 __host__ __device__ __forceinline__ int group_slots(int n) {       // hash slots: at least 2 n
   int h = 64;
@@ -168,7 +167,7 @@ embed_norm_kernel(const int* __restrict__ ids, const T* __restrict__ G, long lon
   const int n32 = (Tn + 31) & ~31, slots = group_slots(Tn);
   int* keys = sm_i + 3 * n32;
   int* first = keys + slots;
-  const TokenGroups g{sm_i, sm_i + n32, sm_i + 2 * n32, keys, first};
+  const TokenGroups g{sm_i, sm_i + n32, sm_i + 2 * n32, keys};
   int* s_start = keys + n32;             // group start in the order, at the first occurrence
   int* s_ord = first;                    // rows in order; sign bit = group end
 
@@ -351,7 +350,7 @@ sort_one_block_kernel(const int* __restrict__ ids, int n, int V, int* __restrict
   __shared__ int wsum[33];
   const int n32 = (n + 31) & ~31, slots = group_slots(n);
   int* keys = sm_i + 3 * n32;
-  const TokenGroups g{sm_i, sm_i + n32, sm_i + 2 * n32, keys, keys + slots};
+  const TokenGroups g{sm_i, sm_i + n32, sm_i + 2 * n32, keys};
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int v = threadIdx.x; v <= V; v += kSortThreads) seg[v] = 0;
   load_ids(ids, n, V, g.id, dev_status);
@@ -406,7 +405,7 @@ sort_rank_kernel(const int* __restrict__ ids, int n, int V, int chunk_len, int* 
   const int chunk = blockIdx.x, j0 = chunk * chunk_len, m = min(chunk_len, n - j0);
   const int n32 = (m + 31) & ~31, slots = group_slots(m);
   int* keys = sm_i + 3 * n32;
-  const TokenGroups g{sm_i, sm_i + n32, sm_i + 2 * n32, keys, keys + slots};
+  const TokenGroups g{sm_i, sm_i + n32, sm_i + 2 * n32, keys};
   load_ids(ids + j0, m, V, g.id, dev_status);
   group_tokens(g, keys, keys + slots, slots, m);
   // tokens per 1024 ids, added up for the chunk first (ids below 1024 are the most frequent)
@@ -702,11 +701,9 @@ embed_scatter_combine_kernel(const int* __restrict__ ids, const int* __restrict_
         long_head = (s0 == k) && (n > kScatShort);
       }
     }
-    const unsigned m = __ballot_sync(0xffffffffu, long_head);
     if (threadIdx.x == 0) s_n = 0;
     __syncwarp();
     if (long_head) { s_v = v; s_k0 = k; s_n = n; }
-    (void)m;
   }
   __syncthreads();
   const int n = s_n;
