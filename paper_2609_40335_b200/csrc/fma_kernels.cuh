@@ -53,9 +53,11 @@ struct EmbedSortWs {
 };
 constexpr int kSortChunk = 1024;
 // One block sorts by itself in one launch instead of four, but its walk over the tokens and its scan over the ids are
-// serial.  One block and chunks, Zipf ids: 5.8 and 8.5 us at 64 tokens and 1000 ids, 14.7 and 16.4 at 2048 and 4000; 18.3 and
-// 16.7 at 3072 and 4000, 18.9 and 16.8 at 2048 and 8192, 11.2 and 8.2 at 64 and 8192.
-constexpr int kSortOneBlock = 2048, kSortOneBlockIds = 4096;
+// serial.  One block and chunks, Zipf ids, replayed as a graph: 5.8 and 8.5 us at 64 tokens and 1000 ids, 14.7 and 16.4 at 2048 and
+// 4000; 18.9 and 16.8 at 2048 and 8192, 11.2 and 8.2 at 64 and 8192, 22.6 and 17.7 at 3072 and 8192.  The line over the ids lies where a
+// small step still gains: launched call by call the three launches are 8 us of the host's time, which bounds it (34 -> 42 us at
+// 64 tokens and 4500 ids).
+constexpr int kSortOneBlock = 2048, kSortOneBlockIds = 8192;
 inline bool sort_in_one_block(int n, int V) { return n <= kSortOneBlock && V <= kSortOneBlockIds; }
 // Chunks whose counts a token adds up when it is placed; with more, sort_prefix_kernel adds them up once: 22.7 us with it
 // against 21.9 at 4 chunks, 24.9 against 25.4 at 16, 55 against 77 at 64, 0.84 against 14.7 ms at 1024 (V = 50257).

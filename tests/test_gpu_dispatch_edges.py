@@ -69,9 +69,9 @@ def test_token_sort_at_the_edges_of_its_variants(B, T, V):
     assert (got[len(want_perm):] == -7).all()
 
 
-# one block up to 2048 tokens and 4096 ids; counts of up to 8 chunks are added up token by token, of more once for
+# one block up to 2048 tokens and 8192 ids; counts of up to 8 chunks are added up token by token, of more once for
 # all; tokens per 1024 ids are counted in shared memory up to 262144 ids
-@pytest.mark.parametrize("B,T,V", [(1, 2048, 4096), (1, 2049, 4096), (1, 64, 4097), (2, 4096, 6000),
+@pytest.mark.parametrize("B,T,V", [(1, 2048, 8192), (1, 2049, 8192), (1, 64, 8193), (2, 4096, 6000),
                                    (1, 8193, 6000), (9, 4096, 1025), (8, 4097, 262144), (2, 4096, 262145), (300, 2048, 5000)])
 def test_token_sort_at_the_lines_of_its_rules(B, T, V):
     test_token_sort_at_the_edges_of_its_variants(B, T, V)
