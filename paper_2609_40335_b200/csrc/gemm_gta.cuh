@@ -32,7 +32,90 @@ struct GtaNoise {
   const uint32_t* tensor_ids;   // [n_layers]
 };
 
-// terms = 3: the operands are (2B, T, .) planes of high and low bf16 terms (fp32 inputs) and a product
+// How a clipped sum walks its contraction.  The token rows of a batch lie one after the other (row i*T + t, one
+// pitch), so the tensor map has them as one dimension and a K step is 64 consecutive rows whatever examples they
+// belong to; the scaler warps look up a clip factor per row where a step holds several.  Steps that end with
+// their example instead were filled up with zeros: at T = 203 84 steps of 64 for 21 examples, 67 now; at T = 77 two
+// steps an example, at T = 16 one, three quarters of it zeros.  The step of DistilGPT2 with all its parameters at B = 21, T = 203
+// 1383 -> 1295 us, of GPT-2 small at B = 3, T = 77 349 -> 344; at B = 32, T = 128 (the same steps) 940 -> 945, within the runs'
+// differences.  Coordinates are 32-bit: a batch of 2^31 rows keeps
+// steps per example (per_example).
+struct GtaRows {
+  int B, T;                // planes along K, rows of each, as the tensor map has them
+  bool per_example;
+};
+inline GtaRows gta_rows(int B, int T) {
+  const long long rows = (long long)B * T;
+  if (rows > 0x7fffffffLL - 64) return {B, T, true};
+  return {1, int(rows), false};
+}
+
+// Clip factors of a K step's rows: lane k holds those of rows k and k + 32.
+struct RowFactors { float lo, hi; };
+// step: K step of the contraction; rows: all token rows, 0: `tsteps` steps belong to each example
+__device__ __forceinline__ RowFactors row_factors(const float* clip, int step, int lane, int T, int rows, int tsteps) {
+  if (rows == 0) {
+    const float r = __ldg(clip + step / tsteps);
+    return {r, r};
+  }
+  const unsigned first = unsigned(step) * 64u + unsigned(lane), last = unsigned(rows) - 1u;
+  return {__ldg(clip + min(first, last) / unsigned(T)), __ldg(clip + min(first + 32u, last) / unsigned(T))};
+}
+
+// One warp multiplies a 16 KiB operand part (two boxes of 64 rows x 128 bytes; the 128-byte swizzle moves 16-byte
+// chunks inside a row only) by its rows' factors.  r = r_hi + r_lo with both parts in bf16 (16 mantissa bits in
+// total); x*r is formed as fma(x, r_hi, x*r_lo) on packed bf16 pairs: one rounding of the exact x*r_hi plus a tiny
+// correction, i.e. the correctly rounded bf16 product up to 2^-17 relative.  16-byte chunks, eight at a time.
+__device__ __forceinline__ void scale_part(uint4* part, RowFactors f, int lane) {
+  const float r = __shfl_sync(0xffffffffu, f.lo, 0);
+  const bool one = __all_sync(0xffffffffu, f.lo == r && f.hi == r);
+  if (one && r == 1.0f) return;
+  auto split = [](float x) {                       // r_hi in the low half, r_lo in the high one
+    const __nv_bfloat16 h = __float2bfloat16_rn(x), l = __float2bfloat16_rn(x - __bfloat162float(h));
+    return uint32_t(__bfloat16_as_ushort(h)) | (uint32_t(__bfloat16_as_ushort(l)) << 16);
+  };
+  const uint32_t w_lo = split(f.lo), w_hi = split(f.hi);
+  auto pair = [](uint32_t w, uint32_t sel) {
+    const uint32_t b = __byte_perm(w, w, sel);
+    return *reinterpret_cast<const __nv_bfloat162*>(&b);
+  };
+  uint4* x = part + lane;
+  if (one) {
+    const __nv_bfloat162 rh2 = pair(w_lo, 0x1010), rl2 = pair(w_lo, 0x3232);
+#pragma unroll 1
+    for (int c0 = 0; c0 < 32; c0 += 8) {
+      uint4 v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = x[(c0 + q) * 32];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&v[q]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) e[k] = __hfma2(e[k], rh2, __hmul2(e[k], rl2));
+        x[(c0 + q) * 32] = v[q];
+      }
+    }
+    return;
+  }
+#pragma unroll 1
+  for (int c0 = 0; c0 < 32; c0 += 8) {             // chunk (c0 + q) * 32 + lane lies in row 4 (c0 + q) + lane / 8 of 64
+    const uint32_t mine = (c0 & 8) ? w_hi : w_lo;
+    uint4 v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = x[(c0 + q) * 32];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const uint32_t w = __shfl_sync(0xffffffffu, mine, 4 * q + (lane >> 3));
+      const __nv_bfloat162 rh2 = pair(w, 0x1010), rl2 = pair(w, 0x3232);
+      __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&v[q]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) e[k] = __hfma2(e[k], rh2, __hmul2(e[k], rl2));
+      x[(c0 + q) * 32] = v[q];
+    }
+  }
+}
+
+// terms = 3: the operands are planes of high and, behind them all, of low bf16 terms (fp32 inputs) and a product
 // takes three K steps per 64 tokens; terms = 1: plain bf16 operands.
 //
 // Order of a contraction's K steps.  With three terms, first lo hi' and hi lo' of all its 64-token blocks, then
@@ -44,10 +127,10 @@ struct GtaNoise {
 // at run time the step of GPT-2 medium at B = 16, T = 128 came out 0.4 % slower than with a fixed order, in this form 0.4 % faster.
 template <bool kSplit>
 struct GtaWalk {
-  int ex, ts, tblocks;                 // example, block in it, blocks per example
+  int ex, ts, tblocks;                 // plane (example, or all of them), block in it, blocks per plane
   int term = 0, ex0 = 0, ts0 = 0, left = 0;      // split: which product, where the contraction starts, blocks left in this round
 
-  // blocks [b0, b1), counted from example `first`
+  // blocks [b0, b1), counted from plane `first`
   __device__ __forceinline__ GtaWalk(int first, int b0, int b1, int tblocks_) : tblocks(tblocks_) {
     ex = first + b0 / tblocks;
     ts = b0 % tblocks;
@@ -60,8 +143,8 @@ struct GtaWalk {
     term = 0;
     if (--left == 0) { ex = ex0; ts = ts0; term = 2; }
   }
-  // plane of the A or G operand
-  __device__ __forceinline__ int plane(bool is_a) const { return kSplit ? 2 * ex + (term == (is_a ? 0 : 1)) : ex; }
+  // plane of the A or G operand; `low`: the first plane of low terms
+  __device__ __forceinline__ int plane(bool is_a, int low) const { return kSplit && term == (is_a ? 0 : 1) ? ex + low : ex; }
 };
 
 long long gta_tiles(const dp_linear_desc& L);           // output tiles of one layer

@@ -79,7 +79,9 @@ struct __align__(64) BigParams {
   CUtensorMap tmA[kGtaMaxLayers];
   BigLayer layer[kGtaMaxLayers];
   int n_layers;
-  int tsteps, ksteps;        // K steps per example (split fp32: three per 64 tokens), K steps in all
+  int tsteps, ksteps;        // K steps per plane (split fp32: three per 64 tokens), K steps in all
+  int low_plane;             // split operands: first plane of low terms
+  int example_rows, rows;    // scaling: tokens per example, all rows (0: steps per example)
   int skew;                  // K steps that sub-tile 1 of an item lags behind
   int n_big, n_big_total;    // two-tile items run as such, and in all (the rest as two singles each)
   int total_items;
@@ -230,7 +232,7 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
           if (go)
 #pragma unroll
             for (int b = 0; b < kHalf / 64; ++b)
-              ptx::tma_load_3d_a(dst + b * kBoxBytes, tm, bar, c0 + b * 64, at.ts * kBK, at.plane(!is_g));
+              ptx::tma_load_3d_a(dst + b * kBoxBytes, tm, bar, c0 + b * 64, at.ts * kBK, at.plane(!is_g, P.low_plane));
         }
         __syncwarp();
         ++issued;
@@ -304,8 +306,8 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
     }
   } else if (warp < kEpiWarp0) {
     // ------------------------------------------------------------------ scalers
-    // Every scaler warp owns every fourth K step: it waits for the stage, multiplies X by the example's
-    // clip factor where that has not been done yet, and tells rank 0's issuer (see gemm_gta_tc.cu for the
+    // Every scaler warp owns every fourth K step: it waits for the stage, multiplies X's rows by their
+    // examples' clip factors where that has not been done yet, and tells rank 0's issuer (see gemm_gta_tc.cu for the
     // barriers' reasoning: the wait on `empty` makes the parity of `full` exact).
     const int sw = warp - kScalerWarp0;
     const uint32_t ready_remote = ptx::mapa_u32(ready_a, 0);
@@ -317,38 +319,21 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
       const Item it = decode_item(P, item, lay);
       const bool scale_here = P.clip && !P.layer[it.layer].prescaled;
       const int steps = P.ksteps + (it.nsub == 2 ? P.skew : 0);
-      auto factor = [&](int j) {               // clip factor of step j (the last `skew` steps are the first again)
-        return (scale_here && j < steps) ? __ldg(P.clip + (j < P.ksteps ? j : j - P.ksteps) / P.tsteps) : 1.f;
+      auto factors = [&](int j) {              // of step j (the last `skew` steps are the first again)
+        if (!scale_here || j >= steps) return RowFactors{1.f, 1.f};
+        return row_factors(P.clip, j < P.ksteps ? j : j - P.ksteps, lane, P.example_rows, P.rows, P.tsteps);
       };
       int j = int((uint32_t(sw) + kScalerWarps - cnt % kScalerWarps) % kScalerWarps);
       uint32_t c = cnt + uint32_t(j);
-      float r_next = factor(j);
+      RowFactors r_next = factors(j);
       for (; j < steps; j += kScalerWarps, c += kScalerWarps) {
-        const float r = r_next;
-        r_next = factor(j + kScalerWarps);
+        const RowFactors r = r_next;
+        r_next = factors(j + kScalerWarps);
         const uint32_t stage = c % kStages, fill = c / kStages, phase = fill & 1u;
         if (fill > 0 && !ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
         if (!ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit)) { ok = false; break; }
-        if (r != 1.0f) {
-          // r = r_hi + r_lo with both parts in bf16; fma(x, r_hi, x*r_lo) on packed pairs is the
-          // correctly rounded bf16 product up to 2^-17 relative
-          const __nv_bfloat16 rh = __float2bfloat16_rn(r);
-          const __nv_bfloat16 rl = __float2bfloat16_rn(r - __bfloat162float(rh));
-          const __nv_bfloat162 rh2 = __halves2bfloat162(rh, rh), rl2 = __halves2bfloat162(rl, rl);
-          uint4* x = reinterpret_cast<uint4*>(tiles + size_t(stage) * kStageBytes) + lane;
-#pragma unroll 1
-          for (int c0 = 0; c0 < kPartBytes / 16 / 32; c0 += 8) {
-            uint4 v[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = x[(c0 + q) * 32];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              __nv_bfloat162* w = reinterpret_cast<__nv_bfloat162*>(&v[q]);
-#pragma unroll
-              for (int e = 0; e < 4; ++e) w[e] = __hfma2(w[e], rh2, __hmul2(w[e], rl2));
-              x[(c0 + q) * 32] = v[q];
-            }
-          }
+        if (scale_here) {
+          scale_part(reinterpret_cast<uint4*>(tiles + size_t(stage) * kStageBytes), r, lane);
           ptx::fence_proxy_async_smem();
         }
         __syncwarp();
@@ -495,13 +480,14 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
                          const GtaNoise* noise, int* dev_status, cudaStream_t st) {
   BigParams P;
   memset(&P, 0, sizeof(P));
-  const int planes = terms > 1 ? 2 * B : B;
+  const GtaRows K = gta_rows(B, T);
+  const int planes = terms > 1 ? 2 * K.B : K.B;
   int bigs = 0, singles = 0;
   for (int k = 0; k < n; ++k) {
     const GtaBigJob& J = jobs[k];
-    dp_status s = make_tmap_bf16_3d(&P.tmG[k], J.G, J.ldg, J.p, T, planes, 64, kBK);
+    dp_status s = make_tmap_bf16_3d(&P.tmG[k], J.G, J.ldg, J.p, K.T, planes, 64, kBK);
     if (s != DP_OK) return s;
-    s = make_tmap_bf16_3d(&P.tmA[k], J.A, J.lda, J.d, T, planes, 64, kBK);
+    s = make_tmap_bf16_3d(&P.tmA[k], J.A, J.lda, J.d, K.T, planes, 64, kBK);
     if (s != DP_OK) return s;
     BigLayer& L = P.layer[k];
     L.out = J.out; L.ldo = J.ldo; L.M = J.p; L.N = J.d;
@@ -524,7 +510,8 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
   P.n_big = (rest && convert < keep) ? bigs - rest : bigs;
   P.total_items = P.n_big + 2 * (bigs - P.n_big) + singles;
   P.n_layers = n;
-  P.tsteps = terms * ceil_div(T, kBK); P.ksteps = B * P.tsteps;
+  P.tsteps = terms * ceil_div(K.T, kBK); P.ksteps = K.B * P.tsteps; P.low_plane = K.B;
+  P.example_rows = T; P.rows = K.per_example ? 0 : K.T;
   // Long enough to read one accumulator, and to draw its noise, while the other is fed: with noise 4, 6, 8,
   // 10, 12, 24 and 40 steps gave 2341, 2278, 2252, 2265, 2283, 2407 and 2513 us (B = 16, T = 512).  The same
   // without noise, which would do with 2 or none, so that a sum does not depend on whether noise is fused.

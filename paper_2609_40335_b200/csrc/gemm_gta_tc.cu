@@ -7,11 +7,11 @@
 //
 // Both operands are contiguous along M / N (token rows are the K dimension), so shared
 // memory holds MN-major tiles: every TMA box is 64 token rows x 64 columns (128-byte rows,
-// 128-byte swizzle).  A K step never straddles two examples (the tensor map is 3-D:
-// column, token, example; the token tail of an example is zero-filled), so one clip factor
-// applies to a whole stage: a "scaler" warp multiplies the G tile by R_i in shared memory
-// (packed bf16 FMAs with R_i split into two bf16 parts) between the TMA-full and MMA-ready
-// barriers; four such warps work on four consecutive stages at once.
+// 128-byte swizzle).  In (a) the K steps run over the rows of the whole batch (see GtaRows), in (b)
+// over one example's (tensor map column, token, example; its token tail is zero-filled).  A "scaler" warp
+// multiplies the rows of a G tile by their R_i in shared memory (packed bf16 FMAs with R_i split into two
+// bf16 parts) between the TMA-full and MMA-ready barriers; four such warps work on four consecutive stages
+// at once.
 //
 // Roles per CTA (736 threads): warps 0 and 2 TMA producers (G and A), warp 1 MMA issuer, warps 3-6 scalers,
 // warps 7-22 epilogue (four per TMEM lane quarter, two 32-column chunks each; they also draw
@@ -73,7 +73,9 @@ struct __align__(64) GtaParams {
   CUtensorMap tmA[kGtaMaxLayers];
   GtaLayer layer[kGtaMaxLayers];
   int n_layers;
-  int B, T, tsteps;          // tsteps = terms * ceil(T / 64) K steps per example
+  int B, T, tsteps;          // planes along K and rows of each; tsteps = terms * ceil(T / 64) K steps per plane
+  int low_plane;             // split operands: first plane of low terms
+  int example_rows, rows;    // scaling: tokens per example, all rows (0: steps per example)
   int nsplit, ksteps_per_split;   // K splits, the same for all layers of a call; multiples of `terms` steps
   float beta;
   int total_items;
@@ -204,7 +206,7 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
           const uint32_t dst = tiles_a + stage * kStageBytes + (is_a ? kGBytes : 0);
           ptx::mbar_arrive_expect_tx_a(bar, my_bytes);
           for (int j = 0; j < nbox; ++j)
-            ptx::tma_load_3d_a(dst + j * kBoxBytes, tm, bar, c0 + j * 64, at.ts * kBK, at.plane(is_a));
+            ptx::tma_load_3d_a(dst + j * kBoxBytes, tm, bar, c0 + j * 64, at.ts * kBK, at.plane(is_a, P.low_plane));
           ++issued;
           at.next();
           if (++stage == kStages) { stage = 0; phase ^= 1; }
@@ -292,11 +294,13 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
         uint32_t c = cnt + uint32_t(ks - it.k0);
         // no scaling here when the operand arrives scaled: clip == NULL (the split fp32 path) or a
         // layer whose narrow operand was multiplied by R_i in a pass of its own (see prescale)
-        float r_next = (scale_here && ks < it.k1) ? __ldg(P.clip + ks / P.tsteps) : 1.f;
+        RowFactors r_next{1.f, 1.f};
+        if (scale_here && ks < it.k1) r_next = row_factors(P.clip, ks, lane, P.example_rows, P.rows, P.tsteps);
         for (; ks < it.k1; ks += kScalerWarps, c += kScalerWarps) {
-          const float r = r_next;
-          // the factor of this warp's next K step is fetched before the waits, off the stage's path
-          if (scale_here && ks + kScalerWarps < it.k1) r_next = __ldg(P.clip + (ks + kScalerWarps) / P.tsteps);
+          const RowFactors r = r_next;
+          // the factors of this warp's next K step are fetched before the waits, off the stage's path
+          if (scale_here && ks + kScalerWarps < it.k1)
+            r_next = row_factors(P.clip, ks + kScalerWarps, lane, P.example_rows, P.rows, P.tsteps);
           const uint32_t stage = c % kStages, fill = c / kStages, phase = fill & 1u;
           // A warp hops between stages, so it has not seen the previous fill of this one, and the
           // parity of `full` alone cannot tell "fill n landed" from "fill n-1 still in flight".
@@ -305,29 +309,8 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
           // or "fill n landed".
           if (fill > 0 && !ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
           if (!ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit)) { ok = false; break; }
-          if (r != 1.0f) {
-            // r = r_hi + r_lo with both parts in bf16 (16 mantissa bits in total); g*r is formed
-            // as fma(g, r_hi, g*r_lo) on packed bf16 pairs: one rounding of the exact g*r_hi plus
-            // a tiny correction, i.e. the correctly rounded bf16 product up to 2^-17 relative.
-            const __nv_bfloat16 rh = __float2bfloat16_rn(r);
-            const __nv_bfloat16 rl = __float2bfloat16_rn(r - __bfloat162float(rh));
-            const __nv_bfloat162 rh2 = __halves2bfloat162(rh, rh), rl2 = __halves2bfloat162(rl, rl);
-            // kChunks 16-byte chunks per lane, eight at a time
-            constexpr int kChunks = kGBytes / 16 / 32;
-            uint4* g = reinterpret_cast<uint4*>(tiles + size_t(stage) * kStageBytes) + lane;
-#pragma unroll 1
-            for (int c0 = 0; c0 < kChunks; c0 += 8) {
-              uint4 v[8];
-#pragma unroll
-              for (int q = 0; q < 8; ++q) v[q] = g[(c0 + q) * 32];
-#pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                __nv_bfloat162* w = reinterpret_cast<__nv_bfloat162*>(&v[q]);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) w[e] = __hfma2(w[e], rh2, __hmul2(w[e], rl2));
-                g[(c0 + q) * 32] = v[q];
-              }
-            }
+          if (scale_here) {
+            scale_part(reinterpret_cast<uint4*>(tiles + size_t(stage) * kStageBytes), r, lane);
             ptx::fence_proxy_async_smem();
           }
           __syncwarp();
@@ -660,11 +643,12 @@ static long long gta_tiles(const dp_linear_desc* layers, int n_layers) {
 bool gta_prescales(const dp_linear_desc& L) { return prescale_layer(L); }
 
 int gta_choose_nsplit(long long tiles, int B, int T, int terms, int sms) {
-  const int ksteps = B * terms * ceil_div(T, kBK);
+  const GtaRows K = gta_rows(B, T);
+  const int ksteps = K.B * terms * ceil_div(K.T, kBK);
   const int units = kUsePair ? sms / 2 : sms;          // persistent CTAs or CTA pairs
   if (tiles >= 2LL * units) return 1;
   long long ns = std::max<long long>(1, (2LL * units) / std::max<long long>(tiles, 1));
-  ns = std::min<long long>(ns, std::max(1, ksteps / 4));
+  ns = std::min<long long>(ns, std::max(1, (ksteps + terms - 1) / 4));      // a split is whole blocks of `terms` steps
   return (int)std::max<long long>(1, ns);
 }
 
@@ -684,8 +668,9 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
                                     int* dev_status, cudaStream_t st) {
   dp_status s = DP_OK;
   const int sms = sm_count();
-  const int tsteps = terms * ceil_div(T, kBK), planes = terms > 1 ? 2 * B : B;
-  const int ksteps = B * tsteps;
+  const GtaRows K = gta_rows(B, T);
+  const int tsteps = terms * ceil_div(K.T, kBK), planes = terms > 1 ? 2 * K.B : K.B;
+  const int ksteps = K.B * tsteps;
   int nsplit = gta_choose_nsplit(gta_tiles(layers, n_layers), B, T, terms, sms);
   const int kps = terms * ceil_div(ksteps / terms, nsplit);   // whole 64-token blocks
   nsplit = ceil_div(ksteps, kps);                       // drop empty trailing splits
@@ -725,9 +710,9 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
         L.prescaled = 1;
       }
       if (!use_big) {
-        s = make_tmap_bf16_3d(&P.tmG[g - g0], D.G, D.ldg, D.p, T, planes, 64, kBK);
+        s = make_tmap_bf16_3d(&P.tmG[g - g0], D.G, D.ldg, D.p, K.T, planes, 64, kBK);
         if (s != DP_OK) return s;
-        s = make_tmap_bf16_3d(&P.tmA[g - g0], D.A, D.lda, D.d, T, planes, 64, kBK);
+        s = make_tmap_bf16_3d(&P.tmA[g - g0], D.A, D.lda, D.d, K.T, planes, 64, kBK);
         if (s != DP_OK) return s;
       }
       L.out = outs[g]; L.ldo = ldos[g];
@@ -752,7 +737,8 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
       P.noise_step = noise->step; P.noise_scale = noise->scale;
       P.step_dev = g_step_dev;
     }
-    P.n_layers = g1 - g0; P.B = B; P.T = T; P.tsteps = tsteps;
+    P.n_layers = g1 - g0; P.B = K.B; P.T = K.T; P.tsteps = tsteps; P.low_plane = K.B;
+    P.example_rows = T; P.rows = K.per_example ? 0 : K.T;
     P.total_items = items;
     P.nsplit = nsplit; P.ksteps_per_split = kps; P.beta = beta;
     P.clip = clip;
@@ -820,7 +806,7 @@ dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& p
       items += B * plan.direct[li].tiles_m * plan.direct[li].tiles_n;
     }
     P.n_layers = int(g1 - g0);
-    P.B = B; P.T = T; P.tsteps = terms * ceil_div(T, kBK);
+    P.B = B; P.T = T; P.tsteps = terms * ceil_div(T, kBK); P.low_plane = B;
     P.total_items = items;
     P.nsplit = 1;
     P.sq_partials = partials; P.n_per = plan.n_per;

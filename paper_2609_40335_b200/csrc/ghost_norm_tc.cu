@@ -95,7 +95,7 @@ __device__ __forceinline__ uint32_t add_f32(uint32_t a, uint32_t b) {
   return __float_as_uint(__uint_as_float(a) + __uint_as_float(b));
 }
 
-// kSplit: fp32 operands stored as two bf16 planes per example (see split_kernels.cu).  Every Gram
+// kSplit: fp32 operands stored as bf16 planes of high and low terms (see split_kernels.cu).  Every Gram
 // tile is then S = hi hi^T + hi lo^T + lo hi^T, three MMAs per K step on tiles loaded once.  An MMA rounds its sum
 // towards zero, by as much as the sum is large, and the diagonal of S is a sum of positive terms: the two small
 // products have an accumulator of their own, the second buffer's, which leaves a third of the roundings.
@@ -160,7 +160,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
       const Item it = decode_item(P, item, lay);
       const bool diag = kDiagOnly || (it.ti == it.tj);
       const uint32_t bytes = diag ? term_bytes : stage_bytes;
-      const int ex = kSplit ? 2 * it.example : it.example;     // (high) plane of the example
+      const int ex = it.example, low = ex + P.B;               // planes of the example (split: high and low terms)
       for (int pass = 0; pass < 2 && ok; ++pass) {
         const uint64_t tm = reinterpret_cast<uint64_t>(pass == 0 ? &P.tmA[it.layer] : &P.tmG[it.layer]);
         const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
@@ -176,12 +176,12 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
               if (b >= nb) break;
               ptx::tma_load_3d_a(dst + b * term_bytes, tm, bar, (k + b) * kKStep, it.ti * kTile, ex);
               if (kSplit)
-                ptx::tma_load_3d_a(dst + b * term_bytes + tile_bytes, tm, bar, (k + b) * kKStep, it.ti * kTile, ex + 1);
+                ptx::tma_load_3d_a(dst + b * term_bytes + tile_bytes, tm, bar, (k + b) * kKStep, it.ti * kTile, low);
             }
             if (!diag) {
               ptx::tma_load_3d_a(dst + term_bytes, tm, bar, k * kKStep, it.tj * kTile, ex);
               if (kSplit)
-                ptx::tma_load_3d_a(dst + term_bytes + tile_bytes, tm, bar, k * kKStep, it.tj * kTile, ex + 1);
+                ptx::tma_load_3d_a(dst + term_bytes + tile_bytes, tm, bar, k * kKStep, it.tj * kTile, low);
             }
           }
           __syncwarp();

@@ -47,7 +47,7 @@ GhostPlan plan_ghost_norms(const dp_linear_desc* layers, int n_layers, int B, in
 dp_status launch_ghost_norm_pair(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
                                  float* partials, int* dev_status, cudaStream_t st);
 
-// split: the operands are (2B, T, .) planes of high and low bf16 terms (fp32 inputs).
+// split: the operands are (2, B, T, .) planes of high and of low bf16 terms (fp32 inputs).
 dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
                                float* partials, int* dev_status, cudaStream_t st, bool split = false);
 

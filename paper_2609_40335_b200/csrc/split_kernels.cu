@@ -5,9 +5,9 @@
 // the "3 x TF32" scheme with 16 instead of 21 mantissa bits, far inside the 1e-4 the fp32 path has
 // to meet, and at three bf16 MMAs cheaper than three TF32 MMAs (which run at half the bf16 rate).
 //
-// An operand is stored once, as two planes per example (as many bytes as the fp32 original); the
-// Gram and G^T A kernels pick the plane of each side of each product by the tensor map's example
-// coordinate.  (Widened copies [hi | hi | lo] and [hi | lo | hi] took three to six times the
+// An operand is stored once, the high terms of all examples and behind them the low ones (as many bytes as the fp32
+// original); the Gram and G^T A kernels pick the plane of each side of each product by the tensor map's outer
+// coordinate, and a contraction over tokens finds the rows of all examples in one piece.  (Widened copies [hi | hi | lo] and [hi | lo | hi] took three to six times the
 // workspace and traffic and, the workspace being sized for one layer, a dozen launches per layer:
 // 24 layers and a head of DistilGPT2 at B = 8, T = 128 took 236 launches, now 12.)
 // For the clipped sum the clip factor R_i (Eq. 7) multiplies the narrower operand in fp32 BEFORE the
@@ -54,7 +54,7 @@ split_kernel(const __grid_constant__ SplitParams P) {
   const bool vec = ((reinterpret_cast<uintptr_t>(S.src) & 15) == 0) && ((S.lds & 3) == 0);
   const long long total = P.rows * S.per_row;
   const long long first = (long long)(int(blockIdx.x) - S.block_begin) * kChunksPerBlock;
-  const size_t plane = size_t(P.T) * S.per_row * 8;        // elements of one plane
+  const size_t plane = size_t(P.rows) * S.per_row * 8;     // elements of the high terms
   const long long row0 = first / S.per_row;                // the block's first row and chunk in it
   const unsigned off0 = unsigned(first - row0 * S.per_row);
 #pragma unroll
@@ -64,11 +64,10 @@ split_kernel(const __grid_constant__ SplitParams P) {
     if (first + k * 256 + threadIdx.x >= total) break;
     const unsigned r = unsigned(row0) + dr;                // token row i*T + t
     const int col = int(off - dr * S.per_row) * 8;
-    const int i = int(r / unsigned(P.T)), t = int(r - unsigned(i) * P.T);
     float v[8];
     load8<float>(S.src + (long long)r * S.lds + col, S.c - col, vec, v);      // columns >= c read as zero
     if (S.scaled) {
-      const float f = __ldg(P.clip + i);
+      const float f = __ldg(P.clip + r / unsigned(P.T));
 #pragma unroll
       for (int j = 0; j < 8; ++j) v[j] *= f;
     }
@@ -81,7 +80,7 @@ split_kernel(const __grid_constant__ SplitParams P) {
       const float2 b = __bfloat1622float2(h2[j]);
       l2[j] = __floats2bfloat162_rn(v[2 * j] - b.x, v[2 * j + 1] - b.y);
     }
-    __nv_bfloat16* d = S.dst + size_t(2 * i) * plane + size_t(t) * S.per_row * 8 + col;
+    __nv_bfloat16* d = S.dst + size_t(r) * S.per_row * 8 + col;
     *reinterpret_cast<uint4*>(d) = h;
     *reinterpret_cast<uint4*>(d + plane) = l;
   }

@@ -7,8 +7,7 @@ namespace dpg {
 
 // operand width rounded up to 8 columns (a 16-byte pitch for the TMA tensor maps)
 inline int split_padded(int c) { return (c + 7) / 8 * 8; }
-// bytes of one split operand: (2B, T, padded(c)) bf16, plane 2i the high and 2i+1 the low terms of
-// example i
+// bytes of one split operand: (2, B, T, padded(c)) bf16, the high terms of all examples, then the low ones
 inline size_t split_bytes(long long rows, int c) {
   return align_up(size_t(rows) * 2 * size_t(split_padded(c)) * 2, 256);
 }

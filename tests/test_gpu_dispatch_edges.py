@@ -188,6 +188,22 @@ def test_two_tile_items(shapes, beta, noise, B, T):
     assert int(st.item()) == 0
 
 
+# K steps run over the rows of the whole batch: one example or many per 64 rows, a step that begins and ends inside
+# one, the last step short; the one-tile kernel (K split and not), the two-tile one, either operand scaled
+@pytest.mark.parametrize("B,T", [(1, 1), (70, 1), (37, 3), (9, 16), (5, 63), (5, 65), (3, 100), (4, 203), (2, 320)])
+@pytest.mark.parametrize("d,p", [(64, 72), (768, 14300), (14300, 768)])
+def test_every_row_gets_its_own_clip_factor(B, T, d, p):
+    layer = dp.Linear(bf16((B, T, d), 1.0, T, ld=(d + 7) // 8 * 8), bf16((B, T, p), 0.1, B, ld=(p + 7) // 8 * 8), d=d, p=p)
+    clip = torch.tensor([2.0 ** -(i % 5) for i in range(B)], device="cuda")
+    out, st = torch.empty(p, d, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    dp.dp_clip_accumulate_grouped([layer], B, T, None, 1.0, [out], clip=clip, dev_status=st)
+    g = layer.G[..., :p].double() * clip.double()[:, None, None]
+    want = g.reshape(-1, p).T @ layer.A[..., :d].double().reshape(-1, d)
+    # powers of two: R_i * x is exact in bf16, what is left is fp32 accumulation
+    assert float((out.double() - want).norm() / want.norm()) < 1e-5
+    assert int(st.item()) == 0
+
+
 def test_two_tile_items_give_up_cleanly():
     """A wait limit of zero: the kernel flags DP_DEV_TIMEOUT and returns; the same call then succeeds."""
     B, T, d, p = 32, 128, 512, 19000               # long enough a contraction that some wait is not over at once
