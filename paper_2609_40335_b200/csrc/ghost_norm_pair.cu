@@ -15,6 +15,12 @@
 // next item before S_G is complete, and they multiply S_G against those registers while the next
 // item's S_A is being accumulated.
 //
+// Row blocks are as tall as the sequence needs: ceil(T / 256) blocks of equal height, in steps of 32 rows (kHalf
+// rows from each CTA; the N of an MMA is the block's height, its M stays 256, the rows beyond are nobody's).
+// With blocks of 256 rows the last one was multiplied, and its zeros written to shared memory, as if it were full.
+// Where all of T is one block every tile pair is a diagonal one (kDiag) and a stage holds two column steps of it.
+// DistilGPT2 at B = 21, T = 203 (blocks of 224 rows): step 1297 -> 1276 us; T a multiple of 256: no difference.
+//
 // Roles per CTA (640 threads): warp 0 TMA producer, warp 1 MMA issuer (rank 0 only), warp 2 tells
 // rank 0 that this CTA's half of a stage has landed, warp 3 idle, warps 4..19 epilogue (four per
 // TMEM lane quarter, 64 columns each).  Every wait is bounded.
@@ -33,24 +39,31 @@ namespace dpg {
 
 namespace {
 
-constexpr int kRows = 128;                        // rows of a block that one CTA supplies
-constexpr int kTile2 = 2 * kRows;                 // Gram tile edge of the pair
+constexpr int kMmaRows = 128;                     // rows that an MMA reads of each CTA's first operand
+constexpr int kTile2 = 2 * kMmaRows;              // largest block height; columns of one accumulator
 constexpr int kKStep = 64;                        // bf16 columns per stage row (128 bytes)
-constexpr int kTileBytes = kRows * kKStep * 2;    // 16 KiB
-constexpr int kStageBytes = 2 * kTileBytes;       // rows of block I, rows of block J
-constexpr int kStages = 7;
-constexpr size_t kSmemBytes = size_t(kStages) * kStageBytes + 1024 /*alignment slack*/ + 1024;
+constexpr int kRingBytes = 7 * 32 * 1024;
+constexpr size_t kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 1024;
+
+// kHalf: rows of a block that one CTA supplies, a multiple of 16
+template <int kHalf>
+struct Geo {
+  static constexpr int kBlock = 2 * kHalf;                 // rows of a block, edge of a Gram tile
+  static constexpr int kTileBytes = kHalf * kKStep * 2;
+  static constexpr int kStageBytes = 2 * kTileBytes;       // rows of block I and of block J, or two column steps of one
+  // the MMAs of the last tile read kMmaRows rows as well
+  static constexpr int kStages = (kRingBytes - (kMmaRows - kHalf) * kKStep * 2) / kStageBytes;
+};
 constexpr int kEpiWarp0 = 4, kEpiWarps = 16;
 constexpr int kThreads = (kEpiWarp0 + kEpiWarps) * 32;
 constexpr int kTmemCols = 512;
-constexpr int kColsPerWarp = kTile2 / (kEpiWarps / 4);    // 64
 
 struct __align__(64) PairParams {
   CUtensorMap tmA[kGhostMaxLayers];
   CUtensorMap tmG[kGhostMaxLayers];
   GhostLayerPlan layer[kGhostMaxLayers];
   int n_layers;
-  int B, T, nt, ntp;         // nt = ceil(T / 256) row blocks, ntp = nt (nt + 1) / 2 tile pairs
+  int B, T, nt, ntp;         // nt row blocks, ntp = nt (nt + 1) / 2 tile pairs
   int total_items;
   int n_per;
   float* partials;           // [B][n_per]; an item owns two consecutive slots (one per CTA)
@@ -90,15 +103,19 @@ __device__ __forceinline__ Item decode_item(const PairParams& P, int item, int& 
   return it;
 }
 
+template <int kHalf, bool kDiag>
 __global__ void __launch_bounds__(kThreads, 1)
 ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
+  using G = Geo<kHalf>;
+  constexpr int kStages = G::kStages, kStageBytes = G::kStageBytes, kTileBytes = G::kTileBytes;
+  constexpr int kSteps = kDiag ? 2 : 1;            // column steps per stage
   const uint32_t rank = ptx::cluster_ctarank();
   const int first_item = int(blockIdx.x >> 1);
   const int item_stride = int(gridDim.x >> 1);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                               ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + size_t(kStages) * kStageBytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + kRingBytes);
   uint64_t* full = bars;                       // [kStages] this CTA's TMA landed
   uint64_t* ready = bars + kStages;            // [kStages] both CTAs' tiles landed (rank 0's copy)
   uint64_t* empty = bars + 2 * kStages;        // [kStages] MMAs retired
@@ -147,21 +164,22 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
     bool ok = true;
     for (int item = first_item; item < P.total_items && ok; item += item_stride) {
       const Item it = decode_item(P, item, lay);
-      const bool diag = it.ti == it.tj;
-      const uint32_t bytes = diag ? kTileBytes : kStageBytes;
-      const int row_i = it.ti * kTile2 + int(rank) * kRows;     // this CTA's rows of block I
-      const int row_j = it.tj * kTile2 + int(rank) * kRows;     // and of block J
+      const bool diag = kDiag || it.ti == it.tj;
+      const int row_i = it.ti * G::kBlock + int(rank) * kHalf;  // this CTA's rows of block I
+      const int row_j = it.tj * G::kBlock + int(rank) * kHalf;  // and of block J
       for (int pass = 0; pass < 2 && ok; ++pass) {
         const uint64_t tm = reinterpret_cast<uint64_t>(pass == 0 ? &P.tmA[it.layer] : &P.tmG[it.layer]);
         const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
-        for (int k = k0; k < k1; ++k) {
+        for (int k = k0; k < k1; k += kSteps) {
           ok = ptx::warp_ok(ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit));
           if (!ok) break;
           const uint32_t dst = tiles_a + stage * kStageBytes, bar = full_a + 8 * stage;
+          const bool second = kDiag ? k + 1 < k1 : !diag;
           if (ptx::elect_one()) {
-            ptx::mbar_arrive_expect_tx_a(bar, bytes);
+            ptx::mbar_arrive_expect_tx_a(bar, second ? kStageBytes : kTileBytes);
             ptx::tma_load_3d_a(dst, tm, bar, k * kKStep, row_i, it.example);
-            if (!diag) ptx::tma_load_3d_a(dst + kTileBytes, tm, bar, k * kKStep, row_j, it.example);
+            if (second)
+              ptx::tma_load_3d_a(dst + kTileBytes, tm, bar, (kDiag ? k + 1 : k) * kKStep, kDiag ? row_i : row_j, it.example);
           }
           __syncwarp();
           ++issued;
@@ -177,7 +195,7 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
   } else if (warp == 1) {
     // --------------------------------------------------------------- MMA issuer
     if (rank == 0) {
-      constexpr uint32_t idesc = ptx::idesc_bf16_f32(kTile2, kTile2, 0, 0);
+      constexpr uint32_t idesc = ptx::idesc_bf16_f32(kTile2, G::kBlock, 0, 0);
       constexpr uint64_t dbase = ptx::smem_desc_base(16, 1024, ptx::SWIZZLE_128B);   // K-major
       constexpr uint32_t desc_hi = uint32_t(dbase >> 32);
       const uint32_t desc_lo0 = uint32_t(dbase) | ((tiles_a >> 4) & 0x3FFF);
@@ -187,7 +205,7 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
       bool ok = true;
       for (int item = first_item; item < P.total_items && ok; item += item_stride, ++n_item) {
         const Item it = decode_item(P, item, lay);
-        const bool diag = it.ti == it.tj;
+        const bool diag = kDiag || it.ti == it.tj;
         const uint32_t ph = n_item & 1;
         for (int pass = 0; pass < 2 && ok; ++pass) {
           // the accumulator of this pass must have been read out for the previous item
@@ -197,7 +215,7 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
           ptx::tc_fence_after();
           const uint32_t d_tmem = tmem_base + pass * kTile2;
           const int nsteps = pass == 0 ? it.a1 - it.a0 : it.g1 - it.g0;
-          for (int k = 0; k < nsteps; ++k) {
+          for (int k = 0; k < nsteps; k += kSteps) {
             ok = ptx::warp_ok(ptx::mbar_wait_cluster_a(ready_a + 8 * stage, phase, abort_flag, P.wait_limit));
             if (!ok) break;
             ptx::tc_fence_after();
@@ -207,8 +225,14 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
 #pragma unroll
               for (int kk = 0; kk < kKStep / 16; ++kk)
                 ptx::mma_bf16_ss_pair_lh(d_tmem, sa + kk * 2, sb + kk * 2, desc_hi, idesc, (k > 0 || kk > 0) ? 1u : 0u);
+              if (kDiag && k + 1 < nsteps) {
+                const uint32_t s1 = sa + (kTileBytes >> 4);
+#pragma unroll
+                for (int kk = 0; kk < kKStep / 16; ++kk)
+                  ptx::mma_bf16_ss_pair_lh(d_tmem, s1 + kk * 2, s1 + kk * 2, desc_hi, idesc, 1u);
+              }
               ptx::mma_commit_pair_a(empty_a + 8 * stage, 3);
-              if (k + 1 == nsteps) ptx::mma_commit_pair(pass == 0 ? sa_full : sg_full, 3);
+              if (k + kSteps >= nsteps) ptx::mma_commit_pair(pass == 0 ? sa_full : sg_full, 3);
             }
             __syncwarp();
             if (++stage == kStages) { stage = 0; phase ^= 1; }
@@ -235,8 +259,8 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
     bool ok = true;
     for (int item = first_item; item < P.total_items && ok; item += item_stride) {
       const Item it = decode_item(P, item, lay);
-      const int nsteps = (it.a1 - it.a0) + (it.g1 - it.g0);
-      for (int k = 0; k < nsteps; ++k) {
+      const int stages = (it.a1 - it.a0 + kSteps - 1) / kSteps + (it.g1 - it.g0 + kSteps - 1) / kSteps;
+      for (int k = 0; k < stages; ++k) {
         ok = ptx::warp_ok(ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit));
         if (!ok) break;
         if (ptx::elect_one()) {
@@ -255,8 +279,10 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
     // ----------------------------------------------------------------- epilogue
     const int q = warp & 3;                          // TMEM lane quarter this warp may read
     const int ew = warp - kEpiWarp0;
-    const int cg = ew >> 2;                          // which 64 of the 256 columns
-    const uint32_t t_sa = tmem_base + (uint32_t(q * 32) << 16) + cg * kColsPerWarp;
+    const int cg = ew >> 2;                          // which quarter of the columns
+    constexpr int kCols = G::kBlock / (kEpiWarps / 4), kChunks = kCols / 8;      // of a warp; in chunks of eight
+    const uint32_t t_sa = tmem_base + (uint32_t(q * 32) << 16) + cg * kCols;
+    const bool mine = q * 32 + lane < kHalf;         // a row of the block
     const uint32_t t_sg = t_sa + kTile2;
     uint32_t n_item = 0;
     int lay = 0;
@@ -267,9 +293,9 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
       // S_A -> registers, then the accumulator is free for the next item
       if (!ptx::mbar_wait_relaxed(sa_full, ph, abort_flag, P.wait_limit)) { ok = false; break; }
       ptx::tc_fence_after();
-      uint32_t sa0[32], sa1[32];
-      ptx::tmem_ld_32x32b_x32(t_sa, sa0);
-      ptx::tmem_ld_32x32b_x32(t_sa + 32, sa1);
+      uint32_t sa[kCols];
+#pragma unroll
+      for (int c = 0; c < kChunks; ++c) ptx::tmem_ld_32x32b_x8(t_sa + c * 8, sa + c * 8);
       ptx::tmem_ld_wait();
       ptx::tc_fence_before();
       __syncwarp();
@@ -279,16 +305,16 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
       ptx::tc_fence_after();
       float acc = 0.f;
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
+      for (int c = 0; c < kChunks; c += 2) {
         uint32_t g[16];
-        ptx::tmem_ld_32x32b_x16(t_sg + c * 16, g);
+        ptx::tmem_ld_32x32b_x8(t_sg + c * 8, g);
+        if (c + 1 < kChunks) ptx::tmem_ld_32x32b_x8(t_sg + c * 8 + 8, g + 8);
         ptx::tmem_ld_wait();
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const uint32_t a = (c < 2) ? sa0[(c & 1) * 16 + j] : sa1[(c & 1) * 16 + j];
-          acc = fmaf(__uint_as_float(a), __uint_as_float(g[j]), acc);
-        }
+        for (int j = 0; j < (c + 1 < kChunks ? 16 : 8); ++j)
+          acc = fmaf(__uint_as_float(sa[c * 8 + j]), __uint_as_float(g[j]), acc);
       }
+      if (kHalf < kMmaRows && !mine) acc = 0.f;      // whatever lay in the rows beyond
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive_cluster(sg_empty, 0);
@@ -323,13 +349,35 @@ ghost_norm_pair_kernel(const __grid_constant__ PairParams P) {
   }
 }
 
+template <int kHalf, bool kDiag>
+dp_status launch_variant(const PairParams& P, cudaStream_t st) {
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_pair_kernel<kHalf, kDiag>)))
+    DP_CUDA_OK((allow_shared(ghost_norm_pair_kernel<kHalf, kDiag>, kSmemBytes)));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * std::min(P.total_items, sm_count() / 2), 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  DP_CUDA_OK(cudaLaunchKernelEx(&cfg, ghost_norm_pair_kernel<kHalf, kDiag>, P));
+  ++g_kernel_launches;
+  return DP_OK;
+}
+
+template <int kHalf>
+dp_status launch_half(const PairParams& P, cudaStream_t st) {
+  return P.nt == 1 ? launch_variant<kHalf, true>(P, st) : launch_variant<kHalf, false>(P, st);
+}
+
 }  // namespace
 
 dp_status launch_ghost_norm_pair(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
                                  float* partials, int* dev_status, cudaStream_t st) {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_pair_kernel)))
-    DP_CUDA_OK(allow_shared(ghost_norm_pair_kernel, kSmemBytes));
   const int nt = ceil_div(T, kTile2);
+  const int half = ceil_div(ceil_div(T, nt), 32) * 16;         // T > 128: 80, 96, 112 or 128
   for (size_t g0 = 0; g0 < plan.ghost_layers.size(); g0 += kGhostMaxLayers) {
     const size_t g1 = std::min(plan.ghost_layers.size(), g0 + kGhostMaxLayers);
     PairParams P;
@@ -338,9 +386,9 @@ dp_status launch_ghost_norm_pair(const dp_linear_desc* layers, const GhostPlan& 
     for (size_t g = g0; g < g1; ++g) {
       const int li = plan.ghost_layers[g];
       const dp_linear_desc& L = layers[li];
-      dp_status s = make_tmap_bf16_3d(&P.tmA[g - g0], L.A, L.lda, L.d, T, B, kKStep, kRows);
+      dp_status s = make_tmap_bf16_3d(&P.tmA[g - g0], L.A, L.lda, L.d, T, B, kKStep, half);
       if (s != DP_OK) return s;
-      s = make_tmap_bf16_3d(&P.tmG[g - g0], L.G, L.ldg, L.p, T, B, kKStep, kRows);
+      s = make_tmap_bf16_3d(&P.tmG[g - g0], L.G, L.ldg, L.p, T, B, kKStep, half);
       if (s != DP_OK) return s;
       GhostLayerPlan lp = plan.layer[li];
       lp.item_begin = items;
@@ -354,18 +402,9 @@ dp_status launch_ghost_norm_pair(const dp_linear_desc* layers, const GhostPlan& 
     P.partials = partials;
     P.dev_status = dev_status;
     P.wait_limit = g_wait_limit;
-    const int units = std::min(items, sm_count() / 2);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * units, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = kSmemBytes;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    DP_CUDA_OK(cudaLaunchKernelEx(&cfg, ghost_norm_pair_kernel, P));
-    ++g_kernel_launches;
+    const dp_status s = half <= 80 ? launch_half<80>(P, st) : half == 96 ? launch_half<96>(P, st)
+                        : half == 112 ? launch_half<112>(P, st) : launch_half<128>(P, st);
+    if (s != DP_OK) return s;
   }
   return DP_OK;
 }

@@ -465,3 +465,21 @@ def test_gram_tiles_of_short_sequences(T, dtype):
     # exact products, fp32 sums of at most 2500 terms
     assert (np.abs(sq.double().cpu().numpy() / want - 1) < 1e-5).all()
     assert int(st.item()) == 0
+
+
+# row blocks of equal height in steps of 32 rows: one, two and three blocks of every height, an odd number of column steps
+@pytest.mark.parametrize("T", [129, 160, 161, 192, 200, 224, 225, 256, 257, 300, 330, 384, 390, 430, 448, 512, 513, 600, 768])
+def test_gram_blocks_of_longer_sequences(T):
+    B, shapes = 2, [(64, 72), (300, 64), (136, 2500)]
+    layers = [dp.Linear(bf16((B, T, d), 1.0, k, ld=(d + 7) // 8 * 8), bf16((B, T, p), 0.1, 50 + k, ld=(p + 7) // 8 * 8),
+                        d=d, p=p, mode=dp.DP_NORM_GHOST) for k, (d, p) in enumerate(shapes)]
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for _ in range(2):                                     # the second call finds the first one's shared memory
+        sq = torch.zeros(B, device="cuda")
+        dp.dp_ghost_norms(layers, B, T, sq, dev_status=st)
+    want = np.zeros(B)
+    for l in layers:
+        want += (np.einsum("btp,btd->bpd", f64(l.G, l.p), f64(l.A, l.d)) ** 2).sum((1, 2))
+    # exact products, fp32 sums of at most 2500 terms
+    assert (np.abs(sq.double().cpu().numpy() / want - 1) < 1e-5).all()
+    assert int(st.item()) == 0
