@@ -312,13 +312,15 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
  * scratch, as are ws (the largest *_ws_bytes of the calls on `stream`, dp_step_ws_bytes if fp32 layers
  * are to be split once instead of for the norms and again for the sums, and the norms of short ones to
  * take one launch instead of one per layer, and
- * dp_clip_accumulate_embed_ws_bytes when tied) and side_ws (the largest of dp_embed_norms_ws_bytes,
+ * dp_clip_accumulate_embed_ws_bytes when tied; with dp_step_vectors_ws_bytes behind all of that, and ws on a
+ * 16-byte boundary, a DP_STEP_ALL call reads the vectors' G and X once instead of twice) and side_ws (the largest of dp_embed_norms_ws_bytes,
  * dp_embed_sort_ws_bytes and dp_clip_accumulate_embed_ws_bytes over both tables; with
  * dp_embed_norms_ws_bytes more per table one kernel adds up all the norms' partial sums).  events: four
  * cudaEvent_t of the caller that order the two streams; `stream` has waited for `side_stream` at the
  * end.  phases: DP_STEP_ALL, or the three phases one after the other with the same descriptor (so
  * that a caller can time them, or change the clip factors on `stream` before the second). */
 size_t dp_step_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype dt, int32_t B, int32_t T);
+size_t dp_step_vectors_ws_bytes(const dp_vector_desc* vectors, int32_t n, int32_t B, int32_t T);
 enum { DP_STEP_NORMS = 1, DP_STEP_GEMM = 2, DP_STEP_REST = 4, DP_STEP_ALL = 7 };
 typedef struct {
   dp_linear_desc* layers;  float* const* outs;  const int64_t* ldos;  const uint32_t* tensor_ids;

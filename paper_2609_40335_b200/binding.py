@@ -55,7 +55,8 @@ EXPORTS = ["dp_vector_norms", "dp_vector_norms_ws_bytes", "dp_clip_accumulate_ve
            "dp_last_cuda_error", "dp_version", "dp_kernel_launches", "dp_debug_force_fma",
            "dp_debug_noise_error_scan", "dp_debug_bounds_checked", "dp_debug_bounds_probe",
            "dp_debug_tensor_map_encodes", "dp_debug_set_wait_limit",
-           "dp_debug_ghost_single", "dp_set_reserved_sms", "dp_step_enqueue", "dp_step_ws_bytes"]
+           "dp_debug_ghost_single", "dp_set_reserved_sms", "dp_step_enqueue", "dp_step_ws_bytes",
+           "dp_step_vectors_ws_bytes"]
 
 
 def lib_path() -> str:
@@ -80,6 +81,8 @@ def load():
     VP = C.POINTER(_VectorDesc)
     L.dp_vector_norms.argtypes = [VP, i32, i32, i32, i32, vp, vp, sz, vp]
     L.dp_vector_norms_ws_bytes.argtypes = [VP, i32, i32, i32]
+    L.dp_step_vectors_ws_bytes.argtypes = [VP, i32, i32, i32]
+    L.dp_step_vectors_ws_bytes.restype = sz
     L.dp_vector_norms_ws_bytes.restype = sz
     L.dp_clip_accumulate_vectors.argtypes = [VP, i32, i32, i32, i32, vp, f32, vp, C.POINTER(vp), f32, i32,
                                              f32, f32, C.c_uint64, C.POINTER(C.c_uint32), C.c_uint32,
@@ -555,6 +558,11 @@ def dp_fill_noise(out: torch.Tensor, sigma: float, C_: float, scale: float, seed
 def dp_step_ws_bytes(layers: Sequence[Linear], B: int, T: int) -> int:
     """Workspace with which a step splits fp32 layers once (0: nothing to gain); see the header."""
     return int(load().dp_step_ws_bytes(_descs(layers), len(layers), _dt(layers[0].A), B, T))
+
+
+def dp_step_vectors_ws_bytes(params: Sequence[Vector], B: int, T: int) -> int:
+    """Workspace with which a step reads its vectors once (0: nothing to gain); see the header."""
+    return int(load().dp_step_vectors_ws_bytes(_vdescs(params), len(params), B, T))
 
 
 def dp_step_enqueue(layers, outs, tensor_ids, vectors, vector_outs, vector_ids, *, ids, G_emb, pos_ids, wte, wpe,

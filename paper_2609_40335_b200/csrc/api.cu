@@ -527,7 +527,8 @@ size_t dp_vector_norms_ws_bytes(const dp_vector_desc* prm, int32_t n, int32_t B,
 }
 
 static dp_status vector_norms_impl(const dp_vector_desc* prm, int32_t n, dp_dtype dt, int32_t B, int32_t T,
-                                   float* sq, void* ws, size_t ws_bytes, void* stream, NormSource* left) {
+                                   float* sq, void* ws, size_t ws_bytes, void* stream, NormSource* left,
+                                   float* keep = nullptr) {
   const dp_status c = check_vectors(prm, n, B, T);
   if (c != DP_OK) return c;
   if (!sq || (dt != DP_F32 && dt != DP_BF16)) return DP_ERR_INVALID_ARG;
@@ -535,7 +536,7 @@ static dp_status vector_norms_impl(const dp_vector_desc* prm, int32_t n, dp_dtyp
   cudaStream_t st = (cudaStream_t)stream;
   float* partials = static_cast<float*>(ws);
   const int n_per = vector_total_slabs(prm, n);
-  dp_status s = launch_vector_norms(prm, n, dt, B, T, partials, n_per, st);
+  dp_status s = launch_vector_norms(prm, n, dt, B, T, partials, n_per, st, keep);
   if (s != DP_OK) return s;
   if (left) { *left = NormSource{partials, n_per, 1.f, nullptr}; return DP_OK; }
   return launch_reduce_partials(partials, n_per, B, sq, 1.f, nullptr, st);
@@ -960,6 +961,13 @@ size_t dp_step_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype
   return need + fma_norms_bytes(layers, n_layers, dt, B, T);
 }
 
+// Row sums of the vectors' examples, from the norms of a step to its clipped sums.  Reading G again costs 2T or 4T bytes
+// per column and example, these 8; below eight tokens there is nothing to gain.
+size_t dp_step_vectors_ws_bytes(const dp_vector_desc* vectors, int32_t n, int32_t B, int32_t T) {
+  if (check_vectors(vectors, n, B, T) != DP_OK || T < 8) return 0;
+  return align_up(vector_keep_bytes(vectors, n, B), 256);
+}
+
 // All that can be wrong with a step, before anything is enqueued: an error found halfway would leave work on two
 // streams.  Workspaces as the requested phases use them; plan: of the layers' norms, if those are among them.
 static dp_status check_step(const dp_step_desc* S, int32_t phases, GhostPlan* plan) {
@@ -1031,7 +1039,7 @@ static dp_status start_table(const dp_step_desc* S, float* table, int64_t ld, in
 
 // events: [0] the step began, [1] embedding norms done, [2] row sums done, [3] clip factors exist (as the clipped sums
 // take them)
-static dp_status step_norms(const dp_step_desc* S, const GhostPlan& plan, SplitGroup* kept) {
+static dp_status step_norms(const dp_step_desc* S, const GhostPlan& plan, SplitGroup* kept, float* row_sums) {
   cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
   const dp_dtype embed_dt = (dp_dtype)S->embed_dtype;
   const int B = S->B, T = S->T;
@@ -1104,7 +1112,7 @@ static dp_status step_norms(const dp_step_desc* S, const GhostPlan& plan, SplitG
     s = room(need);
     if (s != DP_OK) return s;
     s = vector_norms_impl(S->vectors, S->n_vectors, (dp_dtype)S->vector_dtype, B, T, S->sq, ws + held, S->ws_bytes - held,
-                          main, &N.src[N.n]);
+                          main, &N.src[N.n], row_sums);
     if (s != DP_OK) return s;
     ++N.n;
     held += need;
@@ -1136,13 +1144,18 @@ static dp_status step_gemm(const dp_step_desc* S, const SplitGroup* kept) {
                               S->stream, kept);
 }
 
-static dp_status step_rest(const dp_step_desc* S) {
+static dp_status step_rest(const dp_step_desc* S, const float* row_sums) {
   cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
   const dp_dtype dt = (dp_dtype)S->embed_dtype;
   dp_status s;
   // Row sums of tables that no GEMM writes need the clip factors only: on the side stream they run
   // where the GEMM's last wave leaves SMs idle.
   DP_CUDA_OK(cudaStreamWaitEvent(side, (cudaEvent_t)S->events[3], 0));
+  if (row_sums) {
+    s = launch_vector_kept_sums(S->vectors, S->n_vectors, S->B, S->T, row_sums, S->clip, S->vector_outs, 0.f, S->with_noise,
+                                S->sigma * S->C, 1.f, S->seed, S->vector_ids, S->step, side);
+    if (s != DP_OK) return s;
+  }
   if (!S->tied) {
     s = dp_clip_accumulate_embed_sorted(S->ids, S->G_emb, S->ldge, dt, S->B, S->T, S->d, S->V, nullptr, S->C,
                                         S->clip, S->wte, S->ld_wte, 1.f, S->perm, S->seg, S->side_ws,
@@ -1163,26 +1176,46 @@ static dp_status step_rest(const dp_step_desc* S) {
                                         S->ws_bytes, S->dev_status, main);
     if (s != DP_OK) return s;
   }
-  if (S->n_vectors)
+  if (S->n_vectors && !row_sums)
     return dp_clip_accumulate_vectors(S->vectors, S->n_vectors, (dp_dtype)S->vector_dtype, S->B, S->T, nullptr, S->C, S->clip,
                                       S->vector_outs, 0.f, S->with_noise, S->sigma, 1.f, S->seed,
                                       S->vector_ids, S->step, S->ws, S->ws_bytes, main);
   return DP_OK;
 }
 
-dp_status dp_step_enqueue(const dp_step_desc* S, int32_t phases) {
+dp_status dp_step_enqueue(const dp_step_desc* step, int32_t phases) {
   GhostPlan plan;
-  dp_status s = check_step(S, phases, &plan);
+  dp_status s = DP_ERR_WORKSPACE;
+  dp_step_desc desc;
+  const dp_step_desc* S = step;
+  // The vectors' row sums lie at the end of ws, where it has room for them beside all else.
+  float* row_sums = nullptr;
+  if (step && phases == DP_STEP_ALL && step->n_vectors > 0 && step->vectors && step->ws && aligned16(step->ws)) {
+    const size_t all = step->ws_bytes & ~size_t(255);
+    const size_t rows = dp_step_vectors_ws_bytes(step->vectors, step->n_vectors, step->B, step->T);
+    // (room that split fp32 layers can use comes first)
+    const size_t layers = dp_step_ws_bytes(step->layers, step->n_layers, (dp_dtype)step->layer_dtype, step->B, step->T);
+    if (rows && all >= rows + layers) {
+      desc = *step;
+      desc.ws_bytes = all - rows;
+      s = check_step(&desc, phases, &plan);
+      if (s == DP_OK) {
+        S = &desc;
+        row_sums = reinterpret_cast<float*>(static_cast<char*>(step->ws) + desc.ws_bytes);
+      }
+    }
+  }
+  if (s == DP_ERR_WORKSPACE) s = check_step(step, phases, &plan);
   if (s != DP_OK) return s;
   // fp32 layers: within one call the sums can use the norms' split operands
   SplitGroup split;
   SplitGroup* kept = phases == DP_STEP_ALL && S->layer_dtype == DP_F32 ? &split : nullptr;
-  if (phases & DP_STEP_NORMS) s = step_norms(S, plan, kept);
+  if (phases & DP_STEP_NORMS) s = step_norms(S, plan, kept, row_sums);
   // a call of its own: what `stream` did in between (other clip factors, say) comes before the row sums as well
   if ((phases & (DP_STEP_NORMS | DP_STEP_GEMM)) == DP_STEP_GEMM)
     DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[3], (cudaStream_t)S->stream));
   if (s == DP_OK && (phases & DP_STEP_GEMM)) s = step_gemm(S, kept);
-  if (s == DP_OK && (phases & DP_STEP_REST)) s = step_rest(S);
+  if (s == DP_OK && (phases & DP_STEP_REST)) s = step_rest(S, row_sums);
   if (s != DP_OK) {
     // a launch failed: whatever the side stream still does to the caller's tensors, `stream` waits for it
     const int error = g_last_cuda_error;

@@ -137,7 +137,7 @@ def allocate(ds: DeviceStep, split_once: bool = True) -> None:
     """Output tensors (one per parameter tensor) and one workspace large enough for every call.
     split_once: of fp32 layers, room for the split operands of all of them (as large as the inputs, up to
     16 GiB), so that a step splits them once; without it, or where that much is not free, for those of the
-    largest layer three times over."""
+    largest layer three times over.  Of vectors, room for their examples' row sums, so that a step reads them once."""
     dev = ds.sq.device
     f32 = dict(dtype=torch.float32, device=dev)
     for k, l in enumerate(ds.linears):
@@ -183,6 +183,8 @@ def _ws_bytes(ds: DeviceStep, split_once: bool) -> int:
             if ds.tied:
                 once += int(L.dp_tied_cross_term_ws_bytes(ds.B, ds.T, ds.d_model, ds.V))
         need = max(need, once)
+    if ds.vectors and split_once:
+        need = (need + 255) // 256 * 256 + dp.dp_step_vectors_ws_bytes(ds.vectors, ds.B, ds.T)
     return need
 
 

@@ -272,3 +272,33 @@ def test_fp32_step_in_the_least_memory(monkeypatch):
     monkeypatch.setattr(torch, "empty", full)
     pipeline.allocate(ds)
     assert ds.ws.numel() == small
+
+
+# vectors read once (row sums kept from the norms) or twice; widths around a slab of 256 columns and a Philox counter of
+# four, one more vector than a launch holds, fewer tokens than pay
+@pytest.mark.parametrize("dtype", [BF16, F32])
+@pytest.mark.parametrize("B,T,widths", [(3, 40, [1, 3, 4, 255, 256, 257, 700]), (9, 8, [64] * 97), (2, 7, [64, 70]), (1, 9, [513])])
+def test_vectors_read_once_and_twice(dtype, B, T, widths):
+    ds = make_step(vectors=dtype, B=B, T=T)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    rand = lambda p, std: torch.empty(B, T, p, dtype=dtype, device="cuda").normal_(0.0, std, generator=g)
+    ds.vectors = [dp.Vector(rand(p, 0.05), rand(p, 1.0) if k % 2 else None, p=p) for k, p in enumerate(widths)]
+    pipeline.allocate(ds)
+    keep = dp.dp_step_vectors_ws_bytes(ds.vectors, B, T)
+    assert (keep == 0) == (T < 8)
+    results, launches = [], []
+    for ws in (ds.ws, ds.ws[:ds.ws.numel() - max(keep, 256)], ds.ws[4:]):      # with room, with less, off the boundary
+        ds.ws = ws
+        for noise in (True, False):
+            wipe(ds)
+            n0 = dp.dp_kernel_launches()
+            pipeline.dp_step(ds, seed=3, step=2, noise=noise)
+            launches.append(dp.dp_kernel_launches() - n0)
+            results.append(state(ds))
+    groups = (len(widths) + 95) // 96
+    assert launches[4] - launches[0] == (groups if T >= 8 else 0) and launches[2] in (launches[0], launches[4])
+    for got, want in ((0, 2), (1, 3), (4, 2), (5, 3)):
+        # at most 360 products in fp32, added up in another order
+        assert_same(results[got], results[want], rel=360 * 2.0 ** -24)
+    assert int(ds.dev_status.item()) == 0
