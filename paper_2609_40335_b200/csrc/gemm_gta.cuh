@@ -39,64 +39,72 @@ struct GtaNoise {
 // steps an example, at T = 16 one, three quarters of it zeros.  The step of DistilGPT2 with all its parameters at B = 21, T = 203
 // 1383 -> 1295 us, of GPT-2 small at B = 3, T = 77 349 -> 344; at B = 32, T = 128 (the same steps) 940 -> 945, within the runs'
 // differences.  Coordinates are 32-bit: a batch of 2^31 rows keeps
-// steps per example (per_example).
+// steps per example.
 struct GtaRows {
   int B, T;                // planes along K, rows of each, as the tensor map has them
-  bool per_example;
+  int scaled_rows, scaled_steps;   // scaling: all rows, or 0 and the steps of an example where each has its own
 };
 inline GtaRows gta_rows(int B, int T) {
   const long long rows = (long long)B * T;
-  if (rows > 0x7fffffffLL - 64) return {B, T, true};
-  return {1, int(rows), false};
+  const int steps = (T + 63) / 64;
+  if (rows > 0x7fffffffLL - 64) return {B, T, 0, steps};
+  return {1, int(rows), T % 64 == 0 ? 0 : int(rows), steps};
 }
 
-// Clip factors of a K step's rows: lane k holds those of rows k and k + 32.
-struct RowFactors { float lo, hi; };
-// step: K step of the contraction; rows: all token rows, 0: `tsteps` steps belong to each example
+// Clip factors of a K step's rows: lane k holds those of rows k and k + 32; `one`: they are all the same.
+struct RowFactors { float lo, hi; bool one; };
+// step: K step of the contraction; rows: all token rows, 0: `tsteps` steps belong to each example.  The lanes look their
+// rows up only where a step holds several examples (done always, 16 layers at B = 16, T = 512 took 791 us instead of 783).
 __device__ __forceinline__ RowFactors row_factors(const float* clip, int step, int lane, int T, int rows, int tsteps) {
   if (rows == 0) {
     const float r = __ldg(clip + step / tsteps);
-    return {r, r};
+    return {r, r, true};
   }
-  const unsigned first = unsigned(step) * 64u + unsigned(lane), last = unsigned(rows) - 1u;
-  return {__ldg(clip + min(first, last) / unsigned(T)), __ldg(clip + min(first + 32u, last) / unsigned(T))};
+  const unsigned first = unsigned(step) * 64u, ex = first / unsigned(T);
+  if (first + 64u <= (ex + 1u) * unsigned(T)) {
+    const float r = __ldg(clip + ex);
+    return {r, r, true};
+  }
+  const unsigned last = unsigned(rows) - 1u, mine = first + unsigned(lane);
+  return {__ldg(clip + min(mine, last) / unsigned(T)), __ldg(clip + min(mine + 32u, last) / unsigned(T)), false};
 }
 
 // One warp multiplies a 16 KiB operand part (two boxes of 64 rows x 128 bytes; the 128-byte swizzle moves 16-byte
 // chunks inside a row only) by its rows' factors.  r = r_hi + r_lo with both parts in bf16 (16 mantissa bits in
 // total); x*r is formed as fma(x, r_hi, x*r_lo) on packed bf16 pairs: one rounding of the exact x*r_hi plus a tiny
 // correction, i.e. the correctly rounded bf16 product up to 2^-17 relative.  16-byte chunks, eight at a time.
-__device__ __forceinline__ void scale_part(uint4* part, RowFactors f, int lane) {
-  const float r = __shfl_sync(0xffffffffu, f.lo, 0);
-  const bool one = __all_sync(0xffffffffu, f.lo == r && f.hi == r);
-  if (one && r == 1.0f) return;
+__device__ __forceinline__ void scale_part(uint4* part, float r, int lane) {
+  const __nv_bfloat16 rh = __float2bfloat16_rn(r);
+  const __nv_bfloat16 rl = __float2bfloat16_rn(r - __bfloat162float(rh));
+  const __nv_bfloat162 rh2 = __halves2bfloat162(rh, rh), rl2 = __halves2bfloat162(rl, rl);
+  uint4* x = part + lane;
+#pragma unroll 1
+  for (int c0 = 0; c0 < 32; c0 += 8) {
+    uint4 v[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = x[(c0 + q) * 32];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&v[q]);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) e[k] = __hfma2(e[k], rh2, __hmul2(e[k], rl2));
+      x[(c0 + q) * 32] = v[q];
+    }
+  }
+}
+
+// The same with a factor per row.  Out of line: inside the scalers' loop it cost the steps that need none of it 1 %.
+static __device__ __noinline__ void scale_rows(uint4* part, float lo, float hi, int lane) {
   auto split = [](float x) {                       // r_hi in the low half, r_lo in the high one
     const __nv_bfloat16 h = __float2bfloat16_rn(x), l = __float2bfloat16_rn(x - __bfloat162float(h));
     return uint32_t(__bfloat16_as_ushort(h)) | (uint32_t(__bfloat16_as_ushort(l)) << 16);
   };
-  const uint32_t w_lo = split(f.lo), w_hi = split(f.hi);
   auto pair = [](uint32_t w, uint32_t sel) {
     const uint32_t b = __byte_perm(w, w, sel);
     return *reinterpret_cast<const __nv_bfloat162*>(&b);
   };
+  const uint32_t w_lo = split(lo), w_hi = split(hi);
   uint4* x = part + lane;
-  if (one) {
-    const __nv_bfloat162 rh2 = pair(w_lo, 0x1010), rl2 = pair(w_lo, 0x3232);
-#pragma unroll 1
-    for (int c0 = 0; c0 < 32; c0 += 8) {
-      uint4 v[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = x[(c0 + q) * 32];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&v[q]);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) e[k] = __hfma2(e[k], rh2, __hmul2(e[k], rl2));
-        x[(c0 + q) * 32] = v[q];
-      }
-    }
-    return;
-  }
 #pragma unroll 1
   for (int c0 = 0; c0 < 32; c0 += 8) {             // chunk (c0 + q) * 32 + lane lies in row 4 (c0 + q) + lane / 8 of 64
     const uint32_t mine = (c0 & 8) ? w_hi : w_lo;

@@ -81,7 +81,7 @@ struct __align__(64) BigParams {
   int n_layers;
   int tsteps, ksteps;        // K steps per plane (split fp32: three per 64 tokens), K steps in all
   int low_plane;             // split operands: first plane of low terms
-  int example_rows, rows;    // scaling: tokens per example, all rows (0: steps per example)
+  int example_rows, rows, example_steps;     // scaling: tokens per example; all rows, or 0 and the steps of an example
   int skew;                  // K steps that sub-tile 1 of an item lags behind
   int n_big, n_big_total;    // two-tile items run as such, and in all (the rest as two singles each)
   int total_items;
@@ -320,8 +320,8 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
       const bool scale_here = P.clip && !P.layer[it.layer].prescaled;
       const int steps = P.ksteps + (it.nsub == 2 ? P.skew : 0);
       auto factors = [&](int j) {              // of step j (the last `skew` steps are the first again)
-        if (!scale_here || j >= steps) return RowFactors{1.f, 1.f};
-        return row_factors(P.clip, j < P.ksteps ? j : j - P.ksteps, lane, P.example_rows, P.rows, P.tsteps);
+        if (!scale_here || j >= steps) return RowFactors{1.f, 1.f, true};
+        return row_factors(P.clip, j < P.ksteps ? j : j - P.ksteps, lane, P.example_rows, P.rows, P.example_steps);
       };
       int j = int((uint32_t(sw) + kScalerWarps - cnt % kScalerWarps) % kScalerWarps);
       uint32_t c = cnt + uint32_t(j);
@@ -332,10 +332,10 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
         const uint32_t stage = c % kStages, fill = c / kStages, phase = fill & 1u;
         if (fill > 0 && !ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
         if (!ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit)) { ok = false; break; }
-        if (scale_here) {
-          scale_part(reinterpret_cast<uint4*>(tiles + size_t(stage) * kStageBytes), r, lane);
-          ptx::fence_proxy_async_smem();
-        }
+        uint4* part = reinterpret_cast<uint4*>(tiles + size_t(stage) * kStageBytes);
+        if (!r.one) scale_rows(part, r.lo, r.hi, lane);
+        else if (r.lo != 1.0f) scale_part(part, r.lo, lane);
+        if (scale_here) ptx::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
           if (rank == 0) ptx::mbar_arrive_expect_tx_a(ready_a + 8 * stage, 4);
@@ -511,7 +511,7 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
   P.total_items = P.n_big + 2 * (bigs - P.n_big) + singles;
   P.n_layers = n;
   P.tsteps = terms * ceil_div(K.T, kBK); P.ksteps = K.B * P.tsteps; P.low_plane = K.B;
-  P.example_rows = T; P.rows = K.per_example ? 0 : K.T;
+  P.example_rows = T; P.rows = K.scaled_rows; P.example_steps = K.scaled_steps;
   // Long enough to read one accumulator, and to draw its noise, while the other is fed: with noise 4, 6, 8,
   // 10, 12, 24 and 40 steps gave 2341, 2278, 2252, 2265, 2283, 2407 and 2513 us (B = 16, T = 512).  The same
   // without noise, which would do with 2 or none, so that a sum does not depend on whether noise is fused.

@@ -75,7 +75,7 @@ struct __align__(64) GtaParams {
   int n_layers;
   int B, T, tsteps;          // planes along K and rows of each; tsteps = terms * ceil(T / 64) K steps per plane
   int low_plane;             // split operands: first plane of low terms
-  int example_rows, rows;    // scaling: tokens per example, all rows (0: steps per example)
+  int example_rows, rows, example_steps;     // scaling: tokens per example; all rows, or 0 and the steps of an example
   int nsplit, ksteps_per_split;   // K splits, the same for all layers of a call; multiples of `terms` steps
   float beta;
   int total_items;
@@ -294,13 +294,13 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
         uint32_t c = cnt + uint32_t(ks - it.k0);
         // no scaling here when the operand arrives scaled: clip == NULL (the split fp32 path) or a
         // layer whose narrow operand was multiplied by R_i in a pass of its own (see prescale)
-        RowFactors r_next{1.f, 1.f};
-        if (scale_here && ks < it.k1) r_next = row_factors(P.clip, ks, lane, P.example_rows, P.rows, P.tsteps);
+        RowFactors r_next{1.f, 1.f, true};
+        if (scale_here && ks < it.k1) r_next = row_factors(P.clip, ks, lane, P.example_rows, P.rows, P.example_steps);
         for (; ks < it.k1; ks += kScalerWarps, c += kScalerWarps) {
           const RowFactors r = r_next;
           // the factors of this warp's next K step are fetched before the waits, off the stage's path
           if (scale_here && ks + kScalerWarps < it.k1)
-            r_next = row_factors(P.clip, ks + kScalerWarps, lane, P.example_rows, P.rows, P.tsteps);
+            r_next = row_factors(P.clip, ks + kScalerWarps, lane, P.example_rows, P.rows, P.example_steps);
           const uint32_t stage = c % kStages, fill = c / kStages, phase = fill & 1u;
           // A warp hops between stages, so it has not seen the previous fill of this one, and the
           // parity of `full` alone cannot tell "fill n landed" from "fill n-1 still in flight".
@@ -309,10 +309,10 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
           // or "fill n landed".
           if (fill > 0 && !ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
           if (!ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit)) { ok = false; break; }
-          if (scale_here) {
-            scale_part(reinterpret_cast<uint4*>(tiles + size_t(stage) * kStageBytes), r, lane);
-            ptx::fence_proxy_async_smem();
-          }
+          uint4* part = reinterpret_cast<uint4*>(tiles + size_t(stage) * kStageBytes);
+          if (!r.one) scale_rows(part, r.lo, r.hi, lane);
+          else if (r.lo != 1.0f) scale_part(part, r.lo, lane);
+          if (scale_here) ptx::fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
             if (!kPair) ptx::mbar_arrive(&ready[stage]);
@@ -738,7 +738,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
       P.step_dev = g_step_dev;
     }
     P.n_layers = g1 - g0; P.B = K.B; P.T = K.T; P.tsteps = tsteps; P.low_plane = K.B;
-    P.example_rows = T; P.rows = K.per_example ? 0 : K.T;
+    P.example_rows = T; P.rows = K.scaled_rows; P.example_steps = K.scaled_steps;
     P.total_items = items;
     P.nsplit = nsplit; P.ksteps_per_split = kps; P.beta = beta;
     P.clip = clip;
