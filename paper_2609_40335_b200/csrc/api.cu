@@ -11,6 +11,7 @@
 #include "fma_kernels.cuh"
 #include "gemm_gta.cuh"
 #include "ghost_plan.cuh"
+#include "small_step.cuh"
 #include "split_kernels.cuh"
 #include "tma_host.cuh"
 #include "vector_kernels.cuh"
@@ -1183,6 +1184,21 @@ static dp_status step_rest(const dp_step_desc* S, const float* row_sums) {
   return DP_OK;
 }
 
+// A step short of work uses `stream` alone.  What `side_stream` still has to do, an earlier fill of a table say, comes
+// before it, as when the step used both; inside a capture `side_stream` joins first.
+static dp_status small_step(const dp_step_desc* S) {
+  cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
+  cudaStreamCaptureStatus capture;
+  DP_CUDA_OK(cudaStreamIsCapturing(main, &capture));
+  if (capture != cudaStreamCaptureStatusNone) {
+    DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[0], main));
+    DP_CUDA_OK(cudaStreamWaitEvent(side, (cudaEvent_t)S->events[0], 0));
+  }
+  DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[2], side));
+  DP_CUDA_OK(cudaStreamWaitEvent(main, (cudaEvent_t)S->events[2], 0));
+  return launch_small_step(*S, main);
+}
+
 dp_status dp_step_enqueue(const dp_step_desc* step, int32_t phases) {
   GhostPlan plan;
   dp_status s = DP_ERR_WORKSPACE;
@@ -1207,6 +1223,7 @@ dp_status dp_step_enqueue(const dp_step_desc* step, int32_t phases) {
   }
   if (s == DP_ERR_WORKSPACE) s = check_step(step, phases, &plan);
   if (s != DP_OK) return s;
+  if (phases == DP_STEP_ALL && small_step_fits(*S)) return small_step(S);
   // fp32 layers: within one call the sums can use the norms' split operands
   SplitGroup split;
   SplitGroup* kept = phases == DP_STEP_ALL && S->layer_dtype == DP_F32 ? &split : nullptr;
