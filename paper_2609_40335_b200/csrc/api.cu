@@ -77,6 +77,12 @@ GhostPlan plan_ghost_norms(const dp_linear_desc* layers, int n_layers, int B, in
     plan.mode_used[l] = mode;
     (mode == DP_NORM_GHOST ? plan.ghost_layers : plan.direct_layers).push_back(l);
   }
+  // as many examples per tile as fit, while two items per SM remain; the rows of the batch are counted in 32 bits
+  if (T <= 64 && (long long)B * T <= 0x7fffffffLL - 128) {
+    const long long most = (long long)B * (long long)plan.ghost_layers.size() / (2LL * units);
+    plan.pack = (int)std::max(1LL, std::min(most, (long long)std::min(B, 128 / T)));
+  }
+  const int groups = ceil_div(B, plan.pack);
   // Column chunking of wide operands.  The per-item step budget shrinks until there are at
   // least two items per SM (or the budget bottoms out).  Split operands have sums no longer than those of layers
   // planned one by one on widened operands (24 steps at d = 768, with 2.4 times the error per step): see
@@ -95,7 +101,7 @@ GhostPlan plan_ghost_norms(const dp_linear_desc* layers, int n_layers, int B, in
       L.nsplit = ceil_div(large, chunk);
       L.chunk_steps = ceil_div(large, L.nsplit);
       L.nsplit = ceil_div(large, L.chunk_steps);
-      items += (long long)B * plan.ntp * L.nsplit;
+      items += (long long)groups * plan.ntp * L.nsplit;
     }
     if (items >= 2LL * units || budget <= 8 || plan.ghost_layers.empty()) break;
     budget /= 2;

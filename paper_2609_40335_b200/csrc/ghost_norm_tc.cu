@@ -34,15 +34,17 @@ constexpr int kTileBytes = kTile * kKStep * 2;   // 16 KiB
 // pair is diagonal, so stages shrink to one tile and twice as many are kept in flight (the
 // kernel is HBM-bound there: bytes in flight are what counts).  Split operands (fp32 inputs) bring
 // two tiles, high and low terms, for each.
-// Up to 64 tokens a stage of 16 KiB took the 550 cycles of its hand-offs for a half or a quarter of the
-// data, the rest zeros.  kBoxes = 2 or 4: tiles of T rounded up to 16 rows, and two or four of them, 64
-// columns each, per stage.  B = 16, T = 64, 48 GPT-2-small layers 87.5 -> 71.9 us, B = 32, T = 48, 24 layers 78.9 ->
-// 61.3, B = 37, T = 35, 12 layers of d = 1024 64.3 -> 47.9, B = 6, T = 16, 24 of d = 512 20.3 -> 14.2.  Above 64 tokens
-// short tiles and sizes known at run time cost more than they save (115 -> 122 us at B = 32, T = 128):
-// kBoxes = 1 has full tiles and everything constant.
+// Up to 64 tokens a tile holds several examples (kPacked): the rows of a batch lie one after the other, so 128 / T of them
+// fill it, its Gram matrix has theirs on the diagonal, and the epilogue multiplies only those blocks.  An example by itself
+// took the 550 cycles of a stage's hand-offs, an item's start and its epilogue for a few KiB.  Tiles are as tall as their
+// examples, rounded up to 16 rows; where the whole batch fills less than half of one, a stage holds two or four of them, 64
+// columns each (kBoxes).  97 layers of d = 128 at B = 95, T = 17 115 -> 50 us, 49 at B = 91, T = 39 70 -> 50; never so many
+// examples that fewer than two items per SM remain (5 fp32 layers at B = 2, T = 54: 7.7 -> 10.2 with both in one tile).  Above 64 tokens
+// short tiles and sizes known at run time cost more than they save (115 -> 122 us at B = 32, T = 128): there
+// tiles are full and everything is constant.
 constexpr int kRingBytes = 12 * kTileBytes;
 constexpr int kMaxStages = 32;
-constexpr size_t kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 1024 /*barriers*/;
+constexpr size_t kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 1024 /*barriers*/ + 4 * kTile * sizeof(float) /*row sums*/;
 constexpr int kThreads = 192;
 constexpr int kTmemCols = 512;                   // 2 buffers x (S_A 128 + S_G 128) columns; split: hi hi, small products
 
@@ -52,7 +54,10 @@ struct __align__(64) GhostParams {
   GhostLayerPlan layer[kGhostMaxLayers];
   int n_layers;
   int B, T, nt, ntp;
-  int rows, stages;          // kBoxes > 1: tokens of a tile, stages of the ring
+  int rows, stages;          // packed: rows of a tile, stages of the ring
+  int pack;                  // packed: examples per tile ...
+  int row_step, plane_step;  // ... and where the rows of the next tile begin: so many rows on, or so many planes
+  int low_plane;             // split operands: first plane of low terms
   int total_items;
   int n_per;                 // partial sums per example in the workspace
   float* partials;           // [B][n_per]
@@ -61,11 +66,12 @@ struct __align__(64) GhostParams {
 };
 
 struct Item {
-  int layer, example, ti, tj, a0, a1, g0, g1, pidx;
+  int layer, example, ti, tj, a0, a1, g0, g1, pidx;      // packed: which tile of examples; its place in an example's sums
 };
 
 // `l` is the caller's running layer index: a role's items ascend, so the search goes on from the layer
 // of its previous item instead of walking the list (a constant-memory line per layer) every time.
+template <bool kPacked>
 __device__ __forceinline__ Item decode_item(const GhostParams& P, int item, int& l) {
   Item it;
   while (l + 1 < P.n_layers && item >= P.layer[l + 1].item_begin) ++l;
@@ -87,7 +93,7 @@ __device__ __forceinline__ Item decode_item(const GhostParams& P, int item, int&
     it.g0 = 0; it.g1 = L.g_steps;
     it.a0 = c0; it.a1 = min(c0 + L.chunk_steps, L.a_steps);
   }
-  it.pidx = it.example * P.n_per + L.col_begin + tp * L.nsplit + s;
+  it.pidx = (kPacked ? 0 : it.example * P.n_per) + L.col_begin + tp * L.nsplit + s;
   return it;
 }
 
@@ -102,18 +108,18 @@ __device__ __forceinline__ uint32_t add_f32(uint32_t a, uint32_t b) {
 // 25 layers of DistilGPT2's shapes at B = 64, T = 256, error against 64 bits: 2.2e-5 with all three in one, now
 // 1.4e-5.  The epilogue no longer overlaps the next item's MMAs; fewer chunks of wide operands make up for it (the fp32
 // step of DistilGPT2 at B = 8, T = 128: no difference beyond 0.5 %).
-template <bool kDiagOnly, bool kSplit, int kBoxes>
+template <bool kDiagOnly, bool kSplit, bool kPacked, int kBoxes>
 __global__ void __launch_bounds__(kThreads, 1)
 ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
-  static_assert(kBoxes == 1 || kDiagOnly, "several column tiles per stage: diagonal pairs only");
+  static_assert(kDiagOnly || !kPacked, "packed examples: diagonal pairs only");
+  static_assert(kPacked || kBoxes == 1, "several column tiles per stage: packed examples only");
   // an MMA reads 128 rows of its first operand whatever `rows` is: rows beyond it come from the next
   // stages (the ring ends a whole tile after its last tile begins) and fill accumulator rows nobody reads
-  constexpr bool kShort = kBoxes > 1;
-  const int rows = kShort ? P.rows : kTile;
+  const int rows = kPacked ? P.rows : kTile;
   const uint32_t tile_bytes = uint32_t(rows) * (kKStep * 2);
   const uint32_t term_bytes = (kSplit ? 2 : 1) * tile_bytes;             // one row tile, all its terms
   const uint32_t stage_bytes = (kDiagOnly ? kBoxes : 2) * term_bytes;
-  const int n_stages = kShort ? P.stages : kRingBytes / int((kDiagOnly ? 1 : 2) * (kSplit ? 2 : 1) * kTileBytes);
+  const int n_stages = kPacked ? P.stages : kRingBytes / int((kDiagOnly ? 1 : 2) * (kSplit ? 2 : 1) * kTileBytes);
   extern __shared__ uint8_t smem_raw[];
   // 128-byte swizzled tiles need 1024-byte alignment
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -127,7 +133,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
   uint64_t* red_bar = mma_done + 1;        // [4]        epilogue warps -> epilogue warp 0
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(red_bar + 4);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* epi_red = reinterpret_cast<float*>(tmem_slot + 2);   // [4][4]
+  float* epi_red = reinterpret_cast<float*>(tmem_slot + 2);   // [4][4]; packed: [4][kTile], a sum for each row
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -157,10 +163,11 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
     int lay = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x) {
-      const Item it = decode_item(P, item, lay);
+      const Item it = decode_item<kPacked>(P, item, lay);
       const bool diag = kDiagOnly || (it.ti == it.tj);
       const uint32_t bytes = diag ? term_bytes : stage_bytes;
-      const int ex = it.example, low = ex + P.B;               // planes of the example (split: high and low terms)
+      const int ex = kPacked ? it.example * P.plane_step : it.example, low = ex + P.low_plane;   // planes (split: high and low terms)
+      const int row_i = kPacked ? it.example * P.row_step : it.ti * kTile;
       for (int pass = 0; pass < 2 && ok; ++pass) {
         const uint64_t tm = reinterpret_cast<uint64_t>(pass == 0 ? &P.tmA[it.layer] : &P.tmG[it.layer]);
         const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
@@ -168,15 +175,15 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
           ok = ptx::warp_ok(ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit));
           if (!ok) break;
           const uint32_t dst = tiles_a + stage * stage_bytes, bar = full_a + 8 * stage;
-          const int nb = kShort ? min(kBoxes, k1 - k) : 1;
+          const int nb = kPacked ? min(kBoxes, k1 - k) : 1;
           if (ptx::elect_one()) {
-            ptx::mbar_arrive_expect_tx_a(bar, kShort ? nb * term_bytes : bytes);
+            ptx::mbar_arrive_expect_tx_a(bar, kPacked ? nb * term_bytes : bytes);
 #pragma unroll
             for (int b = 0; b < kBoxes; ++b) {
               if (b >= nb) break;
-              ptx::tma_load_3d_a(dst + b * term_bytes, tm, bar, (k + b) * kKStep, it.ti * kTile, ex);
+              ptx::tma_load_3d_a(dst + b * term_bytes, tm, bar, (k + b) * kKStep, row_i, ex);
               if (kSplit)
-                ptx::tma_load_3d_a(dst + b * term_bytes + tile_bytes, tm, bar, (k + b) * kKStep, it.ti * kTile, low);
+                ptx::tma_load_3d_a(dst + b * term_bytes + tile_bytes, tm, bar, (k + b) * kKStep, row_i, low);
             }
             if (!diag) {
               ptx::tma_load_3d_a(dst + term_bytes, tm, bar, k * kKStep, it.tj * kTile, ex);
@@ -207,7 +214,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
     int lay = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x, ++n_item) {
-      const Item it = decode_item(P, item, lay);
+      const Item it = decode_item<kPacked>(P, item, lay);
       const bool diag = kDiagOnly || (it.ti == it.tj);
       const uint32_t buf = kSplit ? 0 : n_item & 1, acc_phase = (kSplit ? n_item : n_item >> 1) & 1;
       ok = ptx::warp_ok(ptx::mbar_wait(&acc_empty[buf], acc_phase ^ 1, abort_flag, P.wait_limit));
@@ -220,7 +227,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
           ok = ptx::warp_ok(ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit));
           if (!ok) break;
           ptx::tc_fence_after();
-          const int nb = kShort ? min(kBoxes, nsteps - k) : 1;
+          const int nb = kPacked ? min(kBoxes, nsteps - k) : 1;
           if (ptx::elect_one()) {
 #pragma unroll
             for (int b = 0; b < kBoxes; ++b) {
@@ -258,48 +265,55 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
     int lay = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < P.total_items && ok; item += gridDim.x, ++n_item) {
-      const Item it = decode_item(P, item, lay);
+      const Item it = decode_item<kPacked>(P, item, lay);
       const uint32_t buf = kSplit ? 0 : n_item & 1, acc_phase = (kSplit ? n_item : n_item >> 1) & 1;
       if (!ptx::mbar_wait_relaxed(&acc_full[buf], acc_phase, abort_flag, P.wait_limit)) { ok = false; break; }
       ptx::tc_fence_after();
       const uint32_t t0 = tmem_base + (uint32_t(q * 32) << 16) + buf * 256;
       float acc = 0.f;
+      // packed: this row's example and the columns of its tokens; the warp's rows have those of [c_lo, c_hi)
+      const int row = q * 32 + lane, own = kPacked ? row / P.T * P.T : 0;
+      const int c_lo = kPacked ? (q * 32 / P.T * P.T) & ~15 : 0;
+      const int c_hi = kPacked ? min(rows, (q * 32 + 31) / P.T * P.T + P.T) : rows;
 #pragma unroll 1
-      for (int c = 0; c + 32 <= rows; c += 32) {
+      for (int c = c_lo; c < c_hi; c += 32) {
         uint32_t ra[32], rg[32];
-        ptx::tmem_ld_32x32b_x32(t0 + c, ra);
-        ptx::tmem_ld_32x32b_x32(t0 + 128 + c, rg);
-        if (kSplit) {
-          uint32_t sa[32], sg[32];
-          ptx::tmem_ld_32x32b_x32(t0 + 256 + c, sa);
-          ptx::tmem_ld_32x32b_x32(t0 + 384 + c, sg);
-          ptx::tmem_ld_wait();
+        if (!kPacked || c + 32 <= rows) {
+          ptx::tmem_ld_32x32b_x32(t0 + c, ra);
+          ptx::tmem_ld_32x32b_x32(t0 + 128 + c, rg);
+          if (kSplit) {
+            uint32_t sa[32], sg[32];
+            ptx::tmem_ld_32x32b_x32(t0 + 256 + c, sa);
+            ptx::tmem_ld_32x32b_x32(t0 + 384 + c, sg);
+            ptx::tmem_ld_wait();
 #pragma unroll
-          for (int j = 0; j < 32; ++j) { ra[j] = add_f32(ra[j], sa[j]); rg[j] = add_f32(rg[j], sg[j]); }
-        } else {
-          ptx::tmem_ld_wait();
+            for (int j = 0; j < 32; ++j) { ra[j] = add_f32(ra[j], sa[j]); rg[j] = add_f32(rg[j], sg[j]); }
+          } else {
+            ptx::tmem_ld_wait();
+          }
+        } else {                                       // the last 16 columns
+          uint32_t ha[16], hg[16];
+          ptx::tmem_ld_32x32b_x16(t0 + c, ha);
+          ptx::tmem_ld_32x32b_x16(t0 + 128 + c, hg);
+          if (kSplit) {
+            uint32_t sa[16], sg[16];
+            ptx::tmem_ld_32x32b_x16(t0 + 256 + c, sa);
+            ptx::tmem_ld_32x32b_x16(t0 + 384 + c, sg);
+            ptx::tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 16; ++j) { ha[j] = add_f32(ha[j], sa[j]); hg[j] = add_f32(hg[j], sg[j]); }
+          } else {
+            ptx::tmem_ld_wait();
+          }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) { ra[j] = ha[j]; rg[j] = hg[j]; ra[16 + j] = 0u; rg[16 + j] = 0u; }
         }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) acc = fmaf(__uint_as_float(ra[j]), __uint_as_float(rg[j]), acc);
-      }
-      if (kShort && (rows & 16)) {
-        uint32_t ra[16], rg[16];
-        ptx::tmem_ld_32x32b_x16(t0 + rows - 16, ra);
-        ptx::tmem_ld_32x32b_x16(t0 + 128 + rows - 16, rg);
-        if (kSplit) {
-          uint32_t sa[16], sg[16];
-          ptx::tmem_ld_32x32b_x16(t0 + 256 + rows - 16, sa);
-          ptx::tmem_ld_32x32b_x16(t0 + 384 + rows - 16, sg);
-          ptx::tmem_ld_wait();
-#pragma unroll
-          for (int j = 0; j < 16; ++j) { ra[j] = add_f32(ra[j], sa[j]); rg[j] = add_f32(rg[j], sg[j]); }
-        } else {
-          ptx::tmem_ld_wait();
+        for (int j = 0; j < 32; ++j) {
+          if (!kPacked || unsigned(c + j - own) < unsigned(P.T))
+            acc = fmaf(__uint_as_float(ra[j]), __uint_as_float(rg[j]), acc);
         }
-#pragma unroll
-        for (int j = 0; j < 16; ++j) acc = fmaf(__uint_as_float(ra[j]), __uint_as_float(rg[j]), acc);
       }
-      if (kShort && q * 32 + lane >= P.T) acc = 0.f;     // a row beyond the tile: whatever lay there
       ptx::tc_fence_before();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&acc_empty[buf]);   // accumulators may be overwritten
@@ -307,12 +321,29 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
       // gave up above never arrives, and warp 0's wait for the others is bounded like every other.
       // Four slots: the other warps can run at most two items ahead of a waiting warp 0 (they
       // need its acc_empty arrivals), so a slot is never rewritten before it has been read.
-      acc = warp_sum(acc);
       const uint32_t slot = n_item & 3, red_phase = (n_item >> 2) & 1;
-      if (lane == 0) { epi_red[slot * 4 + ew] = acc; ptx::mbar_arrive(&red_bar[slot]); }
+      if (kPacked) {
+        epi_red[slot * kTile + row] = acc;
+        __syncwarp();
+      } else {
+        acc = warp_sum(acc);
+        if (lane == 0) epi_red[slot * 4 + ew] = acc;
+      }
+      if (lane == 0) ptx::mbar_arrive(&red_bar[slot]);
       if (ew == 0) {
         if (!ptx::mbar_wait_relaxed(&red_bar[slot], red_phase, abort_flag, P.wait_limit)) { ok = false; break; }
-        if (lane == 0 && dp_in_range(it.pidx, (long long)P.B * P.n_per, P.dev_status)) {
+        if (kPacked) {
+          for (int e = lane; e < P.pack; e += 32) {      // a lane adds up the rows of an example
+            const int example = it.example * P.pack + e;
+            const long long at = (long long)example * P.n_per + it.pidx;
+            if (example >= P.B || !dp_in_range(at, (long long)P.B * P.n_per, P.dev_status)) break;
+            const float* of = epi_red + slot * kTile + e * P.T;
+            float s = 0.f;
+#pragma unroll 8
+            for (int k = 0; k < P.T; ++k) s += of[k];
+            P.partials[at] = s;
+          }
+        } else if (lane == 0 && dp_in_range(it.pidx, (long long)P.B * P.n_per, P.dev_status)) {
           const float s = (epi_red[slot * 4 + 0] + epi_red[slot * 4 + 1]) +
                           (epi_red[slot * 4 + 2] + epi_red[slot * 4 + 3]);
           P.partials[it.pidx] = (it.ti == it.tj) ? s : 2.f * s;
@@ -363,12 +394,12 @@ dp_status launch_reduce_partials(const float* partials, int n_per, int B, float*
 
 namespace {
 
-template <bool kDiagOnly, bool kSplit, int kBoxes>
+template <bool kDiagOnly, bool kSplit, bool kPacked, int kBoxes>
 dp_status launch_variant(const GhostParams& P, cudaStream_t st) {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_tc_kernel<kDiagOnly, kSplit, kBoxes>)))
-    DP_CUDA_OK((allow_shared(ghost_norm_tc_kernel<kDiagOnly, kSplit, kBoxes>, kSmemBytes)));
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_tc_kernel<kDiagOnly, kSplit, kPacked, kBoxes>)))
+    DP_CUDA_OK((allow_shared(ghost_norm_tc_kernel<kDiagOnly, kSplit, kPacked, kBoxes>, kSmemBytes)));
   const int grid = std::min(P.total_items, sm_count());
-  ghost_norm_tc_kernel<kDiagOnly, kSplit, kBoxes><<<grid, kThreads, kSmemBytes, st>>>(P);
+  ghost_norm_tc_kernel<kDiagOnly, kSplit, kPacked, kBoxes><<<grid, kThreads, kSmemBytes, st>>>(P);
   DP_LAUNCH_OK();
   return DP_OK;
 }
@@ -380,10 +411,12 @@ dp_status launch_variant(const GhostParams& P, cudaStream_t st) {
 dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
                                float* partials, int* dev_status, cudaStream_t st, bool split) {
   const int nt = ceil_div(T, kTile);
-  const int planes = split ? 2 * B : B;
-  const int boxes = T > 64 ? 1 : T > 32 || split ? 2 : 4;       // split operands: T >= 32
-  const int rows = boxes > 1 ? (T + 15) / 16 * 16 : kTile, tile_bytes = rows * kKStep * 2;
+  const bool packed = T <= 64, flat = plan.pack > 1 || B == 1;       // flat: the rows of the batch as one dimension
+  const int rows = packed ? (plan.pack * T + 15) / 16 * 16 : kTile, tile_bytes = rows * kKStep * 2;
+  const int map_rows = packed && flat ? B * T : T, examples = packed && flat ? 1 : B, planes = (split ? 2 : 1) * examples;
+  const int boxes = !packed || rows > 64 ? 1 : rows > 32 || split ? 2 : 4;
   const int stages = std::min(kMaxStages, (kRingBytes - (kTileBytes - tile_bytes)) / (boxes * (split ? 2 : 1) * tile_bytes));
+  const int groups = packed ? ceil_div(B, plan.pack) : B;
   // layers are processed in groups that fit one parameter block
   for (size_t g0 = 0; g0 < plan.ghost_layers.size(); g0 += kGhostMaxLayers) {
     const size_t g1 = std::min(plan.ghost_layers.size(), g0 + kGhostMaxLayers);
@@ -393,18 +426,19 @@ dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& pl
     for (size_t g = g0; g < g1; ++g) {
       const int li = plan.ghost_layers[g];
       const dp_linear_desc& L = layers[li];
-      dp_status s = make_tmap_bf16_3d(&P.tmA[g - g0], L.A, L.lda, L.d, T, planes, kKStep, rows);
+      dp_status s = make_tmap_bf16_3d(&P.tmA[g - g0], L.A, L.lda, L.d, map_rows, planes, kKStep, rows);
       if (s != DP_OK) return s;
-      s = make_tmap_bf16_3d(&P.tmG[g - g0], L.G, L.ldg, L.p, T, planes, kKStep, rows);
+      s = make_tmap_bf16_3d(&P.tmG[g - g0], L.G, L.ldg, L.p, map_rows, planes, kKStep, rows);
       if (s != DP_OK) return s;
       GhostLayerPlan lp = plan.layer[li];
       lp.item_begin = items;
-      items += B * plan.ntp * lp.nsplit;
+      items += groups * plan.ntp * lp.nsplit;
       P.layer[g - g0] = lp;
     }
     P.n_layers = int(g1 - g0);
     P.B = B; P.T = T; P.nt = nt; P.ntp = plan.ntp;
-    P.rows = rows; P.stages = stages;
+    P.rows = rows; P.stages = stages; P.pack = plan.pack; P.low_plane = examples;
+    P.row_step = flat ? plan.pack * T : 0; P.plane_step = flat ? 0 : 1;
     P.total_items = items;
     P.n_per = plan.n_per;
     P.partials = partials;
@@ -412,11 +446,14 @@ dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& pl
     P.wait_limit = g_wait_limit;
     dp_status s;
     if (split)
-      s = nt > 1 ? launch_variant<false, true, 1>(P, st)
-                 : boxes == 1 ? launch_variant<true, true, 1>(P, st) : launch_variant<true, true, 2>(P, st);
-    else if (nt > 1) s = launch_variant<false, false, 1>(P, st);
-    else if (boxes == 1) s = launch_variant<true, false, 1>(P, st);
-    else s = boxes == 2 ? launch_variant<true, false, 2>(P, st) : launch_variant<true, false, 4>(P, st);
+      s = nt > 1 ? launch_variant<false, true, false, 1>(P, st)
+          : !packed ? launch_variant<true, true, false, 1>(P, st)
+          : boxes == 1 ? launch_variant<true, true, true, 1>(P, st) : launch_variant<true, true, true, 2>(P, st);
+    else
+      s = nt > 1 ? launch_variant<false, false, false, 1>(P, st)
+          : !packed ? launch_variant<true, false, false, 1>(P, st)
+          : boxes == 1 ? launch_variant<true, false, true, 1>(P, st)
+          : boxes == 2 ? launch_variant<true, false, true, 2>(P, st) : launch_variant<true, false, true, 4>(P, st);
     if (s != DP_OK) return s;
   }
   return DP_OK;

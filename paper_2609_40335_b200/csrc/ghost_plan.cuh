@@ -31,6 +31,7 @@ struct DirectLayerPlan {
 struct GhostPlan {
   bool pair = false;                    // T > 128: 256 x 256 tiles on CTA pairs (two partial sums per item)
   int ntp = 0;                          // tile pairs (ti <= tj) of a T x T Gram matrix
+  int pack = 1;                         // examples whose rows share a 128-row tile (T <= 64)
   int n_per = 0;                        // partial sums per example over all layers
   std::vector<GhostLayerPlan> layer;    // indexed like the caller's layer array
   std::vector<DirectLayerPlan> direct;  // indexed like the caller's layer array

@@ -467,6 +467,38 @@ def test_gram_tiles_of_short_sequences(T, dtype):
     assert int(st.item()) == 0
 
 
+# several examples per Gram tile up to 64 tokens: as many as fit and one more or less, tiles of every multiple of 16 rows,
+# examples across the quarters of a tile; one example that is not a number leaves the others alone
+@pytest.mark.parametrize("B,T", [(300, 1), (127, 1), (2, 7), (40, 3), (8, 16), (9, 16), (7, 17), (15, 17), (33, 31), (4, 32), (5, 32), (4, 33),
+                                 (7, 42), (2, 43), (5, 57), (1, 64), (4, 64)])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_gram_tiles_of_several_examples(B, T, dtype):
+    shapes = [(64, 72), (300, 64), (136, 2500)]
+    layers = [dp.Linear(bf16((B, T, d), 1.0, k, ld=(d + 7) // 8 * 8), bf16((B, T, p), 0.1, 50 + k, ld=(p + 7) // 8 * 8),
+                        d=d, p=p, mode=dp.DP_NORM_GHOST) for k, (d, p) in enumerate(shapes)]
+    if B > 2:
+        layers[1].A[1, T - 1, 5] = float("nan")
+    if dtype == "f32":
+        layers = [dp.Linear(l.A[..., :l.d].float().contiguous(), l.G[..., :l.p].float().contiguous(), d=l.d, p=l.p,
+                            mode=dp.DP_NORM_GHOST) for l in layers]
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    before = dp.dp_set_reserved_sms(146)                   # with two SMs left, tiles are filled however few the items
+    try:
+        for _ in range(2):                                 # the second call finds the first one's shared memory
+            sq = torch.zeros(B, device="cuda")
+            dp.dp_ghost_norms(layers + layers, B, T, sq, dev_status=st)
+    finally:
+        dp.dp_set_reserved_sms(before)
+    got, want = sq.double().cpu().numpy(), np.zeros(B)
+    for l in layers + layers:
+        want += (np.einsum("btp,btd->bpd", f64(l.G, l.p), f64(l.A, l.d)) ** 2).sum((1, 2))
+    keep = np.arange(B) != 1 if B > 2 else np.ones(B, bool)
+    assert keep.all() or np.isnan(got[1])
+    # exact products (f32: the inputs are bf16 numbers), fp32 sums of at most 2500 terms
+    assert (np.abs(got[keep] / want[keep] - 1) < 1e-5).all()
+    assert int(st.item()) == 0
+
+
 # row blocks of equal height in steps of 32 rows: one, two and three blocks of every height, an odd number of column steps
 @pytest.mark.parametrize("T", [129, 160, 161, 192, 200, 224, 225, 256, 257, 300, 330, 384, 390, 430, 448, 512, 513, 600, 768])
 def test_gram_blocks_of_longer_sequences(T):
