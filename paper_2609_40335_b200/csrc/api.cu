@@ -160,7 +160,8 @@ static int resolve_mode(const dp_linear_desc& L, int T) {
 // *_ws_bytes functions see to that), and so several ordinary layers beside a head-sized one.
 struct SplitGroup {
   std::vector<int> index;               // into the caller's layers
-  std::vector<dp_linear_desc> desc;     // the same layers on their split operands
+  std::vector<dp_linear_desc> source;   // the layers
+  std::vector<dp_linear_desc> desc;     // the same on their split operands
   std::vector<SplitJob> jobs;
   size_t bytes = 0;                     // workspace taken by the split operands
   size_t bound = 0;                     // norms: by all of it, at most
@@ -179,6 +180,7 @@ struct SplitGroup {
     jobs.push_back({static_cast<const float*>(L.G), L.ldg, L.p, scale && L.d > L.p, base + bytes});
     bytes += split_bytes(rows, L.p);
     index.push_back(l);
+    source.push_back(L);
     desc.push_back(D);
     tiles += gta_tiles(L);
     out_bytes += align_up(size_t(L.p) * size_t(L.d) * sizeof(float), 256);
@@ -202,10 +204,24 @@ static size_t f32_norm_bytes(const dp_linear_desc& L, int B, int T, int sms) {
 // the place of the partial sums)
 static dp_status f32_norm_group(const SplitGroup& g, int B, int T, float* sq, char* ws, int* dev_status,
                                 cudaStream_t st, bool overwrite, NormSource* left) {
-  const GhostPlan plan = plan_ghost_norms(g.desc.data(), (int)g.desc.size(), B, T, sm_count(), true);
+  GhostPlan plan = plan_ghost_norms(g.desc.data(), (int)g.desc.size(), B, T, sm_count(), true);
   float* partials = reinterpret_cast<float*>(ws + g.bytes);
-  dp_status s = launch_split(g.jobs.data(), (int)g.jobs.size(), B, T, nullptr, st);
+  // ghost norms that split their operands on the way, and what is split beforehand
+  std::vector<int> fused;
+  std::vector<SplitJob> before;
+  std::vector<char> is_fused(g.desc.size(), 0);
+  for (int l : plan.ghost_layers)
+    if (ghost_norm_splits(g.source[size_t(l)], B, T)) { fused.push_back(l); is_fused[size_t(l)] = 1; }
+  for (size_t l = 0; l < g.desc.size(); ++l)
+    if (!is_fused[l]) { before.push_back(g.jobs[2 * l]); before.push_back(g.jobs[2 * l + 1]); }
+  dp_status s = launch_split(before.data(), (int)before.size(), B, T, nullptr, st);
   if (s != DP_OK) return s;
+  if (!fused.empty()) {
+    s = launch_ghost_norm_split(g.source.data(), g.jobs.data(), fused, plan, B, T, partials, dev_status, st);
+    if (s != DP_OK) return s;
+  }
+  plan.ghost_layers.erase(std::remove_if(plan.ghost_layers.begin(), plan.ghost_layers.end(),
+                                         [&](int l) { return is_fused[size_t(l)] != 0; }), plan.ghost_layers.end());
   if (!plan.ghost_layers.empty()) {
     s = launch_ghost_norm_tc(g.desc.data(), plan, B, T, partials, dev_status, st, true);
     if (s != DP_OK) return s;

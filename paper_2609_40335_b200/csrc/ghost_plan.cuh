@@ -52,4 +52,10 @@ dp_status launch_ghost_norm_pair(const dp_linear_desc* layers, const GhostPlan& 
 dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
                                float* partials, int* dev_status, cudaStream_t st, bool split = false);
 
+// fp32 layers of 32 to 128 tokens on a 16-byte boundary and pitch: norm and split in one pass (ghost_norm_split.cu).
+struct SplitJob;
+bool ghost_norm_splits(const dp_linear_desc& L, int B, int T);
+dp_status launch_ghost_norm_split(const dp_linear_desc* layers, const SplitJob* jobs, const std::vector<int>& index,
+                                  const GhostPlan& plan, int B, int T, float* partials, int* dev_status, cudaStream_t st);
+
 }  // namespace dpg

@@ -19,4 +19,8 @@ dp_status make_tmap_bf16_3d(CUtensorMap* out, const void* base, int64_t ld, int 
 // driver encodes made so far (cache misses)
 long long tmap_encode_count();
 
+// the same of fp32 tensors, without a swizzle
+dp_status make_tmap_f32_3d(CUtensorMap* out, const void* base, int64_t ld, int cols, int rows,
+                           int batch, int box_cols, int box_rows);
+
 }  // namespace dpg

@@ -368,6 +368,42 @@ def test_fp32_step_with_kept_operands(ample, kind):
     assert int(ds.dev_status.item()) == 0
 
 
+# fp32 norms that split their operands on the way, for the sums to use: every height of a tile, several examples in one,
+# widths that end inside a step of 64 columns or a word of 8, layers cut into chunks; one whose rows TMA cannot read among them
+@pytest.mark.parametrize("B,T", [(3, 32), (8, 32), (5, 33), (7, 42), (3, 64), (2, 65), (3, 77), (2, 96), (1, 100), (3, 127), (2, 128), (3, 129)])
+def test_fp32_norms_split_on_the_way(B, T):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B * T)
+
+    def normal(cols, std, ld=None):
+        t = torch.full((B, T, ld or cols), float("nan"), device="cuda")
+        t[..., :cols] = torch.randn(B, T, cols, generator=g, device="cuda") * std
+        return t
+
+    shapes = [(64, 64, None), (72, 300, None), (132, 68, 140), (68, 9000, None), (5000, 64, None), (67, 130, 133)]
+    linears = [dp.Linear(normal(i, 1.0, ld), normal(o, 0.05, ld), d=i, p=o) for i, o, ld in shapes]
+    linears[4].mode = dp.DP_NORM_DIRECT
+    vec = dict(dtype=torch.float32, device="cuda")
+    ds = pipeline.DeviceStep(
+        B=B, T=T, V=50, C=1.0, sigma=0.8, tied=False, positions=False, linears=linears, lm=None,
+        ids=torch.zeros(B, T, dtype=torch.int32, device="cuda"), pos_ids=None, G_emb=normal(64, 0.05), d_model=64,
+        sq=torch.zeros(B, **vec), clip=torch.zeros(B, **vec), norms=torch.zeros(B, **vec), cross=None,
+        dev_status=torch.zeros(1, dtype=torch.int32, device="cuda"))
+    pipeline.allocate(ds)
+    for _ in range(2):                                     # the second step finds the first one's workspace
+        ds.ws.fill_(255)
+        pipeline.dp_step(ds, noise=False)
+    want = (ds.G_emb.double().sum(1) ** 2).sum(1)
+    for l in linears:
+        want += (torch.einsum("btp,btd->bpd", l.G[..., :l.p].double(), l.A[..., :l.d].double()) ** 2).sum((1, 2))
+    assert ((ds.sq.double() / want - 1).abs() < 4e-5).all()          # two bf16 terms: 2^-16 of a product at most
+    R = ds.clip.double()[:, None, None]
+    for k, l in enumerate(linears):
+        ref = torch.einsum("btp,btd->pd", R * l.G[..., :l.p].double(), l.A[..., :l.d].double())
+        assert float((ds.outs[f"linear{k}"].double() - ref).norm() / ref.norm()) < 2e-5, k
+    assert int(ds.dev_status.item()) == 0
+
+
 # tiles of 128 tokens x 32 positions, several per block from 2 x 148 tiles on
 @pytest.mark.parametrize("B,T,d,V", [(1, 1, 64, 40), (2, 31, 72, 300), (3, 33, 64, 300), (2, 129, 136, 1000), (75, 128, 64, 100),
                                      (130, 97, 64, 64)])
