@@ -38,17 +38,19 @@ struct GtaNoise {
 // their example instead were filled up with zeros: at T = 203 84 steps of 64 for 21 examples, 67 now; at T = 77 two
 // steps an example, at T = 16 one, three quarters of it zeros.  The step of DistilGPT2 with all its parameters at B = 21, T = 203
 // 1383 -> 1295 us, of GPT-2 small at B = 3, T = 77 349 -> 344; at B = 32, T = 128 (the same steps) 940 -> 945, within the runs'
-// differences.  Coordinates are 32-bit: a batch of 2^31 rows keeps
-// steps per example.
+// differences.  Scaling row by row costs more, so the batch is walked whole only where that saves a sixth of the steps (7 layers
+// of d = 576 at B = 23, T = 57, 21 steps or 23: step 232 us against 217).  Coordinates are 32-bit: a batch of 2^31 rows
+// keeps steps per example.
 struct GtaRows {
   int B, T;                // planes along K, rows of each, as the tensor map has them
   int scaled_rows, scaled_steps;   // scaling: all rows, or 0 and the steps of an example where each has its own
 };
-inline GtaRows gta_rows(int B, int T) {
+inline GtaRows gta_rows(int B, int T, int terms) {
   const long long rows = (long long)B * T;
   const int steps = (T + 63) / 64;
-  if (rows > 0x7fffffffLL - 64) return {B, T, 0, steps};
-  return {1, int(rows), T % 64 == 0 ? 0 : int(rows), steps};
+  if ((T % 64 == 0 || terms > 1) && rows <= 0x7fffffffLL - 64) return {1, int(rows), 0, steps};      // no factors by row
+  if (rows > 0x7fffffffLL - 64 || 6 * ((rows + 63) / 64) > 5LL * B * steps) return {B, T, 0, steps};
+  return {1, int(rows), int(rows), steps};
 }
 
 // Clip factors of a K step's rows: lane k holds those of rows k and k + 32; `one`: they are all the same.
@@ -105,20 +107,24 @@ static __device__ __noinline__ void scale_rows(uint4* part, float lo, float hi, 
   };
   const uint32_t w_lo = split(lo), w_hi = split(hi);
   uint4* x = part + lane;
+  // chunk 32 i + lane of a box lies in row 4 i + lane / 8: four rows of both boxes at a time
 #pragma unroll 1
-  for (int c0 = 0; c0 < 32; c0 += 8) {             // chunk (c0 + q) * 32 + lane lies in row 4 (c0 + q) + lane / 8 of 64
-    const uint32_t mine = (c0 & 8) ? w_hi : w_lo;
+  for (int i0 = 0; i0 < 16; i0 += 4) {
+    const uint32_t mine = i0 & 8 ? w_hi : w_lo;
     uint4 v[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = x[(c0 + q) * 32];
+    for (int q = 0; q < 8; ++q) v[q] = x[(i0 + (q >> 1) + 16 * (q & 1)) * 32];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const uint32_t w = __shfl_sync(0xffffffffu, mine, 4 * q + (lane >> 3));
+    for (int q = 0; q < 8; q += 2) {
+      const uint32_t w = __shfl_sync(0xffffffffu, mine, (4 * (i0 + (q >> 1)) + (lane >> 3)) & 31);
       const __nv_bfloat162 rh2 = pair(w, 0x1010), rl2 = pair(w, 0x3232);
-      __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&v[q]);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) e[k] = __hfma2(e[k], rh2, __hmul2(e[k], rl2));
-      x[(c0 + q) * 32] = v[q];
+      for (int h = 0; h < 2; ++h) {
+        __nv_bfloat162* e = reinterpret_cast<__nv_bfloat162*>(&v[q + h]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) e[k] = __hfma2(e[k], rh2, __hmul2(e[k], rl2));
+        x[(i0 + (q >> 1) + 16 * h) * 32] = v[q + h];
+      }
     }
   }
 }

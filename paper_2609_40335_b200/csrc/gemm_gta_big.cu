@@ -158,14 +158,15 @@ struct Slots {
 // straight code of its own there: with one path for all the epilogue took 180 instructions per counter, 137 of them the
 // generator's, and where few tokens meet many parameters its rate is the step's.  48 GPT-2-small layers at B = 3, T = 77
 // 196.4 -> 179.0 us, 96 of GPT-2 medium at B = 16, T = 128 1470 -> 1443, 24 of GPT-2 small at B = 32, T = 128 377 -> 374.
-// (The same for sums without noise, or the two kernels' epilogues as one function: slower by up to 3 %.)
+// Sums without noise have a kernel without it: 119.5 -> 113.7 us at B = 3, T = 77, 160 -> 153.5 at B = 4, T = 128.
 static __device__ __noinline__ float4 normals4_call(unsigned long long q, const NoiseKeys& K, uint32_t id, uint32_t step) {
   float z[4];
   normals4(q, K, id, step, z);
   return make_float4(z[0], z[1], z[2], z[3]);
 }
 
-template <bool kSplit>
+// kNoise: some layer's noise is drawn in the epilogue
+template <bool kSplit, bool kNoise>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
   const uint32_t rank = ptx::cluster_ctarank();
@@ -384,7 +385,7 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
       const long long ld = L.ldo;
       const bool vec8 = ((ld & 7) == 0) && ((reinterpret_cast<uintptr_t>(L.out) & 31) == 0);
       const bool vec4 = ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(L.out) & 15) == 0);
-      const bool noisy = L.noise_amp >= 0.f;
+      const bool noisy = kNoise && L.noise_amp >= 0.f;
       const float amp = L.noise_amp;
       const uint32_t tensor_id = L.tensor_id;
       const bool common = noisy && vec8 && P.beta == 0.f && P.noise_scale == 1.f;
@@ -483,10 +484,10 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
 
 }  // namespace
 
-template <bool kSplit>
+template <bool kSplit, bool kNoise>
 static dp_status launch_big(const BigParams& P, int units, cudaStream_t st) {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_big_kernel<kSplit>)))
-    DP_CUDA_OK(allow_shared(gemm_gta_big_kernel<kSplit>, kSmemBytes));
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_big_kernel<kSplit, kNoise>)))
+    DP_CUDA_OK((allow_shared(gemm_gta_big_kernel<kSplit, kNoise>, kSmemBytes)));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * units, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -496,7 +497,7 @@ static dp_status launch_big(const BigParams& P, int units, cudaStream_t st) {
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  DP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_gta_big_kernel<kSplit>, P));
+  DP_CUDA_OK((cudaLaunchKernelEx(&cfg, gemm_gta_big_kernel<kSplit, kNoise>, P)));
   ++g_kernel_launches;
   return DP_OK;
 }
@@ -506,7 +507,7 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
                          const GtaNoise* noise, int* dev_status, cudaStream_t st) {
   BigParams P;
   memset(&P, 0, sizeof(P));
-  const GtaRows K = gta_rows(B, T);
+  const GtaRows K = gta_rows(B, T, terms);
   const int planes = terms > 1 ? 2 * K.B : K.B;
   int bigs = 0, singles = 0;
   for (int k = 0; k < n; ++k) {
@@ -554,7 +555,8 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
   P.dev_status = dev_status;
   P.wait_limit = g_wait_limit;
   const int units = std::min(P.total_items, pairs);
-  return terms > 1 ? launch_big<true>(P, units, st) : launch_big<false>(P, units, st);
+  if (terms > 1) return noise ? launch_big<true, true>(P, units, st) : launch_big<true, false>(P, units, st);
+  return noise ? launch_big<false, true>(P, units, st) : launch_big<false, false>(P, units, st);
 }
 
 }  // namespace dpg

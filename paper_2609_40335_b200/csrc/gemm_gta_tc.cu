@@ -643,7 +643,7 @@ static long long gta_tiles(const dp_linear_desc* layers, int n_layers) {
 bool gta_prescales(const dp_linear_desc& L) { return prescale_layer(L); }
 
 int gta_choose_nsplit(long long tiles, int B, int T, int terms, int sms) {
-  const GtaRows K = gta_rows(B, T);
+  const GtaRows K = gta_rows(B, T, terms);
   const int ksteps = K.B * terms * ceil_div(K.T, kBK);
   const int units = kUsePair ? sms / 2 : sms;          // persistent CTAs or CTA pairs
   if (tiles >= 2LL * units) return 1;
@@ -668,7 +668,7 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
                                     int* dev_status, cudaStream_t st) {
   dp_status s = DP_OK;
   const int sms = sm_count();
-  const GtaRows K = gta_rows(B, T);
+  const GtaRows K = gta_rows(B, T, terms);
   const int tsteps = terms * ceil_div(K.T, kBK), planes = terms > 1 ? 2 * K.B : K.B;
   const int ksteps = K.B * tsteps;
   int nsplit = gta_choose_nsplit(gta_tiles(layers, n_layers), B, T, terms, sms);
