@@ -122,8 +122,20 @@ __device__ __forceinline__ void stream_rows(const VecParam& q, long long row_bas
   else stream_rows_t<T, kWeighted, false>(q, row_base, r0, r1, c, nvalid, Tn, clip, acc);
 }
 
+// 0 * (a column's terms), which is 0 or, where one of them is not finite, not a number
+template <typename T>
+__device__ __noinline__ float zero_times_terms(const VecParam& q, long long row_base, int rows, int c) {
+  float z = 0.f;
+  for (int r = 0; r < rows; ++r) {
+    const float g = to_f32(static_cast<const T*>(q.G)[(row_base + r) * q.ldg + c]);
+    z = fmaf(0.f, q.X ? g * to_f32(static_cast<const T*>(q.X)[(row_base + r) * q.ldx + c]) : g, z);
+  }
+  return z;
+}
+
 // grid = (slabs of all parameters, examples): || sum_t G*X ||^2 restricted to the block's columns
-// keep: [B][n_per][256] or nullptr, the block's columns of v_i
+// keep: [B][n_per][256] or nullptr, the block's columns of v_i.  A sum that overflowed is not kept: its example has
+// no finite norm, so its factor is 0 and the clipped sum takes 0 times each of its terms, not 0 times infinity.
 template <typename T>
 __global__ void __launch_bounds__(256, 4)
 vector_norm_kernel(const __grid_constant__ VecParams P, float* __restrict__ partials, int n_per,
@@ -146,7 +158,11 @@ vector_norm_kernel(const __grid_constant__ VecParams P, float* __restrict__ part
 #pragma unroll
   for (int ww = 0; ww < 8; ++ww) v += part[ww][threadIdx.x];
   const size_t at = size_t(i) * n_per + col0_partial + slab;
-  if (keep) keep[at * kVecCols + threadIdx.x] = v;
+  if (keep) {
+    const int cc = (slab - q.slab_begin) * kVecCols + threadIdx.x;
+    const bool finite = fabsf(v) <= 3.402823466e38f;
+    keep[at * kVecCols + threadIdx.x] = finite ? v : zero_times_terms<T>(q, (long long)i * P.T, P.T, cc);
+  }
   const float s = block_sum(v * v, red);
   if (threadIdx.x == 0) partials[at] = s;
 }

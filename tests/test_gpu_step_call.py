@@ -302,3 +302,33 @@ def test_vectors_read_once_and_twice(dtype, B, T, widths):
         # at most 360 products in fp32, added up in another order
         assert_same(results[got], results[want], rel=360 * 2.0 ** -24)
     assert int(ds.dev_status.item()) == 0
+
+
+# finite gradients of one example that overflow when they are summed over its tokens: no finite norm, factor 0, and the
+# example leaves every sum; a term that is itself infinite or not a number shows in its column.  With and without kept sums
+@pytest.mark.parametrize("dtype", [BF16, F32])
+def test_vector_sums_that_overflow_drop_out(dtype):
+    ds = make_step(vectors=dtype, B=5, T=24)
+    big = torch.finfo(dtype).max
+    gain, bias = ds.vectors
+    bias.G[1, :, 3] = big                         # +inf, and with the second pair of signs inf - inf between two warps' rows
+    bias.G[1, ::2, 4], bias.G[1, 1::2, 4] = big, -big
+    gain.G[1, :, 5], gain.X[1, :, 5] = 1e25, 1e10
+    gain.G[2, 7, 6], gain.X[2, 7, 6] = 1e25, 1e25            # the term itself is infinite
+    bias.G[3, 9, 7] = float("nan")
+    results = []
+    for ws in (ds.ws, ds.ws[:ds.ws.numel() - dp.dp_step_vectors_ws_bytes(ds.vectors, ds.B, ds.T)]):
+        ds.ws = ws
+        wipe(ds)
+        pipeline.dp_step(ds, noise=False)
+        results.append(state(ds))
+    kept, read_again = results
+    assert kept["clip"].tolist()[1:4] == [0.0, 0.0, 0.0] and bool((kept["clip"][[0, 4]] > 0).all())
+    for k, (v, bad) in enumerate([(gain, 6), (bias, 7)]):
+        terms = v.G.double() * (v.X.double() if v.X is not None else 1.0)
+        want = (kept["clip"][[0, 4]].double()[:, None] * terms[[0, 4]].sum(1)).sum(0)
+        for got in (kept[f"vector{k}"], read_again[f"vector{k}"]):
+            fine = torch.arange(v.p, device="cuda") != bad
+            assert bool(got[bad].isnan())
+            # at most 48 products in fp32
+            assert float((got.double() - want)[fine].norm()) <= 48 * 2.0 ** -24 * float(want[fine].norm())
