@@ -303,7 +303,8 @@ dp_status dp_fill_noise(float* out, int64_t n, float sigma, float C, float scale
  * `side_stream` the embedding norms, the token sorts, the tables' noise (or zeros) and, once the
  * clip factors exist, the row sums of tables that no GEMM writes.  A caller that steps thousands of
  * times pays one call instead of a dozen.  Nothing is kept between calls.  A DP_STEP_ALL call short of work (a few hundred
- * tokens, small layers, no vectors, positions or tied head) uses `stream` alone, after all that `side_stream` has to do.
+ * tokens, small layers, no vectors, positions or tied head) uses `stream` alone, after all that `side_stream` has to do.  Work that
+ * is put on `side_stream` after the call comes after what the step writes to tables that no GEMM writes.
  * layers [host, n_layers; the LM head, if any, is the last one], with outs / ldos / tensor_ids as in
  * dp_clip_accumulate_noise_grouped (tied: the head's out is wte).  vectors, vector_outs, vector_ids
  * as in dp_clip_accumulate_vectors.  layer_dtype, vector_dtype, embed_dtype: the storage types of the

@@ -1207,18 +1207,24 @@ static dp_status step_rest(const dp_step_desc* S, const float* row_sums) {
 }
 
 // A step short of work uses `stream` alone.  What `side_stream` still has to do, an earlier fill of a table say, comes
-// before it, as when the step used both; inside a capture `side_stream` joins first.
+// before it, and what is put there later comes after it, as when the step used both; inside a capture `side_stream`
+// joins first and is joined again.
 static dp_status small_step(const dp_step_desc* S) {
   cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
   cudaStreamCaptureStatus capture;
   DP_CUDA_OK(cudaStreamIsCapturing(main, &capture));
-  if (capture != cudaStreamCaptureStatusNone) {
-    DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[0], main));
-    DP_CUDA_OK(cudaStreamWaitEvent(side, (cudaEvent_t)S->events[0], 0));
-  }
-  DP_CUDA_OK(cudaEventRecord((cudaEvent_t)S->events[2], side));
-  DP_CUDA_OK(cudaStreamWaitEvent(main, (cudaEvent_t)S->events[2], 0));
-  return launch_small_step(*S, main);
+  auto after = [](cudaStream_t later, cudaStream_t earlier, void* event) {
+    DP_CUDA_OK(cudaEventRecord((cudaEvent_t)event, earlier));
+    DP_CUDA_OK(cudaStreamWaitEvent(later, (cudaEvent_t)event, 0));
+    return DP_OK;
+  };
+  dp_status s = DP_OK;
+  if (capture != cudaStreamCaptureStatusNone) s = after(side, main, S->events[0]);
+  if (s == DP_OK) s = after(main, side, S->events[2]);
+  if (s == DP_OK) s = launch_small_step(*S, main);
+  if (s == DP_OK) s = after(side, main, S->events[0]);
+  if (s == DP_OK && capture != cudaStreamCaptureStatusNone) s = after(main, side, S->events[2]);
+  return s;
 }
 
 dp_status dp_step_enqueue(const dp_step_desc* step, int32_t phases) {

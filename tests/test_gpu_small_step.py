@@ -142,3 +142,34 @@ def test_small_step_comes_after_the_side_stream():
         pipeline.dp_step(ds, seed=5, step=k)
     torch.cuda.synchronize()
     check(ds, 5, 19, True)
+
+
+@pytest.mark.parametrize("captured", [False, True])
+def test_side_stream_comes_after_the_small_step(captured):
+    """Work put on the side stream after the step finds the table as the step wrote it, also inside a capture."""
+    ds = make(F32, F32, 8, 64, 128, [(128, 128)], 8192)
+    pipeline.dp_step(ds, seed=5, step=0)                 # makes the side stream
+    got = torch.empty_like(ds.outs["wte"])
+    torch.cuda.synchronize()
+
+    def step_and_read():
+        torch.cuda._sleep(20_000_000)                    # some 10 ms: the step has not begun when the copy is enqueued
+        n0 = dp.dp_kernel_launches()
+        pipeline.dp_step(ds, seed=5, step=4)
+        assert dp.dp_kernel_launches() - n0 == 2
+        with torch.cuda.stream(ds.side_stream):
+            got.copy_(ds.outs["wte"])
+        torch.cuda.current_stream().wait_stream(ds.side_stream)
+
+    if captured:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            step_and_read()
+        for t in ds.outs.values():
+            t.fill_(9.0)
+        graph.replay()
+    else:
+        step_and_read()
+    torch.cuda.synchronize()
+    check(ds, 5, 4, True)
+    assert torch.equal(got, ds.outs["wte"])
