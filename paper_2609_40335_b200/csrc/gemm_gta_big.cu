@@ -154,19 +154,21 @@ struct Slots {
   }
 };
 
-// Out of line, for the epilogue's general path.  Noise at scale 1 onto an output that is written whole, 32 bytes at a time, has
-// straight code of its own there: with one path for all the epilogue took 180 instructions per counter, 137 of them the
-// generator's, and where few tokens meet many parameters its rate is the step's.  48 GPT-2-small layers at B = 3, T = 77
-// 196.4 -> 179.0 us, 96 of GPT-2 medium at B = 16, T = 128 1470 -> 1443, 24 of GPT-2 small at B = 32, T = 128 377 -> 374.
-// Sums without noise have a kernel without it: 119.5 -> 113.7 us at B = 3, T = 77, 160 -> 153.5 at B = 4, T = 128.
+// What the epilogue writes.  kPlain: sums without noise.  kStraight: noise at scale 1 onto outputs that are written whole, 32 bytes
+// at a time, has straight code of its own, and what little else there is calls the generator: with one path for all the epilogue took 180
+// instructions per counter, 137 of them the generator's, and where few tokens meet many parameters its rate is the step's (the call for
+// 48 GPT-2-small layers at B = 3, T = 77 202 -> 183 us, for 96 of GPT-2 medium at B = 16, T = 128 1310 -> 1255).
+// kGeneral: everything else, the generator in line (called from there, 48 GPT-2-small layers at B = 3, T = 77 with scale 1/B took
+// 276 us instead of 206, with beta = 1 401 instead of 294).
+enum Epilogue { kPlain, kStraight, kGeneral };
+
 static __device__ __noinline__ float4 normals4_call(unsigned long long q, const NoiseKeys& K, uint32_t id, uint32_t step) {
   float z[4];
   normals4(q, K, id, step, z);
   return make_float4(z[0], z[1], z[2], z[3]);
 }
 
-// kNoise: some layer's noise is drawn in the epilogue
-template <bool kSplit, bool kNoise>
+template <bool kSplit, Epilogue kEpilogue>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
   const uint32_t rank = ptx::cluster_ctarank();
@@ -385,10 +387,10 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
       const long long ld = L.ldo;
       const bool vec8 = ((ld & 7) == 0) && ((reinterpret_cast<uintptr_t>(L.out) & 31) == 0);
       const bool vec4 = ((ld & 3) == 0) && ((reinterpret_cast<uintptr_t>(L.out) & 15) == 0);
-      const bool noisy = kNoise && L.noise_amp >= 0.f;
+      const bool noisy = kEpilogue != kPlain && L.noise_amp >= 0.f;
       const float amp = L.noise_amp;
       const uint32_t tensor_id = L.tensor_id;
-      const bool common = noisy && vec8 && P.beta == 0.f && P.noise_scale == 1.f;
+      const bool straight = kEpilogue == kStraight && noisy && vec8;
       for (int h = 0; h < it.nsub; ++h) {
         const uint32_t slot = slots.first(it.nsub) + h;
         if (!ptx::mbar_wait_relaxed(&acc_full[slot], slots.uses(slot) & 1, abort_flag, P.wait_limit)) { ok = false; break; }
@@ -405,7 +407,7 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
           ptx::tmem_ld_wait();
           // free as soon as the last part is in registers, before its noise is drawn
           if (c + 1 == kChunks) free_acc(slot);
-          if (common && row < L.M && col0 + 32 <= L.N) {
+          if (straight && row < L.M && col0 + 32 <= L.N) {
             const unsigned long long q0 = ((unsigned long long)row * L.N + col0) >> 2;
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
@@ -444,8 +446,13 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
                 if (noisy) {
 #pragma unroll
                   for (int k = 0; k < 2; ++k) {
-                    const float4 z4 = normals4_call(q0 + 2 * g + k, P.noise_keys, tensor_id, step);
-                    const float z[4] = {z4.x, z4.y, z4.z, z4.w};
+                    float z[4];
+                    if (kEpilogue == kGeneral) {
+                      normals4(q0 + 2 * g + k, P.noise_keys, tensor_id, step, z);
+                    } else {
+                      const float4 f = normals4_call(q0 + 2 * g + k, P.noise_keys, tensor_id, step);
+                      z[0] = f.x; z[1] = f.y; z[2] = f.z; z[3] = f.w;
+                    }
 #pragma unroll
                     for (int e = 0; e < 4; ++e) v[4 * k + e] = noised(v[4 * k + e], z[e], amp, P.noise_scale);
                   }
@@ -484,10 +491,10 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
 
 }  // namespace
 
-template <bool kSplit, bool kNoise>
+template <bool kSplit, Epilogue kEpilogue>
 static dp_status launch_big(const BigParams& P, int units, cudaStream_t st) {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_big_kernel<kSplit, kNoise>)))
-    DP_CUDA_OK((allow_shared(gemm_gta_big_kernel<kSplit, kNoise>, kSmemBytes)));
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_big_kernel<kSplit, kEpilogue>)))
+    DP_CUDA_OK((allow_shared(gemm_gta_big_kernel<kSplit, kEpilogue>, kSmemBytes)));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * units, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -497,9 +504,16 @@ static dp_status launch_big(const BigParams& P, int units, cudaStream_t st) {
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  DP_CUDA_OK((cudaLaunchKernelEx(&cfg, gemm_gta_big_kernel<kSplit, kNoise>, P)));
+  DP_CUDA_OK((cudaLaunchKernelEx(&cfg, gemm_gta_big_kernel<kSplit, kEpilogue>, P)));
   ++g_kernel_launches;
   return DP_OK;
+}
+
+template <bool kSplit>
+static dp_status launch_big(const BigParams& P, Epilogue epilogue, int units, cudaStream_t st) {
+  return epilogue == kPlain      ? launch_big<kSplit, kPlain>(P, units, st)
+         : epilogue == kStraight ? launch_big<kSplit, kStraight>(P, units, st)
+                                 : launch_big<kSplit, kGeneral>(P, units, st);
 }
 
 // One launch over at most kGtaMaxLayers layers without a K split.
@@ -510,8 +524,13 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
   const GtaRows K = gta_rows(B, T, terms);
   const int planes = terms > 1 ? 2 * K.B : K.B;
   int bigs = 0, singles = 0;
+  long long outputs = 0, odd = 0;               // with noise; of these, not in a full chunk of 32 columns on a 32-byte boundary
   for (int k = 0; k < n; ++k) {
     const GtaBigJob& J = jobs[k];
+    if (J.noise_amp >= 0.f) {
+      outputs += (long long)J.p * J.d;
+      odd += (long long)J.p * (reinterpret_cast<uintptr_t>(J.out) % 32 == 0 && J.ldo % 8 == 0 ? J.d % 32 : J.d);
+    }
     dp_status s = make_tmap_bf16_3d(&P.tmG[k], J.G, J.ldg, J.p, K.T, planes, 64, kBK);
     if (s != DP_OK) return s;
     s = make_tmap_bf16_3d(&P.tmA[k], J.A, J.lda, J.d, K.T, planes, 64, kBK);
@@ -555,8 +574,9 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
   P.dev_status = dev_status;
   P.wait_limit = g_wait_limit;
   const int units = std::min(P.total_items, pairs);
-  if (terms > 1) return noise ? launch_big<true, true>(P, units, st) : launch_big<true, false>(P, units, st);
-  return noise ? launch_big<false, true>(P, units, st) : launch_big<false, false>(P, units, st);
+  // A called generator costs a third of an output's time, the straight code saves a twelfth: one output in eight may be odd.
+  const Epilogue epilogue = !noise ? kPlain : beta == 0.f && noise->scale == 1.f && 8 * odd <= outputs ? kStraight : kGeneral;
+  return terms > 1 ? launch_big<true>(P, epilogue, units, st) : launch_big<false>(P, epilogue, units, st);
 }
 
 }  // namespace dpg

@@ -188,6 +188,27 @@ def test_two_tile_items(shapes, beta, noise, B, T):
     assert int(st.item()) == 0
 
 
+# straight code for noise at scale 1 onto aligned outputs, a few odd columns beside it (chunks of 32 columns, words of
+# eight, widths whose noise is drawn later), the general code from one odd output in eight on, and for scales, beta and alignments of its own
+@pytest.mark.parametrize("widths", [(768,), (800,), (776, 1284), (772, 130), (288, 40, 36, 33), (40,)])
+@pytest.mark.parametrize("scale,beta,pad,offset", [(1.0, 0.0, 0, 0), (0.25, 0.0, 0, 0), (1.0, 1.0, 0, 0), (1.0, 0.0, 8, 0), (1.0, 0.0, 4, 0),
+                                                   (1.0, 0.0, 0, 4), (1.0, 0.0, 1, 3)])
+def test_noise_onto_outputs_of_every_kind(widths, scale, beta, pad, offset):
+    B, T, p = 2, 40, 40000
+    layers = [dp.Linear(bf16((B, T, d), 1.0, k, ld=(d + 7) // 8 * 8), bf16((B, T, p), 0.1, 50 + k), d=d, p=p) for k, d in enumerate(widths)]
+    clip, ids = torch.tensor([0.5, 1.0], device="cuda"), list(range(3, 3 + len(widths)))
+
+    def outs(d_all):
+        return [torch.full((p * (d + pad) + offset,), 0.5, device="cuda")[offset:].view(p, d + pad)[:, :d] for d in d_all]
+
+    got, want = outs(widths), [torch.full((p, d), 0.5, device="cuda") for d in widths]
+    dp.dp_clip_accumulate_noise_grouped(layers, B, T, None, 1.0, got, 0.9, scale, 7, ids, 1, beta=beta, clip=clip)
+    dp.dp_clip_accumulate_grouped(layers, B, T, None, 1.0, want, beta=beta, clip=clip)
+    for g, w, i in zip(got, want, ids):
+        dp.dp_add_noise(w, 0.9, 1.0, scale, 7, i, 1)
+        assert torch.equal(g, w)
+
+
 # K steps run over the rows of the whole batch: one example or many per 64 rows, a step that begins and ends inside
 # one, the last step short; the one-tile kernel (K split and not), the two-tile one, either operand scaled
 @pytest.mark.parametrize("B,T", [(1, 1), (70, 1), (37, 3), (9, 16), (5, 63), (5, 65), (3, 100), (4, 203), (2, 320)])
