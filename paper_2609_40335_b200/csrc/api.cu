@@ -1167,7 +1167,7 @@ static dp_status step_gemm(const dp_step_desc* S, const SplitGroup* kept) {
                               S->stream, kept);
 }
 
-static dp_status step_rest(const dp_step_desc* S, const float* row_sums) {
+static dp_status step_rest(const dp_step_desc* S, float* row_sums) {
   cudaStream_t main = (cudaStream_t)S->stream, side = (cudaStream_t)S->side_stream;
   const dp_dtype dt = (dp_dtype)S->embed_dtype;
   dp_status s;

@@ -219,25 +219,30 @@ vector_combine_kernel(const __grid_constant__ VecParams P, const float* __restri
   q.out[cc] = v;
 }
 
-// The same from the v_i that vector_norm_kernel kept: one block per slab, a lane's four columns are one Philox
-// counter; examples e, e + 2, ... in half e of the block, eight loads in flight.  It runs beside the persistent GEMM,
-// hence 128 threads of 32 registers (see embed_kernels.cu).
+// The same from the v_i that vector_norm_kernel kept: a lane's four columns are one Philox counter; rows e, e + 2, ... of
+// a block's in half e of it, four loads in flight.  It runs beside the persistent GEMM, hence 128 threads of 32 registers (see
+// embed_kernels.cu).  A block walks `rows` rows that lie `row_step` examples apart, weighted with clip unless that is nullptr.  Large
+// batches take two launches: with `rows_per_part` > 0 block y sums that many rows and leaves the result in the first of them, which nobody else
+// reads; then one block per slab adds these up.
 constexpr int kKeptThreads = 128;
+constexpr int kKeptAlone = 112;        // examples that one block walks: at 96 two launches took 50.0 us a step instead of 48.4, at 128 53.1 instead of 54.6
+constexpr int kKeptRows = 64;          // rows of a part
 __global__ void __launch_bounds__(kKeptThreads, 16)
-vector_kept_sum_kernel(const __grid_constant__ VecParams P, const float* __restrict__ keep, int n_per, int col0,
-                       const float* __restrict__ clip, float beta, int with_noise, float amp, float scale,
+vector_kept_sum_kernel(const __grid_constant__ VecParams P, float* keep, int n_per, int col0, const float* __restrict__ clip,
+                       int rows, int row_step, int rows_per_part, float beta, int with_noise, float amp, float scale,
                        const __grid_constant__ NoiseKeys keys, uint32_t step, const uint32_t* __restrict__ step_dev) {
   __shared__ float4 part[kVecCols / 4];
   const int slab = blockIdx.x;
   const VecParam& q = P.prm[find_param(P, slab)];
   const int half = threadIdx.x >> 6, quad = threadIdx.x & 63;
-  const float4* src = reinterpret_cast<const float4*>(keep + size_t(col0 + slab) * kVecCols) + quad;
-  const size_t pitch = size_t(n_per) * (kVecCols / 4);
+  const int r0 = int(blockIdx.y) * rows_per_part, r1 = rows_per_part ? min(rows, r0 + rows_per_part) : rows;
+  float4* src = reinterpret_cast<float4*>(keep + size_t(col0 + slab) * kVecCols) + quad;
+  const size_t pitch = size_t(n_per) * (kVecCols / 4) * row_step;
   float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-  for (int i = half; i < P.B; i += 2) {
-    const float4 v = __ldg(src + size_t(i) * pitch);
-    const float r = __ldg(clip + i);
+  for (int i = r0 + half; i < r1; i += 2) {
+    const float4 v = src[size_t(i) * pitch];
+    const float r = clip ? __ldg(clip + i) : 1.f;
     a.x = fmaf(r, v.x, a.x); a.y = fmaf(r, v.y, a.y); a.z = fmaf(r, v.z, a.z); a.w = fmaf(r, v.w, a.w);
   }
   if (half) part[quad] = a;
@@ -245,6 +250,7 @@ vector_kept_sum_kernel(const __grid_constant__ VecParams P, const float* __restr
   if (half) return;
   const float4 b = part[quad];
   float v[4] = {a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w};
+  if (rows_per_part) { src[size_t(r0) * pitch] = make_float4(v[0], v[1], v[2], v[3]); return; }
   const int c = (slab - q.slab_begin) * kVecCols + 4 * quad;
   if (c >= q.p) return;
   float z[4] = {0.f, 0.f, 0.f, 0.f};
@@ -340,17 +346,28 @@ size_t vector_keep_bytes(const dp_vector_desc* prm, int n, int B) {
   return size_t(B) * vector_total_slabs(prm, n) * kVecCols * sizeof(float);
 }
 
-dp_status launch_vector_kept_sums(const dp_vector_desc* prm, int n, int B, int T, const float* keep, const float* clip,
+dp_status launch_vector_kept_sums(const dp_vector_desc* prm, int n, int B, int T, float* keep, const float* clip,
                                   float* const* outs, float beta, int with_noise, float amp, float scale, uint64_t seed,
                                   const uint32_t* tensor_ids, uint32_t step, cudaStream_t st) {
   if (first_use_on_this_device(reinterpret_cast<const void*>(&vector_kept_sum_kernel)))
     DP_CUDA_OK(prefer_max_shared(vector_kept_sum_kernel));
   const int n_per = vector_total_slabs(prm, n);
+  // one block per slab as long as its serial walk is short; beyond, parts at least as long as there are parts.  Step of six biases of 768
+  // at T = 8 and B = 256, 1024, 4096: 72, 168, 481 us with G read twice, 75, 240, 950 with one block per slab, 65, 164, 432 now.
+  int per_part = 0;
+  if (B > kKeptAlone) for (per_part = kKeptRows; (long long)per_part * per_part < B; per_part *= 2) {}
+  const int parts = per_part ? ceil_div(B, per_part) : 1;
   int col0 = 0;
   for (int n0 = 0; n0 < n; n0 += kVecMaxParams) {
     VecParams P;
     const int slabs = fill_params(P, prm, n0, std::min(n, n0 + kVecMaxParams), outs, tensor_ids, B, T);
-    vector_kept_sum_kernel<<<slabs, kKeptThreads, 0, st>>>(P, keep, n_per, col0, clip, beta, with_noise, amp, scale,
+    if (per_part) {
+      vector_kept_sum_kernel<<<dim3(slabs, parts), kKeptThreads, 0, st>>>(P, keep, n_per, col0, clip, B, 1, per_part, 0.f, 0, 0.f,
+                                                                         1.f, expand_noise_keys(seed), step, g_step_dev);
+      DP_LAUNCH_OK();
+    }
+    vector_kept_sum_kernel<<<slabs, kKeptThreads, 0, st>>>(P, keep, n_per, col0, per_part ? nullptr : clip, per_part ? parts : B,
+                                                          per_part ? per_part : 1, 0, beta, with_noise, amp, scale,
                                                           expand_noise_keys(seed), step, g_step_dev);
     DP_LAUNCH_OK();
     col0 += slabs;

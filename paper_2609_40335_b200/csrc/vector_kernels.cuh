@@ -15,7 +15,8 @@ int vector_row_splits(const dp_vector_desc* prm, int n, int B, int T, int sms);
 dp_status launch_vector_norms(const dp_vector_desc* prm, int n, dp_dtype dt, int B, int T,
                               float* partials, int n_per, cudaStream_t st, float* keep = nullptr);
 size_t vector_keep_bytes(const dp_vector_desc* prm, int n, int B);
-dp_status launch_vector_kept_sums(const dp_vector_desc* prm, int n, int B, int T, const float* keep, const float* clip,
+// (the kept sums of large batches are used up)
+dp_status launch_vector_kept_sums(const dp_vector_desc* prm, int n, int B, int T, float* keep, const float* clip,
                                   float* const* outs, float beta, int with_noise, float amp, float scale, uint64_t seed,
                                   const uint32_t* tensor_ids, uint32_t step, cudaStream_t st);
 // partial_ws: [row splits][sum of p over one launch's parameters] floats

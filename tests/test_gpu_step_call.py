@@ -332,3 +332,31 @@ def test_vector_sums_that_overflow_drop_out(dtype):
             assert bool(got[bad].isnan())
             # at most 48 products in fp32
             assert float((got.double() - want)[fine].norm()) <= 48 * 2.0 ** -24 * float(want[fine].norm())
+
+
+# kept sums of more examples than a block walks by itself: one more, one short part, parts of more than 64 (beyond 4096)
+@pytest.mark.parametrize("B", [112, 113, 128, 130, 4097])
+def test_kept_sums_of_large_batches(B):
+    ds = make_step(vectors=F32, B=B, T=8, V=100, lm=False)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B)
+    ds.vectors = [dp.Vector(torch.randn(B, 8, p, generator=g, device="cuda") * 0.05, None, p=p) for p in (3, 64, 300)]
+    pipeline.allocate(ds)
+    wipe(ds)
+    n0 = dp.dp_kernel_launches()
+    pipeline.dp_step(ds, seed=3, step=2)
+    with_room = dp.dp_kernel_launches() - n0
+    got = state(ds)
+    tid = pipeline.tensor_ids(ds)
+    for k, v in enumerate(ds.vectors):
+        z = torch.zeros((v.p + 3) // 4 * 4, device="cuda")
+        dp.dp_fill_noise(z, ds.sigma, 1.0, 1.0, 3, tid[f"vector{k}"], 2)
+        terms = v.G.double() * got["clip"].double()[:, None, None]
+        # at most 8 B products in fp32, and the noise's own rounding
+        bound = 2.0 ** -24 * (8 * B * terms.abs().sum((0, 1)) / B + 4 * z[:v.p].double().abs() + terms.abs().sum((0, 1)))
+        assert ((got[f"vector{k}"].double() - terms.sum((0, 1)) - z[:v.p].double()).abs() <= bound).all(), k
+    ds.ws = ds.ws[:ds.ws.numel() - dp.dp_step_vectors_ws_bytes(ds.vectors, B, 8)]
+    n0 = dp.dp_kernel_launches()
+    pipeline.dp_step(ds, seed=3, step=2)
+    assert dp.dp_kernel_launches() - n0 - with_room == (1 if B <= 112 else 0)
+    assert_same(state(ds), got, rel=8 * 64 * 2.0 ** -24)
