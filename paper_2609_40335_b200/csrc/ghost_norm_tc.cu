@@ -34,11 +34,11 @@ constexpr int kTileBytes = kTile * kKStep * 2;   // 16 KiB
 // pair is diagonal, so stages shrink to one tile and twice as many are kept in flight (the
 // kernel is HBM-bound there: bytes in flight are what counts).  Split operands (fp32 inputs) bring
 // two tiles, high and low terms, for each.
-// Up to 64 tokens a tile holds several examples (kPacked): the rows of a batch lie one after the other, so 128 / T of them
-// fill it, its Gram matrix has theirs on the diagonal, and the epilogue multiplies only those blocks.  An example by itself
-// took the 550 cycles of a stage's hand-offs, an item's start and its epilogue for a few KiB.  Tiles are as tall as their
-// examples, rounded up to 16 rows; where the whole batch fills less than half of one, a stage holds two or four of them, 64
-// columns each (kBoxes).  97 layers of d = 128 at B = 95, T = 17 115 -> 50 us, 49 at B = 91, T = 39 70 -> 50; never so many
+// Up to 64 tokens tiles are as tall as their examples, rounded up to 16 rows (kShort), and where that is less than half of one a stage
+// holds two or four of them, 64 columns each (kBoxes): a stage's hand-offs take 550 cycles whatever it carries.  Where there is work enough
+// a tile holds several examples (kPacked): the rows of a batch lie one after the other, so 128 / T of them fill it, its Gram matrix has
+// theirs on the diagonal, and the epilogue multiplies only those blocks.  An example by itself has the plainer epilogue (a GPT-2-small
+// block at B = 1, 2 and 4, T = 64 10.0, 10.8 and 10.8 us with the other, 9.7, 10.3 and 10.3 with its own).  97 layers of d = 128 at B = 95, T = 17 115 -> 50 us, 49 at B = 91, T = 39 70 -> 50; never so many
 // examples that fewer than two items per SM remain (5 fp32 layers at B = 2, T = 54: 7.7 -> 10.2 with both in one tile).  Above 64 tokens
 // short tiles and sizes known at run time cost more than they save (115 -> 122 us at B = 32, T = 128): there
 // tiles are full and everything is constant.
@@ -48,15 +48,17 @@ constexpr size_t kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 1024 /*bar
 constexpr int kThreads = 192;
 constexpr int kTmemCols = 512;                   // 2 buffers x (S_A 128 + S_G 128) columns; split: hi hi, small products
 
+// rows of a tile: a tile of one example's; one short example's; several short examples'
+enum Rows { kFullTile, kShortTile, kPackedTile };
+
 struct __align__(64) GhostParams {
   CUtensorMap tmA[kGhostMaxLayers];
   CUtensorMap tmG[kGhostMaxLayers];
   GhostLayerPlan layer[kGhostMaxLayers];
   int n_layers;
   int B, T, nt, ntp;
-  int rows, stages;          // packed: rows of a tile, stages of the ring
-  int pack;                  // packed: examples per tile ...
-  int row_step, plane_step;  // ... and where the rows of the next tile begin: so many rows on, or so many planes
+  int rows, stages;          // short: rows of a tile, stages of the ring
+  int pack;                  // packed: examples per tile
   int low_plane;             // split operands: first plane of low terms
   int total_items;
   int n_per;                 // partial sums per example in the workspace
@@ -108,18 +110,19 @@ __device__ __forceinline__ uint32_t add_f32(uint32_t a, uint32_t b) {
 // 25 layers of DistilGPT2's shapes at B = 64, T = 256, error against 64 bits: 2.2e-5 with all three in one, now
 // 1.4e-5.  The epilogue no longer overlaps the next item's MMAs; fewer chunks of wide operands make up for it (the fp32
 // step of DistilGPT2 at B = 8, T = 128: no difference beyond 0.5 %).
-template <bool kDiagOnly, bool kSplit, bool kPacked, int kBoxes>
+template <bool kDiagOnly, bool kSplit, Rows kRows, int kBoxes>
 __global__ void __launch_bounds__(kThreads, 1)
 ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
-  static_assert(kDiagOnly || !kPacked, "packed examples: diagonal pairs only");
-  static_assert(kPacked || kBoxes == 1, "several column tiles per stage: packed examples only");
+  constexpr bool kShort = kRows != kFullTile, kPacked = kRows == kPackedTile;
+  static_assert(kDiagOnly || !kShort, "short tiles: diagonal pairs only");
+  static_assert(kShort || kBoxes == 1, "several column tiles per stage: short tiles only");
   // an MMA reads 128 rows of its first operand whatever `rows` is: rows beyond it come from the next
   // stages (the ring ends a whole tile after its last tile begins) and fill accumulator rows nobody reads
-  const int rows = kPacked ? P.rows : kTile;
+  const int rows = kShort ? P.rows : kTile;
   const uint32_t tile_bytes = uint32_t(rows) * (kKStep * 2);
   const uint32_t term_bytes = (kSplit ? 2 : 1) * tile_bytes;             // one row tile, all its terms
   const uint32_t stage_bytes = (kDiagOnly ? kBoxes : 2) * term_bytes;
-  const int n_stages = kPacked ? P.stages : kRingBytes / int((kDiagOnly ? 1 : 2) * (kSplit ? 2 : 1) * kTileBytes);
+  const int n_stages = kShort ? P.stages : kRingBytes / int((kDiagOnly ? 1 : 2) * (kSplit ? 2 : 1) * kTileBytes);
   extern __shared__ uint8_t smem_raw[];
   // 128-byte swizzled tiles need 1024-byte alignment
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -166,8 +169,8 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
       const Item it = decode_item<kPacked>(P, item, lay);
       const bool diag = kDiagOnly || (it.ti == it.tj);
       const uint32_t bytes = diag ? term_bytes : stage_bytes;
-      const int ex = kPacked ? it.example * P.plane_step : it.example, low = ex + P.low_plane;   // planes (split: high and low terms)
-      const int row_i = kPacked ? it.example * P.row_step : it.ti * kTile;
+      const int ex = kPacked ? 0 : it.example, low = ex + P.low_plane;       // planes (split: high and low terms)
+      const int row_i = kPacked ? it.example * P.pack * P.T : it.ti * kTile;
       for (int pass = 0; pass < 2 && ok; ++pass) {
         const uint64_t tm = reinterpret_cast<uint64_t>(pass == 0 ? &P.tmA[it.layer] : &P.tmG[it.layer]);
         const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
@@ -175,9 +178,9 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
           ok = ptx::warp_ok(ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit));
           if (!ok) break;
           const uint32_t dst = tiles_a + stage * stage_bytes, bar = full_a + 8 * stage;
-          const int nb = kPacked ? min(kBoxes, k1 - k) : 1;
+          const int nb = kShort ? min(kBoxes, k1 - k) : 1;
           if (ptx::elect_one()) {
-            ptx::mbar_arrive_expect_tx_a(bar, kPacked ? nb * term_bytes : bytes);
+            ptx::mbar_arrive_expect_tx_a(bar, kShort ? nb * term_bytes : bytes);
 #pragma unroll
             for (int b = 0; b < kBoxes; ++b) {
               if (b >= nb) break;
@@ -227,7 +230,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
           ok = ptx::warp_ok(ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit));
           if (!ok) break;
           ptx::tc_fence_after();
-          const int nb = kPacked ? min(kBoxes, nsteps - k) : 1;
+          const int nb = kShort ? min(kBoxes, nsteps - k) : 1;
           if (ptx::elect_one()) {
 #pragma unroll
             for (int b = 0; b < kBoxes; ++b) {
@@ -278,7 +281,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
 #pragma unroll 1
       for (int c = c_lo; c < c_hi; c += 32) {
         uint32_t ra[32], rg[32];
-        if (!kPacked || c + 32 <= rows) {
+        if (!kShort || c + 32 <= rows) {
           ptx::tmem_ld_32x32b_x32(t0 + c, ra);
           ptx::tmem_ld_32x32b_x32(t0 + 128 + c, rg);
           if (kSplit) {
@@ -326,6 +329,7 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
         epi_red[slot * kTile + row] = acc;
         __syncwarp();
       } else {
+        if (kShort && row >= P.T) acc = 0.f;         // a row beyond the tile: whatever lay there
         acc = warp_sum(acc);
         if (lane == 0) epi_red[slot * 4 + ew] = acc;
       }
@@ -394,12 +398,12 @@ dp_status launch_reduce_partials(const float* partials, int n_per, int B, float*
 
 namespace {
 
-template <bool kDiagOnly, bool kSplit, bool kPacked, int kBoxes>
+template <bool kDiagOnly, bool kSplit, Rows kRows, int kBoxes>
 dp_status launch_variant(const GhostParams& P, cudaStream_t st) {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_tc_kernel<kDiagOnly, kSplit, kPacked, kBoxes>)))
-    DP_CUDA_OK((allow_shared(ghost_norm_tc_kernel<kDiagOnly, kSplit, kPacked, kBoxes>, kSmemBytes)));
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_tc_kernel<kDiagOnly, kSplit, kRows, kBoxes>)))
+    DP_CUDA_OK((allow_shared(ghost_norm_tc_kernel<kDiagOnly, kSplit, kRows, kBoxes>, kSmemBytes)));
   const int grid = std::min(P.total_items, sm_count());
-  ghost_norm_tc_kernel<kDiagOnly, kSplit, kPacked, kBoxes><<<grid, kThreads, kSmemBytes, st>>>(P);
+  ghost_norm_tc_kernel<kDiagOnly, kSplit, kRows, kBoxes><<<grid, kThreads, kSmemBytes, st>>>(P);
   DP_LAUNCH_OK();
   return DP_OK;
 }
@@ -411,10 +415,11 @@ dp_status launch_variant(const GhostParams& P, cudaStream_t st) {
 dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& plan, int B, int T,
                                float* partials, int* dev_status, cudaStream_t st, bool split) {
   const int nt = ceil_div(T, kTile);
-  const bool packed = T <= 64, flat = plan.pack > 1 || B == 1;       // flat: the rows of the batch as one dimension
-  const int rows = packed ? (plan.pack * T + 15) / 16 * 16 : kTile, tile_bytes = rows * kKStep * 2;
-  const int map_rows = packed && flat ? B * T : T, examples = packed && flat ? 1 : B, planes = (split ? 2 : 1) * examples;
-  const int boxes = !packed || rows > 64 ? 1 : rows > 32 || split ? 2 : 4;
+  const Rows kind = T > 64 ? kFullTile : plan.pack == 1 ? kShortTile : kPackedTile;
+  const bool packed = kind == kPackedTile;                     // the rows of the batch as one dimension
+  const int rows = kind == kFullTile ? kTile : (plan.pack * T + 15) / 16 * 16, tile_bytes = rows * kKStep * 2;
+  const int map_rows = packed ? B * T : T, examples = packed ? 1 : B, planes = (split ? 2 : 1) * examples;
+  const int boxes = kind == kFullTile || rows > 64 ? 1 : rows > 32 || split ? 2 : 4;
   const int stages = std::min(kMaxStages, (kRingBytes - (kTileBytes - tile_bytes)) / (boxes * (split ? 2 : 1) * tile_bytes));
   const int groups = packed ? ceil_div(B, plan.pack) : B;
   // layers are processed in groups that fit one parameter block
@@ -438,7 +443,6 @@ dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& pl
     P.n_layers = int(g1 - g0);
     P.B = B; P.T = T; P.nt = nt; P.ntp = plan.ntp;
     P.rows = rows; P.stages = stages; P.pack = plan.pack; P.low_plane = examples;
-    P.row_step = flat ? plan.pack * T : 0; P.plane_step = flat ? 0 : 1;
     P.total_items = items;
     P.n_per = plan.n_per;
     P.partials = partials;
@@ -446,14 +450,19 @@ dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& pl
     P.wait_limit = g_wait_limit;
     dp_status s;
     if (split)
-      s = nt > 1 ? launch_variant<false, true, false, 1>(P, st)
-          : !packed ? launch_variant<true, true, false, 1>(P, st)
-          : boxes == 1 ? launch_variant<true, true, true, 1>(P, st) : launch_variant<true, true, true, 2>(P, st);
+      s = nt > 1              ? launch_variant<false, true, kFullTile, 1>(P, st)
+          : kind == kFullTile ? launch_variant<true, true, kFullTile, 1>(P, st)
+          : !packed           ? launch_variant<true, true, kShortTile, 2>(P, st)
+          : boxes == 1        ? launch_variant<true, true, kPackedTile, 1>(P, st)
+                              : launch_variant<true, true, kPackedTile, 2>(P, st);
     else
-      s = nt > 1 ? launch_variant<false, false, false, 1>(P, st)
-          : !packed ? launch_variant<true, false, false, 1>(P, st)
-          : boxes == 1 ? launch_variant<true, false, true, 1>(P, st)
-          : boxes == 2 ? launch_variant<true, false, true, 2>(P, st) : launch_variant<true, false, true, 4>(P, st);
+      s = nt > 1              ? launch_variant<false, false, kFullTile, 1>(P, st)
+          : kind == kFullTile ? launch_variant<true, false, kFullTile, 1>(P, st)
+          : !packed           ? (boxes == 2 ? launch_variant<true, false, kShortTile, 2>(P, st)
+                                            : launch_variant<true, false, kShortTile, 4>(P, st))
+          : boxes == 1        ? launch_variant<true, false, kPackedTile, 1>(P, st)
+          : boxes == 2        ? launch_variant<true, false, kPackedTile, 2>(P, st)
+                              : launch_variant<true, false, kPackedTile, 4>(P, st);
     if (s != DP_OK) return s;
   }
   return DP_OK;
