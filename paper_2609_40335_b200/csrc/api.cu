@@ -174,10 +174,10 @@ struct SplitGroup {
     const long long rows = (long long)B * T;
     D.mode = resolve_mode(L, T);
     D.A = base + bytes; D.lda = split_padded(L.d);
-    jobs.push_back({static_cast<const float*>(L.A), L.lda, L.d, scale && L.d <= L.p, base + bytes});
+    jobs.push_back({static_cast<const float*>(L.A), L.lda, L.d, scale && a_is_scaled(L), base + bytes});
     bytes += split_bytes(rows, L.d);
     D.G = base + bytes; D.ldg = split_padded(L.p);
-    jobs.push_back({static_cast<const float*>(L.G), L.ldg, L.p, scale && L.d > L.p, base + bytes});
+    jobs.push_back({static_cast<const float*>(L.G), L.ldg, L.p, scale && !a_is_scaled(L), base + bytes});
     bytes += split_bytes(rows, L.p);
     index.push_back(l);
     source.push_back(L);
@@ -201,9 +201,9 @@ static size_t f32_norm_bytes(const dp_linear_desc& L, int B, int T, int sms) {
 }
 
 // norms of a group of fp32 layers: split, Gram or gradient-tile kernels, one reduction (or, with `left`,
-// the place of the partial sums)
+// the place of the partial sums).  keep: split operands that clipped sums can use are in place afterwards
 static dp_status f32_norm_group(const SplitGroup& g, int B, int T, float* sq, char* ws, int* dev_status,
-                                cudaStream_t st, bool overwrite, NormSource* left) {
+                                cudaStream_t st, bool overwrite, NormSource* left, bool keep) {
   GhostPlan plan = plan_ghost_norms(g.desc.data(), (int)g.desc.size(), B, T, sm_count(), true);
   float* partials = reinterpret_cast<float*>(ws + g.bytes);
   // ghost norms that split their operands on the way, and what is split beforehand
@@ -217,7 +217,7 @@ static dp_status f32_norm_group(const SplitGroup& g, int B, int T, float* sq, ch
   dp_status s = launch_split(before.data(), (int)before.size(), B, T, nullptr, st);
   if (s != DP_OK) return s;
   if (!fused.empty()) {
-    s = launch_ghost_norm_split(g.source.data(), g.jobs.data(), fused, plan, B, T, partials, dev_status, st);
+    s = launch_ghost_norm_split(g.source.data(), g.jobs.data(), fused, plan, B, T, keep, partials, dev_status, st);
     if (s != DP_OK) return s;
   }
   plan.ghost_layers.erase(std::remove_if(plan.ghost_layers.begin(), plan.ghost_layers.end(),
@@ -396,13 +396,13 @@ static dp_status ghost_norms_impl(const GhostPlan& plan, dp_linear_desc* layers,
       if (s != DP_OK) return s;
       overwrite = false;
     }
-    int flushed = 0;
-    auto flush = [&]() {
+    bool one_group = true;               // so far
+    auto flush = [&](bool last) {
       if (group.index.empty()) return DP_OK;
-      const bool all = (int)group.index.size() == n_layers;
-      const dp_status s = f32_norm_group(group, B, T, sq, base, dev_status, st, overwrite, all ? left : nullptr);
-      overwrite = false;
-      if (kept) { if (flushed++ == 0) *kept = std::move(group); else *kept = SplitGroup(); }
+      const bool all = (int)group.index.size() == n_layers, keep = kept && last && one_group;
+      const dp_status s = f32_norm_group(group, B, T, sq, base, dev_status, st, overwrite, all ? left : nullptr, keep);
+      overwrite = one_group = false;
+      if (keep) *kept = std::move(group);
       group = SplitGroup();
       return s;
     };
@@ -411,7 +411,7 @@ static dp_status ghost_norms_impl(const GhostPlan& plan, dp_linear_desc* layers,
       if (together && !on_tensor_cores(layers[l], dt, T) && plan.mode_used[l] == DP_NORM_GHOST) continue;
       if (dt == DP_F32 && f32_on_tensor_cores(layers[l], T)) {
         const size_t more = f32_norm_bytes(layers[l], B, T, sm_count());
-        if (group.bound + more > ws_bytes) s = flush();
+        if (group.bound + more > ws_bytes) s = flush(false);
         if (s != DP_OK) return s;
         group.bound += more;
         group.add(layers[l], l, B, T, false, base);
@@ -422,7 +422,7 @@ static dp_status ghost_norms_impl(const GhostPlan& plan, dp_linear_desc* layers,
       if (s != DP_OK) return s;
       layers[l].mode_used = plan.mode_used[l];
     }
-    return flush();
+    return flush(true);
   }
   float* partials = static_cast<float*>(ws);
   dp_status s = DP_OK;
@@ -699,12 +699,12 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
     std::vector<int> fma;                // layers on the fp32 kernels: one launch for all of them
     if (kept && !kept->index.empty() && !sq &&
         kept->bytes + gta_partial_bytes(kept->desc.data(), (int)kept->desc.size(), B, T, 3, sm_count()) <= ws_bytes) {
-      // the norms' split operands are still there: only the narrower one of each layer is split again, scaled
+      // the norms' split operands are still there, but for the narrower one of each layer, which is split (again), scaled
       group = *kept;
       base = static_cast<char*>(ws);
       group.jobs.clear();
       for (size_t k = 0; k < kept->index.size(); ++k) {
-        SplitJob J = kept->jobs[2 * k + (layers[kept->index[k]].d <= layers[kept->index[k]].p ? 0 : 1)];
+        SplitJob J = kept->jobs[2 * k + (a_is_scaled(layers[kept->index[k]]) ? 0 : 1)];
         J.scaled = true;
         group.jobs.push_back(J);
       }

@@ -1,14 +1,15 @@
 // Ghost norm of fp32 layers of at most 128 tokens, and their split into two bf16 terms, in one pass over the operands.
 //
 // The Gram products are those of ghost_norm_tc.cu on split operands (S = hi hi^T + hi lo^T + lo hi^T, the two small
-// products in an accumulator of their own); the terms are those of split_kernels.cu and go to the same place, where the
-// clipped sums find them.  There the split read 4 bytes per value and wrote 4, and the Gram kernel read 4 again.  Here
-// the tiles arrive in fp32 and eight converter warps make both terms on the way: into shared memory, in the swizzled
-// layout that the MMAs read, and into the planes.  Each column of the wider operand is some item's own; the narrower one,
-// which every chunk of a layer multiplies, is written by the first.
+// products in an accumulator of their own); the terms are those of split_kernels.cu.  There the split read 4 bytes per value and
+// wrote 4, and the Gram kernel read 4 again.  Here the tiles arrive in fp32 and eight converter warps make both terms on the way, into
+// shared memory, in the swizzled layout that the MMAs read; and, where clipped sums follow that can use them, into the planes where
+// these look for them.  That is the wider operand of a layer: the narrower one is split again, scaled, for the sums.  Each column of the
+// operand that is cut into chunks is some item's own; the other, which every chunk of a layer multiplies, is written by the first.
 //
-// Bound by HBM (4 bytes in, 4 out per value: 157 us for DistilGPT2's 25 layers at B = 8, T = 128, where split and Gram kernel took
-// 152 each) and by its last wave (156 steps on the busiest SM, 119 on average).  The step 870 -> 830 us.
+// Bound by HBM (4 bytes in, and 4 out for the values that are kept) and by its last wave (156 steps on the busiest SM, 119 on average).
+// Norms alone of DistilGPT2's 25 layers at B = 8, T = 128: 275 us split first, 227 with every plane stored, 145 with none; the step
+// 876 -> 841, stores of the narrower operand included or not.
 //
 // A tile holds the rows of as many whole examples as fit into 128 (one above 64 tokens; see ghost_norm_tc.cu), rounded up to
 // 16 rows.  Roles per CTA (448 threads): warp 0 TMA producer, warp 1 MMA issuer, warps 2 - 5 epilogue, warps 6 - 13
@@ -42,7 +43,7 @@ constexpr size_t kRingBytes = size_t(kStagesIn + kStages) * kStageBytes;
 constexpr size_t kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 1024 /*barriers*/ + 4 * kTile * sizeof(float);
 
 struct SplitPlanes {
-  __nv_bfloat16* hi;
+  __nv_bfloat16* hi;                               // nullptr: not kept
   __nv_bfloat16* lo;
   int cols;                                        // pitch, a multiple of 8
 };
@@ -209,7 +210,7 @@ ghost_norm_split_kernel(const __grid_constant__ SplitGramParams P) {
       const int own = (int)min((long long)P.pack * P.T, batch_rows - row0);        // rows of this tile's examples
       for (int pass = 0; pass < 2 && ok; ++pass) {
         const SplitPlanes& D = pass == 0 ? P.A[it.layer] : P.G[it.layer];
-        const bool write = pass == 0 ? it.write_a : it.write_g;
+        const bool write = D.hi && (pass == 0 ? it.write_a : it.write_g);
         const int k0 = pass == 0 ? it.a0 : it.g0, k1 = pass == 0 ? it.a1 : it.g1;
         for (int k = k0; k < k1; ++k) {
           ok = ptx::mbar_wait_a(in_full_a + 8 * s_in, ph_in, abort_flag, P.wait_limit) &&
@@ -340,9 +341,10 @@ bool ghost_norm_splits(const dp_linear_desc& L, int B, int T) {
          L.lda % 4 == 0 && L.ldg % 4 == 0;
 }
 
-// index: layers of the plan, with the fp32 operands in `layers`; jobs: their split, A and G of layer k at 2k and 2k + 1
+// index: layers of the plan, with the fp32 operands in `layers`; jobs: their split, A and G of layer k at 2k and 2k + 1;
+// keep: the wider operand's is stored
 dp_status launch_ghost_norm_split(const dp_linear_desc* layers, const SplitJob* jobs, const std::vector<int>& index,
-                                  const GhostPlan& plan, int B, int T, float* partials, int* dev_status, cudaStream_t st) {
+                                  const GhostPlan& plan, int B, int T, bool keep, float* partials, int* dev_status, cudaStream_t st) {
   if (first_use_on_this_device(reinterpret_cast<const void*>(&ghost_norm_split_kernel)))
     DP_CUDA_OK(allow_shared(ghost_norm_split_kernel, kSmemBytes));
   const int rows = (plan.pack * T + 15) / 16 * 16, groups = ceil_div(B, plan.pack);
@@ -363,8 +365,7 @@ dp_status launch_ghost_norm_split(const dp_linear_desc* layers, const SplitJob* 
         __nv_bfloat16* hi = static_cast<__nv_bfloat16*>(J.dst);
         return SplitPlanes{hi, hi + size_t(B) * T * split_padded(J.c), split_padded(J.c)};
       };
-      P.A[k] = planes(jobs[2 * li]);
-      P.G[k] = planes(jobs[2 * li + 1]);
+      if (keep) (a_is_scaled(L) ? P.G[k] : P.A[k]) = planes(jobs[a_is_scaled(L) ? 2 * li + 1 : 2 * li]);
       P.layer[k] = plan.layer[li];
       P.layer[k].item_begin = items;
       items += groups * plan.layer[li].nsplit;

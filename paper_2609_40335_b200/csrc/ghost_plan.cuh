@@ -56,6 +56,6 @@ dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& pl
 struct SplitJob;
 bool ghost_norm_splits(const dp_linear_desc& L, int B, int T);
 dp_status launch_ghost_norm_split(const dp_linear_desc* layers, const SplitJob* jobs, const std::vector<int>& index,
-                                  const GhostPlan& plan, int B, int T, float* partials, int* dev_status, cudaStream_t st);
+                                  const GhostPlan& plan, int B, int T, bool keep, float* partials, int* dev_status, cudaStream_t st);
 
 }  // namespace dpg

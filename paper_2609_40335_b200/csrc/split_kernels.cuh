@@ -5,6 +5,9 @@
 
 namespace dpg {
 
+// the operand that the clipped sums scale is the narrower one: A, unless it is wider than G
+inline bool a_is_scaled(const dp_linear_desc& L) { return L.d <= L.p; }
+
 // operand width rounded up to 8 columns (a 16-byte pitch for the TMA tensor maps)
 inline int split_padded(int c) { return (c + 7) / 8 * 8; }
 // bytes of one split operand: (2, B, T, padded(c)) bf16, the high terms of all examples, then the low ones

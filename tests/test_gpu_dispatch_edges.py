@@ -425,6 +425,17 @@ def test_fp32_norms_split_on_the_way(B, T):
     assert int(ds.dev_status.item()) == 0
 
 
+def test_fp32_norms_alone_store_no_split_operands():
+    """Nobody reads them there: only the partial sums behind them are written."""
+    B, T = 3, 40
+    layers = [dp.Linear(torch.randn(B, T, d, device="cuda"), torch.randn(B, T, p, device="cuda"), d=d, p=p) for d, p in [(72, 304), (304, 72), (64, 64)]]
+    ws = torch.full((dp.dp_ghost_norms_ws_bytes(layers, B, T),), 255, dtype=torch.uint8, device="cuda")
+    sq = torch.zeros(B, device="cuda")
+    dp.dp_ghost_norms(layers[:2], B, T, sq, ws=ws)
+    planes = 2 * B * T * 2 * (72 + 304) * 2                # of two layers, every one a multiple of 256 bytes
+    assert bool((ws[:planes] == 255).all()) and not bool((ws[planes:] == 255).all())
+
+
 # tiles of 128 tokens x 32 positions, several per block from 2 x 148 tiles on
 @pytest.mark.parametrize("B,T,d,V", [(1, 1, 64, 40), (2, 31, 72, 300), (3, 33, 64, 300), (2, 129, 136, 1000), (75, 128, 64, 100),
                                      (130, 97, 64, 64)])
