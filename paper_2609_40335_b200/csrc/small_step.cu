@@ -29,6 +29,7 @@ namespace {
 
 constexpr int kMaxLayers = 8, kMaxTokens = 512, kMaxT = 64, kMaxB = 64, kMaxCols = 256;
 constexpr int kMaxBlocks = 148;          // Gram items, and output tiles: one per SM
+constexpr size_t kMostBf16Smem = 150 * 1024;       // bf16 layers: shared memory of the norms' blocks on the busiest SM
 constexpr int kThreads = 256;
 constexpr int kGramTile = 32;
 constexpr int kEmbedCols = 64;         // columns per embedding item
@@ -462,10 +463,15 @@ int partials_per_example(const dp_step_desc& S) {
 
 }  // namespace
 
-// At most 512 tokens in sequences of at most 64, eight layers of at most 256 columns, a table of at most 2^20 values, and no
-// more blocks than run at the same time.  Step of one 256 x 256 layer at 512 tokens, call by call and as a graph: fp32 56 and 36 -> 27
-// and 29 us, bf16 48 and 33 -> 28 and 29; of four, fp32 61 and 39 -> 35 and 37, but bf16 50 and 33 -> 36 and 37, hence the
-// line at 148 blocks.  Widths in whole words of four values, as everything here is read.
+// At most 512 tokens in sequences of at most 64, eight layers of at most 256 columns, a table of at most 2^20 values, and at most
+// as many Gram items, and output tiles, as there are SMs (the embedding items come on top).  Step of one 256 x 256 layer at 512 tokens, call by
+// call and as a graph: fp32 56 and 36 -> 27 and 29 us, bf16 48 and 33 -> 28 and 29; of four, fp32 61 and 39 -> 35 and 37, but bf16
+// 50 and 33 -> 36 and 37, hence the line.  bf16 steps, whose Gram products the general path takes on the tensor cores, also go there where
+// the norms' blocks fill an SM's shared memory and many are Gram items: two 256 x 256 layers at B = 64, T = 8 and a table of 256 columns (384 blocks of 66 KiB) 43
+// and 31 -> 35 and 37, three of 256 x 192 at B = 49, T = 10 (343 of 58) 44 and 33 -> 34 and 35, but with 64 table columns (192 of 66) 42
+// and 33 -> 24 and 27, and with one layer (64 Gram items of 320 blocks) 41 and 32 -> 25 and 27; fp32 ones were faster in all of these, both ways.  At the line bf16 graphs are even (two 256 x 256 layers at B = 12,
+// T = 42 and B = 16, T = 32: 32.5 and 30.0 -> 32.8 and 30.7) and calls a third faster.  Widths in whole words of four values, as
+// everything here is read.
 bool small_step_fits(const dp_step_desc& S) {
   if (g_force_fma || S.tied || S.n_vectors || S.pos_ids || S.n_layers > kMaxLayers) return false;
   if (S.T > kMaxT || S.B > kMaxB || (long long)S.B * S.T > kMaxTokens) return false;
@@ -482,6 +488,9 @@ bool small_step_fits(const dp_step_desc& S) {
     if (L.mode == DP_NORM_DIRECT || (L.mode == DP_NORM_AUTO && (long long)S.T * S.T > (long long)L.d * L.p)) return false;
   }
   if (items > kMaxBlocks || tiles > kMaxBlocks) return false;
+  const long long blocks = items + (long long)S.B * ceil_div(S.d, kEmbedCols);
+  if (S.layer_dtype == DP_BF16 && 2 * items > kMaxBlocks &&
+      size_t((blocks + kMaxBlocks - 1) / kMaxBlocks) * gram_smem(S) > kMostBf16Smem) return false;
   return S.ws && (reinterpret_cast<uintptr_t>(S.ws) & 3) == 0 && size_t(S.B) * partials_per_example(S) * sizeof(float) <= S.ws_bytes;
 }
 

@@ -173,3 +173,16 @@ def test_side_stream_comes_after_the_small_step(captured):
     torch.cuda.synchronize()
     check(ds, 5, 4, True)
     assert torch.equal(got, ds.outs["wte"])
+
+
+# bf16 layers whose norms would fill an SM's shared memory go the general way; fp32 ones, fewer table columns or layers do not
+@pytest.mark.parametrize("layers,d,n,taken", [(BF16, 256, 2, False), (F32, 256, 2, True), (BF16, 64, 2, True), (BF16, 256, 1, True)])
+def test_bf16_steps_of_many_wide_blocks(layers, d, n, taken):
+    ds = make(layers, layers, 64, 8, d, [(256, 256)] * n, 300)
+    assert (launches(ds, seed=2, step=1, noise=False) == 2) == taken
+    want, sq = {n: t.clone() for n, t in ds.outs.items()}, ds.sq.clone()
+    pipeline.dp_step(ds, seed=2, step=1, noise=False, overlap=False)
+    assert torch.allclose(ds.sq, sq, rtol=1e-5)
+    for n, t in ds.outs.items():
+        # bf16 tensor cores round R_i * g once, by 2^-9 at most
+        assert float((t - want[n]).norm()) <= (2e-5 if layers == F32 else 2.0 ** -8) * float(t.norm()), n
