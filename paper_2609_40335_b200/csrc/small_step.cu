@@ -155,7 +155,8 @@ small_norms_kernel(const __grid_constant__ SmallParams P) {
 #pragma unroll
     for (int e = 0; e < 4; ++e) acc = fmaf(sa[e >> 1][e & 1], sg[e >> 1][e & 1], acc);
     const float tot = block_sum(acc, red);
-    if (threadIdx.x == 0) P.partials[i * P.n_per + l * P.ntp + tp] = two ? 2.f * tot : tot;
+    const int slot = i * P.n_per + l * P.ntp + tp;
+    if (threadIdx.x == 0 && dp_in_range(slot, P.B * P.n_per, P.dev_status)) P.partials[slot] = two ? 2.f * tot : tot;
     return;
   }
   // embedding: || sum over the tokens of an id ||^2, over the ids of the example
@@ -198,7 +199,7 @@ small_norms_kernel(const __grid_constant__ SmallParams P) {
 #pragma unroll
   for (int k = 0; k < kMaxT / 4; ++k) at += s_first[4 * k + part] < first;
   at = add4(at) + rank;                                  // tokens beyond T come last, each by itself
-  if (part == 0 && t < T) s_order[at] = ((id >= 0 ? t : T) * pitch) | (rank + 1 == size ? int(0x80000000u) : 0);
+  if (part == 0 && t < T && dp_in_range(at, T, P.dev_status)) s_order[at] = ((id >= 0 ? t : T) * pitch) | (rank + 1 == size ? int(0x80000000u) : 0);
   __syncthreads();
   float tot = 0.f;
   if (int(threadIdx.x) < cols) {
@@ -219,7 +220,8 @@ small_norms_kernel(const __grid_constant__ SmallParams P) {
     }
   }
   const float s = block_sum(tot, red);
-  if (threadIdx.x == 0) P.partials[i * P.n_per + P.n_main + slab] = s;
+  const int slot = i * P.n_per + P.n_main + slab;
+  if (threadIdx.x == 0 && dp_in_range(slot, P.B * P.n_per, P.dev_status)) P.partials[slot] = s;
 }
 
 // clip factors of all examples into shared memory (the norms' kernel is waited for first); block 0 writes the outputs
@@ -368,7 +370,7 @@ small_sums_kernel(const __grid_constant__ SmallParams P) {
   }
 #pragma unroll
   for (int h = 0; h < 2; ++h)
-    if (row[h] >= 0) {
+    if (row[h] >= 0 && dp_in_range(row[h], rows, P.dev_status) && dp_in_range(before, n, P.dev_status)) {
       s_pos[before] = short(2 * threadIdx.x + h);
       s_row[before] = static_cast<unsigned char>(row[h]);
       atomicOr(&s_touched, 1u << row[h]);
@@ -380,6 +382,7 @@ small_sums_kernel(const __grid_constant__ SmallParams P) {
   // the row's noise (or zeros) plus `sum`
   auto write = [&](int r, const float4& sum) {
     const long long v = block + (long long)r * P.table_blocks;
+    if (!dp_in_range(v, P.V, P.dev_status)) return;
     float x[4] = {sum.x, sum.y, sum.z, sum.w};
     if (noisy) {
       float z[4];
@@ -404,6 +407,7 @@ small_sums_kernel(const __grid_constant__ SmallParams P) {
       for (int k = part; k < entries; k += parts) {
         if (s_row[k] != r) continue;
         const int t = s_pos[k];
+        if (!dp_in_range(t, n, P.dev_status)) continue;
         const float f = s_clip[t / P.T];
         const float4 g = load4(G + t * P.ldge);
         acc.x = fmaf(f, g.x, acc.x); acc.y = fmaf(f, g.y, acc.y); acc.z = fmaf(f, g.z, acc.z); acc.w = fmaf(f, g.w, acc.w);

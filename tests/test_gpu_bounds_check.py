@@ -65,3 +65,21 @@ def test_small_shape_parity_suite_is_clean_under_the_checked_build():
     tail = (r.stdout + r.stderr)[-1500:]
     assert r.returncode == 0, tail
     assert " passed" in r.stdout and "failed" not in r.stdout, tail
+
+
+# kernels that no parity test of a small shape is sure to select: steps of two kernels, norms that split their operands on
+# the way, Gram tiles of several examples and row blocks of every height, factors per row, vectors read once
+EDGES = [("test_gpu_small_step.py", "small_step_against_float64 or ids_out_of_range"),
+         ("test_gpu_dispatch_edges.py", "norms_split_on_the_way or gram_tiles or gram_blocks or own_clip_factor"),
+         ("test_gpu_step_call.py", "vectors_read_once or kept_sums")]
+
+
+@pytest.mark.parametrize("file,select", EDGES)
+def test_kernels_of_small_and_short_shapes_are_clean_under_the_checked_build(file, select):
+    if not os.path.exists(CHECK_LIB):
+        from paper_2609_40335_b200 import build
+        build.build(check=True)
+    r = subprocess.run([sys.executable, "-m", "pytest", os.path.join(ROOT, "tests", file), "-x", "-q", "-m", "gpu", "-k", select,
+                        "-p", "no:cacheprovider"],
+                       env=dict(os.environ, DP_GHOST_LIB=CHECK_LIB), cwd=ROOT, capture_output=True, text=True, timeout=900)
+    assert r.returncode == 0 and " passed" in r.stdout, (r.stdout + r.stderr)[-1500:]
