@@ -55,10 +55,13 @@ inline GtaRows gta_rows(int B, int T, int terms) {
 
 // Clip factors of a K step's rows: lane k holds those of rows k and k + 32; `one`: they are all the same.
 struct RowFactors { float lo, hi; bool one; };
-// step: K step of the contraction; rows: all token rows, 0: `tsteps` steps belong to each example.  The lanes look their
-// rows up only where a step holds several examples (done always, 16 layers at B = 16, T = 512 took 791 us instead of 783).
+// step: K step of the contraction.  kByRow: of the `rows` token rows of the batch, or else `tsteps` steps belong to each
+// example; the kernels that never meet several in a step are compiled without the code for them, whose mere presence cost
+// them more than its use saves (4 GPT-2-small layers at B = 88, T = 272 346 us without, 365 with).  The lanes look their
+// rows up only where a step holds several examples.
+template <bool kByRow>
 __device__ __forceinline__ RowFactors row_factors(const float* clip, int step, int lane, int T, int rows, int tsteps) {
-  if (rows == 0) {
+  if (!kByRow) {
     const float r = __ldg(clip + step / tsteps);
     return {r, r, true};
   }
@@ -95,7 +98,7 @@ __device__ __forceinline__ void scale_part(uint4* part, float r, int lane) {
   }
 }
 
-// The same with a factor per row.  Out of line: inside the scalers' loop it cost the steps that need none of it 1 %.
+// The same with a factor per row.  Out of line: inside the scalers' loop it cost the steps that need none of it more.
 static __device__ __noinline__ void scale_rows(uint4* part, float lo, float hi, int lane) {
   auto split = [](float x) {                       // r_hi in the low half, r_lo in the high one
     const __nv_bfloat16 h = __float2bfloat16_rn(x), l = __float2bfloat16_rn(x - __bfloat162float(h));

@@ -168,7 +168,7 @@ static __device__ __noinline__ float4 normals4_call(unsigned long long q, const 
   return make_float4(z[0], z[1], z[2], z[3]);
 }
 
-template <bool kSplit, Epilogue kEpilogue>
+template <bool kSplit, bool kByRow, Epilogue kEpilogue>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
   const uint32_t rank = ptx::cluster_ctarank();
@@ -335,7 +335,7 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
       const int steps = P.ksteps + (it.nsub == 2 ? P.skew : 0);
       auto factors = [&](int j) {              // of step j (the last `skew` steps are the first again)
         if (!scale_here || j >= steps) return RowFactors{1.f, 1.f, true};
-        return row_factors(P.clip, j < P.ksteps ? j : j - P.ksteps, lane, P.example_rows, P.rows, P.example_steps);
+        return row_factors<kByRow>(P.clip, j < P.ksteps ? j : j - P.ksteps, lane, P.example_rows, P.rows, P.example_steps);
       };
       int j = int((uint32_t(sw) + kScalerWarps - cnt % kScalerWarps) % kScalerWarps);
       uint32_t c = cnt + uint32_t(j);
@@ -347,7 +347,7 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
         if (fill > 0 && !ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
         if (!ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit)) { ok = false; break; }
         uint4* part = reinterpret_cast<uint4*>(tiles + size_t(stage) * kStageBytes);
-        if (!r.one) scale_rows(part, r.lo, r.hi, lane);
+        if (kByRow && !r.one) scale_rows(part, r.lo, r.hi, lane);
         else if (r.lo != 1.0f) scale_part(part, r.lo, lane);
         if (scale_here) ptx::fence_proxy_async_smem();
         __syncwarp();
@@ -491,10 +491,10 @@ gemm_gta_big_kernel(const __grid_constant__ BigParams P) {
 
 }  // namespace
 
-template <bool kSplit, Epilogue kEpilogue>
+template <bool kSplit, bool kByRow, Epilogue kEpilogue>
 static dp_status launch_big(const BigParams& P, int units, cudaStream_t st) {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_big_kernel<kSplit, kEpilogue>)))
-    DP_CUDA_OK((allow_shared(gemm_gta_big_kernel<kSplit, kEpilogue>, kSmemBytes)));
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_big_kernel<kSplit, kByRow, kEpilogue>)))
+    DP_CUDA_OK((allow_shared(gemm_gta_big_kernel<kSplit, kByRow, kEpilogue>, kSmemBytes)));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * units, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -504,16 +504,16 @@ static dp_status launch_big(const BigParams& P, int units, cudaStream_t st) {
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  DP_CUDA_OK((cudaLaunchKernelEx(&cfg, gemm_gta_big_kernel<kSplit, kEpilogue>, P)));
+  DP_CUDA_OK((cudaLaunchKernelEx(&cfg, gemm_gta_big_kernel<kSplit, kByRow, kEpilogue>, P)));
   ++g_kernel_launches;
   return DP_OK;
 }
 
-template <bool kSplit>
+template <bool kSplit, bool kByRow>
 static dp_status launch_big(const BigParams& P, Epilogue epilogue, int units, cudaStream_t st) {
-  return epilogue == kPlain      ? launch_big<kSplit, kPlain>(P, units, st)
-         : epilogue == kStraight ? launch_big<kSplit, kStraight>(P, units, st)
-                                 : launch_big<kSplit, kGeneral>(P, units, st);
+  return epilogue == kPlain      ? launch_big<kSplit, kByRow, kPlain>(P, units, st)
+         : epilogue == kStraight ? launch_big<kSplit, kByRow, kStraight>(P, units, st)
+                                 : launch_big<kSplit, kByRow, kGeneral>(P, units, st);
 }
 
 // One launch over at most kGtaMaxLayers layers without a K split.
@@ -576,7 +576,9 @@ dp_status launch_gta_big(const GtaBigJob* jobs, int n, int B, int T, int terms, 
   const int units = std::min(P.total_items, pairs);
   // A called generator costs a third of an output's time, the straight code saves a twelfth: one output in eight may be odd.
   const Epilogue epilogue = !noise ? kPlain : beta == 0.f && noise->scale == 1.f && 8 * odd <= outputs ? kStraight : kGeneral;
-  return terms > 1 ? launch_big<true>(P, epilogue, units, st) : launch_big<false>(P, epilogue, units, st);
+  return terms > 1       ? launch_big<true, false>(P, epilogue, units, st)
+         : K.scaled_rows ? launch_big<false, true>(P, epilogue, units, st)
+                         : launch_big<false, false>(P, epilogue, units, st);
 }
 
 }  // namespace dpg

@@ -119,7 +119,7 @@ __device__ __forceinline__ Item decode_item(const GtaParams& P, int item, int& l
   return it;
 }
 
-template <bool kScale, bool kSqsum, bool kPair, bool kSplit>
+template <bool kScale, bool kSqsum, bool kPair, bool kSplit, bool kByRow>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_gta_kernel(const __grid_constant__ GtaParams P) {
   static_assert(kScale || !kPair, "CTA pairs need the scaler warps' cross-CTA stage hand-off");
@@ -295,12 +295,12 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
         // no scaling here when the operand arrives scaled: clip == NULL (the split fp32 path) or a
         // layer whose narrow operand was multiplied by R_i in a pass of its own (see prescale)
         RowFactors r_next{1.f, 1.f, true};
-        if (scale_here && ks < it.k1) r_next = row_factors(P.clip, ks, lane, P.example_rows, P.rows, P.example_steps);
+        if (scale_here && ks < it.k1) r_next = row_factors<kByRow>(P.clip, ks, lane, P.example_rows, P.rows, P.example_steps);
         for (; ks < it.k1; ks += kScalerWarps, c += kScalerWarps) {
           const RowFactors r = r_next;
           // the factors of this warp's next K step are fetched before the waits, off the stage's path
           if (scale_here && ks + kScalerWarps < it.k1)
-            r_next = row_factors(P.clip, ks + kScalerWarps, lane, P.example_rows, P.rows, P.example_steps);
+            r_next = row_factors<kByRow>(P.clip, ks + kScalerWarps, lane, P.example_rows, P.rows, P.example_steps);
           const uint32_t stage = c % kStages, fill = c / kStages, phase = fill & 1u;
           // A warp hops between stages, so it has not seen the previous fill of this one, and the
           // parity of `full` alone cannot tell "fill n landed" from "fill n-1 still in flight".
@@ -310,7 +310,7 @@ gemm_gta_kernel(const __grid_constant__ GtaParams P) {
           if (fill > 0 && !ptx::mbar_wait_a(empty_a + 8 * stage, phase ^ 1, abort_flag, P.wait_limit)) { ok = false; break; }
           if (!ptx::mbar_wait_a(full_a + 8 * stage, phase, abort_flag, P.wait_limit)) { ok = false; break; }
           uint4* part = reinterpret_cast<uint4*>(tiles + size_t(stage) * kStageBytes);
-          if (!r.one) scale_rows(part, r.lo, r.hi, lane);
+          if (kByRow && !r.one) scale_rows(part, r.lo, r.hi, lane);
           else if (r.lo != 1.0f) scale_part(part, r.lo, lane);
           if (scale_here) ptx::fence_proxy_async_smem();
           __syncwarp();
@@ -605,10 +605,10 @@ constexpr bool kClipScale = true;
 constexpr bool kUsePair = true;
 
 // Launch on `units` persistent CTAs (single) or CTA pairs (cluster of 2).
-template <bool kScale, bool kSqsum, bool kPair, bool kSplit>
+template <bool kScale, bool kSqsum, bool kPair, bool kSplit, bool kByRow>
 dp_status launch_gta(const GtaParams& P, int units, cudaStream_t st) {
-  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_kernel<kScale, kSqsum, kPair, kSplit>)))
-    DP_CUDA_OK(allow_shared(gemm_gta_kernel<kScale, kSqsum, kPair, kSplit>, Geo<kPair>::kSmemBytes));
+  if (first_use_on_this_device(reinterpret_cast<const void*>(&gemm_gta_kernel<kScale, kSqsum, kPair, kSplit, kByRow>)))
+    DP_CUDA_OK(allow_shared(gemm_gta_kernel<kScale, kSqsum, kPair, kSplit, kByRow>, Geo<kPair>::kSmemBytes));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kPair ? 2 * units : units, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -621,7 +621,7 @@ dp_status launch_gta(const GtaParams& P, int units, cudaStream_t st) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  DP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_gta_kernel<kScale, kSqsum, kPair, kSplit>, P));
+  DP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_gta_kernel<kScale, kSqsum, kPair, kSplit, kByRow>, P));
   ++g_kernel_launches;
   return DP_OK;
 }
@@ -746,8 +746,9 @@ dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, 
     P.wait_limit = g_wait_limit;
     const int units = std::min(items, kUsePair ? sms / 2 : sms);
     s = use_big ? launch_gta_big(big.data(), (int)big.size(), B, T, terms, clip, beta, noise, dev_status, st)
-        : terms > 1 ? launch_gta<kClipScale, false, kUsePair, true>(P, units, st)
-                    : launch_gta<kClipScale, false, kUsePair, false>(P, units, st);
+        : terms > 1     ? launch_gta<kClipScale, false, kUsePair, true, false>(P, units, st)
+        : K.scaled_rows ? launch_gta<kClipScale, false, kUsePair, false, true>(P, units, st)
+                        : launch_gta<kClipScale, false, kUsePair, false, false>(P, units, st);
     if (s != DP_OK) return s;
     if (nsplit > 1) {
       ReduceParams R;
@@ -812,8 +813,8 @@ dp_status launch_direct_norm_tc(const dp_linear_desc* layers, const GhostPlan& p
     P.sq_partials = partials; P.n_per = plan.n_per;
     P.dev_status = dev_status;
     P.wait_limit = g_wait_limit;
-    s = terms > 1 ? launch_gta<false, true, false, true>(P, std::min(items, sms), st)
-                  : launch_gta<false, true, false, false>(P, std::min(items, sms), st);
+    s = terms > 1 ? launch_gta<false, true, false, true, false>(P, std::min(items, sms), st)
+                  : launch_gta<false, true, false, false, false>(P, std::min(items, sms), st);
     if (s != DP_OK) return s;
   }
   return DP_OK;
