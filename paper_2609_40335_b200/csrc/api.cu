@@ -165,8 +165,6 @@ struct SplitGroup {
   std::vector<SplitJob> jobs;
   size_t bytes = 0;                     // workspace taken by the split operands
   size_t bound = 0;                     // norms: by all of it, at most
-  long long tiles = 0;                  // sums: output tiles
-  size_t out_bytes = 0;                 // and one fp32 plane of every output
 
   // scale: the narrower operand is to be multiplied by the clip factors
   void add(const dp_linear_desc& L, int l, int B, int T, bool scale, char* base) {
@@ -182,8 +180,6 @@ struct SplitGroup {
     index.push_back(l);
     source.push_back(L);
     desc.push_back(D);
-    tiles += gta_tiles(L);
-    out_bytes += align_up(size_t(L.p) * size_t(L.d) * sizeof(float), 256);
   }
 };
 
@@ -629,12 +625,12 @@ size_t dp_clip_accumulate_grouped_ws_bytes(const dp_linear_desc* layers, int32_t
   if (!layers || n_layers <= 0 || B <= 0 || T <= 0) return 0;
   size_t n = align_up(size_t(B) * sizeof(float), 256);          // clip factors
   if (dt == DP_BF16 && !g_force_fma) n += gta_partial_bytes(layers, n_layers, B, T, 1, sm_count());
-  if (dt == DP_F32) {            // split operands of the largest layer, half as much again, and its K-split planes
+  if (dt == DP_F32) {            // split operands of the largest layer, half as much again, and its K-split planes or more
     size_t need = 0;
     for (int l = 0; l < n_layers; ++l)
       if (f32_on_tensor_cores(layers[l], T))
         need = std::max(need, split_layer_bytes(layers[l], B, T) * 3 / 2 +
-                                  gta_partial_bytes(layers + l, 1, B, T, 3, sm_count()));
+                                  gta_partial_bytes(layers + l, 1, B, T, 3, sm_count(), true));
     n += need;
   }
   return n;
@@ -696,6 +692,24 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
       group = SplitGroup();
       return s;
     };
+    // The layers that go together from layer l on, up to the one returned: as many as fit with the K split, and so the planes of
+    // partial sums, that all their tiles give (fewer layers are split more, so a part of them may not fit where all do).
+    auto group_end = [&](int first) {
+      size_t bytes = head, out_bytes = 0;
+      long long tiles = 0;
+      int end = first + 1;
+      for (int l = first; l < n_layers; ++l) {
+        if (!f32_on_tensor_cores(layers[l], T)) continue;
+        bytes += split_layer_bytes(layers[l], B, T);
+        if (l > first && bytes > ws_bytes) break;
+        tiles += gta_tiles(layers[l]);
+        out_bytes += align_up(size_t(layers[l].p) * size_t(layers[l].d) * sizeof(float), 256);
+        const int ns = gta_choose_nsplit(tiles, B, T, 3, sm_count());
+        if (bytes + (ns > 1 ? size_t(ns) * out_bytes : 0) <= ws_bytes) end = l + 1;
+      }
+      return end;
+    };
+    int end = 0;
     std::vector<int> fma;                // layers on the fp32 kernels: one launch for all of them
     if (kept && !kept->index.empty() && !sq &&
         kept->bytes + gta_partial_bytes(kept->desc.data(), (int)kept->desc.size(), B, T, 3, sm_count()) <= ws_bytes) {
@@ -716,12 +730,11 @@ static dp_status clip_accumulate_impl(const dp_linear_desc* layers, int32_t n_la
     for (int l = 0; l < n_layers; ++l) {
       if (dt == DP_F32 && f32_on_tensor_cores(layers[l], T)) {
         if (kept) continue;
-        // the K split, and with it the planes of partial sums, follows from the group's tiles
-        const size_t out = align_up(size_t(layers[l].p) * size_t(layers[l].d) * sizeof(float), 256);
-        const int ns = gta_choose_nsplit(group.tiles + gta_tiles(layers[l]), B, T, 3, sm_count());
-        const size_t planes = ns > 1 ? size_t(ns) * (group.out_bytes + out) : 0;
-        if (head + group.bytes + split_layer_bytes(layers[l], B, T) + planes > ws_bytes) s = flush();
-        if (s != DP_OK) return s;
+        if (l >= end) {
+          s = flush();
+          if (s != DP_OK) return s;
+          end = group_end(l);
+        }
         group.add(layers[l], l, B, T, true, base);
         continue;
       }
@@ -979,7 +992,7 @@ size_t dp_step_ws_bytes(const dp_linear_desc* layers, int32_t n_layers, dp_dtype
       need += f32_norm_bytes(layers[l], B, T, sm_count());
       on.push_back(layers[l]);
     }
-  if (!on.empty()) need += gta_partial_bytes(on.data(), (int)on.size(), B, T, 3, sm_count());
+  if (!on.empty()) need += gta_partial_bytes(on.data(), (int)on.size(), B, T, 3, sm_count(), true);
   if (need > (size_t(16) << 30)) need = f32_norms_bytes(layers, n_layers, dt, B, T);
   return need + fma_norms_bytes(layers, n_layers, dt, B, T);
 }

@@ -169,7 +169,8 @@ bool gta_prescales(const dp_linear_desc& L);            // terms = 1: a scaled c
 int gta_choose_nsplit(long long tiles, int B, int T, int terms, int sms);
 // scratch of a grouped call behind the clip factors: K-split planes (if any) and, terms = 1, the
 // pre-scaled copies of very narrow operands
-size_t gta_partial_bytes(const dp_linear_desc* layers, int n_layers, int B, int T, int terms, int sms);
+// ample: planes of as many splits as if K steps ended with their examples, at least as many; room in which more layers go together
+size_t gta_partial_bytes(const dp_linear_desc* layers, int n_layers, int B, int T, int terms, int sms, bool ample = false);
 
 // One persistent launch over the output tiles of all layers (plus split-K reduces if needed).
 dp_status launch_clip_accumulate_tc(const dp_linear_desc* layers, int n_layers, int B, int T, int terms,

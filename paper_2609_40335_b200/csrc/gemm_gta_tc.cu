@@ -642,18 +642,25 @@ static long long gta_tiles(const dp_linear_desc* layers, int n_layers) {
 
 bool gta_prescales(const dp_linear_desc& L) { return prescale_layer(L); }
 
-int gta_choose_nsplit(long long tiles, int B, int T, int terms, int sms) {
-  const GtaRows K = gta_rows(B, T, terms);
-  const int ksteps = K.B * terms * ceil_div(K.T, kBK);
+static int choose_nsplit(long long tiles, int ksteps, int sms) {
   const int units = kUsePair ? sms / 2 : sms;          // persistent CTAs or CTA pairs
   if (tiles >= 2LL * units) return 1;
   long long ns = std::max<long long>(1, (2LL * units) / std::max<long long>(tiles, 1));
-  ns = std::min<long long>(ns, std::max(1, (ksteps + terms - 1) / 4));      // a split is whole blocks of `terms` steps
+  ns = std::min<long long>(ns, std::max(1, ksteps / 4));
   return (int)std::max<long long>(1, ns);
 }
 
-size_t gta_partial_bytes(const dp_linear_desc* layers, int n_layers, int B, int T, int terms, int sms) {
-  const int ns = gta_choose_nsplit(gta_tiles(layers, n_layers), B, T, terms, sms);
+// Two splits of one 64-token block each, three K steps, are no gain: 6 steps stay whole (fp32 at B = 1, T = 128: 4 GPT-2-small
+// layers of d = 256 14.7 us, 17.6 in two).
+int gta_choose_nsplit(long long tiles, int B, int T, int terms, int sms) {
+  const GtaRows K = gta_rows(B, T, terms);
+  return choose_nsplit(tiles, K.B * terms * ceil_div(K.T, kBK), sms);
+}
+
+
+size_t gta_partial_bytes(const dp_linear_desc* layers, int n_layers, int B, int T, int terms, int sms, bool ample) {
+  const long long tiles = gta_tiles(layers, n_layers);
+  const int ns = ample ? choose_nsplit(tiles, B * terms * ceil_div(T, kBK), sms) : gta_choose_nsplit(tiles, B, T, terms, sms);
   size_t n = 0;
   for (int l = 0; l < n_layers; ++l) {
     if (ns > 1) n += align_up(size_t(ns) * size_t(layers[l].p) * size_t(layers[l].d) * sizeof(float), 256);

@@ -425,6 +425,23 @@ def test_fp32_norms_split_on_the_way(B, T):
     assert int(ds.dev_status.item()) == 0
 
 
+# layers that fit the workspace together go together, although the first few of them alone would be split along K into more planes
+# than it holds; 64-token blocks 2, 3 and 5
+@pytest.mark.parametrize("B,T", [(1, 77), (1, 128), (3, 64), (4, 77)])
+def test_fp32_sums_of_layers_that_fit_go_together(B, T):
+    shapes = [(576, 1728), (576, 576), (576, 2304), (2304, 576)]
+    layers = [dp.Linear(torch.randn(B, T, d, device="cuda"), torch.randn(B, T, p, device="cuda") * 0.1, d=d, p=p) for d, p in shapes]
+    outs, clip = [torch.empty(p, d, device="cuda") for d, p in shapes], torch.rand(B, device="cuda")
+    need = max(dp.dp_step_ws_bytes(layers, B, T), dp.dp_clip_accumulate_grouped_ws_bytes(layers, B, T))
+    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    n0 = dp.dp_kernel_launches()
+    dp.dp_clip_accumulate_grouped(layers, B, T, None, 1.0, outs, clip=clip, ws=ws)
+    assert dp.dp_kernel_launches() - n0 == 2                 # the split, the sums
+    for l, o in zip(layers, outs):
+        want = torch.einsum("btp,btd->pd", l.G.double() * clip.double()[:, None, None], l.A.double())
+        assert float((o.double() - want).norm() / want.norm()) < 2e-5         # two bf16 terms
+
+
 def test_fp32_norms_alone_store_no_split_operands():
     """Nobody reads them there: only the partial sums behind them are written."""
     B, T = 3, 40
