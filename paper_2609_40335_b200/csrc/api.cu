@@ -207,7 +207,9 @@ static dp_status f32_norm_group(const SplitGroup& g, int B, int T, float* sq, ch
   std::vector<SplitJob> before;
   std::vector<char> is_fused(g.desc.size(), 0);
   for (int l : plan.ghost_layers)
-    if (ghost_norm_splits(g.source[size_t(l)], B, T)) { fused.push_back(l); is_fused[size_t(l)] = 1; }
+    if (ghost_norm_splits(g.source[size_t(l)], B, T)) fused.push_back(l);
+  if (!ghost_norm_split_pays(fused, plan, B, T, keep, sm_count())) fused.clear();
+  for (int l : fused) is_fused[size_t(l)] = 1;
   for (size_t l = 0; l < g.desc.size(); ++l)
     if (!is_fused[l]) { before.push_back(g.jobs[2 * l]); before.push_back(g.jobs[2 * l + 1]); }
   dp_status s = launch_split(before.data(), (int)before.size(), B, T, nullptr, st);

@@ -341,6 +341,29 @@ bool ghost_norm_splits(const dp_linear_desc& L, int B, int T) {
          L.lda % 4 == 0 && L.ldg % 4 == 0;
 }
 
+// Whether one pass over the layers in `index` takes less time than the split and the Gram kernel after it.  A K step takes 0.6 us here
+// whatever its rows, and more on the busiest SM than on average; there 12 bytes per value go through memory, 0.014 us per row and
+// step of the average SM, here 4, or with stores 7.  The lines, in steps of the busiest SM over the average: rows / 42, with stores rows / 55.
+// Norms alone, split first -> in one pass: 24 GPT-2-small layers at T = 128, B = 1, 2, 8 (2.05, 1.03, 1.03 against 3.0) 29, 44, 165 -> 27, 28,
+// 104 us, at T = 64, B = 1, 2, 8 (the same against 1.5) 21.5, 26, 92 -> 22, 22, 69, at T = 32 (against 0.8) 19, 20, 63 -> 21, 21, 61; one
+// of them, T = 128, B = 1 and 8 (48 and 6) 21 and 23 -> 25 and 26.  Steps, with stores: 24 layers at T = 64, B = 2, 8 (1.03 against 1.16) 97, 226
+// -> 91, 214, 4 of d = 576 at T = 64, B = 16 (1.54) 82 -> 92, at T = 128, B = 8 (1.54 against 2.3) 89 -> 85, one layer at T = 128, B = 1 38 -> 45.
+// Norms alone of a dozen steps at most are launches only: 4 layers of d = 256, B = 1, T = 32 and 64 12.7 and 13.1 -> 12.2 and 12.6, beyond 80 rows
+// longer (15 -> 16).
+bool ghost_norm_split_pays(const std::vector<int>& index, const GhostPlan& plan, int B, int T, bool keep, int sms) {
+  const int rows = (plan.pack * T + 15) / 16 * 16, groups = ceil_div(B, plan.pack);
+  long long total = 0, busiest = 0, items = 0, next = 0;       // the first SM has the longest item of every wave
+  for (int l : index) {
+    const GhostLayerPlan& L = plan.layer[size_t(l)];
+    const int narrow = std::min(L.a_steps, L.g_steps), wide = std::max(L.a_steps, L.g_steps);
+    items += (long long)groups * L.nsplit;
+    total += (long long)groups * (L.nsplit * narrow + wide);
+    for (; next < items; next += sms) busiest += narrow + L.chunk_steps;
+  }
+  if (!keep && busiest <= 12 && rows <= 80) return true;
+  return busiest * sms * (keep ? 55 : 42) <= total * rows;
+}
+
 // index: layers of the plan, with the fp32 operands in `layers`; jobs: their split, A and G of layer k at 2k and 2k + 1;
 // keep: the wider operand's is stored
 dp_status launch_ghost_norm_split(const dp_linear_desc* layers, const SplitJob* jobs, const std::vector<int>& index,

@@ -55,6 +55,7 @@ dp_status launch_ghost_norm_tc(const dp_linear_desc* layers, const GhostPlan& pl
 // fp32 layers of 32 to 128 tokens on a 16-byte boundary and pitch: norm and split in one pass (ghost_norm_split.cu).
 struct SplitJob;
 bool ghost_norm_splits(const dp_linear_desc& L, int B, int T);
+bool ghost_norm_split_pays(const std::vector<int>& index, const GhostPlan& plan, int B, int T, bool keep, int sms);
 dp_status launch_ghost_norm_split(const dp_linear_desc* layers, const SplitJob* jobs, const std::vector<int>& index,
                                   const GhostPlan& plan, int B, int T, bool keep, float* partials, int* dev_status, cudaStream_t st);
 

@@ -425,6 +425,30 @@ def test_fp32_norms_split_on_the_way(B, T):
     assert int(ds.dev_status.item()) == 0
 
 
+# the same where the pass over fp32 operands pays: two SMs, which it fills
+@pytest.mark.parametrize("B,T", [(3, 32), (8, 32), (5, 33), (7, 42), (3, 64), (2, 65), (3, 77), (2, 96), (1, 100), (3, 127), (2, 128)])
+def test_fp32_norms_split_on_the_way_on_two_sms(B, T):
+    before = dp.dp_set_reserved_sms(146)
+    try:
+        test_fp32_norms_split_on_the_way(B, T)
+    finally:
+        dp.dp_set_reserved_sms(before)
+
+
+# one pass where it is short or fills the chip, split first where it would wait for a few SMs or has few rows per tile
+@pytest.mark.parametrize("shapes,B,T,launches", [([(256, 768), (256, 256)], 1, 64, 2), ([(256, 768), (256, 256)], 1, 128, 3),
+                                                 ([(768, 2304)], 8, 128, 3), ([(768, 2304)] * 12, 16, 128, 2), ([(768, 2304)] * 12, 8, 32, 3)])
+def test_fp32_norms_take_the_way_that_pays(shapes, B, T, launches):
+    layers = [dp.Linear(torch.randn(B, T, d, device="cuda"), torch.randn(B, T, p, device="cuda") * 0.05, d=d, p=p) for d, p in shapes]
+    ws = torch.empty(max(dp.dp_ghost_norms_ws_bytes(layers, B, T), dp.dp_step_ws_bytes(layers, B, T)), dtype=torch.uint8, device="cuda")
+    sq = torch.zeros(B, device="cuda")
+    n0 = dp.dp_kernel_launches()
+    dp.dp_ghost_norms(layers, B, T, sq, ws=ws)
+    assert dp.dp_kernel_launches() - n0 == launches
+    want = sum((torch.einsum("btp,btd->bpd", l.G.double(), l.A.double()) ** 2).sum((1, 2)) for l in layers)
+    assert ((sq.double() / want - 1).abs() < 4e-5).all()             # two bf16 terms: 2^-16 of a product at most
+
+
 # layers that fit the workspace together go together, although the first few of them alone would be split along K into more planes
 # than it holds; 64-token blocks 2, 3 and 5
 @pytest.mark.parametrize("B,T", [(1, 77), (1, 128), (3, 64), (4, 77)])
