@@ -277,45 +277,54 @@ ghost_norm_tc_kernel(const __grid_constant__ GhostParams P) {
       // packed: this row's example and the columns of its tokens; the warp's rows have those of [c_lo, c_hi)
       const int row = q * 32 + lane, own = kPacked ? row / P.T * P.T : 0;
       const int c_lo = kPacked ? (q * 32 / P.T * P.T) & ~15 : 0;
-      const int c_hi = kPacked ? min(rows, (q * 32 + 31) / P.T * P.T + P.T) : rows;
-#pragma unroll 1
-      for (int c = c_lo; c < c_hi; c += 32) {
+      const int c_hi = kPacked ? min(rows, (q * 32 + 31) / P.T * P.T + P.T) : 0;
+      auto add32 = [&](int c) {
         uint32_t ra[32], rg[32];
-        if (!kShort || c + 32 <= rows) {
-          ptx::tmem_ld_32x32b_x32(t0 + c, ra);
-          ptx::tmem_ld_32x32b_x32(t0 + 128 + c, rg);
-          if (kSplit) {
-            uint32_t sa[32], sg[32];
-            ptx::tmem_ld_32x32b_x32(t0 + 256 + c, sa);
-            ptx::tmem_ld_32x32b_x32(t0 + 384 + c, sg);
-            ptx::tmem_ld_wait();
+        ptx::tmem_ld_32x32b_x32(t0 + c, ra);
+        ptx::tmem_ld_32x32b_x32(t0 + 128 + c, rg);
+        if (kSplit) {
+          uint32_t sa[32], sg[32];
+          ptx::tmem_ld_32x32b_x32(t0 + 256 + c, sa);
+          ptx::tmem_ld_32x32b_x32(t0 + 384 + c, sg);
+          ptx::tmem_ld_wait();
 #pragma unroll
-            for (int j = 0; j < 32; ++j) { ra[j] = add_f32(ra[j], sa[j]); rg[j] = add_f32(rg[j], sg[j]); }
-          } else {
-            ptx::tmem_ld_wait();
-          }
-        } else {                                       // the last 16 columns
-          uint32_t ha[16], hg[16];
-          ptx::tmem_ld_32x32b_x16(t0 + c, ha);
-          ptx::tmem_ld_32x32b_x16(t0 + 128 + c, hg);
-          if (kSplit) {
-            uint32_t sa[16], sg[16];
-            ptx::tmem_ld_32x32b_x16(t0 + 256 + c, sa);
-            ptx::tmem_ld_32x32b_x16(t0 + 384 + c, sg);
-            ptx::tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) { ha[j] = add_f32(ha[j], sa[j]); hg[j] = add_f32(hg[j], sg[j]); }
-          } else {
-            ptx::tmem_ld_wait();
-          }
-#pragma unroll
-          for (int j = 0; j < 16; ++j) { ra[j] = ha[j]; rg[j] = hg[j]; ra[16 + j] = 0u; rg[16 + j] = 0u; }
+          for (int j = 0; j < 32; ++j) { ra[j] = add_f32(ra[j], sa[j]); rg[j] = add_f32(rg[j], sg[j]); }
+        } else {
+          ptx::tmem_ld_wait();
         }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
+        for (int j = 0; j < 32; ++j)
           if (!kPacked || unsigned(c + j - own) < unsigned(P.T))
             acc = fmaf(__uint_as_float(ra[j]), __uint_as_float(rg[j]), acc);
+      };
+      auto add16 = [&](int c) {                          // the last 16 columns
+        uint32_t ra[16], rg[16];
+        ptx::tmem_ld_32x32b_x16(t0 + c, ra);
+        ptx::tmem_ld_32x32b_x16(t0 + 128 + c, rg);
+        if (kSplit) {
+          uint32_t sa[16], sg[16];
+          ptx::tmem_ld_32x32b_x16(t0 + 256 + c, sa);
+          ptx::tmem_ld_32x32b_x16(t0 + 384 + c, sg);
+          ptx::tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) { ra[j] = add_f32(ra[j], sa[j]); rg[j] = add_f32(rg[j], sg[j]); }
+        } else {
+          ptx::tmem_ld_wait();
         }
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          if (!kPacked || unsigned(c + j - own) < unsigned(P.T))
+            acc = fmaf(__uint_as_float(ra[j]), __uint_as_float(rg[j]), acc);
+      };
+      if (kPacked) {
+#pragma unroll 1
+        for (int c = c_lo; c < c_hi; c += 32)
+          if (c + 32 <= rows) add32(c);
+          else add16(c);
+      } else {
+#pragma unroll 1
+        for (int c = 0; c + 32 <= rows; c += 32) add32(c);
+        if (kShort && (rows & 16)) add16(rows - 16);
       }
       ptx::tc_fence_before();
       __syncwarp();
