@@ -225,6 +225,29 @@ def test_every_row_gets_its_own_clip_factor(B, T, d, p):
     assert int(st.item()) == 0
 
 
+@pytest.mark.parametrize("B,T", [(37, 3), (9, 16), (3, 100), (4, 203), (6, 64)])
+@pytest.mark.parametrize("d,p", [(64, 72), (768, 14300), (14300, 768)])
+def test_factors_of_any_value_are_applied_in_two_parts(B, T, d, p):
+    """R_i x is the correctly rounded bf16 product, for rows of one K step with factors of their own too: 1.4e-4 from rounding it once
+    (one element in 1400 is rounded up instead of down or the other way); with R_i's upper half alone 2.7e-3."""
+    layer = dp.Linear(bf16((B, T, d), 1.0, T, ld=(d + 7) // 8 * 8), bf16((B, T, p), 0.1, B, ld=(p + 7) // 8 * 8), d=d, p=p)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B + T)
+    clip = torch.rand(B, generator=g, device="cuda") * 0.9 + 0.05
+    out = torch.empty(p, d, device="cuda")
+    dp.dp_clip_accumulate_grouped([layer], B, T, None, 1.0, [out], clip=clip)
+    G, A, R = layer.G[..., :p].double(), layer.A[..., :d].double(), clip.double()[:, None, None]
+    rounded = lambda x: (R * x).to(torch.bfloat16).double()
+    errors, size = [], 0.0
+    for r0 in range(0, p, 256):                          # which operand is scaled is each output tile's own
+        both = [torch.einsum("btp,btd->pd", g_[..., r0:r0 + 256], a_) for g_, a_ in ((rounded(G), A), (G, rounded(A)))]
+        for c0 in range(0, d, 256):
+            got = out[r0:r0 + 256, c0:c0 + 256].double()
+            errors.append(min(float((got - w[:, c0:c0 + 256]).norm()) ** 2 for w in both))
+        size += float(both[0].norm()) ** 2
+    assert (sum(errors) / size) ** 0.5 < 5e-4
+
+
 def test_two_tile_items_give_up_cleanly():
     """A wait limit of zero: the kernel flags DP_DEV_TIMEOUT and returns; the same call then succeeds."""
     B, T, d, p = 32, 128, 512, 19000               # long enough a contraction that some wait is not over at once
