@@ -55,13 +55,13 @@ inline GtaRows gta_rows(int B, int T, int terms) {
 
 // Clip factors of a K step's rows: lane k holds those of rows k and k + 32; `one`: they are all the same.
 struct RowFactors { float lo, hi; bool one; };
-// step: K step of the contraction.  kByRow: of the `rows` token rows of the batch, or else `tsteps` steps belong to each
-// example; the kernels that never meet several in a step are compiled without the code for them, whose mere presence cost
-// them more than its use saves (4 GPT-2-small layers at B = 88, T = 272 346 us without, 365 with).  The lanes look their
+// step: K step of the contraction; rows: all token rows, 0: `tsteps` steps belong to each example, as always without kByRow:
+// kernels that never meet several examples in a step are compiled without the code for them, whose mere presence costs
+// more than its use saves (4 GPT-2-small layers at B = 88, T = 272 346 us without, 365 with).  The lanes look their
 // rows up only where a step holds several examples.
 template <bool kByRow>
 __device__ __forceinline__ RowFactors row_factors(const float* clip, int step, int lane, int T, int rows, int tsteps) {
-  if (!kByRow) {
+  if (!kByRow || rows == 0) {
     const float r = __ldg(clip + step / tsteps);
     return {r, r, true};
   }

@@ -509,10 +509,13 @@ static dp_status launch_big(const BigParams& P, int units, cudaStream_t st) {
   return DP_OK;
 }
 
+// The straight epilogue runs beside the scalers that know factors per row, used or not: without that code the scalers are ready
+// sooner and poll more beside warps that are bound by their instructions (24 GPT-2-small layers at B = 32, T = 128 with noise 373 us, 377
+// without; sums alone 368 and 367).
 template <bool kSplit, bool kByRow>
 static dp_status launch_big(const BigParams& P, Epilogue epilogue, int units, cudaStream_t st) {
   return epilogue == kPlain      ? launch_big<kSplit, kByRow, kPlain>(P, units, st)
-         : epilogue == kStraight ? launch_big<kSplit, kByRow, kStraight>(P, units, st)
+         : epilogue == kStraight ? launch_big<kSplit, !kSplit, kStraight>(P, units, st)
                                  : launch_big<kSplit, kByRow, kGeneral>(P, units, st);
 }
 
