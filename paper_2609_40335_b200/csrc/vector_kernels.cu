@@ -219,39 +219,46 @@ vector_combine_kernel(const __grid_constant__ VecParams P, const float* __restri
   q.out[cc] = v;
 }
 
-// The same from the v_i that vector_norm_kernel kept: a lane's four columns are one Philox counter; rows e, e + 2, ... of
-// a block's in half e of it, four loads in flight.  It runs beside the persistent GEMM, hence 128 threads of 32 registers (see
-// embed_kernels.cu).  A block walks `rows` rows that lie `row_step` examples apart, weighted with clip unless that is nullptr.  Large
-// batches take two launches: with `rows_per_part` > 0 block y sums that many rows and leaves the result in the first of them, which nobody else
-// reads; then one block per slab adds these up.
-constexpr int kKeptThreads = 128;
-constexpr int kKeptAlone = 112;        // examples that one block walks: at 96 two launches took 50.0 us a step instead of 48.4, at 128 53.1 instead of 54.6
-constexpr int kKeptRows = 64;          // rows of a part
+// The same from the v_i that vector_norm_kernel kept.  It runs beside the persistent GEMM, hence 128 threads of 32 registers (see
+// embed_kernels.cu); where there is none, the walk over the examples is what counts, so a block has 64 columns, a lane's four are
+// one Philox counter, and eight parts of 16 lanes take every eighth row each, four loads in flight (with 256 columns and two parts
+// the step of six biases of 768 at B = 96, T = 8 took 38.1 us, 35.5 with the gradients read twice, now 33.1).  A block walks `rows` rows that lie
+// `row_step` examples apart, weighted with clip unless that is nullptr.  Large batches take two launches: with `rows_per_part` > 0
+// block y sums that many rows and leaves the result in the first of them, which nobody else reads; then one block adds these up.
+constexpr int kKeptThreads = 128, kKeptCols = 64, kKeptLanes = kKeptCols / 4, kKeptParts = kKeptThreads / kKeptLanes;
+constexpr int kKeptAlone = 448;        // examples that one block walks
+constexpr int kKeptRows = 128;         // rows of a part
 __global__ void __launch_bounds__(kKeptThreads, 16)
 vector_kept_sum_kernel(const __grid_constant__ VecParams P, float* keep, int n_per, int col0, const float* __restrict__ clip,
                        int rows, int row_step, int rows_per_part, float beta, int with_noise, float amp, float scale,
                        const __grid_constant__ NoiseKeys keys, uint32_t step, const uint32_t* __restrict__ step_dev) {
-  __shared__ float4 part[kVecCols / 4];
-  const int slab = blockIdx.x;
+  __shared__ float4 sums[kKeptParts][kKeptLanes];
+  const int slab = blockIdx.x / (kVecCols / kKeptCols), col = int(blockIdx.x) % (kVecCols / kKeptCols) * kKeptCols;
   const VecParam& q = P.prm[find_param(P, slab)];
-  const int half = threadIdx.x >> 6, quad = threadIdx.x & 63;
+  const int c0 = (slab - q.slab_begin) * kVecCols + col;
+  if (c0 >= q.p) return;
+  const int lane = threadIdx.x & (kKeptLanes - 1), part = threadIdx.x / kKeptLanes;
   const int r0 = int(blockIdx.y) * rows_per_part, r1 = rows_per_part ? min(rows, r0 + rows_per_part) : rows;
-  float4* src = reinterpret_cast<float4*>(keep + size_t(col0 + slab) * kVecCols) + quad;
+  float4* src = reinterpret_cast<float4*>(keep + size_t(col0 + slab) * kVecCols + col) + lane;
   const size_t pitch = size_t(n_per) * (kVecCols / 4) * row_step;
   float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-  for (int i = r0 + half; i < r1; i += 2) {
+  for (int i = r0 + part; i < r1; i += kKeptParts) {
     const float4 v = src[size_t(i) * pitch];
     const float r = clip ? __ldg(clip + i) : 1.f;
     a.x = fmaf(r, v.x, a.x); a.y = fmaf(r, v.y, a.y); a.z = fmaf(r, v.z, a.z); a.w = fmaf(r, v.w, a.w);
   }
-  if (half) part[quad] = a;
+  sums[part][lane] = a;
   __syncthreads();
-  if (half) return;
-  const float4 b = part[quad];
-  float v[4] = {a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w};
-  if (rows_per_part) { src[size_t(r0) * pitch] = make_float4(v[0], v[1], v[2], v[3]); return; }
-  const int c = (slab - q.slab_begin) * kVecCols + 4 * quad;
+  if (part) return;
+#pragma unroll
+  for (int k = 1; k < kKeptParts; ++k) {
+    const float4 x = sums[k][lane];
+    a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+  }
+  if (rows_per_part) { src[size_t(r0) * pitch] = a; return; }
+  const float v[4] = {a.x, a.y, a.z, a.w};
+  const int c = c0 + 4 * lane;
   if (c >= q.p) return;
   float z[4] = {0.f, 0.f, 0.f, 0.f};
   if (with_noise) normals4((unsigned long long)(c >> 2), keys, q.tensor_id, effective_step(step, step_dev), z);
@@ -352,8 +359,8 @@ dp_status launch_vector_kept_sums(const dp_vector_desc* prm, int n, int B, int T
   if (first_use_on_this_device(reinterpret_cast<const void*>(&vector_kept_sum_kernel)))
     DP_CUDA_OK(prefer_max_shared(vector_kept_sum_kernel));
   const int n_per = vector_total_slabs(prm, n);
-  // one block per slab as long as its serial walk is short; beyond, parts at least as long as there are parts.  Step of six biases of 768
-  // at T = 8 and B = 256, 1024, 4096: 72, 168, 481 us with G read twice, 75, 240, 950 with one block per slab, 65, 164, 432 now.
+  // one block walks all examples as long as that is short; beyond, parts at least as long as there are parts.  Step of six biases of 768
+  // at T = 8 and B = 256, 1024, 4096: 72, 167, 478 us with G read twice, 64, 151, 431 now.
   int per_part = 0;
   if (B > kKeptAlone) for (per_part = kKeptRows; (long long)per_part * per_part < B; per_part *= 2) {}
   const int parts = per_part ? ceil_div(B, per_part) : 1;
@@ -361,12 +368,13 @@ dp_status launch_vector_kept_sums(const dp_vector_desc* prm, int n, int B, int T
   for (int n0 = 0; n0 < n; n0 += kVecMaxParams) {
     VecParams P;
     const int slabs = fill_params(P, prm, n0, std::min(n, n0 + kVecMaxParams), outs, tensor_ids, B, T);
+    const int blocks = slabs * (kVecCols / kKeptCols);
     if (per_part) {
-      vector_kept_sum_kernel<<<dim3(slabs, parts), kKeptThreads, 0, st>>>(P, keep, n_per, col0, clip, B, 1, per_part, 0.f, 0, 0.f,
+      vector_kept_sum_kernel<<<dim3(blocks, parts), kKeptThreads, 0, st>>>(P, keep, n_per, col0, clip, B, 1, per_part, 0.f, 0, 0.f,
                                                                          1.f, expand_noise_keys(seed), step, g_step_dev);
       DP_LAUNCH_OK();
     }
-    vector_kept_sum_kernel<<<slabs, kKeptThreads, 0, st>>>(P, keep, n_per, col0, per_part ? nullptr : clip, per_part ? parts : B,
+    vector_kept_sum_kernel<<<blocks, kKeptThreads, 0, st>>>(P, keep, n_per, col0, per_part ? nullptr : clip, per_part ? parts : B,
                                                           per_part ? per_part : 1, 0, beta, with_noise, amp, scale,
                                                           expand_noise_keys(seed), step, g_step_dev);
     DP_LAUNCH_OK();
