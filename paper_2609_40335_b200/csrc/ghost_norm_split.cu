@@ -9,7 +9,7 @@
 //
 // Bound by HBM (4 bytes in, and 4 out for the values that are kept) and by its last wave (156 steps on the busiest SM, 119 on average).
 // Norms alone of DistilGPT2's 25 layers at B = 8, T = 128: 275 us split first, 227 with every plane stored, 145 with none; the step
-// 876 -> 841, stores of the narrower operand included or not.
+// 850 -> 801.
 //
 // A tile holds the rows of as many whole examples as fit into 128 (one above 64 tokens; see ghost_norm_tc.cu), rounded up to
 // 16 rows.  Roles per CTA (448 threads): warp 0 TMA producer, warp 1 MMA issuer, warps 2 - 5 epilogue, warps 6 - 13

@@ -34,14 +34,15 @@ constexpr int kTileBytes = kTile * kKStep * 2;   // 16 KiB
 // pair is diagonal, so stages shrink to one tile and twice as many are kept in flight (the
 // kernel is HBM-bound there: bytes in flight are what counts).  Split operands (fp32 inputs) bring
 // two tiles, high and low terms, for each.
-// Up to 64 tokens tiles are as tall as their examples, rounded up to 16 rows (kShort), and where that is less than half of one a stage
-// holds two or four of them, 64 columns each (kBoxes): a stage's hand-offs take 550 cycles whatever it carries.  Where there is work enough
-// a tile holds several examples (kPacked): the rows of a batch lie one after the other, so 128 / T of them fill it, its Gram matrix has
-// theirs on the diagonal, and the epilogue multiplies only those blocks.  An example by itself has the plainer epilogue (a GPT-2-small
-// block at B = 1, 2 and 4, T = 64 10.0, 10.8 and 10.8 us with the other, 9.7, 10.3 and 10.3 with its own).  97 layers of d = 128 at B = 95, T = 17 115 -> 50 us, 49 at B = 91, T = 39 70 -> 50; never so many
-// examples that fewer than two items per SM remain (5 fp32 layers at B = 2, T = 54: 7.7 -> 10.2 with both in one tile).  Above 64 tokens
-// short tiles and sizes known at run time cost more than they save (115 -> 122 us at B = 32, T = 128): there
-// tiles are full and everything is constant.
+// Up to 64 tokens tiles are as tall as their examples, rounded up to 16 rows (kShort), and where that is less than half
+// of one a stage holds two or four of them, 64 columns each (kBoxes): a stage's hand-offs take 550 cycles whatever it
+// carries.  Where there is work enough a tile holds several examples (kPacked): the rows of a batch lie one after the
+// other, so 128 / T of them fill it, its Gram matrix has theirs on the diagonal, and the epilogue multiplies only those
+// blocks.  An example by itself has the plainer epilogue (a GPT-2-small block at B = 1, 2 and 4, T = 64 10.0, 10.8 and
+// 10.8 us with the other, 9.7, 10.3 and 10.3 with its own).  97 layers of d = 128 at B = 95, T = 17 115 -> 50 us, 49 at
+// B = 91, T = 39 70 -> 50; never so many examples that fewer than two items per SM remain (5 fp32 layers at B = 2, T =
+// 54: 7.7 -> 10.2 with both in one tile).  Above 64 tokens short tiles and sizes known at run time cost more than they
+// save (115 -> 122 us at B = 32, T = 128): there tiles are full and everything is constant.
 constexpr int kRingBytes = 12 * kTileBytes;
 constexpr int kMaxStages = 32;
 constexpr size_t kSmemBytes = kRingBytes + 1024 /*alignment slack*/ + 1024 /*barriers*/ + 4 * kTile * sizeof(float) /*row sums*/;

@@ -14,7 +14,7 @@
 // Everything is fp32 and in a fixed order.
 //
 // Bound by latency: launch, one round trip to memory, and the serial sums of a block.  Step of one 64 x 64 fp32 layer and a 1000-row
-// table at B = 4, T = 16: 30 -> 12.5 us, as a graph 22.6 -> 10.3 (12.4 without the early launch of the second kernel).
+// table at B = 4, T = 16: 30 -> 13 us, as a graph 22.6 -> 10.3 (12.4 without the early launch of the second kernel).
 #include <algorithm>
 #include <cstring>
 
@@ -467,15 +467,16 @@ int partials_per_example(const dp_step_desc& S) {
 
 }  // namespace
 
-// At most 512 tokens in sequences of at most 64, eight layers of at most 256 columns, a table of at most 2^20 values, and at most
-// as many Gram items, and output tiles, as there are SMs (the embedding items come on top).  Step of one 256 x 256 layer at 512 tokens, call by
-// call and as a graph: fp32 56 and 36 -> 27 and 29 us, bf16 48 and 33 -> 28 and 29; of four, fp32 61 and 39 -> 35 and 37, but bf16
-// 50 and 33 -> 36 and 37, hence the line.  bf16 steps, whose Gram products the general path takes on the tensor cores, also go there where
-// the norms' blocks fill an SM's shared memory and many are Gram items: two 256 x 256 layers at B = 64, T = 8 and a table of 256 columns (384 blocks of 66 KiB) 43
-// and 31 -> 35 and 37, three of 256 x 192 at B = 49, T = 10 (343 of 58) 44 and 33 -> 34 and 35, but with 64 table columns (192 of 66) 42
-// and 33 -> 24 and 27, and with one layer (64 Gram items of 320 blocks) 41 and 32 -> 25 and 27; fp32 ones were faster in all of these, both ways.  At the line bf16 graphs are even (two 256 x 256 layers at B = 12,
-// T = 42 and B = 16, T = 32: 32.5 and 30.0 -> 32.8 and 30.7) and calls a third faster.  Widths in whole words of four values, as
-// everything here is read.
+// At most 512 tokens in sequences of at most 64, eight layers of at most 256 columns, a table of at most 2^20 values, and at
+// most as many Gram items, and output tiles, as there are SMs (the embedding items come on top).  Step of one 256 x 256 layer
+// at 512 tokens, call by call and as a graph: fp32 56 and 36 -> 27 and 29 us, bf16 48 and 33 -> 28 and 29; of four, fp32 61 and
+// 39 -> 35 and 37, but bf16 50 and 33 -> 36 and 37, hence the line.  bf16 steps, whose Gram products the general path takes on
+// the tensor cores, also go there where the norms' blocks fill an SM's shared memory and many are Gram items: two 256 x 256
+// layers at B = 64, T = 8 and a table of 256 columns (384 blocks of 66 KiB) 43 and 31 -> 35 and 37, three of 256 x 192 at B =
+// 49, T = 10 (343 of 58) 44 and 33 -> 34 and 35, but with 64 table columns (192 of 66) 42 and 33 -> 24 and 27, and with one
+// layer (64 Gram items of 320 blocks) 41 and 32 -> 25 and 27; fp32 ones were faster in all of these, both ways.  At the line
+// bf16 graphs are even (two 256 x 256 layers at B = 12, T = 42 and B = 16, T = 32: 32.5 and 30.0 -> 32.8 and 30.7) and calls a
+// third faster.  Widths in whole words of four values, as everything here is read.
 bool small_step_fits(const dp_step_desc& S) {
   if (g_force_fma || S.tied || S.n_vectors || S.pos_ids || S.n_layers > kMaxLayers) return false;
   if (S.T > kMaxT || S.B > kMaxB || (long long)S.B * S.T > kMaxTokens) return false;
